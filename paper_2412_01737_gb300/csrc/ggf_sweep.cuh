@@ -10,77 +10,145 @@ constexpr int NWARP = 8;
 
 __device__ __forceinline__ double magc(cxd v) { return fabs(v.x) + fabs(v.y); }
 
-// warp argmax over lanes (ties: lowest index).  The result is taken from
-// lane 0 so that every lane follows the same pivot even when a NaN makes the
-// comparisons inconsistent (the callers branch on it around __syncwarp).
-__device__ __forceinline__ int warp_argmax(double v, int idx) {
-    for (int o = 16; o > 0; o >>= 1) {
-        double ov = __shfl_xor_sync(0xffffffffu, v, o);
-        int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+// ---- FP64 scalars of the link steps: double for the diagonal pairs, cxd for
+// the pairs n < m ----
+__device__ __forceinline__ double magc(double v) { return fabs(v); }
+__device__ __forceinline__ bool is_zero(double v) { return v == 0.0; }
+__device__ __forceinline__ bool is_zero(cxd v) { return v.x == 0.0 && v.y == 0.0; }
+__device__ __forceinline__ bool is_fin(double v) { return isfinite(v); }
+__device__ __forceinline__ bool is_fin(cxd v) { return isfinite(v.x) && isfinite(v.y); }
+__device__ __forceinline__ double recip(double v) { return 1.0 / v; }
+// one division where |v|^2 is well inside the range, Smith's method elsewhere
+__device__ __forceinline__ cxd recip(cxd v) {
+    const double m = v.x * v.x + v.y * v.y;
+    if (m > 1e-280 && m < 1e280) {
+        const double t = 1.0 / m;
+        return {v.x * t, -v.y * t};
     }
-    return __shfl_sync(0xffffffffu, idx, 0);
+    return cxd{1.0, 0.0} / v;
+}
+__device__ __forceinline__ void fmac(double& r, double a, double b) { r = fma(a, b, r); }
+__device__ __forceinline__ void fmac(cxd& r, cxd a, cxd b) {
+    r.x = fma(a.x, b.x, r.x); r.x = fma(-a.y, b.y, r.x);
+    r.y = fma(a.x, b.y, r.y); r.y = fma(a.y, b.x, r.y);
+}
+__device__ __forceinline__ void fmsc(double& r, double a, double b) { r = fma(-a, b, r); }
+__device__ __forceinline__ void fmsc(cxd& r, cxd a, cxd b) {
+    r.x = fma(-a.x, b.x, r.x); r.x = fma(a.y, b.y, r.x);
+    r.y = fma(-a.x, b.y, r.y); r.y = fma(-a.y, b.x, r.y);
+}
+__device__ __forceinline__ cxd to_c(double v) { return {v, 0.0}; }
+__device__ __forceinline__ cxd to_c(cxd v) { return v; }
+
+// Lane of the largest magnitude among the lanes that take part (ties: the
+// lowest lane), one warp, all lanes call: a redux over the upper words of the
+// FP64 magnitudes, and over the lower words where those tie, instead of five
+// shuffle rounds of three words (the search was a third of an elimination
+// step).  The result is the same in every lane, so that callers branch alike
+// whatever the values (NaN magnitudes order above all others).
+__device__ __forceinline__ int warp_pivot(double m, bool part) {
+    const unsigned hi = part ? (unsigned)__double2hiint(m) & 0x7fffffffu : 0u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, hi);
+    unsigned cand = __ballot_sync(0xffffffffu, part && hi == top);
+    if (__popc(cand) > 1) {
+        const bool in = (cand >> (threadIdx.x & 31)) & 1;
+        const unsigned lo = in ? (unsigned)__double2loint(m) : 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, lo);
+        cand = __ballot_sync(0xffffffffu, in && lo == best);
+    }
+    return __ffs(cand) - 1;
 }
 
-// Pfaffian of an n x n (n <= 32) antisymmetric matrix in shared memory, by one
-// warp (skew Gaussian elimination with pivoting).  A is destroyed.
-__device__ cxd warp_pfaffian(cxd* A, int n) {
+// Pfaffian of an n x n (n <= 16) antisymmetric matrix in shared memory, by one
+// warp (skew Gaussian elimination with pivoting).  A is destroyed.  An FP32
+// inverse is antisymmetric only to its rounding, and which of two mirrored
+// entries is read shows in the ratio: the multipliers come from the columns
+// below the pivot, as everywhere in this library.  The update itself is
+// antisymmetric, so each product is formed once for both triangles (12
+// instead of 16 FP64 instructions; the FP64 unit issues two lanes per clock
+// and SM), in three rounds of the warp at most.  Pairs are counted from the
+// last row, so that a lane's (row, column) offsets are the same at every step.
+template <class T>
+__device__ __forceinline__ T warp_pfaffian(T* A, int n) {
     const int lane = threadIdx.x & 31;
-    cxd res = {1.0, 0.0};
+    int pi[3], pj[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const int e = lane + 32 * t;
+        int i = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)e)) * 0.5f);
+        if (i * (i - 1) / 2 > e) --i;
+        if ((i + 1) * i / 2 <= e) ++i;
+        pi[t] = i;
+        pj[t] = e - i * (i - 1) / 2;
+    }
+    T res = Sc<T>::one();
     for (int k = 0; k < n - 1; k += 2) {
-        double m = (lane >= k + 1 && lane < n) ? magc(A[lane * n + k]) : -1.0;
-        int p = warp_argmax(m, lane);
         const int q = k + 1;
+        const bool part = lane > k && lane < n;
+        const int p = warp_pivot(part ? magc(A[lane * n + k]) : 0.0, part);
         if (p != q) {
             if (lane >= k && lane < n) {
-                cxd t = A[q * n + lane]; A[q * n + lane] = A[p * n + lane]; A[p * n + lane] = t;
+                const T t = A[q * n + lane]; A[q * n + lane] = A[p * n + lane]; A[p * n + lane] = t;
             }
             __syncwarp();
             if (lane >= k && lane < n) {
-                cxd t = A[lane * n + q]; A[lane * n + q] = A[lane * n + p]; A[lane * n + p] = t;
+                const T t = A[lane * n + q]; A[lane * n + q] = A[lane * n + p]; A[lane * n + p] = t;
             }
             __syncwarp();
             res = -res;
         }
-        cxd piv = A[q * n + k];
-        if (piv.x == 0.0 && piv.y == 0.0) { __syncwarp(); return {0.0, 0.0}; }
+        const T piv = A[q * n + k];
+        if (is_zero(piv)) { __syncwarp(); return Sc<T>::zero(); }
         res = res * A[k * n + q];
-        const cxd ipiv = cxd{1.0, 0.0} / piv;
-        int mm = n - k - 2;
+        if (k + 2 >= n) break;
+        const T ip = recip(piv);
         // multipliers l_i = A[i][k] / A[q][k], one per row, in column k
         // (column k is not read again)
-        if (lane < mm) A[(k + 2 + lane) * n + k] = A[(k + 2 + lane) * n + k] * ipiv;
+        if (lane > q && lane < n) A[lane * n + k] = A[lane * n + k] * ip;
         __syncwarp();
-        for (int e = lane; e < mm * mm; e += 32) {
-            int i = k + 2 + e / mm, j = k + 2 + e % mm;
-            A[i * n + j] += A[i * n + k] * A[j * n + q] - A[i * n + q] * A[j * n + k];
+        const int mm = n - k - 2, cnt = mm * (mm - 1) / 2;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            if (32 * t >= cnt) break;
+            if (lane + 32 * t < cnt) {
+                const int i = n - 1 - pi[t], j = n - 1 - pj[t];
+                T u = A[i * n + k] * A[j * n + q];
+                fmsc(u, A[i * n + q], A[j * n + k]);
+                A[i * n + j] += u;
+                A[j * n + i] -= u;
+            }
         }
         __syncwarp();
     }
+    __syncwarp();
     return res;
 }
 
 // Solve [A | B] (r x 2r, row-major, stride 2r) in place by Gauss-Jordan with
-// partial pivoting; the right half becomes A^{-1} B.  fcol: r scratch.
-__device__ bool warp_solve(cxd* A, int r, cxd* fcol) {
+// partial pivoting; the right half becomes A^{-1} B (columns up to the pivot
+// are not read again and keep their values).  fcol: r scratch.
+template <class T>
+__device__ __forceinline__ bool warp_solve(T* A, int r, T* fcol) {
     const int lane = threadIdx.x & 31;
     const int w = 2 * r;
     for (int k = 0; k < r; ++k) {
-        double m = (lane >= k && lane < r) ? magc(A[lane * w + k]) : -1.0;
-        int p = warp_argmax(m, lane);
+        const bool part = lane >= k && lane < r;
+        const int p = warp_pivot(part ? magc(A[lane * w + k]) : 0.0, part);
         if (p != k) {
-            if (lane < w) { cxd t = A[k * w + lane]; A[k * w + lane] = A[p * w + lane]; A[p * w + lane] = t; }
+            if (lane < w) { T t = A[k * w + lane]; A[k * w + lane] = A[p * w + lane]; A[p * w + lane] = t; }
             __syncwarp();
         }
-        cxd d = A[k * w + k];
-        if (d.x == 0.0 && d.y == 0.0) return false;
+        const T d = A[k * w + k];
+        if (is_zero(d)) return false;
+        const T id = recip(d);
         __syncwarp();
-        if (lane < w) A[k * w + lane] = A[k * w + lane] / d;
+        if (lane > k && lane < w) A[k * w + lane] = A[k * w + lane] * id;
         if (lane < r) fcol[lane] = A[lane * w + k];
         __syncwarp();
-        for (int e = lane; e < r * w; e += 32) {
-            int i = e / w, j = e % w;
-            if (i != k) A[i * w + j] -= fcol[i] * A[k * w + j];
+        const int cols = w - k - 1;
+        for (int e = lane; e < r * cols; e += 32) {
+            const int i = e / cols, j = k + 1 + e % cols;
+            if (i != k) fmsc(A[i * w + j], fcol[i], A[k * w + j]);
         }
         __syncwarp();
     }
@@ -236,21 +304,21 @@ __device__ __forceinline__ void twist_table(const Geometry& g, const Proposal& q
 
 // Pf(M') / Pf(M) = Pf([[Delta, -1], [1, W_SS]]) (r/2 = 2 n_v even: no extra
 // sign), one warp; Bw is 2r x 2r scratch.
-__device__ __forceinline__ cxd bordered_ratio(const cxd* D, const cxd* Ws, cxd* Bw, int r) {
+template <class T>
+__device__ __forceinline__ T bordered_ratio(const T* D, const T* Ws, T* Bw, int r) {
     const int lane = threadIdx.x & 31, n2 = 2 * r;
     // a non-finite block (an inverse that overflowed) gives ratio 0: the
     // proposal is rejected
     bool fin = true;
-    for (int e = lane; e < r * r; e += 32)
-        fin = fin && isfinite(Ws[e].x) && isfinite(Ws[e].y) && isfinite(D[e].x) && isfinite(D[e].y);
-    if (!__all_sync(0xffffffffu, fin)) return {0.0, 0.0};
+    for (int e = lane; e < r * r; e += 32) fin = fin && is_fin(Ws[e]) && is_fin(D[e]);
+    if (!__all_sync(0xffffffffu, fin)) return Sc<T>::zero();
     for (int e = lane; e < n2 * n2; e += 32) {
         int i = e / n2, j = e % n2;
-        cxd v = {0.0, 0.0};
+        T v = Sc<T>::zero();
         if (i < r && j < r) v = D[i * r + j];
         else if (i >= r && j >= r) v = Ws[(i - r) * r + (j - r)];
-        else if (i < r && j == i + r) v = {-1.0, 0.0};
-        else if (i >= r && j == i - r) v = {1.0, 0.0};
+        else if (i < r && j == i + r) v = -Sc<T>::one();
+        else if (i >= r && j == i - r) v = Sc<T>::one();
         Bw[e] = v;
     }
     __syncwarp();
@@ -309,22 +377,23 @@ __device__ __forceinline__ void combine_pairs(const DevConst& dc, const cxd* ell
 
 // Z = (1 + Delta W_SS)^{-1} Delta (r x r) into Zout, one warp; Aug is r x 2r
 // scratch, fcol r.  Returns false for a singular system.
-__device__ __forceinline__ bool pair_z(const cxd* D, const cxd* Ws, cxd* Aug, cxd* fcol, int r, cxd* Zout) {
+template <class T, class Z>
+__device__ __forceinline__ bool pair_z(const T* D, const T* Ws, T* Aug, T* fcol, int r, Z* Zout) {
     const int lane = threadIdx.x & 31, w2 = 2 * r;
-    for (int e = lane; e < r * w2; e += 32) {
-        int i = e / w2, j = e % w2;
-        cxd v;
-        if (j < r) {
-            v = {i == j ? 1.0 : 0.0, 0.0};
-            for (int z = 0; z < r; ++z) v += D[i * r + z] * Ws[z * r + j];
-        } else {
-            v = D[i * r + (j - r)];
-        }
-        Aug[e] = v;
+    for (int e = lane; e < r * r; e += 32) {
+        const int i = e / r, j = e % r;
+        T v = i == j ? Sc<T>::one() : Sc<T>::zero();
+        for (int z = 0; z < r; ++z) fmac(v, D[i * r + z], Ws[z * r + j]);
+        Aug[i * w2 + j] = v;
+        Aug[i * w2 + r + j] = D[e];
     }
     __syncwarp();
     const bool ok = warp_solve(Aug, r, fcol);
-    for (int e = lane; e < r * r; e += 32) Zout[e] = Aug[(e / r) * w2 + r + e % r];
+    for (int e = lane; e < r * r; e += 32) {
+        const T v = Aug[(e / r) * w2 + r + e % r];
+        if constexpr (sizeof(Z) == sizeof(T)) Zout[e] = v;
+        else Zout[e] = to_c(v);
+    }
     __syncwarp();
     return ok;
 }

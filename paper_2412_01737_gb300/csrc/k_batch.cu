@@ -8,11 +8,11 @@
 // j r + xi of T is Majorana xi of link l0 + j).  Every proposal of the batch
 // needs only the block of the current inverse on T.  With W the inverse at
 // the start of the batch, C = W[:, T], Y = W[T, :], G0 = W[T, T]:
-//   batch_gather  C -> U panel, Y^T -> V^T panel, G := G0, X := 0 (C read as
+//   batch_gather  C -> U panel, Y^T -> V^T panel, G := G0 (C read as
 //                 the true columns: -Y^T, equal in exact arithmetic, makes
 //                 the rounding error grow geometrically)
-//   batch_steps   one CTA per chain runs the kb link steps on the small
-//                 matrices: ratio from G[S_j, S_j], decision, and on accept,
+//   batch_steps   one cluster per chain (k_steps.cu) runs the kb link steps on
+//                 the small matrices, from X = 0: ratio from G[S_j, S_j], decision, and on accept,
 //                 with Z = (1 + Delta G[S, S])^{-1} Delta,
 //                   G[F, F] -= G[F, S] Z G[S, F]   (F: the later links' rows)
 //                   X       += P Z Q,  P = E_S - X G0[:, S],
@@ -37,7 +37,7 @@ namespace {
 // ---- gather -------------------------------------------------------------------
 // Grid (ceil(N / BR), family pairs, chains), 256 threads.  Rows i0 .. i0+BR-1
 // of the U panel (C = W[:, T]) and of the V^T panel (Y^T = W[T, :]^T); the
-// rows of G := W[T, T] whose T index falls in the block; X := 0 there.
+// rows of G := W[T, T] whose T index falls in the block.
 template <class T>
 __global__ void __launch_bounds__(256) batch_gather(Geometry g, int l0, int kb, int fam_pairs, int KRM, int BR,
                                                     const T* W, typename Sc<T>::R* Pan, T* Sm) {
@@ -59,7 +59,6 @@ __global__ void __launch_bounds__(256) batch_gather(Geometry g, int l0, int kb, 
     RR* U = Pan + base * 2 * PanelIO<T>::PLANES * NK;
     RR* Vt = U + PanelIO<T>::PLANES * NK;
     T* Gm = Sm + base * 2 * KRM * KRM;
-    T* Xm = Gm + (size_t)KRM * KRM;
     // V^T rows: tile[ii][q] = W[T_q][i0 + ii], read along rows of W
     for (int e = threadIdx.x; e < kr * BR; e += blockDim.x) {
         int q = e / BR, ii = e - q * BR;
@@ -87,242 +86,8 @@ __global__ void __launch_bounds__(256) batch_gather(Geometry g, int l0, int kb, 
         if (ii < 0 || ii >= nb) continue;
         for (int q = lane; q < kr; q += 32) {
             Gm[(size_t)a * KRM + q] = tile[ii * ld + q];   // W[T_a][T_q] = U[T_a][q]
-            Xm[(size_t)a * KRM + q] = Sc<T>::zero();
         }
     }
-}
-
-// ---- link steps on the small matrices ----------------------------------------
-struct BatchArgs {
-    DevConst dc;
-    const unsigned long long* d_sweep;
-    int l0, kb, KRM;
-    uint64_t seed;
-    uint64_t coff;         // Philox key word 1 = coff + chain
-    double width;
-    void* links;
-    cxd* ell;
-    int* since_refresh;
-    int* sweep_acc;
-    unsigned long long* counters;
-    int* pend;
-    const void* Pr;   // U panels: G0 = U[T, 0 .. kr)
-    const void* Pc;
-    void* Sr;         // small matrices [n][K][2][KRM][KRM]: G then X
-    void* Sc_;        // [n][Kc][2][KRM][KRM]
-};
-
-// Rank-r update of one pair's small matrices after link j of the batch was
-// accepted (all threads of the CTA).  Gm, Xm: KRM x KRM; U: the pair's U
-// panel (planes of N x KRM); Z: r x r (FP64); st: 4 KRM r scratch scalars.
-template <class T, int r>
-__device__ __forceinline__ void small_update(T* Gm, T* Xm, const typename Sc<T>::R* U, size_t NK, int NP,
-                                             const int* Tl, int j, int kb, int KRM, const cxd* Z, T* st) {
-    const int jr = j * r, m = jr + r, kr = kb * r, nf = kr - m;
-    T* A1 = st;                    // G[F, S] Z, later G0[0:jr, S], later P Z
-    T* A2 = A1 + (size_t)KRM * r;  // G[S, F], later G0[S, 0:jr]
-    T* A3 = A2 + (size_t)KRM * r;  // P  (m x r)
-    T* A4 = A3 + (size_t)KRM * r;  // Q  (r x m)
-    // (a) later links: G[F, F] -= (G[F, S] Z) G[S, F]
-    if (nf > 0) {
-        for (int e = threadIdx.x; e < nf * r; e += blockDim.x) {
-            int i = e / r, b = e - i * r;
-            T acc = Sc<T>::zero();
-            for (int a = 0; a < r; ++a) acc += Gm[(size_t)(m + i) * KRM + jr + a] * Sc<T>::from(Z[a * r + b]);
-            A1[e] = acc;
-        }
-        for (int e = threadIdx.x; e < r * nf; e += blockDim.x) {
-            int b = e / nf, jj = e - b * nf;
-            A2[e] = Gm[(size_t)(jr + b) * KRM + m + jj];
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) {
-            int i = e / nf, jj = e - i * nf;
-            T* gp = Gm + (size_t)(m + i) * KRM + m + jj;
-            T acc = *gp;
-            for (int b = 0; b < r; ++b) acc -= A1[i * r + b] * A2[b * nf + jj];
-            *gp = acc;
-        }
-        __syncthreads();
-    }
-    // (b) X += P Z Q on the leading m x m block
-    for (int e = threadIdx.x; e < jr * r; e += blockDim.x) {
-        int a = e / r, b = e - a * r;
-        A1[e] = PanelIO<T>::ld(U, NK, pidx(Tl[a], jr + b, NP));        // G0[a][S_b]
-        A2[b * jr + a] = PanelIO<T>::ld(U, NK, pidx(Tl[jr + b], a, NP));   // G0[S_b][a]
-    }
-    __syncthreads();
-    // P (m x r): rows a < jr are -X[a, 0:jr] G0[0:jr, S], rows jr.. the identity;
-    // Q (r x m): columns cc < jr are -G0[S, 0:jr] X[0:jr, cc], then the identity.
-    // One thread per row a of P (resp. column cc of Q) keeps its r outputs in
-    // registers, so every element of X is loaded once per product.
-    const T one = Sc<T>::from(cxd{1.0, 0.0});
-    for (int a = threadIdx.x; a < m; a += blockDim.x) {
-        T acc[r];
-#pragma unroll
-        for (int b = 0; b < r; ++b) acc[b] = Sc<T>::zero();
-        if (a < jr) {
-            const T* xr = Xm + (size_t)a * KRM;
-            for (int q = 0; q < jr; ++q) {
-                const T x = xr[q];
-#pragma unroll
-                for (int b = 0; b < r; ++b) acc[b] -= x * A1[q * r + b];
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < r; ++b) A3[a * r + b] = (a >= jr && b == a - jr) ? one : acc[b];
-    }
-    for (int cc = threadIdx.x; cc < m; cc += blockDim.x) {
-        T acc[r];
-#pragma unroll
-        for (int b = 0; b < r; ++b) acc[b] = Sc<T>::zero();
-        if (cc < jr) {
-            for (int q = 0; q < jr; ++q) {
-                const T x = Xm[(size_t)q * KRM + cc];
-#pragma unroll
-                for (int b = 0; b < r; ++b) acc[b] -= A2[b * jr + q] * x;
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < r; ++b) A4[b * m + cc] = (cc >= jr && b == cc - jr) ? one : acc[b];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < m * r; e += blockDim.x) {
-        int a = e / r, b = e - a * r;
-        T acc = Sc<T>::zero();
-        for (int q = 0; q < r; ++q) acc += A3[a * r + q] * Sc<T>::from(Z[q * r + b]);
-        A1[e] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int a = e / m, cc = e - a * m;
-        T* xp = Xm + (size_t)a * KRM + cc;
-        T acc = *xp;
-        for (int b = 0; b < r; ++b) acc += A1[a * r + b] * A4[b * m + cc];
-        *xp = acc;
-    }
-    __syncthreads();
-}
-
-// One CTA (NWARP warps) per chain runs the batch's kb link steps in order.
-// SU2: SU(2) links (quaternion proposal and doublet twist); the Z2 and U(1)
-// instantiations (SU2 = false) do not contain that code.
-template <class RW, class CW, bool SU2>
-__global__ void __launch_bounds__(NWARP * 32, 2) batch_steps(BatchArgs a) {
-    extern __shared__ cxd sm[];
-    const Geometry& g = a.dc.g;
-    const int P = a.dc.P, K = a.dc.K, Kc = P - K, r = g.r, N = g.N, KRM = a.KRM;
-    const int c = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the ratio phase's arrays and the update scratch share the front of
-    // shared memory; Z and the T list follow
-    const size_t front_ratio = (size_t)(2 * P * r * r + NWARP * 4 * r * r + P + NWARP * r);
-    const size_t front_upd = (4 * (size_t)KRM * r * sizeof(CW) + sizeof(cxd) - 1) / sizeof(cxd);
-    const size_t front = front_ratio > front_upd ? front_ratio : front_upd;
-    cxd* Delta = sm;                       // [P][r][r]
-    cxd* Wss = Delta + P * r * r;          // [P][r][r]
-    cxd* Bord = Wss + P * r * r;           // [NWARP][2r][2r]
-    cxd* rho = Bord + NWARP * 4 * r * r;   // [P]
-    cxd* fcol = rho + P;                   // [NWARP][r]
-    cxd* Zs = sm + front;                  // [P][r][r]
-    int* Tl = (int*)(Zs + P * r * r);      // [kb r]
-    __shared__ Proposal s_q;
-    __shared__ double s_cs[8];
-    __shared__ double s_su2[36];          // SU2: new quaternion, old and new doublet rotations
-    __shared__ int s_accept, s_any;
-    typedef typename Sc<RW>::R RR;
-    const size_t NK = panel_plane(N, KRM), SS = (size_t)KRM * KRM;
-    const int NP = panel_rows(N);
-    const int kr = a.kb * r;
-    for (int q = threadIdx.x; q < kr; q += blockDim.x) {
-        int a0, b0;
-        link_ends(g, a.l0 + q / r, a0, b0);
-        Tl[q] = link_majorana(g, a0, b0, q % r);
-    }
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    const unsigned long long sweep = *a.d_sweep;
-
-    for (int j = 0; j < a.kb; ++j) {
-        const int l = a.l0 + j, jr = j * r;
-        if constexpr (SU2) {
-            if (threadIdx.x == 0) {
-                Proposal qq{};
-                qq.u_acc = draw_su2(g, a.links, c, l, sweep, a.seed, a.width, s_su2, s_su2 + 4, s_su2 + 20,
-                                   a.coff);
-                s_q = qq;
-            }
-        } else {
-            if (threadIdx.x == 0) s_q = draw_proposal(g, a.links, c, l, sweep, a.seed, a.width, a.coff);
-        }
-        __syncthreads();
-        const Proposal q = s_q;
-        if constexpr (!SU2) twist_table(g, q, s_cs);
-        __syncthreads();
-        for (int p = warp; p < P; p += NWARP) {
-            cxd* D = Delta + p * r * r;
-            cxd* Ws = Wss + p * r * r;
-            if constexpr (SU2) pair_delta_su2(a.dc, p, l, s_su2 + 4, s_su2 + 20, D);
-            else pair_delta(a.dc, p, l, q, s_cs, D);
-            for (int e = lane; e < r * r; e += 32) {
-                const size_t off = (size_t)(jr + e / r) * KRM + jr + e % r;
-                if (p < K) Ws[e] = loadc((const RW*)a.Sr + ((size_t)c * K + p) * 2 * SS + off);
-                else Ws[e] = loadc((const CW*)a.Sc_ + ((size_t)c * Kc + (p - K)) * 2 * SS + off);
-            }
-            __syncwarp();
-            cxd pf = bordered_ratio(D, Ws, Bord + warp * 4 * r * r, r);
-            if (lane == 0) rho[p] = pf;
-            __syncwarp();
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sn, so;
-            combine_pairs(a.dc, a.ell + (size_t)c * P, rho, sn, so);
-            const int acc = (sn > 0.0 && so > 0.0 && q.u_acc < sn / so) ? 1 : 0;
-            atomicAdd(&a.counters[0], 1ULL);
-            s_accept = acc;
-            if (acc) {
-                s_any = 1;
-                atomicAdd(&a.counters[1], 1ULL);
-                a.since_refresh[c] += 1;
-                a.sweep_acc[c] += 1;
-                if constexpr (SU2) {
-                    double* dst = (double*)a.links + ((size_t)c * g.n_links + l) * 4;
-                    for (int k = 0; k < 4; ++k) dst[k] = s_su2[k];
-                } else {
-                    if (g.group == GGF_Z2) ((int8_t*)a.links)[(size_t)c * g.n_links + l] = (int8_t)q.g_new;
-                    else ((double*)a.links)[(size_t)c * g.n_links + l] = q.th_new;
-                }
-            }
-        }
-        __syncthreads();
-        if (!s_accept) continue;
-        for (int p = warp; p < P; p += NWARP) {
-            pair_z(Delta + p * r * r, Wss + p * r * r, Bord + warp * 4 * r * r, fcol + warp * r, r, Zs + p * r * r);
-            if (lane == 0) ell_add(a.ell[(size_t)c * P + p], rho[p], p < K);
-            __syncwarp();
-        }
-        __syncthreads();
-        for (int p = 0; p < K; ++p) {
-            RW* Gm = (RW*)a.Sr + ((size_t)c * K + p) * 2 * SS;
-            const RR* U = (const RR*)a.Pr + ((size_t)c * K + p) * 2 * PanelIO<RW>::PLANES * NK;
-            if (r == 4) small_update<RW, 4>(Gm, Gm + SS, U, NK, NP, Tl, j, a.kb, KRM, Zs + p * r * r, (RW*)sm);
-            else small_update<RW, 8>(Gm, Gm + SS, U, NK, NP, Tl, j, a.kb, KRM, Zs + p * r * r, (RW*)sm);
-        }
-        for (int p = 0; p < Kc; ++p) {
-            CW* Gm = (CW*)a.Sc_ + ((size_t)c * Kc + p) * 2 * SS;
-            const RR* U = (const RR*)a.Pc + ((size_t)c * Kc + p) * 2 * PanelIO<CW>::PLANES * NK;
-            if (r == 4) small_update<CW, 4>(Gm, Gm + SS, U, NK, NP, Tl, j, a.kb, KRM, Zs + (K + p) * r * r, (CW*)sm);
-            else small_update<CW, 8>(Gm, Gm + SS, U, NK, NP, Tl, j, a.kb, KRM, Zs + (K + p) * r * r, (CW*)sm);
-        }
-    }
-    if (threadIdx.x == 0) a.pend[c] = s_any ? a.kb : 0;
-}
-
-size_t steps_smem(int P, int r, int KRM, size_t cw_bytes) {
-    size_t front = std::max((size_t)(2 * P * r * r + NWARP * 4 * r * r + P + NWARP * r),
-                            (4 * (size_t)KRM * r * cw_bytes + sizeof(cxd) - 1) / sizeof(cxd));
-    return (front + (size_t)P * r * r) * sizeof(cxd) + (size_t)KRM * sizeof(int);
 }
 
 // ---- V^T <- V^T X^T -----------------------------------------------------------
@@ -424,6 +189,9 @@ int gather_rows(int kr, size_t tb) {
 }  // namespace
 
 ggf_status ggf_flush(ggf_ctx* ctx, cudaStream_t st);
+ggf_status ggf_prepare_steps(ggf_ctx* ctx);
+bool ggf_steps_fit(ggf_ctx* ctx, int kmax, bool fp64);
+ggf_status ggf_batch_steps(ggf_ctx* ctx, int l0, int kb, void* Sr, void* Sc_, cudaStream_t st);
 ggf_status ggf_apply_tc(ggf_ctx* ctx, bool cplx, int fam_pairs, int kr, float* Pan, const float* Sm, cudaStream_t st);
 
 // Shared-memory caps of the batch kernels (once per device, like the other
@@ -443,10 +211,7 @@ ggf_status ggf_prepare_batch(ggf_ctx* ctx) {
     GGF_TRY(cap((const void*)batch_gather<float>));
     GGF_TRY(cap((const void*)batch_gather<cxd>));
     GGF_TRY(cap((const void*)batch_gather<cxf>));
-    GGF_TRY(cap((const void*)batch_steps<double, cxd, false>));
-    GGF_TRY(cap((const void*)batch_steps<float, cxf, false>));
-    GGF_TRY(cap((const void*)batch_steps<double, cxd, true>));
-    GGF_TRY(cap((const void*)batch_steps<float, cxf, true>));
+    GGF_TRY(ggf_prepare_steps(ctx));
     GGF_TRY(cap((const void*)batch_apply<double, 4>));
     GGF_TRY(cap((const void*)batch_apply<float, 4>));
     GGF_TRY(cap((const void*)batch_apply<cxd, 4>));
@@ -466,9 +231,8 @@ ggf_status ggf_check_batch(ggf_ctx* ctx, int kmax, bool fp64) {
     GGF_CK(cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     const int r = ctx->g.r, KRM = kmax * r;
     const size_t cw = fp64 ? sizeof(cxd) : sizeof(cxf);
-    const size_t need_steps = steps_smem(ctx->P, r, KRM, cw) + 1024;
     const size_t need_apply = apply_smem(2, KRM, cw) + 1024;
-    if (need_steps > (size_t)mx || need_apply > (size_t)mx)
+    if (!ggf_steps_fit(ctx, kmax, fp64) || need_apply > (size_t)mx)
         return ggf_fail(ctx, GGF_EINVAL, "delay too large: batch kernels need more shared memory than the device has");
     return GGF_OK;
 }
@@ -506,36 +270,7 @@ ggf_status ggf_batch(ggf_ctx* ctx, int l0, int kb, cudaStream_t st) {
     }
     const int ev1 = ctx->prof_mark(st);
     ctx->prof_pair(GGF_KT_GATHER, ev0, ev1);
-    {
-        BatchArgs a;
-        a.dc = ctx->dc();
-        a.d_sweep = ch.d_sweep;
-        a.l0 = l0;
-        a.kb = kb;
-        a.KRM = KRM;
-        a.seed = ch.opts.seed;
-        a.coff = ch.opts.chain_offset;
-        a.width = ch.opts.width;
-        a.links = ch.links;
-        a.ell = ch.ell;
-        a.since_refresh = ch.since_refresh;
-        a.sweep_acc = ch.sweep_acc;
-        a.counters = ch.counters;
-        a.pend = ch.pend;
-        a.Pr = ch.Pr;
-        a.Pc = ch.Pc;
-        a.Sr = Sr;
-        a.Sc_ = Sc_;
-        const size_t smem = steps_smem(ctx->P, r, KRM, fp64 ? sizeof(cxd) : sizeof(cxf));
-        if (g.group == GGF_SU2) {
-            if (fp64) batch_steps<double, cxd, true><<<ch.n, NWARP * 32, smem, st>>>(a);
-            else batch_steps<float, cxf, true><<<ch.n, NWARP * 32, smem, st>>>(a);
-        } else {
-            if (fp64) batch_steps<double, cxd, false><<<ch.n, NWARP * 32, smem, st>>>(a);
-            else batch_steps<float, cxf, false><<<ch.n, NWARP * 32, smem, st>>>(a);
-        }
-        GGF_CK(cudaGetLastError());
-    }
+    GGF_TRY(ggf_batch_steps(ctx, l0, kb, Sr, Sc_, st));
     const int ev2 = ctx->prof_mark(st);
     ctx->prof_pair(GGF_KT_RATIO, ev1, ev2);
     {
