@@ -114,22 +114,10 @@ size_t budget_bytes() {
     return std::max<size_t>(std::min(cap, fr / 2), (size_t)64 << 20);
 }
 
-// logpf/phase of dense refactorisations back to their item positions
-__global__ void scatter_pf_kernel(int n, const int* idx, const cxd* lp, const cxd* ph, cxd* logpf, cxd* phase) {
+// log-weights of dense refactorisations to their places: item i -> ell[at[i]]
+__global__ void scatter_pf_kernel(int n, const int* at, bool cplx, const cxd* lp, const cxd* ph, cxd* ell) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    logpf[idx[i]] = lp[i];
-    phase[idx[i]] = ph[i];
-}
-
-// ell[cfg][pair_off + pair] of items with explicit (cfg, pair)
-__global__ void write_items_kernel(int n_items, const int* cfg, const int* pair, int pair_off, int P, bool cplx,
-                                   const cxd* logpf, const cxd* phase, cxd* ell) {
-    int it = blockIdx.x * blockDim.x + threadIdx.x;
-    if (it >= n_items) return;
-    cxd v = {logpf[it].x, 0.0};
-    if (cplx) v.y = atan2(phase[it].y, phase[it].x);
-    ell[(size_t)cfg[it] * P + pair_off + pair[it]] = v;
+    if (i < n) ell[at[i]] = {lp[i].x, cplx ? atan2(ph[i].y, ph[i].x) : 0.0};
 }
 
 // W[chain][p] <- convert(A[item]) and log-weight bookkeeping after a factorisation
@@ -145,83 +133,78 @@ __global__ void scatter_kernel(int N, int fam_pairs, const int* item_chain, cons
     W[((size_t)c * fam_pairs + p) * NN + e] = Sc<TD>::from(v);
 }
 
-// log Pf(M_nm(G)) of explicit (configuration, pair-within-family) items
-// (host lists hc, hp) into d_logpf / d_phase, by the site-by-site FP64
-// elimination; items whose closed sets had no usable pivot are refactored by
-// the dense FP64 Parlett-Reid Pfaffian.  d_cfg, d_pair, d_flag hold
-// hc.size() entries (overwritten).
-ggf_status pf_items(ggf_ctx* ctx, bool cplx, const std::vector<int>& hc, const std::vector<int>& hp,
-                    const void* d_links, int* d_cfg, int* d_pair, int* d_flag, cxd* d_logpf, cxd* d_phase,
-                    cudaStream_t st) {
-    const int items = (int)hc.size();
-    if (items == 0) return GGF_OK;
+// log Pf(M_nm(G)) of every pair of n configurations (d_chains[q], or q; h_chains
+// the same list on the host) into *ell [n][P], in the context's own buffer, by
+// the site-by-site FP64 elimination.  `then` is queued behind it and may run
+// again: items whose closed sets had no usable pivot are refactored by the
+// dense FP64 Parlett-Reid Pfaffian afterwards.  Synchronises the stream.
+template <class Then>
+ggf_status log_pfaffians(ggf_ctx* ctx, int n, const int* d_chains, const std::vector<int>* h_chains,
+                         const void* d_links, cudaStream_t st, Then then) {
+    const int P = ctx->P, K = ctx->K;
+    const size_t total = (size_t)n * P, eb = (total * sizeof(cxd) + 255) / 256 * 256;
+    const size_t need = eb + (total + 1) * sizeof(int);
+    if (need > ctx->lw_bytes) {
+        if (ctx->lw) cudaFree(ctx->lw);
+        ctx->lw = nullptr;
+        ctx->lw_bytes = 0;
+        GGF_CK(cudaMalloc(&ctx->lw, need));
+        ctx->lw_bytes = need;
+    }
+    cxd* ell = (cxd*)ctx->lw;
+    int* d_bad = (int*)((unsigned char*)ctx->lw + eb);
+    GGF_TRY(ggf_front_pfaffian(ctx, n, d_chains, d_links, ell, d_bad, st));
+    GGF_TRY(then(ell));
+    int nbad = 0;
+    GGF_CK(cudaMemcpyAsync(&nbad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    GGF_CK(cudaStreamSynchronize(st));
+    if (nbad == 0) return GGF_OK;
+    ctx->dense_pfaffians += nbad;
+    std::vector<int> list(nbad);
+    GGF_CK(cudaMemcpy(list.data(), d_bad + 1, nbad * sizeof(int), cudaMemcpyDeviceToHost));
+    std::sort(list.begin(), list.end());
     const int N = ctx->g.N;
     const size_t NN = (size_t)N * N;
-    GGF_CK(cudaMemcpyAsync(d_cfg, hc.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-    GGF_CK(cudaMemcpyAsync(d_pair, hp.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-    GGF_TRY(ggf_front_pfaffian(ctx, cplx, items, d_cfg, d_pair, d_links, d_logpf, d_phase, d_flag, st));
-    std::vector<int> hf(items);
-    GGF_CK(cudaMemcpyAsync(hf.data(), d_flag, items * sizeof(int), cudaMemcpyDeviceToHost, st));
+    for (int fam = 0; fam < 2; ++fam) {
+        const bool cplx = fam == 1;
+        const size_t elem = cplx ? sizeof(cxd) : sizeof(double);
+        std::vector<int> at, fc, fp;
+        for (int i : list) {
+            const int q = i / P, p = i % P;
+            if ((p >= K) != cplx) continue;
+            at.push_back(i);
+            fc.push_back(h_chains ? (*h_chains)[q] : q);
+            fp.push_back(cplx ? p - K : p);
+        }
+        const int nf = (int)at.size();
+        if (nf == 0) continue;
+        const int per = (int)std::max<size_t>(1, std::min<size_t>(nf, budget_bytes() / (NN * elem)));
+        const size_t tmp = ggf_factor_tmp_bytes(N, per);
+        GGF_TRY(ggf_workspace(ctx, NN * elem * per + tmp + (size_t)per * (3 * sizeof(int) + 2 * sizeof(cxd)) + 1024));
+        unsigned char* q = (unsigned char*)ctx->work;
+        void* A = q;
+        q += (NN * elem * per + 255) / 256 * 256;
+        void* ftmp = q;
+        q += (tmp + 255) / 256 * 256;
+        cxd* f_logpf = (cxd*)q; q += (size_t)per * sizeof(cxd);
+        cxd* f_phase = (cxd*)q; q += (size_t)per * sizeof(cxd);
+        int* f_cfg = (int*)q; q += (size_t)per * sizeof(int);
+        int* f_pair = (int*)q; q += (size_t)per * sizeof(int);
+        int* f_at = (int*)q;
+        for (int f0 = 0; f0 < nf; f0 += per) {
+            const int nb = std::min(per, nf - f0);
+            GGF_CK(cudaMemcpyAsync(f_cfg, fc.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
+            GGF_CK(cudaMemcpyAsync(f_pair, fp.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
+            GGF_CK(cudaMemcpyAsync(f_at, at.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
+            GGF_TRY(ggf_assemble(ctx, !cplx, nb, f_cfg, f_pair, d_links, A, st));
+            GGF_TRY(ggf_pfaffian_batched(ctx, cplx, N, nb, A, f_logpf, f_phase, ftmp, st));
+            scatter_pf_kernel<<<(nb + 127) / 128, 128, 0, st>>>(nb, f_at, cplx, f_logpf, f_phase, ell);
+            GGF_CK(cudaGetLastError());
+            GGF_CK(cudaStreamSynchronize(st));
+        }
+    }
+    GGF_TRY(then(ell));
     GGF_CK(cudaStreamSynchronize(st));
-    std::vector<int> fi, fc, fp;
-    for (int i = 0; i < items; ++i)
-        if (hf[i]) { fi.push_back(i); fc.push_back(hc[i]); fp.push_back(hp[i]); }
-    ctx->dense_pfaffians += fi.size();
-    if (fi.empty()) return GGF_OK;
-    const size_t elem = cplx ? sizeof(cxd) : sizeof(double);
-    const int nf = (int)fi.size();
-    const int per = (int)std::max<size_t>(1, std::min<size_t>(nf, budget_bytes() / (NN * elem)));
-    const size_t tmp = ggf_factor_tmp_bytes(N, per);
-    GGF_TRY(ggf_workspace(ctx, NN * elem * per + tmp + (size_t)per * (3 * sizeof(int) + 2 * sizeof(cxd)) + 1024));
-    unsigned char* q = (unsigned char*)ctx->work;
-    void* A = q;
-    q += (NN * elem * per + 255) / 256 * 256;
-    void* ftmp = q;
-    q += (tmp + 255) / 256 * 256;
-    cxd* f_logpf = (cxd*)q; q += (size_t)per * sizeof(cxd);
-    cxd* f_phase = (cxd*)q; q += (size_t)per * sizeof(cxd);
-    int* f_cfg = (int*)q; q += (size_t)per * sizeof(int);
-    int* f_pair = (int*)q; q += (size_t)per * sizeof(int);
-    int* f_idx = (int*)q;
-    for (int f0 = 0; f0 < nf; f0 += per) {
-        const int nb = std::min(per, nf - f0);
-        GGF_CK(cudaMemcpyAsync(f_cfg, fc.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
-        GGF_CK(cudaMemcpyAsync(f_pair, fp.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
-        GGF_CK(cudaMemcpyAsync(f_idx, fi.data() + f0, nb * sizeof(int), cudaMemcpyHostToDevice, st));
-        GGF_TRY(ggf_assemble(ctx, !cplx, nb, f_cfg, f_pair, d_links, A, st));
-        GGF_TRY(ggf_pfaffian_batched(ctx, cplx, N, nb, A, f_logpf, f_phase, ftmp, st));
-        scatter_pf_kernel<<<(nb + 127) / 128, 128, 0, st>>>(nb, f_idx, f_logpf, f_phase, d_logpf, d_phase);
-        GGF_CK(cudaGetLastError());
-        GGF_CK(cudaStreamSynchronize(st));
-    }
-    return GGF_OK;
-}
-
-// log Pf of every (configuration, pair) item of one family into ell[cfg][P].
-ggf_status front_family(ggf_ctx* ctx, bool cplx, int n_cfg, int npf, const void* d_links, cxd* ell, cudaStream_t st) {
-    const int P = ctx->P;
-    const long long total = (long long)n_cfg * npf;
-    const int chunk = (int)std::min<long long>(total, 1 << 20);
-    DBuf tab;
-    GGF_TRY(dalloc(ctx, tab, (size_t)chunk * (2 * sizeof(cxd) + 3 * sizeof(int)) + 256));
-    cxd* d_logpf = (cxd*)tab.p;
-    cxd* d_phase = d_logpf + chunk;
-    int* d_cfg = (int*)(d_phase + chunk);
-    int* d_pair = d_cfg + chunk;
-    int* d_flag = d_pair + chunk;
-    std::vector<int> hc, hp;
-    for (long long i0 = 0; i0 < total; i0 += chunk) {
-        const int items = (int)std::min<long long>(chunk, total - i0);
-        hc.resize(items); hp.resize(items);
-        for (int i = 0; i < items; ++i) { hc[i] = (int)((i0 + i) / npf); hp[i] = (int)((i0 + i) % npf); }
-        GGF_TRY(pf_items(ctx, cplx, hc, hp, d_links, d_cfg, d_pair, d_flag, d_logpf, d_phase, st));
-        GGF_CK(cudaMemcpyAsync(d_cfg, hc.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-        GGF_CK(cudaMemcpyAsync(d_pair, hp.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-        write_items_kernel<<<(items + 127) / 128, 128, 0, st>>>(items, d_cfg, d_pair, cplx ? ctx->K : 0, P, cplx,
-                                                                 d_logpf, d_phase, ell);
-        GGF_CK(cudaGetLastError());
-        GGF_CK(cudaStreamSynchronize(st));
-    }
     return GGF_OK;
 }
 
@@ -229,25 +212,25 @@ ggf_status front_family(ggf_ctx* ctx, bool cplx, int n_cfg, int npf, const void*
 // them; a refresh records |l_tracked - l_fresh| (log magnitude plus phase
 // mod 2 pi) as drift and replaces them.  Resets the accept count since the
 // last refresh.
-__global__ void ell_set_kernel(int n_items, int pair_off, int P, bool cplx, bool init, const int* item_chain,
-                               const int* item_pair, const cxd* logpf, const cxd* phase, cxd* ell, double* drift,
-                               int* since, unsigned long long* counters, int* flags) {
-    int it = blockIdx.x * blockDim.x + threadIdx.x;
-    if (it >= n_items) return;
-    int c = item_chain[it], p = pair_off + item_pair[it];
-    cxd& el = ell[(size_t)c * P + p];
-    cxd v = {logpf[it].x, 0.0};
-    if (cplx) v.y = atan2(phase[it].y, phase[it].x);
-    if (!isfinite(v.x)) {
-        atomicAdd(&counters[3], 1ULL);
-        atomicOr(&flags[c], 1);
+__global__ void ell_set_kernel(int n, int K, int P, bool init, const int* chains, const cxd* fresh, cxd* ell,
+                               double* drift, int* since, unsigned long long* counters, int* flags) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const int c = chains[q];
+    for (int p = 0; p < P; ++p) {
+        cxd& el = ell[(size_t)c * P + p];
+        const cxd v = fresh[(size_t)q * P + p];
+        if (!isfinite(v.x)) {
+            atomicAdd(&counters[3], 1ULL);
+            flags[c] |= 1;
+        }
+        if (!init) {
+            double d = fabs(v.x - el.x);
+            if (p >= K) d += fabs(remainder(v.y - el.y, 2 * M_PI));
+            if (!(d <= drift[c])) drift[c] = d;
+        }
+        el = v;
     }
-    if (!init) {
-        double d = fabs(v.x - el.x);
-        if (cplx) d += fabs(remainder(v.y - el.y, 2 * M_PI));
-        if (!(d <= drift[c])) drift[c] = d;
-    }
-    el = v;
     since[c] = 0;
 }
 
@@ -382,30 +365,17 @@ ggf_status newton_inverse(ggf_ctx* ctx, const std::vector<int>& chains, std::vec
 // (dense fallback for items without a usable pivot).
 ggf_status chain_ell(ggf_ctx* ctx, const std::vector<int>& chains, bool init, cudaStream_t st) {
     Chains& ch = ctx->ch;
-    for (int fam = 0; fam < 2; ++fam) {
-        const bool cplx = fam == 1;
-        const int npf = cplx ? ctx->Kc : ctx->K;
-        if (npf == 0) continue;
-        const int items = (int)chains.size() * npf;
-        std::vector<int> hc(items), hp(items);
-        for (size_t i = 0; i < chains.size(); ++i)
-            for (int p = 0; p < npf; ++p) { hc[i * npf + p] = chains[i]; hp[i * npf + p] = p; }
-        DBuf tab;
-        GGF_TRY(dalloc(ctx, tab, (size_t)items * (2 * sizeof(cxd) + 3 * sizeof(int)) + 256));
-        cxd* d_logpf = (cxd*)tab.p;
-        cxd* d_phase = d_logpf + items;
-        int* d_chain = (int*)(d_phase + items);
-        int* d_pair = d_chain + items;
-        int* d_flag = d_pair + items;
-        GGF_TRY(pf_items(ctx, cplx, hc, hp, ch.links, d_chain, d_pair, d_flag, d_logpf, d_phase, st));
-        GGF_CK(cudaMemcpyAsync(d_chain, hc.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-        GGF_CK(cudaMemcpyAsync(d_pair, hp.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
-        ell_set_kernel<<<(items + 127) / 128, 128, 0, st>>>(items, cplx ? ctx->K : 0, ctx->P, cplx, init, d_chain,
-                                                            d_pair, d_logpf, d_phase, ch.ell, ch.drift,
-                                                            ch.since_refresh, ch.counters, ch.flags);
-        GGF_CK(cudaGetLastError());
-        GGF_CK(cudaStreamSynchronize(st));
-    }
+    const int n = (int)chains.size();
+    DBuf list;
+    GGF_TRY(dalloc(ctx, list, (size_t)n * sizeof(int)));
+    GGF_CK(cudaMemcpyAsync(list.p, chains.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, st));
+    const cxd* ell = nullptr;
+    GGF_TRY(log_pfaffians(ctx, n, (const int*)list.p, &chains, ch.links, st,
+                          [&](const cxd* e) { ell = e; return GGF_OK; }));
+    ell_set_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, ctx->K, ctx->P, init, (const int*)list.p, ell, ch.ell, ch.drift,
+                                                    ch.since_refresh, ch.counters, ch.flags);
+    GGF_CK(cudaGetLastError());
+    GGF_CK(cudaStreamSynchronize(st));
     return GGF_OK;
 }
 
@@ -465,6 +435,7 @@ void ggf_destroy(ggf_ctx* ctx) {
     ggf_free_consts(ctx);
     ggf_front_free(ctx);
     if (ctx->work) cudaFree(ctx->work);
+    if (ctx->lw) cudaFree(ctx->lw);
     if (ctx->d_err) cudaFree(ctx->d_err);
     for (cudaEvent_t e : ctx->ev) cudaEventDestroy(e);
     delete ctx;
@@ -540,36 +511,36 @@ ggf_status ggf_logweight(ggf_ctx* ctx, int n_cfg, const void* links, double* log
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const Geometry& g = ctx->g;
-    const int N = g.N, P = ctx->P;
-    const size_t NN = (size_t)N * N;
+    const int P = ctx->P;
     const size_t lbytes = (size_t)n_cfg * g.n_links * link_bytes(g);
-    DBuf dl, dell, dlog;
+    DBuf dl, dlog;
     const void* d_links = links;
     if (mem == GGF_MEM_HOST) {
         GGF_TRY(dalloc(ctx, dl, lbytes));
         GGF_CK(cudaMemcpyAsync(dl.p, links, lbytes, cudaMemcpyHostToDevice, st));
         d_links = dl.p;
     }
-    GGF_TRY(dalloc(ctx, dell, (size_t)n_cfg * P * sizeof(cxd)));
-    for (int fam = 0; fam < 2; ++fam) {
-        const bool cplx = fam == 1;
-        const int npf = cplx ? ctx->Kc : ctx->K;
-        if (npf == 0) continue;
-        GGF_TRY(front_family(ctx, cplx, n_cfg, npf, d_links, (cxd*)dell.p, st));
-    }
     double* d_logN = logN;
     if (mem == GGF_MEM_HOST) {
         GGF_TRY(dalloc(ctx, dlog, (size_t)n_cfg * sizeof(double)));
         d_logN = (double*)dlog.p;
     }
-    GGF_TRY(ggf_combine(ctx, n_cfg, (const cxd*)dell.p, d_logN, st));
-    if (mem == GGF_MEM_HOST) {
-        GGF_CK(cudaMemcpyAsync(logN, d_logN, n_cfg * sizeof(double), cudaMemcpyDeviceToHost, st));
-        if (ell) GGF_CK(cudaMemcpyAsync(ell, dell.p, (size_t)n_cfg * P * sizeof(cxd), cudaMemcpyDeviceToHost, st));
-        GGF_CK(cudaStreamSynchronize(st));
-    } else {
-        if (ell) GGF_CK(cudaMemcpyAsync(ell, dell.p, (size_t)n_cfg * P * sizeof(cxd), cudaMemcpyDeviceToDevice, st));
-        GGF_CK(cudaStreamSynchronize(st));  // scoped temporaries are freed on return
+    // configurations in chunks: 32-bit item positions, and a bounded buffer
+    const int chunk = (int)std::max<long long>(1, std::min<long long>(n_cfg, (1LL << 22) / P));
+    const size_t row = g.n_links * link_bytes(g);
+    const cudaMemcpyKind down = mem == GGF_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    for (int c0 = 0; c0 < n_cfg; c0 += chunk) {
+        const int nc = std::min(chunk, n_cfg - c0);
+        GGF_TRY(log_pfaffians(ctx, nc, nullptr, nullptr, (const unsigned char*)d_links + (size_t)c0 * row, st,
+                              [&](const cxd* e) -> ggf_status {
+                                  GGF_TRY(ggf_combine(ctx, nc, e, d_logN + c0, st));
+                                  if (mem == GGF_MEM_HOST)
+                                      GGF_CK(cudaMemcpyAsync(logN + c0, d_logN + c0, nc * sizeof(double), down, st));
+                                  if (ell)
+                                      GGF_CK(cudaMemcpyAsync(ell + (size_t)c0 * P * 2, e, (size_t)nc * P * sizeof(cxd),
+                                                             down, st));
+                                  return GGF_OK;
+                              }));
     }
     return GGF_OK;
 }

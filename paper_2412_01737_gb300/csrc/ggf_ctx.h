@@ -103,11 +103,17 @@ struct ggf_ctx {
     Chains ch;
     void* work = nullptr;
     size_t work_bytes = 0;
+    // log-weights of one call: [configurations][P], then the list of items to
+    // refactor densely (grown on demand, freed with the context)
+    void* lw = nullptr;
+    size_t lw_bytes = 0;
     // site-by-site Pfaffian (k_front.cu): schedule [slot N | eoff V+1 | elim N]
     // for the lattice it was built for, and a global front workspace for
     // fronts too large for shared memory
     int* d_front = nullptr;
-    int front_F = 0, front_L = -1, front_B = -1;
+    int front_F = 0, front_L = -1, front_B = -1, front_sign = 1;
+    cudaStream_t front_st = nullptr;        // the real family's items run beside the complex ones
+    cudaEvent_t front_fork = nullptr, front_join = nullptr;
     void* front_ws = nullptr;
     size_t front_ws_bytes = 0;
     // refresh bookkeeping since ggf_chains_init: largest Newton residual
@@ -191,11 +197,11 @@ ggf_status ggf_pfaffian_batched(ggf_ctx* ctx, bool cplx, int n, int batch, void*
 // Batched Gauss-Jordan inverse in place: logdet (log|det|, arg) per item.
 ggf_status ggf_invert_batched(ggf_ctx* ctx, bool cplx, int n, int batch, void* A, cxd* d_logdet,
                               void* d_tmp, cudaStream_t st);
-// log Pf(M_nm(G)) by site-by-site elimination along the lattice (FP64):
-// (log|Pf|, 0) and the unit phase per item; flag[item] = 1 where no pivot was
-// usable inside a closed set (refactor those items densely).
-ggf_status ggf_front_pfaffian(ggf_ctx* ctx, bool cplx, int n_items, const int* d_item_cfg, const int* d_item_pair,
-                              const void* d_links, cxd* d_logpf, cxd* d_phase, int* d_flag, cudaStream_t st);
+// log Pf(M_nm(G)) of every pair of n configurations by site-by-site
+// elimination along the lattice (FP64) into d_ell [n][P]; d_bad: count and
+// positions of the items to refactor densely.
+ggf_status ggf_front_pfaffian(ggf_ctx* ctx, int n, const int* d_chains, const void* d_links, cxd* d_ell, int* d_bad,
+                              cudaStream_t st);
 void ggf_front_free(ggf_ctx* ctx);
 // Combine per-config pair log-Pfaffians into log N (device, n_cfg items).
 ggf_status ggf_combine(ggf_ctx* ctx, int n_cfg, const cxd* d_ell, double* d_logN, cudaStream_t st);

@@ -24,40 +24,44 @@
 // global-memory slice per CTA.
 //
 // Sign: Pf(M) = sgn(sigma) prod_t M^(t)_{k_t p_t} with sigma the elimination
-// sequence (k_1, p_1, k_2, p_2, ...).  The parity of sigma is accumulated as
-// the number of earlier-eliminated Majoranas with a larger index, for each
-// eliminated one: with all Majoranas of sites > s still to come (their
-// indices are larger), that count is (N - 1 - v) - #(front entries > v) -
-// (N - (s + 1) B).
+// sequence (k_1, p_1, k_2, p_2, ...): the sign of the schedule's own sequence
+// (known on the host) times one factor -1 per exchange a pivot choice makes.
+//
+// What bounds it: the FP64 unit (two FMAs per clock and SM).  The closed set is
+// eliminated in chunks of at most 16 Majoranas: their rows are copied into a
+// dense panel over the live slots, the pivoted pairs update the panel only,
+// and the rest of the front then takes the chunk's rank-16 update in one
+// pass, 2 x 2 register tiles over a list of the live slots.  Against a rank-2
+// update of the whole triangle per pair (33 % of the FP64 slots useful: dead
+// slots, ragged rows, a shared-memory round trip per product pair) 64 real
+// and 96 complex items of 16 x 16, n_v = 2 took 113 ms and take 50,
+// 1024 real items of 8 x 8 Z2 10.2 ms and 1.7.  Real and complex items
+// run side by side on two streams, because a handful of configurations fills
+// only part of the chip with either.  Fronts of at most 48 slots (8 x 8 Z2:
+// 44) take 64 threads, so that many items share an SM and the barriers of the
+// short steps are cheap; larger ones 256.
 #include <algorithm>
-#include <map>
 #include <vector>
 #include "ggf_ctx.h"
 #include "ggf_geom.cuh"
 
 namespace {
 
-constexpr int FT = 512;                 // threads per CTA
-constexpr int FW = FT / 32;
+constexpr int CHUNK = 16;          // closed Majoranas per panel
+constexpr int SMALL_FRONT = 48;    // slots up to which an item takes 64 threads
 
-__device__ __forceinline__ int tri_row(int i, int F) { return i * (2 * F - i - 1) / 2 - i - 1; }
+__host__ __device__ __forceinline__ int tri_row(int i, int F) { return i * (2 * F - i - 1) / 2 - i - 1; }
 
-template <class T> __device__ __forceinline__ T fzero();
-template <> __device__ __forceinline__ double fzero<double>() { return 0.0; }
-template <> __device__ __forceinline__ cxd fzero<cxd>() { return {0.0, 0.0}; }
-__device__ __forceinline__ double fmag(double v) { return fabs(v); }
-__device__ __forceinline__ double fmag(cxd v) { return hypot(v.x, v.y); }
-__device__ __forceinline__ bool fnz(double v) { return v != 0.0; }
-__device__ __forceinline__ bool fnz(cxd v) { return v.x != 0.0 || v.y != 0.0; }
+__device__ __forceinline__ double fsq(double v) { return v * v; }
+__device__ __forceinline__ double fsq(cxd v) { return fma(v.x, v.x, v.y * v.y); }
 __device__ __forceinline__ double fneg(double v) { return -v; }
 __device__ __forceinline__ cxd fneg(cxd v) { return {-v.x, -v.y}; }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ cxd fdiv(cxd a, cxd b) { return a / b; }
-__device__ __forceinline__ cxd funit(double v) { return {v >= 0 ? 1.0 : -1.0, 0.0}; }
-__device__ __forceinline__ cxd funit(cxd v) {
-    double m = hypot(v.x, v.y);
-    return {v.x / m, v.y / m};
-}
+__device__ __forceinline__ double finv(double v) { return 1.0 / v; }
+__device__ __forceinline__ cxd finv(cxd v) { return cxd{1.0, 0.0} / v; }
+__device__ __forceinline__ double fmul(double a, double b) { return a * b; }
+__device__ __forceinline__ cxd fmul(cxd a, cxd b) { return a * b; }
+__device__ __forceinline__ cxd as_c(double v) { return {v, 0.0}; }
+__device__ __forceinline__ cxd as_c(cxd v) { return v; }
 // r += a * b - c * d
 __device__ __forceinline__ void frank2(double& r, double a, double b, double c, double d) {
     r = fma(a, b, r);
@@ -75,7 +79,7 @@ template <class T>
 __device__ __forceinline__ T sget(const T* S, int F, int a, int b) {
     if (a < b) return S[tri_row(a, F) + b];
     if (a > b) return fneg(S[tri_row(b, F) + a]);
-    return fzero<T>();
+    return Sc<T>::zero();
 }
 
 struct FrontArgs {
@@ -84,138 +88,245 @@ struct FrontArgs {
     const int* slot;    // [N] slot of Majorana i (fixed by the schedule)
     const int* eoff;    // [V + 1] offsets into elim
     const int* elim;    // slots eliminated after adding site s
+    int sign;           // of the schedule's elimination sequence
 };
 
-// One CTA per item (grid-stride over items).  Dynamic shared memory: u[F],
-// v[F] (T), idx[F], es[F] (int), then the packed triangle when it fits.
+// The four link ends of the site being added: link, its value's twist.
+struct EndTab {
+    int link;
+    double gval;
+    double tw[16];      // U(1): cos, sin of q_j theta; SU(2): doublet rotation
+};
+
+// M(i, j) for Majorana a of site s (i = s B + a) and any Majorana j.
 template <class T>
-__global__ void __launch_bounds__(FT, 1)
-front_pf_kernel(DevConst dc, FrontArgs fa, int n_items, const int* item_cfg, const int* item_pair, const void* links,
-                cxd* logpf, cxd* phase, int* flag, T* gws, size_t tri_elems, int in_smem) {
-    extern __shared__ __align__(16) unsigned char fsm[];
-    __shared__ int s_k, s_p, s_bad;
-    const int F = fa.F, N = fa.N, B = fa.B, V = fa.V;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    T* u = (T*)fsm;
-    T* v = u + F;
-    int* idx = (int*)(v + F);
-    int* es = idx + F;
-    T* S = in_smem ? (T*)(fsm + (((size_t)F * (2 * sizeof(T) + 2 * sizeof(int)) + 15) / 16) * 16)
-                   : gws + (size_t)blockIdx.x * tri_elems;
+__device__ __forceinline__ T front_entry(const DevConst& dc, int pair, const EndTab* tab, int s, int a, int j) {
     const Geometry& g = dc.g;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int cfg = item_cfg[item], pair = item_pair[item];
-        for (int a = tid; a < F; a += FT) idx[a] = -1;
+    const int e = a / g.h2, x = a - e * g.h2;
+    const int l = tab[e].link, pi = (e & 1) ? x : g.h2 + x;
+    T v = Sc<T>::zero();
+    int lj, pj;
+    if (j / g.B == s) {
+        const int b = j - s * g.B, eb = b / g.h2, xb = b - eb * g.h2;
+        v = Sc<T>::from(Sc<double>::to(dc.D[((size_t)s * g.B + a) * g.B + b]));
+        lj = tab[eb].link;
+        pj = (eb & 1) ? xb : g.h2 + xb;
+    } else {
+        link_of(g, j, lj, pj);
+    }
+    if (lj == l)
+        v += g.group == GGF_SU2 ? twisted_su2<T>(dc, pair, l, pi, pj, tab[e].tw)
+                                : twisted_tab<T>(dc, pair, l, pi, pj, tab[e].gval, tab[e].tw);
+    return v;
+}
+
+// Byte offsets of an item's shared arrays.
+struct FrontLayout {
+    size_t tab, idx, lv, tri, total;
+};
+__host__ __device__ inline FrontLayout front_layout(int F, size_t elem, bool tri) {
+    FrontLayout l;
+    size_t o = (size_t)CHUNK * F * elem;       // the panel comes first
+    auto take = [&](size_t& at, size_t bytes) { at = o; o = (o + bytes + 15) & ~(size_t)15; };
+    take(l.tab, 4 * sizeof(EndTab));
+    take(l.idx, (size_t)F * sizeof(int));
+    take(l.lv, (size_t)F * sizeof(unsigned short));
+    take(l.tri, tri ? (size_t)F * (F - 1) / 2 * elem : 0);
+    l.total = o;
+    return l;
+}
+
+// One CTA per item (grid-stride); item = q npf + pair of configuration
+// chains[q] (or q).  Its log-weight goes to ell[q][pair_off + pair]; items
+// without a usable pivot are appended to bad[1 ..], counted in bad[0].
+template <class T, int NT>
+__global__ void __launch_bounds__(NT, NT == 64 ? 8 : (sizeof(T) == 8 ? 2 : 1))
+front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains, int npf, int pair_off,
+                const void* links, cxd* ell, int* bad, T* gws, size_t tri_elems, int in_smem) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int s_bad, s_nl;
+    __shared__ T s_inv;
+    __shared__ T s_scale[CHUNK];
+    __shared__ int ord[CHUNK], es[CHUNK];
+    constexpr int NW = NT / 32;
+    const int F = fa.F, B = fa.B, V = fa.V;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const FrontLayout lay = front_layout(F, sizeof(T), in_smem != 0);
+    T* Pn = (T*)fsm;                                     // [CHUNK][F]
+    EndTab* tab = (EndTab*)(fsm + lay.tab);
+    int* idx = (int*)(fsm + lay.idx);                    // Majorana of a slot, -1: dead
+    unsigned short* lv = (unsigned short*)(fsm + lay.lv);
+    T* S = in_smem ? (T*)(fsm + lay.tri) : gws + (size_t)blockIdx.x * tri_elems;
+    const Geometry& g = dc.g;
+    for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const int q = (int)(item / npf), pair = (int)(item - (long long)q * npf);
+        const int cfg = chains ? chains[q] : q;
+        for (int a = tid; a < F; a += NT) idx[a] = -1;
         if (tid == 0) s_bad = 0;
-        double logabs = 0.0;   // meaningful in thread 0
-        cxd ph = {1.0, 0.0};
-        int par = 0;
         __syncthreads();
-        for (int s = 0; s < V && !s_bad; ++s) {
+        // lane 0 of warp 0: prod of the pivots as pr 2^ex
+        cxd pr = {(double)fa.sign, 0.0};
+        long long ex = 0;
+        for (int s = 0; s < V; ++s) {
             // ---- add site s: its B Majoranas take their slots, their rows are M's entries
-            for (int k = tid; k < B; k += FT) idx[fa.slot[s * B + k]] = s * B + k;
+            if (tid < 4) {
+                EndTab& t = tab[tid];
+                int pos;
+                link_of(g, s * B + tid * g.h2, t.link, pos);
+                t.gval = 1.0;
+                if (g.group == GGF_Z2) {
+                    t.gval = (double)((const int8_t*)links)[(size_t)cfg * g.n_links + t.link];
+                } else if (g.group == GGF_U1) {
+                    const double th = ((const double*)links)[(size_t)cfg * g.n_links + t.link];
+                    for (int j = 0; j < g.n_v; ++j) sincos(g.q[j] * th, &t.tw[2 * j + 1], &t.tw[2 * j]);
+                } else {
+                    doublet_rotation(link_quat(g, links, cfg, t.link), t.tw);
+                }
+            }
+            for (int k = tid; k < B; k += NT) idx[fa.slot[s * B + k]] = s * B + k;
             __syncthreads();
-            for (int w = tid; w < B * F; w += FT) {
-                const int k = w / F, b = w - k * F;
+            for (int k = warp; k < B; k += NW) {
                 const int a = fa.slot[s * B + k];
-                const int jb = idx[b];
-                if (b == a || jb < 0) continue;
-                if (jb >= s * B && b < a) continue;        // new-new pair: written once, by the lower slot's row
-                const int lo = min(a, b), hi = max(a, b);
-                const int i = idx[lo], j = idx[hi];
-                T val = fzero<T>();
-                const int si = i / B, sj = j / B;
-                int li, pi, lj, pj;
-                link_of(g, i, li, pi);
-                link_of(g, j, lj, pj);
-                if (si == sj || li == lj) val = assemble_elem<T>(dc, links, cfg, pair, i, j);
-                S[tri_row(lo, F) + hi] = val;
+                for (int b = lane; b < F; b += 32) {
+                    const int jb = idx[b];
+                    if (b == a || jb < 0) continue;
+                    if (jb >= s * B && b < a) continue;        // new-new pair: written once, by the lower slot's row
+                    const T val = front_entry<T>(dc, pair, tab, s, k, jb);
+                    if (a < b) S[tri_row(a, F) + b] = val;
+                    else S[tri_row(b, F) + a] = fneg(val);
+                }
             }
-            // ---- eliminate the closed Majoranas in pivoted pairs
-            const int e0 = fa.eoff[s], e1 = fa.eoff[s + 1];
-            for (int t = tid; t < e1 - e0; t += FT) es[t] = fa.elim[e0 + t];
             __syncthreads();
-            for (int t = 0; t < e1 - e0; t += 2) {
-                if (warp == 0) {
-                    const int ne = e1 - e0 - t;
-                    double best = -1.0;
-                    int bq = 0;
-                    for (int q = lane; q < ne * ne; q += 32) {
-                        const int x = q / ne, y = q - x * ne;
-                        if (x >= y) continue;
-                        const double m = fmag(sget(S, F, es[t + x], es[t + y]));
-                        if (m > best) { best = m; bq = q; }
+            // ---- eliminate the closed Majoranas, a chunk at a time
+            const int e1 = fa.eoff[s + 1];
+            for (int e0 = fa.eoff[s]; e0 < e1; e0 += CHUNK) {
+                const int c = min(CHUNK, e1 - e0);
+                if (tid < c) { es[tid] = fa.elim[e0 + tid]; ord[tid] = tid; }
+                __syncthreads();
+                if (tid < c) idx[es[tid]] = -1;
+                __syncthreads();
+                if (warp == 0) {                        // the live slots, ascending
+                    int n = 0;
+                    for (int b0 = 0; b0 < F; b0 += 32) {
+                        const bool live = b0 + lane < F && idx[b0 + lane] >= 0;
+                        const unsigned m = __ballot_sync(0xffffffffu, live);
+                        if (live) lv[n + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(b0 + lane);
+                        n += __popc(m);
                     }
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const double ob = __shfl_down_sync(0xffffffffu, best, o);
-                        const int oq = __shfl_down_sync(0xffffffffu, bq, o);
-                        if (ob > best || (ob == best && oq < bq)) { best = ob; bq = oq; }
-                    }
-                    if (lane == 0) {
-                        const int x = bq / ne, y = bq - (bq / ne) * ne;
-                        const int k = es[t + x], p = es[t + y];
-                        if (!(best > 1e-8) || !isfinite(best)) s_bad = 1;   // no usable pivot: refactor densely
-                        // move the pair to positions t, t + 1 of the closed list (x < y,
-                        // so the first swap leaves position t + y alone)
-                        es[t + x] = es[t];
-                        es[t] = k;
-                        es[t + y] = es[t + 1];
-                        es[t + 1] = p;
-                        s_k = k;
-                        s_p = p;
-                    }
+                    if (lane == 0) s_nl = n;
                 }
                 __syncthreads();
+                const int nl = s_nl, W = c + nl;
+                for (int t = warp; t < c; t += NW)
+                    for (int w = lane; w < W; w += 32)
+                        Pn[(size_t)t * F + w] = sget(S, F, es[t], w < c ? es[w] : lv[w - c]);
+                __syncthreads();
+                for (int t = 0; t < c; t += 2) {
+                    if (warp == 0) {
+                        // pivot: the largest entry among the chunk's remaining pairs
+                        const int ne = c - t;
+                        double best = -1.0;
+                        int bq = 1;
+                        for (int p = lane; p < ne * (ne - 1) / 2; p += 32) {
+                            int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
+                            if (y * (y - 1) / 2 > p) --y;
+                            if ((y + 1) * y / 2 <= p) ++y;
+                            const int x = p - y * (y - 1) / 2;
+                            const double m = fsq(Pn[(size_t)ord[t + x] * F + ord[t + y]]);
+                            if (m > best || !(m == m)) { best = m; bq = x * 32 + y; }
+                        }
+                        const unsigned key = best >= 0.0 || !(best == best) ? (unsigned)__double2hiint(best) & 0x7fffffffu : 0u;
+                        const unsigned top = __reduce_max_sync(0xffffffffu, key);
+                        const int src = __ffs(__ballot_sync(0xffffffffu, key == top && !(best < 0.0))) - 1;
+                        best = __shfl_sync(0xffffffffu, best, src);
+                        bq = __shfl_sync(0xffffffffu, bq, src);
+                        if (lane == 0) {
+                            const int x = bq / 32, y = bq % 32;
+                            if (!(best > 1e-16) || !isfinite(best)) s_bad = 1;   // no usable pivot: refactor densely
+                            // the pair to positions t, t + 1 (x < y: the first exchange leaves t + y alone)
+                            const int k = ord[t + x], p = ord[t + y];
+                            ord[t + x] = ord[t];
+                            ord[t] = k;
+                            ord[t + y] = ord[t + 1];
+                            ord[t + 1] = p;
+                            const T akp = Pn[(size_t)k * F + p];
+                            const T inv = finv(akp);
+                            s_inv = inv;
+                            s_scale[t] = inv;
+                            pr = pr * as_c(akp);
+                            if ((x > 0) != (y > 1)) pr = -pr;
+                            // keep the product in range by its own power of two
+                            const int e = ((__double2hiint(fmax(fabs(pr.x), fabs(pr.y))) >> 20) & 0x7ff) - 1023;
+                            const double sc = __hiloint2double((1023 - e) << 20, 0);
+                            pr = {pr.x * sc, pr.y * sc};
+                            ex += e;
+                        }
+                    }
+                    __syncthreads();
+                    if (s_bad) break;
+                    // the remaining rows of the chunk: R += (v_R / a) k - (k_R / a) v
+                    const T* rk = Pn + (size_t)ord[t] * F;
+                    const T* rp = Pn + (size_t)ord[t + 1] * F;
+                    const T inv = s_inv;
+                    for (int i = t + 2 + warp; i < c; i += NW) {
+                        const int row = ord[i];
+                        const T vi = fmul(rp[row], inv), ki = fmul(rk[row], inv);
+                        T* r = Pn + (size_t)row * F;
+                        for (int w = lane; w < W; w += 32) {
+                            T x = r[w];
+                            frank2(x, vi, rk[w], ki, rp[w]);
+                            r[w] = x;
+                        }
+                    }
+                    __syncthreads();
+                }
                 if (s_bad) break;
-                const int k = s_k, p = s_p;
-                const T akp = sget(S, F, k, p);
-                if (warp == 0) {
-                    // parity of the elimination sequence: k, then p
-                    const int vk = idx[k], vp = idx[p];
-                    int ck = 0, cp = 0;
-                    for (int b = lane; b < F; b += 32) {
-                        const int j = idx[b];
-                        if (j < 0 || b == k) continue;
-                        ck += j > vk;
-                        if (b != p) cp += j > vp;
-                    }
-                    for (int o = 16; o > 0; o >>= 1) {
-                        ck += __shfl_down_sync(0xffffffffu, ck, o);
-                        cp += __shfl_down_sync(0xffffffffu, cp, o);
-                    }
-                    if (lane == 0) {
-                        const int later = N - (s + 1) * B;
-                        par ^= ((N - 1 - vk) - ck - later) & 1;
-                        par ^= ((N - 1 - vp) - cp - later) & 1;
-                        logabs += log(fmag(akp));
-                        ph = ph * funit(akp);
-                    }
-                }
-                for (int b = tid; b < F; b += FT) {
-                    const bool live = idx[b] >= 0 && b != k && b != p;
-                    u[b] = live ? fdiv(sget(S, F, k, b), akp) : fzero<T>();
-                    v[b] = live ? sget(S, F, p, b) : fzero<T>();
+                // u_t = row k_t / a_t over the live columns
+                for (int t = 2 * warp; t < c; t += 2 * NW) {
+                    T* r = Pn + (size_t)ord[t] * F + c;
+                    const T inv = s_scale[t];
+                    for (int w = lane; w < nl; w += 32) r[w] = fmul(r[w], inv);
                 }
                 __syncthreads();
-                if (tid == 0) { idx[k] = -1; idx[p] = -1; }
-                // C += v u^T - u v^T on the strict upper triangle
-                for (int i = warp; i < F - 1; i += FW) {
-                    const T vi = v[i], ui = u[i];
-                    if (!fnz(vi) && !fnz(ui)) continue;
-                    T* row = S + tri_row(i, F);
-                    for (int j = i + 1 + lane; j < F; j += 32) frank2(row[j], vi, u[j], ui, v[j]);
+                // C += sum_t v_t u_t^T - u_t v_t^T on the pairs of live slots (nl is
+                // even: link ends hold 2 n_v Majoranas), 2 x 2 per thread and turn
+                const int th = nl >> 1;
+                for (int id = tid; id < th * (th + 1) / 2; id += NT) {
+                    int tj = (int)((sqrtf(8.0f * (float)id + 1.0f) - 1.0f) * 0.5f);
+                    if (tj * (tj + 1) / 2 > id) --tj;
+                    if ((tj + 1) * (tj + 2) / 2 <= id) ++tj;
+                    const int i = 2 * (id - tj * (tj + 1) / 2), j = 2 * tj;
+                    const int r0 = lv[i], r1 = lv[i + 1], c0 = lv[j], c1 = lv[j + 1];
+                    T* S0 = S + tri_row(r0, F);
+                    T* S1 = S + tri_row(r1, F);
+                    const bool diag = i == j;
+                    T a00 = diag ? Sc<T>::zero() : S0[c0], a01 = S0[c1];
+                    T a10 = diag ? Sc<T>::zero() : S1[c0], a11 = diag ? Sc<T>::zero() : S1[c1];
+                    for (int t = 0; t < c; t += 2) {
+                        const T* u = Pn + (size_t)ord[t] * F + c;
+                        const T* v = Pn + (size_t)ord[t + 1] * F + c;
+                        const T ui0 = u[i], ui1 = u[i + 1], vi0 = v[i], vi1 = v[i + 1];
+                        const T uj0 = u[j], uj1 = u[j + 1], vj0 = v[j], vj1 = v[j + 1];
+                        frank2(a00, vi0, uj0, ui0, vj0);
+                        frank2(a01, vi0, uj1, ui0, vj1);
+                        frank2(a10, vi1, uj0, ui1, vj0);
+                        frank2(a11, vi1, uj1, ui1, vj1);
+                    }
+                    S0[c1] = a01;
+                    if (!diag) { S0[c0] = a00; S1[c0] = a10; S1[c1] = a11; }
                 }
                 __syncthreads();
             }
+            if (s_bad) break;
         }
         if (tid == 0) {
-            flag[item] = s_bad;
+            cxd* dst = ell + (size_t)q * dc.P + pair_off + pair;
             if (s_bad) {
-                logpf[item] = {NAN, 0.0};
-                phase[item] = {0.0, 0.0};
+                *dst = {NAN, 0.0};
+                bad[1 + atomicAdd(bad, 1)] = (int)((long long)q * dc.P + pair_off + pair);
             } else {
-                logpf[item] = {logabs, 0.0};
-                phase[item] = par ? cxd{-ph.x, -ph.y} : ph;
+                const double m = Sc<T>::CPLX ? hypot(pr.x, pr.y) : fabs(pr.x);
+                *dst = {log(m) + (double)ex * 0.69314718055994530942, Sc<T>::CPLX ? atan2(pr.y, pr.x) : 0.0};
             }
         }
         __syncthreads();
@@ -223,9 +334,11 @@ front_pf_kernel(DevConst dc, FrontArgs fa, int n_items, const int* item_cfg, con
 }
 
 // Elimination schedule for an L x L lattice with B virtual Majoranas per
-// site: slot of every Majorana and the slots closed after each site.
-void build_schedule(const Geometry& g, int& F, std::vector<int>& slot, std::vector<int>& eoff,
-                    std::vector<int>& elim) {
+// site: slot of every Majorana, the slots closed after each site (both ends of
+// a link together, so that a chunk holds whole links) and the sign of the
+// sequence.
+void build_schedule(const Geometry& g, int& F, std::vector<int>& slot, std::vector<int>& eoff, std::vector<int>& elim,
+                    int& sign) {
     const int B = g.B, V = g.V, N = g.N, L = g.L;
     slot.assign(N, -1);
     eoff.assign(V + 1, 0);
@@ -235,7 +348,11 @@ void build_schedule(const Geometry& g, int& F, std::vector<int>& slot, std::vect
         if (e & 1) return d == 0 ? y * L + (x + 1) % L : ((y + 1) % L) * L + x;
         return d == 0 ? y * L + (x + L - 1) % L : ((y + L - 1) % L) * L + x;
     };
-    std::vector<int> free_slots, front;
+    auto link_id = [&](int i) {
+        const int s = i / B, e = (i % B) / g.h2, d = e >> 1;
+        return 2 * ((e & 1) ? s : partner_site(s, e)) + d;
+    };
+    std::vector<int> free_slots, front, seq;
     int next = 0;
     F = 0;
     for (int s = 0; s < V; ++s) {
@@ -252,41 +369,51 @@ void build_schedule(const Geometry& g, int& F, std::vector<int>& slot, std::vect
             front.push_back(s * B + k);
         }
         F = std::max(F, next);
-        std::vector<int> keep;
+        std::vector<int> keep, closed;
         for (int i : front) {
             const int si = i / B, e = (i % B) / g.h2;
-            if (partner_site(si, e) <= s) {
-                elim.push_back(slot[i]);
-                free_slots.push_back(slot[i]);
-            } else {
-                keep.push_back(i);
-            }
+            if (partner_site(si, e) <= s) closed.push_back(i);
+            else keep.push_back(i);
+        }
+        std::stable_sort(closed.begin(), closed.end(), [&](int a, int b) { return link_id(a) < link_id(b); });
+        for (int i : closed) {
+            elim.push_back(slot[i]);
+            free_slots.push_back(slot[i]);
+            seq.push_back(i);
         }
         front.swap(keep);
         eoff[s + 1] = (int)elim.size();
     }
-}
-
-}  // namespace
-
-// Shared memory of the front kernel for F slots (without / with the triangle).
-static size_t front_smem(int F, size_t elem, bool tri) {
-    size_t b = (((size_t)F * (2 * elem + 2 * sizeof(int)) + 15) / 16) * 16;
-    if (tri) b += (size_t)F * (F - 1) / 2 * elem;
-    return b;
+    // sign of the permutation by its cycles
+    std::vector<char> seen(seq.size(), 0);
+    int cycles = 0;
+    for (size_t i = 0; i < seq.size(); ++i) {
+        if (seen[i]) continue;
+        ++cycles;
+        for (size_t j = i; !seen[j]; j = (size_t)seq[j]) seen[j] = 1;
+    }
+    sign = ((int)seq.size() - cycles) % 2 ? -1 : 1;
 }
 
 // opt-in shared memory per CTA (227 KB) less a margin for the static variables
-static const size_t kSmemMax = 227 * 1024 - 1024;
+const size_t kSmemMax = 227 * 1024 - 1024;
+
+template <class T, int NT>
+ggf_status raise_cap(ggf_ctx* ctx) {
+    GGF_CK(cudaFuncSetAttribute(front_pf_kernel<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    return GGF_OK;
+}
+
+}  // namespace
 
 ggf_status ggf_front_prepare(ggf_ctx* ctx) {
     const Geometry& g = ctx->g;
     if (ctx->d_front && ctx->front_L == g.L && ctx->front_B == g.B) return GGF_OK;
     if (ctx->d_front) cudaFree(ctx->d_front);
     ctx->d_front = nullptr;
-    int F = 0;
+    int F = 0, sign = 1;
     std::vector<int> slot, eoff, elim;
-    build_schedule(g, F, slot, eoff, elim);
+    build_schedule(g, F, slot, eoff, elim, sign);
     if ((int)elim.size() != g.N) return ggf_fail(ctx, GGF_ESTATE, "front schedule does not close every Majorana");
     std::vector<int> all;
     all.insert(all.end(), slot.begin(), slot.end());
@@ -294,13 +421,21 @@ ggf_status ggf_front_prepare(ggf_ctx* ctx) {
     all.insert(all.end(), elim.begin(), elim.end());
     GGF_CK(cudaMalloc(&ctx->d_front, all.size() * sizeof(int)));
     GGF_CK(cudaMemcpy(ctx->d_front, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if (!ctx->front_st) {
+        GGF_CK(cudaStreamCreateWithFlags(&ctx->front_st, cudaStreamNonBlocking));
+        GGF_CK(cudaEventCreateWithFlags(&ctx->front_fork, cudaEventDisableTiming));
+        GGF_CK(cudaEventCreateWithFlags(&ctx->front_join, cudaEventDisableTiming));
+    }
     ctx->front_F = F;
+    ctx->front_sign = sign;
     ctx->front_L = g.L;
     ctx->front_B = g.B;
     static bool attr_done[64] = {false};
     if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
-        GGF_CK(cudaFuncSetAttribute(front_pf_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        GGF_CK(cudaFuncSetAttribute(front_pf_kernel<cxd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        GGF_TRY((raise_cap<double, 64>(ctx)));
+        GGF_TRY((raise_cap<double, 256>(ctx)));
+        GGF_TRY((raise_cap<cxd, 64>(ctx)));
+        GGF_TRY((raise_cap<cxd, 256>(ctx)));
         attr_done[ctx->device] = true;
     }
     return GGF_OK;
@@ -309,24 +444,27 @@ ggf_status ggf_front_prepare(ggf_ctx* ctx) {
 void ggf_front_free(ggf_ctx* ctx) {
     if (ctx->d_front) cudaFree(ctx->d_front);
     if (ctx->front_ws) cudaFree(ctx->front_ws);
+    if (ctx->front_st) cudaStreamDestroy(ctx->front_st);
+    if (ctx->front_fork) cudaEventDestroy(ctx->front_fork);
+    if (ctx->front_join) cudaEventDestroy(ctx->front_join);
     ctx->d_front = nullptr;
     ctx->front_ws = nullptr;
     ctx->front_ws_bytes = 0;
+    ctx->front_st = nullptr;
+    ctx->front_fork = ctx->front_join = nullptr;
     ctx->front_L = ctx->front_B = -1;
 }
 
-int ggf_front_slots(ggf_ctx* ctx) { return ctx->front_F; }
-
-// log Pf(M_nm(G)) of n_items (configuration, pair-within-family) items:
-// d_logpf[item] = (log|Pf|, 0), d_phase[item] = Pf/|Pf|, d_flag[item] = 1
-// where a closed set had no usable pivot (the caller refactors those items
-// densely).  Links are device configurations indexed by d_item_cfg.
-ggf_status ggf_front_pfaffian(ggf_ctx* ctx, bool cplx, int n_items, const int* d_item_cfg, const int* d_item_pair,
-                              const void* d_links, cxd* d_logpf, cxd* d_phase, int* d_flag, cudaStream_t st) {
-    if (n_items == 0) return GGF_OK;
+// log Pf(M_nm(G)) of every pair of n configurations (d_chains[q], or q where
+// d_chains is null) of d_links into d_ell [n][P]: (log|Pf|, phase).  Items
+// whose closed sets had no usable pivot are listed in d_bad (1 + n P ints:
+// the count, then positions in d_ell; the caller refactors those densely).
+ggf_status ggf_front_pfaffian(ggf_ctx* ctx, int n, const int* d_chains, const void* d_links, cxd* d_ell, int* d_bad,
+                              cudaStream_t st) {
+    if (n == 0) return GGF_OK;
     GGF_TRY(ggf_front_prepare(ctx));
     const Geometry& g = ctx->g;
-    const int F = ctx->front_F;
+    const int F = ctx->front_F, sms = ctx->n_sms > 0 ? ctx->n_sms : 152;
     FrontArgs fa;
     fa.F = F;
     fa.N = g.N;
@@ -335,32 +473,51 @@ ggf_status ggf_front_pfaffian(ggf_ctx* ctx, bool cplx, int n_items, const int* d
     fa.slot = ctx->d_front;
     fa.eoff = ctx->d_front + g.N;
     fa.elim = ctx->d_front + g.N + g.V + 1;
-    const size_t elem = cplx ? sizeof(cxd) : sizeof(double);
-    const bool in_smem = front_smem(F, elem, true) <= kSmemMax;
+    fa.sign = ctx->front_sign;
     const size_t tri = (size_t)F * (F - 1) / 2;
-    int grid = std::min(n_items, 65535);
-    void* ws = nullptr;
-    if (!in_smem) {
-        const int sms = ctx->n_sms > 0 ? ctx->n_sms : 152;
-        grid = std::min(n_items, 2 * sms);
-        const size_t need = (size_t)grid * tri * elem;
-        if (need > ctx->front_ws_bytes) {
-            if (ctx->front_ws) cudaFree(ctx->front_ws);
-            ctx->front_ws = nullptr;
-            ctx->front_ws_bytes = 0;
-            GGF_CK(cudaMalloc(&ctx->front_ws, need));
-            ctx->front_ws_bytes = need;
-        }
-        ws = ctx->front_ws;
+    int grid[2];
+    bool in_smem[2];
+    size_t need = 0, off[2] = {0, 0};
+    for (int f = 0; f < 2; ++f) {
+        const size_t elem = f ? sizeof(cxd) : sizeof(double);
+        const long long items = (long long)n * (f ? ctx->Kc : ctx->K);
+        in_smem[f] = front_layout(F, elem, true).total <= kSmemMax;
+        grid[f] = (int)std::min<long long>(items, in_smem[f] ? 1 << 20 : 2 * sms);
+        off[f] = need;
+        if (!in_smem[f]) need += ((size_t)grid[f] * tri * elem + 255) / 256 * 256;
     }
-    const size_t smem = front_smem(F, elem, in_smem);
-    ctx->launches += 1;
-    if (cplx)
-        front_pf_kernel<cxd><<<grid, FT, smem, st>>>(ctx->dc(), fa, n_items, d_item_cfg, d_item_pair, d_links, d_logpf,
-                                                     d_phase, d_flag, (cxd*)ws, tri, in_smem ? 1 : 0);
-    else
-        front_pf_kernel<double><<<grid, FT, smem, st>>>(ctx->dc(), fa, n_items, d_item_cfg, d_item_pair, d_links,
-                                                        d_logpf, d_phase, d_flag, (double*)ws, tri, in_smem ? 1 : 0);
+    if (need > ctx->front_ws_bytes) {
+        if (ctx->front_ws) cudaFree(ctx->front_ws);
+        ctx->front_ws = nullptr;
+        ctx->front_ws_bytes = 0;
+        GGF_CK(cudaMalloc(&ctx->front_ws, need));
+        ctx->front_ws_bytes = need;
+    }
+    GGF_CK(cudaMemsetAsync(d_bad, 0, sizeof(int), st));
+    const bool both = ctx->Kc > 0;
+    if (both) {
+        GGF_CK(cudaEventRecord(ctx->front_fork, st));
+        GGF_CK(cudaStreamWaitEvent(ctx->front_st, ctx->front_fork, 0));
+    }
+    const bool small = F <= SMALL_FRONT;
+#define GGF_FRONT(T, NT, f, npf, off_p, stream)                                                                  \
+    front_pf_kernel<T, NT><<<grid[f], NT, front_layout(F, sizeof(T), in_smem[f]).total, stream>>>(                \
+        ctx->dc(), fa, (long long)n * (npf), d_chains, npf, off_p, d_links, d_ell, d_bad,                         \
+        (T*)((unsigned char*)ctx->front_ws + off[f]), tri, in_smem[f] ? 1 : 0)
+    if (both) {      // the complex items, four times as long, are placed first
+        if (small) GGF_FRONT(cxd, 64, 1, ctx->Kc, ctx->K, st);
+        else GGF_FRONT(cxd, 256, 1, ctx->Kc, ctx->K, st);
+        GGF_CK(cudaGetLastError());
+    }
+    cudaStream_t rs = both ? ctx->front_st : st;
+    if (small) GGF_FRONT(double, 64, 0, ctx->K, 0, rs);
+    else GGF_FRONT(double, 256, 0, ctx->K, 0, rs);
     GGF_CK(cudaGetLastError());
+#undef GGF_FRONT
+    ctx->launches += both ? 2 : 1;
+    if (both) {
+        GGF_CK(cudaEventRecord(ctx->front_join, ctx->front_st));
+        GGF_CK(cudaStreamWaitEvent(st, ctx->front_join, 0));
+    }
     return GGF_OK;
 }
