@@ -9,9 +9,6 @@
 #include "ggf_ctx.h"
 
 size_t ggf_factor_tmp_bytes(int n, int batch);
-size_t ggf_refine_bytes(int N, bool cplx);
-ggf_status ggf_refine_inverse(ggf_ctx* ctx, bool cplx, const void* d_links, int cfg, int pair, float* W, void* ws,
-                              int terms, double* rmax, cudaStream_t st);
 // Newton refinement policy for FP32 inverses (largest |I - M W| entry r):
 // r <= kRefineFloor is the FP32 floor (no step); r <= kRefineOne takes one
 // step with one TF32 product; r <= kRefineTol takes three-product steps.
@@ -315,25 +312,45 @@ ggf_status dense_inverse(ggf_ctx* ctx, const std::vector<int>& chains, cudaStrea
     return GGF_OK;
 }
 
-// Newton refinement of one FP32 inverse by the policy above; false when the
+// Newton refinement of a batch by the policy above: ok[i] = 0 where the
 // residual is too large (or does not shrink) and the chain needs refactoring.
-ggf_status refine_one(ggf_ctx* ctx, bool cplx, int c, int p, float* W, bool* ok, cudaStream_t st) {
-    double r = 0.0;
-    GGF_TRY(ggf_refine_inverse(ctx, cplx, ctx->ch.links, c, p, W, ctx->work, 0, &r, st));
-    ctx->refine_rmax = std::max(ctx->refine_rmax, r);
+ggf_status refine_batch(ggf_ctx* ctx, RefineBatch& b, std::vector<int>& ok, cudaStream_t st) {
+    const int n = b.n;
+    std::vector<int> open(n, 1), one(n), three(n), stepped(n);
+    std::vector<double> r(n), after(n);
+    ok.assign(n, 0);
+    GGF_TRY(ggf_refine_measure(ctx, b, ctx->ch.links, open, r, st));
+    for (double v : r) ctx->refine_rmax = std::max(ctx->refine_rmax, v);
     for (int step = 0; step < 3; ++step) {
-        if (r <= kRefineFloor) { *ok = true; return GGF_OK; }
-        if (!(r <= kRefineTol)) break;
-        double unused = 0.0, after = 0.0;
-        GGF_TRY(ggf_refine_inverse(ctx, cplx, ctx->ch.links, c, p, W, ctx->work, r <= kRefineOne ? 1 : 3, &unused, st));
-        GGF_TRY(ggf_refine_inverse(ctx, cplx, ctx->ch.links, c, p, W, ctx->work, 0, &after, st));
-        ctx->refine_steps += 1;
-        // a step that no longer shrinks the residual has met this matrix's
-        // FP32 floor (the rounded exact inverse has the same residual)
-        if (!(after < 0.5 * r)) { r = std::min(r, after); *ok = r <= kRefineOne; return GGF_OK; }
-        r = after;
+        int n1 = 0, n3 = 0;
+        for (int i = 0; i < n; ++i) {
+            one[i] = three[i] = 0;
+            if (!open[i]) continue;
+            if (r[i] <= kRefineFloor) { ok[i] = 1; open[i] = 0; continue; }
+            if (!(r[i] <= kRefineTol)) { open[i] = 0; continue; }
+            if (r[i] <= kRefineOne) { one[i] = 1; ++n1; } else { three[i] = 1; ++n3; }
+        }
+        if (n1 + n3 == 0) return GGF_OK;
+        if (n1) GGF_TRY(ggf_refine_apply(ctx, b, one, 1, st));
+        if (n3) GGF_TRY(ggf_refine_apply(ctx, b, three, 3, st));
+        for (int i = 0; i < n; ++i) stepped[i] = one[i] | three[i];
+        GGF_TRY(ggf_refine_measure(ctx, b, ctx->ch.links, stepped, after, st));
+        ctx->refine_steps += n1 + n3;
+        for (int i = 0; i < n; ++i) {
+            if (!stepped[i]) continue;
+            // a step that no longer shrinks the residual has met this matrix's
+            // FP32 floor (the rounded exact inverse has the same residual)
+            if (!(after[i] < 0.5 * r[i])) {
+                r[i] = std::min(r[i], after[i]);
+                ok[i] = r[i] <= kRefineOne;
+                open[i] = 0;
+            } else {
+                r[i] = after[i];
+            }
+        }
     }
-    *ok = r <= kRefineOne;
+    for (int i = 0; i < n; ++i)
+        if (open[i]) ok[i] = r[i] <= kRefineOne;
     return GGF_OK;
 }
 
@@ -341,22 +358,32 @@ ggf_status refine_one(ggf_ctx* ctx, bool cplx, int c, int p, float* W, bool* ok,
 // chains whose residual is too large for it are returned in `dense`.
 ggf_status newton_inverse(ggf_ctx* ctx, const std::vector<int>& chains, std::vector<int>& dense, cudaStream_t st) {
     Chains& ch = ctx->ch;
-    const int N = ctx->g.N;
-    const size_t NN = (size_t)N * N;
-    GGF_TRY(ggf_workspace(ctx, ggf_refine_bytes(N, ctx->Kc > 0)));
-    for (int c : chains) {
-        bool ok = true;
-        for (int fam = 0; fam < 2 && ok; ++fam) {
-            const bool cplx = fam == 1;
-            const int npf = cplx ? ctx->Kc : ctx->K;
-            for (int p = 0; p < npf && ok; ++p) {
-                float* W = cplx ? (float*)ch.Wc + ((size_t)c * ctx->Kc + p) * NN * 2
-                                : (float*)ch.Wr + ((size_t)c * ctx->K + p) * NN;
-                GGF_TRY(refine_one(ctx, cplx, c, p, W, &ok, st));
+    std::vector<char> bad(ch.n, 0);
+    for (int fam = 0; fam < 2; ++fam) {
+        const bool cplx = fam == 1;
+        const int npf = cplx ? ctx->Kc : ctx->K;
+        std::vector<int> cfg, pair, block, ok;
+        for (int c : chains)
+            for (int p = 0; p < npf && !bad[c]; ++p) {
+                cfg.push_back(c);
+                pair.push_back(p);
+                block.push_back(c * npf + p);
             }
+        if (cfg.empty()) continue;
+        RefineBatch b;
+        ggf_refine_plan(ctx, cplx, (int)cfg.size(), b);
+        GGF_TRY(ggf_workspace(ctx, b.bytes));
+        for (size_t i0 = 0; i0 < cfg.size(); i0 += b.cap) {
+            const int n = (int)std::min<size_t>(b.cap, cfg.size() - i0);
+            GGF_TRY(ggf_refine_begin(ctx, b, n, cfg.data() + i0, pair.data() + i0, block.data() + i0,
+                                     (float*)(cplx ? ch.Wc : ch.Wr), ctx->work, st));
+            GGF_TRY(refine_batch(ctx, b, ok, st));
+            for (int i = 0; i < n; ++i)
+                if (!ok[i]) bad[cfg[i0 + i]] = 1;
         }
-        if (!ok) dense.push_back(c);
     }
+    for (int c : chains)
+        if (bad[c]) dense.push_back(c);
     GGF_CK(cudaStreamSynchronize(st));
     return GGF_OK;
 }
@@ -1252,19 +1279,19 @@ ggf_status ggf_chains_refine(ggf_ctx* ctx, int chain, int pair, int apply, doubl
         return ggf_fail(ctx, GGF_EINVAL, "bad chains_refine arguments");
     if (ch.opts.precision != GGF_FP32) return ggf_fail(ctx, GGF_EINVAL, "chains_refine: FP32 chains only");
     cudaSetDevice(ctx->device);
-    const int N = ctx->g.N;
-    const size_t NN = (size_t)N * N;
     const bool cplx = pair >= ctx->K;
     const int p = cplx ? pair - ctx->K : pair;
-    float* W = cplx ? (float*)ch.Wc + ((size_t)chain * ctx->Kc + p) * NN * 2
-                    : (float*)ch.Wr + ((size_t)chain * ctx->K + p) * NN;
+    const int block = chain * (cplx ? ctx->Kc : ctx->K) + p;
     GGF_CK(cudaDeviceSynchronize());
-    GGF_TRY(ggf_workspace(ctx, ggf_refine_bytes(N, cplx)));
-    GGF_TRY(ggf_refine_inverse(ctx, cplx, ch.links, chain, p, W, ctx->work, 0, rmax, 0));
-    if (apply && *rmax <= kRefineTol) {
-        double unused = 0.0;
-        GGF_TRY(ggf_refine_inverse(ctx, cplx, ch.links, chain, p, W, ctx->work, *rmax <= kRefineOne ? 1 : 3, &unused, 0));
-    }
+    RefineBatch b;
+    ggf_refine_plan(ctx, cplx, 1, b);
+    GGF_TRY(ggf_workspace(ctx, b.bytes));
+    GGF_TRY(ggf_refine_begin(ctx, b, 1, &chain, &p, &block, (float*)(cplx ? ch.Wc : ch.Wr), ctx->work, 0));
+    const std::vector<int> act(1, 1);
+    std::vector<double> r(1);
+    GGF_TRY(ggf_refine_measure(ctx, b, ch.links, act, r, 0));
+    *rmax = r[0];
+    if (apply && *rmax <= kRefineTol) GGF_TRY(ggf_refine_apply(ctx, b, act, *rmax <= kRefineOne ? 1 : 3, 0));
     GGF_CK(cudaDeviceSynchronize());
     return GGF_OK;
 }

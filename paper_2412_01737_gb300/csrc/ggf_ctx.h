@@ -186,6 +186,25 @@ void ggf_free_consts(ggf_ctx* ctx);
 ggf_status ggf_build_constants(ggf_ctx* ctx, const double* gamma_site, int K,
                                const double* gamma_bond, const double* lambda);
 
+// Newton refinement of FP32 inverses, a batch of matrices of one family at a
+// time (k_refine.cu): plan, begin, then measure and apply in turns.
+struct RefineBatch {
+    bool cplx = false, own_ps = false;
+    int cap = 0, n = 0;              // matrices the batch holds, and has
+    size_t bytes = 0;                // workspace
+    float* W = nullptr;              // blocks of N x N
+    float* Pan = nullptr;
+    unsigned char* ps = nullptr;     // pre-split operands, or null
+    int *d_cfg = nullptr, *d_pair = nullptr, *d_block = nullptr, *d_pend = nullptr;
+    unsigned* d_rmax = nullptr;
+};
+void ggf_refine_plan(ggf_ctx* ctx, bool cplx, int items, RefineBatch& b);
+ggf_status ggf_refine_begin(ggf_ctx* ctx, RefineBatch& b, int n, const int* cfg, const int* pair, const int* block,
+                            float* W, void* ws, cudaStream_t st);
+ggf_status ggf_refine_measure(ggf_ctx* ctx, RefineBatch& b, const void* d_links, const std::vector<int>& act,
+                              std::vector<double>& rmax, cudaStream_t st);
+ggf_status ggf_refine_apply(ggf_ctx* ctx, RefineBatch& b, const std::vector<int>& act, int terms, cudaStream_t st);
+
 // linear algebra drivers (k_linalg.cu)
 // Assemble FP64 M for items (cfg index, pair index) into dst (item-major, N*N each).
 // real_family: pairs 0..K-1 (double) else complex pairs (cxd).

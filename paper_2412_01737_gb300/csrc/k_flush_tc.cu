@@ -178,18 +178,25 @@ __device__ __forceinline__ void prefetch_l2(const void* ptr, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ptr), "r"(bytes) : "memory");
 }
 
+// Index of tile t's matrix in W: consecutive (chain, pair) blocks, or the
+// block that wmap names (batches of matrices picked from W).
+__device__ __forceinline__ size_t w_block(const TileInfo& t, const int* wmap, int fam_pairs) {
+    const size_t i = (size_t)t.c * fam_pairs + t.p;
+    return wmap ? (size_t)wmap[i] : i;
+}
+
 // Bulk L2 prefetch of row e of tile t's block of W (the columns j0 .. j0 + 127
 // of that row, one contiguous segment).  The bulk copy needs a 16-byte
 // aligned start and a length that is a multiple of 16 bytes; rows of other
 // widths (possible only in the self-test) are not prefetched.
 template <int ROWS, bool CPLX>
-__device__ __forceinline__ void prefetch_tile_row(const TileInfo& t, const float* W, int fam_pairs, int N, int rowW,
-                                                  int e) {
+__device__ __forceinline__ void prefetch_tile_row(const TileInfo& t, const float* W, const int* wmap, int fam_pairs,
+                                                  int N, int rowW, int e) {
     const int i = t.i0 + e;
     if (e >= ROWS || i >= N) return;
     const int ncol = min(128, N - t.j0);
     if ((rowW & 3) || ((ncol * (CPLX ? 8 : 4)) & 15)) return;
-    const float* ptr = W + ((size_t)t.c * fam_pairs + t.p) * (size_t)N * rowW + (size_t)i * rowW + (CPLX ? 2 : 1) * t.j0;
+    const float* ptr = W + w_block(t, wmap, fam_pairs) * (size_t)N * rowW + (size_t)i * rowW + (CPLX ? 2 : 1) * t.j0;
     prefetch_l2(ptr, (uint32_t)ncol * (CPLX ? 8u : 4u));
 }
 
@@ -334,7 +341,7 @@ __device__ __forceinline__ void stage_next(StageIter& it, long long total, int t
 template <bool CPLX, bool PP>
 __device__ __forceinline__ void epilogue_tiles(int warp, int ew, int lane, long long total, int tiles_i, int tiles_j,
                                                int fam_pairs, const int* pend, int R, int upper, int N, float* W,
-                                               uint32_t tbase, uint64_t* bar_accf, uint64_t* bar_acce,
+                                               const int* wmap, uint32_t tbase, uint64_t* bar_accf, uint64_t* bar_acce,
                                                volatile int& s_fail, int* err) {
     constexpr int ROWS = CPLX ? 128 : 256;        // W rows per tile
     const int rowW = CPLX ? 2 * N : N;            // floats per W row
@@ -351,19 +358,19 @@ __device__ __forceinline__ void epilogue_tiles(int warp, int ew, int lane, long 
         const TileInfo t = decode_tile<ROWS>(tile, tiles_i, tiles_j, fam_pairs, pend, R, upper);
         if (t.K == 0) continue;
         if (first) {
-            prefetch_tile_row<ROWS, CPLX>(t, W, fam_pairs, N, rowW, e_row);
+            prefetch_tile_row<ROWS, CPLX>(t, W, wmap, fam_pairs, N, rowW, e_row);
             first = false;
         }
         for (long long tn = tile + gridDim.x; tn < total; tn += gridDim.x) {
             const TileInfo u = decode_tile<ROWS>(tn, tiles_i, tiles_j, fam_pairs, pend, R, upper);
             if (u.K == 0) continue;
-            prefetch_tile_row<ROWS, CPLX>(u, W, fam_pairs, N, rowW, e_row);
+            prefetch_tile_row<ROWS, CPLX>(u, W, wmap, fam_pairs, N, rowW, e_row);
             break;
         }
         if (!mbar_wait_bounded(smem_u32(&bar_accf[b]), ph, &s_fail)) { raise_fail(&s_fail, err); break; }
         asm volatile("tcgen05.fence::after_thread_sync;");
         const int j = t.j0 + q * 32 + lane;
-        float* Wp = W + ((size_t)t.c * fam_pairs + t.p) * (size_t)N * rowW;
+        float* Wp = W + w_block(t, wmap, fam_pairs) * (size_t)N * rowW;
         const uint32_t tl = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256);
         if (!CPLX) {
             // rows i0 + half*RG + 16 cb + k  <->  TMEM column half*RG + 16 cb + k (RG = 256 / EPI_PARTS)
@@ -545,8 +552,8 @@ __device__ __forceinline__ void mma_tiles(long long total, int tiles_i, int tile
 // TERMS = 3: FP32-accurate TF32 split; TERMS = 1: one TF32 product.
 template <bool CPLX, int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-flush_tc_kernel(int N, int fam_pairs, int n_chains, float* W, const float* Pan, const int* pend, int R, int KRM,
-                int upper, int* err) {
+flush_tc_kernel(int N, int fam_pairs, int n_chains, float* W, const int* wmap, const float* Pan, const int* pend, int R,
+                int KRM, int upper, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar_full[STAGES], bar_empty[STAGES], bar_accf[2], bar_acce[2], bar_done;
     __shared__ uint32_t tmem_slot;
@@ -620,7 +627,7 @@ flush_tc_kernel(int N, int fam_pairs, int n_chains, float* W, const float* Pan, 
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp < MMA_WARP) {
-        epilogue_tiles<CPLX, false>(warp, warp - NPROD, lane, total, tiles_i, tiles_j, fam_pairs, pend, R, upper, N, W, tbase,
+        epilogue_tiles<CPLX, false>(warp, warp - NPROD, lane, total, tiles_i, tiles_j, fam_pairs, pend, R, upper, N, W, wmap, tbase,
                              bar_accf, bar_acce, s_fail, err);
     } else if (lane == 0) {
         mma_tiles<CPLX, TERMS, STAGES>(total, tiles_i, tiles_j, fam_pairs, pend, R, upper, tbase, base, bar_full,
@@ -726,8 +733,8 @@ __global__ void __launch_bounds__(256) ps_split_kernel(int N, int fam_pairs, int
 // them to the wave), operands from the wave's pre-split blocks ps.
 template <bool CPLX, int TERMS>
 __global__ void __launch_bounds__(PS_THREADS, 1)
-flush_ps_kernel(int N, int fam_pairs, int n_chains, float* W, const unsigned char* ps, const int* pend, int R, int KRM,
-                int* err) {
+flush_ps_kernel(int N, int fam_pairs, int n_chains, float* W, const int* wmap, const unsigned char* ps, const int* pend,
+                int R, int KRM, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar_full[PS_STAGES], bar_empty[PS_STAGES], bar_accf[2], bar_acce[2], bar_done;
     __shared__ uint32_t tmem_slot;
@@ -765,7 +772,7 @@ flush_ps_kernel(int N, int fam_pairs, int n_chains, float* W, const unsigned cha
     const uint32_t tbase = tmem_slot;
 
     if (warp < NEPI) {
-        epilogue_tiles<CPLX, GGF_FLUSH_EPI_PP != 0>(warp, warp, lane, total, tiles_i, tiles_j, fam_pairs, pend, R, 0, N, W, tbase, bar_accf,
+        epilogue_tiles<CPLX, GGF_FLUSH_EPI_PP != 0>(warp, warp, lane, total, tiles_i, tiles_j, fam_pairs, pend, R, 0, N, W, wmap, tbase, bar_accf,
                              bar_acce, s_fail, err);
     } else if (warp == PS_COPY_WARP) {
         if (lane == 0) {
@@ -841,7 +848,8 @@ ggf_status ggf_prepare_flush_tc(ggf_ctx* ctx) {
 namespace {
 
 ggf_status launch_flush_tc(ggf_ctx* ctx, bool cplx, int N, int fam_pairs, int n_chains, float* W, const float* Pan,
-                           const int* pend, int R, int KRM, bool upper, int* err, cudaStream_t st, int terms = 3) {
+                           const int* pend, int R, int KRM, bool upper, int* err, cudaStream_t st, int terms = 3,
+                           const int* wmap = nullptr) {
     if (fam_pairs == 0 || n_chains == 0) return GGF_OK;
     if (KRM < 1) return ggf_fail(ctx, GGF_EINVAL, "tensor-core flush: empty panel");
     const int rows = cplx ? 128 : 256;
@@ -851,16 +859,16 @@ ggf_status launch_flush_tc(ggf_ctx* ctx, bool cplx, int N, int fam_pairs, int n_
     GGF_TRY(ggf_prepare_flush_tc(ctx));
     const int up = upper ? 1 : 0;
     if (cplx && terms == 1)
-        flush_tc_kernel<true, 1><<<(unsigned)grid, TC_THREADS, smem_bytes(true), st>>>(N, fam_pairs, n_chains, W, Pan,
+        flush_tc_kernel<true, 1><<<(unsigned)grid, TC_THREADS, smem_bytes(true), st>>>(N, fam_pairs, n_chains, W, wmap, Pan,
                                                                                        pend, R, KRM, up, err);
     else if (cplx)
-        flush_tc_kernel<true, 3><<<(unsigned)grid, TC_THREADS, smem_bytes(true), st>>>(N, fam_pairs, n_chains, W, Pan,
+        flush_tc_kernel<true, 3><<<(unsigned)grid, TC_THREADS, smem_bytes(true), st>>>(N, fam_pairs, n_chains, W, wmap, Pan,
                                                                                        pend, R, KRM, up, err);
     else if (terms == 1)
-        flush_tc_kernel<false, 1><<<(unsigned)grid, TC_THREADS, smem_bytes(false), st>>>(N, fam_pairs, n_chains, W, Pan,
+        flush_tc_kernel<false, 1><<<(unsigned)grid, TC_THREADS, smem_bytes(false), st>>>(N, fam_pairs, n_chains, W, wmap, Pan,
                                                                                          pend, R, KRM, up, err);
     else
-        flush_tc_kernel<false, 3><<<(unsigned)grid, TC_THREADS, smem_bytes(false), st>>>(N, fam_pairs, n_chains, W, Pan,
+        flush_tc_kernel<false, 3><<<(unsigned)grid, TC_THREADS, smem_bytes(false), st>>>(N, fam_pairs, n_chains, W, wmap, Pan,
                                                                                          pend, R, KRM, up, err);
     GGF_CK(cudaGetLastError());
     return GGF_OK;
@@ -931,7 +939,7 @@ namespace {
 // One wave (chains c0 .. c0 + n - 1 of W, Pan and pend): split, then flush.
 template <bool CPLX, int TERMS = 3>
 ggf_status flush_wave(ggf_ctx* ctx, int N, int R, int fam_pairs, int c0, int n, float* W, const float* Pan,
-                      const int* pend, int KRM, unsigned char* ps, cudaStream_t st) {
+                      const int* pend, int KRM, unsigned char* ps, cudaStream_t st, const int* wmap = nullptr) {
     const int sms = ctx->n_sms > 0 ? ctx->n_sms : 152;
     const long long items = (long long)n * fam_pairs * panel_rows(N) * (panel_cols(KRM) / 4);
     const unsigned sgrid = (unsigned)std::min<long long>((items + 255) / 256, (long long)sms * 8);
@@ -940,7 +948,7 @@ ggf_status flush_wave(ggf_ctx* ctx, int N, int R, int fam_pairs, int c0, int n, 
     const long long total = (long long)n * fam_pairs * ((N + rows - 1) / rows) * ((N + 127) / 128);
     const size_t wsz = (size_t)N * N * (CPLX ? 2 : 1);
     flush_ps_kernel<CPLX, TERMS><<<(unsigned)std::min<long long>(total, sms), PS_THREADS, ps_smem_bytes(), st>>>(
-        N, fam_pairs, n, W + (size_t)c0 * fam_pairs * wsz, ps, pend + c0, R, KRM, ctx->d_err);
+        N, fam_pairs, n, W + (size_t)c0 * fam_pairs * wsz, wmap, ps, pend + c0, R, KRM, ctx->d_err);
     GGF_CK(cudaGetLastError());
     return GGF_OK;
 }
@@ -980,22 +988,24 @@ ggf_status ggf_flush_tc(ggf_ctx* ctx, cudaStream_t st, int* launches) {
     return GGF_OK;
 }
 
-// W -= U V for one N x N matrix with rank-K panels (K = pend[0] * R, panel
-// column count KRM), terms = 3 (FP32-accurate TF32 split) or 1 (one TF32
-// product).  Used by the Newton refinement of the inverses (k_refine.cu).
-ggf_status ggf_flush_tc_one(ggf_ctx* ctx, bool cplx, int N, float* W, const float* Pan, const int* pend, int R,
-                            int KRM, int terms, cudaStream_t st) {
-    // through the chains' pre-split scratch when it holds this product's
-    // operands (outside a sweep it is free), else splitting per tile
-    const Chains& ch = ctx->ch;
-    if (ch.ps && ps_bytes(cplx, N, KRM, 1, 1) <= ch.ps_bytes) {
-        GGF_TRY(ggf_prepare_flush_tc(ctx));
-        if (cplx) return terms == 1 ? flush_wave<true, 1>(ctx, N, R, 1, 0, 1, W, Pan, pend, KRM, ch.ps, st)
-                                    : flush_wave<true, 3>(ctx, N, R, 1, 0, 1, W, Pan, pend, KRM, ch.ps, st);
-        return terms == 1 ? flush_wave<false, 1>(ctx, N, R, 1, 0, 1, W, Pan, pend, KRM, ch.ps, st)
-                          : flush_wave<false, 3>(ctx, N, R, 1, 0, 1, W, Pan, pend, KRM, ch.ps, st);
-    }
-    return launch_flush_tc(ctx, cplx, N, 1, 1, W, Pan, pend, R, KRM, false, ctx->d_err, st, terms == 1 ? 1 : 3);
+// Bytes of pre-split operands of one rank-N product of a family.
+size_t ggf_flush_ps_item_bytes(ggf_ctx* ctx, bool cplx) { return ps_bytes(cplx, ctx->g.N, ctx->g.N, 1, 1); }
+
+// W -= U V for n N x N matrices (blocks wmap[i] of W) with rank-N panels of
+// their own (pend[i] * 8 columns pending, 0: left alone), terms = 3
+// (FP32-accurate TF32 split) or 1 (one TF32 product), through the pre-split
+// operands ps (ggf_flush_ps_item_bytes each), or splitting per tile where ps
+// is null.  Used by the Newton refinement of the inverses (k_refine.cu).
+ggf_status ggf_flush_tc_items(ggf_ctx* ctx, bool cplx, int n, float* W, const int* wmap, const float* Pan,
+                              const int* pend, int terms, unsigned char* ps, cudaStream_t st) {
+    const int N = ctx->g.N;
+    GGF_TRY(ggf_prepare_flush_tc(ctx));
+    if (!ps)
+        return launch_flush_tc(ctx, cplx, N, 1, n, W, Pan, pend, 8, N, false, ctx->d_err, st, terms == 1 ? 1 : 3, wmap);
+    if (cplx) return terms == 1 ? flush_wave<true, 1>(ctx, N, 8, 1, 0, n, W, Pan, pend, N, ps, st, wmap)
+                                : flush_wave<true, 3>(ctx, N, 8, 1, 0, n, W, Pan, pend, N, ps, st, wmap);
+    return terms == 1 ? flush_wave<false, 1>(ctx, N, 8, 1, 0, n, W, Pan, pend, N, ps, st, wmap)
+                      : flush_wave<false, 3>(ctx, N, 8, 1, 0, n, W, Pan, pend, N, ps, st, wmap);
 }
 
 extern "C" ggf_status ggf_selftest_flush(ggf_ctx* ctx, int cplx, int N, int rank, double* max_rel_err) {

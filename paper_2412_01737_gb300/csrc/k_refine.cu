@@ -9,13 +9,20 @@
 // FP32 floor of computing R; for a residual below 1e-4 one TF32 product per
 // term suffices (its 2^-11 rounding of a correction that small is below the
 // FP32 rounding of W), larger residuals take the three-product split.
+//
+// Matrices are refined in batches (of one family, from any chains): one
+// residual launch, one read-back of the largest residuals and one product
+// launch for all of them.  One matrix at a time, a refresh of 1 023 chains of
+// 8 x 8 Z2 (N = 512) took 74 ms of kernels of 10 to 49 us that left most of
+// the chip idle, and 37 ms of gaps between them; in batches about 6 ms together.
 #include <algorithm>
-#include <cstring>
+#include <vector>
 #include "ggf_ctx.h"
 #include "ggf_geom.cuh"
 
-ggf_status ggf_flush_tc_one(ggf_ctx* ctx, bool cplx, int N, float* W, const float* Pan, const int* pend, int R,
-                            int KRM, int nprod, cudaStream_t st);
+ggf_status ggf_flush_tc_items(ggf_ctx* ctx, bool cplx, int n, float* W, const int* wmap, const float* Pan,
+                              const int* pend, int terms, unsigned char* ps, cudaStream_t st);
+size_t ggf_flush_ps_item_bytes(ggf_ctx* ctx, bool cplx);
 
 namespace {
 
@@ -30,12 +37,16 @@ template <> struct RefTy<cxd> { typedef cxf S; };
 __device__ __forceinline__ float to_s(double v) { return (float)v; }
 __device__ __forceinline__ cxf to_s(cxd v) { return {(float)v.x, (float)v.y}; }
 
-// V^T panel (chunk-major, row = output column j, rank = output row q) of
-// -R = M W - I for rows q0 .. q0 + 7 and columns j0 .. j0 + 255; the largest
-// |R| entry goes to rmax (float bits, non-negative values compare as ints).
+// V^T panels (chunk-major, row = output column j, rank = output row q) of
+// -R = M W - I for rows q0 .. q0 + 7 of every item (grid.y) with act != 0: the
+// matrix M of (cfg, pair) and block wmap of W; the largest |R| entry goes to
+// rmax[item] (float bits, non-negative values compare as ints).  The
+// coefficients of the eight rows (FP64 twists) are formed once and serve every
+// column block.
 template <class T>
-__global__ void __launch_bounds__(RT) resid_kernel(DevConst dc, const void* links, int cfg, int pair, const float* W,
-                                                   float* Vt, size_t NK, int NP, unsigned* rmax) {
+__global__ void __launch_bounds__(RT) resid_kernel(DevConst dc, const void* links, const int* cfgs, const int* pairs,
+                                                   const int* wmap, const int* act, const float* Wbase, float* Pan,
+                                                   size_t NK, int NP, unsigned* rmax) {
     typedef typename RefTy<T>::S S;
     constexpr bool CPLX = Sc<T>::CPLX;
     __shared__ int cols[MAXC];
@@ -43,9 +54,12 @@ __global__ void __launch_bounds__(RT) resid_kernel(DevConst dc, const void* link
     __shared__ int ncol;
     __shared__ float red[RT / 32];
     const Geometry& g = dc.g;
-    const int N = g.N, B = g.B;
-    const int q0 = blockIdx.y * RB;
-    const int j = blockIdx.x * RT + threadIdx.x;
+    const int N = g.N, B = g.B, item = blockIdx.y;
+    if (!act[item]) return;
+    const int cfg = cfgs[item], pair = pairs[item];
+    const float* W = Wbase + (size_t)wmap[item] * N * N * (CPLX ? 2 : 1);
+    float* Vt = Pan + ((size_t)item * 2 + 1) * (CPLX ? 2 : 1) * NK;
+    const int q0 = blockIdx.x * RB;
     if (threadIdx.x == 0) {
         // columns: the site of q0 .. q0 + 7, then the partner ends of their links
         int n = 0;
@@ -79,7 +93,7 @@ __global__ void __launch_bounds__(RT) resid_kernel(DevConst dc, const void* link
     }
     __syncthreads();
     float mx = 0.f;
-    if (j < N) {
+    for (int j = threadIdx.x; j < N; j += RT) {
         S acc[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) acc[r] = S{};
@@ -139,16 +153,18 @@ __global__ void __launch_bounds__(RT) resid_kernel(DevConst dc, const void* link
     if (threadIdx.x == 0) {
         float m = 0.f;
         for (int w = 0; w < RT / 32; ++w) m = fmaxf(m, red[w]);
-        atomicMax(rmax, __float_as_uint(m));
+        atomicMax(rmax + item, __float_as_uint(m));
     }
 }
 
-// U panel = W: element (row i, rank q) <- W[i][q], eight rank columns per thread
+// U panels = W of the items with pend != 0: element (row i, rank q) <- W[i][q], eight rank columns per thread
 template <bool CPLX>
-__global__ void upanel_kernel(int N, const float* W, float* U, size_t NK, int NP) {
+__global__ void upanel_kernel(int N, const int* wmap, const int* pend, const float* Wbase, float* Pan, size_t NK, int NP) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int q0 = blockIdx.y * 8;
-    if (i >= N) return;
+    const int q0 = blockIdx.y * 8, item = blockIdx.z;
+    if (i >= N || !pend[item]) return;
+    const float* W = Wbase + (size_t)wmap[item] * N * N * (CPLX ? 2 : 1);
+    float* U = Pan + (size_t)item * 2 * (CPLX ? 2 : 1) * NK;
     float* dst = U + pidx(i, q0, NP);
     if (!CPLX) {
         const float* src = W + (size_t)i * N + q0;
@@ -169,55 +185,107 @@ __global__ void upanel_kernel(int N, const float* W, float* U, size_t NK, int NP
     }
 }
 
-__global__ void set_int(int* p, int v) { *p = v; }
+}  // namespace
+
+// ---- batches of matrices of one family -----------------------------------------
+
+namespace {
+
+size_t panel_bytes(int N, bool cplx) { return panel_plane(N, N) * (cplx ? 4 : 2) * sizeof(float); }
+
+size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
 
-// Bytes of the refinement workspace for one matrix (U and V^T panels, rank N).
-size_t ggf_refine_bytes(int N, bool cplx) {
-    return panel_plane(N, N) * (cplx ? 4 : 2) * sizeof(float) + 256;
+// Plans a batch of at most `items` matrices: their number (at least one), the
+// workspace they need, and whether their pre-split operands go into the
+// chains' flush scratch (idle outside a sweep) or into the workspace.  A batch
+// stays within 1 GiB and a quarter of the free memory.
+void ggf_refine_plan(ggf_ctx* ctx, bool cplx, int items, RefineBatch& b) {
+    const int N = ctx->g.N;
+    const Chains& ch = ctx->ch;
+    const size_t pb = panel_bytes(N, cplx), psb = ggf_flush_ps_item_bytes(ctx, cplx);
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    const size_t budget = std::max(ctx->work_bytes, std::min<size_t>((size_t)1 << 30, free_b / 4));
+    b.cplx = cplx;
+    size_t n;
+    if (ch.ps && psb <= ch.ps_bytes) {
+        n = std::min(ch.ps_bytes / psb, budget / pb);
+        b.own_ps = false;
+        b.ps = ch.ps;
+    } else {
+        n = budget / (pb + psb);
+        b.own_ps = n > 0;
+        b.ps = nullptr;                        // n = 0: operands are split per tile
+    }
+    b.cap = (int)std::max<size_t>(1, std::min<size_t>({n, (size_t)items, (size_t)32768}));
+    b.bytes = up256(pb * b.cap) + (b.own_ps ? up256(psb * b.cap) : 0) + 5 * up256((size_t)b.cap * sizeof(int));
 }
 
-// Newton refinement of W (FP32, N x N, real or interleaved complex) for the
-// matrix M of (cfg, pair-within-family), in two calls:
-//   terms = 0: measure, *rmax = max |I - M W| over the entries, and keep
-//              -R = M W - I in the workspace (synchronises the stream);
-//   terms = 1 or 3: apply W <- W + W R with the R the last measure left (one
-//              TF32 product, or the FP32-accurate three-product split).
-// ws holds ggf_refine_bytes(N, cplx) bytes and must not change in between.
-ggf_status ggf_refine_inverse(ggf_ctx* ctx, bool cplx, const void* d_links, int cfg, int pair, float* W, void* ws,
-                              int terms, double* rmax, cudaStream_t st) {
-    const Geometry& g = ctx->g;
-    const int N = g.N, NP = panel_rows(N);
-    if (N % 8) return ggf_fail(ctx, GGF_EINVAL, "refinement needs N divisible by 8");
+// Lays the batch out in ws (b.bytes) and uploads its items: configuration and
+// pair of M, block of W.
+ggf_status ggf_refine_begin(ggf_ctx* ctx, RefineBatch& b, int n, const int* cfg, const int* pair, const int* block,
+                            float* W, void* ws, cudaStream_t st) {
+    const int N = ctx->g.N;
+    unsigned char* q = (unsigned char*)ws;
+    auto take = [&](size_t bytes) { unsigned char* p = q; q += up256(bytes); return p; };
+    b.n = n;
+    b.W = W;
+    b.Pan = (float*)take(panel_bytes(N, b.cplx) * b.cap);
+    if (b.own_ps) b.ps = take(ggf_flush_ps_item_bytes(ctx, b.cplx) * b.cap);
+    const size_t ib = (size_t)b.cap * sizeof(int);
+    b.d_cfg = (int*)take(ib);
+    b.d_pair = (int*)take(ib);
+    b.d_block = (int*)take(ib);
+    b.d_pend = (int*)take(ib);
+    b.d_rmax = (unsigned*)take(ib);
+    GGF_CK(cudaMemcpyAsync(b.d_cfg, cfg, n * sizeof(int), cudaMemcpyHostToDevice, st));
+    GGF_CK(cudaMemcpyAsync(b.d_pair, pair, n * sizeof(int), cudaMemcpyHostToDevice, st));
+    GGF_CK(cudaMemcpyAsync(b.d_block, block, n * sizeof(int), cudaMemcpyHostToDevice, st));
+    return GGF_OK;
+}
+
+// max |I - M W| of the items with act[i] != 0 into rmax[i]; keeps their -R =
+// M W - I for the next product.  Synchronises the stream.
+ggf_status ggf_refine_measure(ggf_ctx* ctx, RefineBatch& b, const void* d_links, const std::vector<int>& act,
+                              std::vector<double>& rmax, cudaStream_t st) {
+    const int N = ctx->g.N, NP = panel_rows(N);
     const size_t NK = panel_plane(N, N);
-    float* Pan = (float*)ws;
-    float* U = Pan;
-    float* Vt = Pan + (cplx ? 2 : 1) * NK;
-    unsigned* d_rmax = (unsigned*)(Pan + (cplx ? 4 : 2) * NK);
-    int* d_pend = (int*)(d_rmax + 1);
-    if (terms != 0) {
-        dim3 ug((N + 255) / 256, N / 8);
-        if (cplx) upanel_kernel<true><<<ug, 256, 0, st>>>(N, W, U, NK, NP);
-        else upanel_kernel<false><<<ug, 256, 0, st>>>(N, W, U, NK, NP);
-        set_int<<<1, 1, 0, st>>>(d_pend, N / 8);
-        GGF_CK(cudaGetLastError());
-        ctx->launches += 3;
-        return ggf_flush_tc_one(ctx, cplx, N, W, Pan, d_pend, 8, N, terms, st);
-    }
-    GGF_CK(cudaMemsetAsync(d_rmax, 0, sizeof(unsigned), st));
-    dim3 grid((N + RT - 1) / RT, (N + RB - 1) / RB);
-    if (cplx)
-        resid_kernel<cxd><<<grid, RT, 0, st>>>(ctx->dc(), d_links, cfg, pair, W, Vt, NK, NP, d_rmax);
+    GGF_CK(cudaMemcpyAsync(b.d_pend, act.data(), b.n * sizeof(int), cudaMemcpyHostToDevice, st));
+    GGF_CK(cudaMemsetAsync(b.d_rmax, 0, b.n * sizeof(unsigned), st));
+    dim3 grid((N + RB - 1) / RB, b.n);
+    if (b.cplx)
+        resid_kernel<cxd><<<grid, RT, 0, st>>>(ctx->dc(), d_links, b.d_cfg, b.d_pair, b.d_block, b.d_pend, b.W, b.Pan, NK,
+                                               NP, b.d_rmax);
     else
-        resid_kernel<double><<<grid, RT, 0, st>>>(ctx->dc(), d_links, cfg, pair, W, Vt, NK, NP, d_rmax);
+        resid_kernel<double><<<grid, RT, 0, st>>>(ctx->dc(), d_links, b.d_cfg, b.d_pair, b.d_block, b.d_pend, b.W, b.Pan,
+                                                  NK, NP, b.d_rmax);
     GGF_CK(cudaGetLastError());
     ctx->launches += 1;
-    unsigned hb = 0;
-    GGF_CK(cudaMemcpyAsync(&hb, d_rmax, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    std::vector<float> h(b.n);
+    GGF_CK(cudaMemcpyAsync(h.data(), b.d_rmax, b.n * sizeof(float), cudaMemcpyDeviceToHost, st));
     GGF_CK(cudaStreamSynchronize(st));
-    float hr;
-    std::memcpy(&hr, &hb, sizeof(float));
-    *rmax = hr;
+    for (int i = 0; i < b.n; ++i)
+        if (act[i]) rmax[i] = h[i];
+    return GGF_OK;
+}
+
+// W <- W + W R of the items with act[i] != 0, with the R of the last measure:
+// one TF32 product, or (terms = 3) the FP32-accurate three-product split.
+ggf_status ggf_refine_apply(ggf_ctx* ctx, RefineBatch& b, const std::vector<int>& act, int terms, cudaStream_t st) {
+    const int N = ctx->g.N, NP = panel_rows(N);
+    if (N % 8) return ggf_fail(ctx, GGF_EINVAL, "refinement needs N divisible by 8");
+    const size_t NK = panel_plane(N, N);
+    std::vector<int> pend(b.n);
+    for (int i = 0; i < b.n; ++i) pend[i] = act[i] ? N / 8 : 0;
+    GGF_CK(cudaMemcpyAsync(b.d_pend, pend.data(), b.n * sizeof(int), cudaMemcpyHostToDevice, st));
+    dim3 ug((N + 255) / 256, N / 8, b.n);
+    if (b.cplx) upanel_kernel<true><<<ug, 256, 0, st>>>(N, b.d_block, b.d_pend, b.W, b.Pan, NK, NP);
+    else upanel_kernel<false><<<ug, 256, 0, st>>>(N, b.d_block, b.d_pend, b.W, b.Pan, NK, NP);
+    GGF_CK(cudaGetLastError());
+    ctx->launches += 3;
+    GGF_TRY(ggf_flush_tc_items(ctx, b.cplx, b.n, b.W, b.d_block, b.Pan, b.d_pend, terms, b.ps, st));
+    GGF_CK(cudaStreamSynchronize(st));     // pend is read by the copy above
     return GGF_OK;
 }
