@@ -16,6 +16,10 @@ size_t ggf_factor_tmp_bytes(int n, int batch);
 // r ends at most kRefineOne (a matrix whose FP32 floor lies above
 // kRefineFloor stalls there), else the chain is refactored by Gauss-Jordan.
 static const double kRefineFloor = 4e-6, kRefineOne = 1e-4, kRefineTol = 5e-2;
+bool ggf_lattice_inverse_use(const ggf_ctx* ctx);
+int ggf_lattice_inverse_plan(ggf_ctx* ctx, bool cplx, int items, size_t budget, size_t& bytes);
+ggf_status ggf_lattice_inverse(ggf_ctx* ctx, bool cplx, int n, const int* cfg, const int* pair, const void* d_links,
+                               std::vector<char>& ok, void** result, int** dev_cfg, int** dev_pair, cudaStream_t st);
 ggf_status ggf_link_step(ggf_ctx* ctx, int link, cudaStream_t st);
 ggf_status ggf_observe(ggf_ctx* ctx, double* d_obs, cudaStream_t st);
 ggf_status ggf_mark_refresh(ggf_ctx* ctx, cudaStream_t st);
@@ -254,6 +258,25 @@ __global__ void status_kernel(int n, int P, const cxd* ell, const double* drift,
     status[c] = bad ? GGF_ESINGULAR : (tol > 0.0 && !(drift[c] <= tol)) ? GGF_EDRIFT : GGF_OK;
 }
 
+// Items of a batch into the chains' W storage.
+ggf_status place_inverses(ggf_ctx* ctx, bool cplx, int n, const int* d_chain, const int* d_pair, const void* A,
+                          cudaStream_t st) {
+    Chains& ch = ctx->ch;
+    const int N = ctx->g.N, npf = cplx ? ctx->Kc : ctx->K;
+    const bool fp64 = ch.opts.precision == GGF_FP64;
+    dim3 grid((unsigned)(((size_t)N * N + 255) / 256), n);
+    if (!cplx) {
+        if (fp64) scatter_kernel<double><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, false, (double*)ch.Wr);
+        else scatter_kernel<float><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, false, (float*)ch.Wr);
+    } else {
+        if (fp64) scatter_kernel<cxd><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, true, (cxd*)ch.Wc);
+        else scatter_kernel<cxf><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, true, (cxf*)ch.Wc);
+    }
+    GGF_CK(cudaGetLastError());
+    ctx->launches += 1;
+    return GGF_OK;
+}
+
 // FP64 Gauss-Jordan inverses of the listed chains' M_nm(G), converted into
 // the chains' W storage.
 ggf_status dense_inverse(ggf_ctx* ctx, const std::vector<int>& chains, cudaStream_t st) {
@@ -294,21 +317,51 @@ ggf_status dense_inverse(ggf_ctx* ctx, const std::vector<int>& chains, cudaStrea
             GGF_CK(cudaMemcpyAsync(d_pair, hp.data(), items * sizeof(int), cudaMemcpyHostToDevice, st));
             GGF_TRY(ggf_assemble(ctx, !cplx, items, d_chain, d_pair, ch.links, A, st));
             GGF_TRY(ggf_invert_batched(ctx, cplx, N, items, A, d_logdet, ftmp, st));
-            dim3 grid((unsigned)((NN + 255) / 256), items);
-            if (!cplx) {
-                if (fp64) scatter_kernel<double><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, false, (double*)ch.Wr);
-                else scatter_kernel<float><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, false, (float*)ch.Wr);
-            } else {
-                if (fp64) scatter_kernel<cxd><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, true, (cxd*)ch.Wc);
-                else scatter_kernel<cxf><<<grid, 256, 0, st>>>(N, npf, d_chain, d_pair, A, true, (cxf*)ch.Wc);
-            }
+            GGF_TRY(place_inverses(ctx, cplx, items, d_chain, d_pair, A, st));
             count_singular_kernel<<<(items + 127) / 128, 128, 0, st>>>(items, d_chain, d_logdet, ch.counters,
                                                                        ch.flags);
-            ctx->launches += 2;
+            ctx->launches += 1;
             GGF_CK(cudaGetLastError());
             GGF_CK(cudaStreamSynchronize(st));  // hc/hp are reused by the next chunk
         }
     }
+    return GGF_OK;
+}
+
+// FP64 inverses of the listed chains along the lattice (k_inverse.cu); the
+// chains it leaves to the dense elimination are returned in `dense`.
+ggf_status lattice_inverse(ggf_ctx* ctx, const std::vector<int>& chains, std::vector<int>& dense, cudaStream_t st) {
+    Chains& ch = ctx->ch;
+    std::vector<char> bad(ch.n, 0);
+    for (int fam = 0; fam < 2; ++fam) {
+        const bool cplx = fam == 1;
+        const int npf = cplx ? ctx->Kc : ctx->K;
+        std::vector<int> cfg, pair;
+        for (int c : chains)
+            for (int p = 0; p < npf && !bad[c]; ++p) { cfg.push_back(c); pair.push_back(p); }
+        if (cfg.empty()) continue;
+        size_t bytes = 0;
+        const int cap = ggf_lattice_inverse_plan(ctx, cplx, (int)cfg.size(), std::max(budget_bytes(), ctx->work_bytes), bytes);
+        if (cap < 1) {                       // no room for one matrix's workspace
+            for (int c : chains) bad[c] = 1;
+            break;
+        }
+        GGF_TRY(ggf_workspace(ctx, bytes));
+        for (size_t i0 = 0; i0 < cfg.size(); i0 += cap) {
+            const int n = (int)std::min<size_t>(cap, cfg.size() - i0);
+            std::vector<char> ok;
+            void* A = nullptr;
+            int *d_chain = nullptr, *d_pair = nullptr;
+            GGF_TRY(ggf_lattice_inverse(ctx, cplx, n, cfg.data() + i0, pair.data() + i0, ch.links, ok, &A, &d_chain,
+                                        &d_pair, st));
+            GGF_TRY(place_inverses(ctx, cplx, n, d_chain, d_pair, A, st));
+            GGF_CK(cudaStreamSynchronize(st));   // the workspace is reused by the next batch
+            for (int i = 0; i < n; ++i)
+                if (!ok[i]) bad[cfg[i0 + i]] = 1;
+        }
+    }
+    for (int c : chains)
+        if (bad[c]) dense.push_back(c);
     return GGF_OK;
 }
 
@@ -407,18 +460,25 @@ ggf_status chain_ell(ggf_ctx* ctx, const std::vector<int>& chains, bool init, cu
 }
 
 // Factor the listed chains: log-weights from the site-by-site FP64 Pfaffian
-// (init: set; refresh: drift recorded), inverses by FP64 Gauss-Jordan at the
-// start and for FP64 chains, by a Newton step on the tensor cores for FP32
-// chains (Gauss-Jordan where the residual is too large for it).
+// (init: set; refresh: drift recorded), inverses in FP64 along the lattice at
+// the start and for FP64 chains (Gauss-Jordan below four rows and where that
+// is not accurate enough), by a Newton step on the tensor cores for FP32
+// chains (the FP64 inverse where the residual is too large for it).
 ggf_status factor_chains(ggf_ctx* ctx, const std::vector<int>& chains, bool init, cudaStream_t st) {
     if (chains.empty()) return GGF_OK;
     GGF_TRY(chain_ell(ctx, chains, init, st));
     const bool newton = !init && ctx->ch.opts.precision == GGF_FP32 && ctx->use_tc && ctx->g.N % 8 == 0;
-    if (!newton) return dense_inverse(ctx, chains, st);
     std::vector<int> dense;
-    GGF_TRY(newton_inverse(ctx, chains, dense, st));
-    ctx->dense_refreshes += dense.size();
-    return dense_inverse(ctx, dense, st);
+    if (newton) {
+        GGF_TRY(newton_inverse(ctx, chains, dense, st));
+        ctx->dense_refreshes += dense.size();
+    } else {
+        dense = chains;
+    }
+    if (dense.empty() || !ggf_lattice_inverse_use(ctx)) return dense_inverse(ctx, dense, st);
+    std::vector<int> rest;
+    GGF_TRY(lattice_inverse(ctx, dense, rest, st));
+    return dense_inverse(ctx, rest, st);
 }
 
 ggf_status require(ggf_ctx* ctx, bool gauss, bool chains) {
