@@ -35,21 +35,61 @@
 // n < m come from its one stored inverse.  With N_nm = e^{logc + ell}
 // (N_mn = conj N_nm) and the pair weights of the sampler's combination,
 //   f_E(G)_l = sum_nm lambda_n^* lambda_m N_nm R_nm / sum_nm lambda_n^* lambda_m N_nm.
-#include "ggf_obs.cuh"
+//
+// What bounds it: latency of short dependent phases (load a block, two small
+// products, the insertion) over many independent items; 32 chains of 8 x 8
+// U(1), K = 2 took 508 us with one thread per (chain, link) and take 93
+// with a group of B lanes (ggf_obs_group.cuh).
+#include "ggf_obs_group.cuh"
 
 namespace {
 
-constexpr int ETHREADS = 128;
-
-// One thread per (chain, link); FIELD: the U(1) electric field instead of J^2.
+// A group of B = 4 H lanes per (chain, link); FIELD: the U(1) electric field
+// instead of J^2.
 template <class RW, class CW, int H, bool FIELD>
-__global__ void __launch_bounds__(ETHREADS) electric_kernel(DevConst dc, int n_chains, int blocks_per_chain,
-                                                            const void* links, const RW* Wr, const CW* Wc,
-                                                            const cxd* ell, cxd* out, cxd* pair_out) {
-    const int c = blockIdx.x / blocks_per_chain;
-    const int l = (blockIdx.x - c * blocks_per_chain) * ETHREADS + threadIdx.x;
-    if (c >= n_chains || l >= dc.g.n_links) return;
-    electric_item<RW, CW, H, FIELD>(dc, c, l, links, Wr, Wc, ell, out, pair_out);
+__global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_per_chain, const void* links, const RW* Wr,
+                                                      const CW* Wc, const cxd* ell, cxd* out, cxd* pair_out) {
+    constexpr int B = 4 * H, NG = OT / B;
+    __shared__ ElectricShared<H> shared[NG];
+    __shared__ cxd np[36];
+    const Geometry& g = dc.g;
+    const int c = blockIdx.x / blocks_per_chain, grp = threadIdx.x / B, lane = threadIdx.x % B;
+    const int want = (blockIdx.x - c * blocks_per_chain) * NG + grp;
+    const int l = min(want, g.n_links - 1);            // idle groups repeat the last link and write nothing
+    const bool live = want < g.n_links;
+    ElectricShared<H>& sh = shared[grp];
+    double gval = 1.0;
+    if (g.group == GGF_SU2) {
+        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), sh.tw);
+    } else if (g.group == GGF_U1) {
+        const double th = ((const double*)links)[(size_t)c * g.n_links + l];
+        if (lane < g.n_v) sincos(g.q[lane] * th, &sh.tw[2 * lane + 1], &sh.tw[2 * lane]);
+    } else {
+        gval = (double)((const int8_t*)links)[(size_t)c * g.n_links + l];
+    }
+    chain_weights(dc, ell + (size_t)c * dc.P, np);
+    const int K = dc.K;
+    const size_t NN = (size_t)g.N * g.N;
+    cxd num = {0.0, 0.0};
+    cxd* po = pair_out ? pair_out + ((size_t)c * g.n_links + l) * K * K : nullptr;
+    for (int p = 0; p < dc.P; ++p) {
+        const bool cplx = p >= K;
+        const cxd v = cplx ? electric_pair<CW, H, FIELD>(dc, p - K, l, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, lane, gval, sh)
+                           : electric_pair<RW, H, FIELD>(dc, p, l, Wr + ((size_t)c * K + p) * NN, lane, gval, sh);
+        // w_p = 2 lambda_n^* lambda_m: the (n, m) term (lane 0) takes E / 2, the
+        // (m, n) term (lane 1) its conjugate; a diagonal pair E once
+        const cxd Np = np[p], E = dc.w[p] * Np;
+        if (lane == 0) num += (cplx ? 0.5 : 1.0) * (E * v);
+        else if (lane == 1 && cplx) num += 0.5 * (conjg(E) * v);
+        if (po && live) {
+            int n, m;
+            pair_nm(K, p, n, m);
+            if (lane == 0) po[n * K + m] = Np * v;
+            else if (lane == 1 && cplx) po[m * K + n] = conjg(Np) * v;
+        }
+    }
+    num = num + shfl_xor_(num, 1);
+    if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = num;
 }
 
 // One thread per chain.
@@ -79,16 +119,14 @@ ggf_status ggf_electric(ggf_ctx* ctx, cxd* d_out, cxd* d_pairs, cudaStream_t st,
     const Geometry& g = ctx->g;
     // pending delayed updates first, so that W is the inverse at the current links
     GGF_TRY(ggf_flush(ctx, st));
-    const int bpc = (g.n_links + ETHREADS - 1) / ETHREADS;
+    const int ng = OT / g.B, bpc = (g.n_links + ng - 1) / ng;
     const long long blocks = (long long)bpc * ch.n;
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
     const void* lk = ch.links;
-#define GGF_EL2(RW, CW, H, F)                                                                            \
-    electric_kernel<RW, CW, H, F><<<(unsigned)blocks, ETHREADS, 0, st>>>(ctx->dc(), ch.n, bpc, lk,       \
-                                                                         (const RW*)ch.Wr,                \
-                                                                         (const CW*)ch.Wc, ch.ell, d_out, \
-                                                                         d_pairs)
+#define GGF_EL2(RW, CW, H, F)                                                                                       \
+    electric_kernel<RW, CW, H, F><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, lk, (const RW*)ch.Wr,             \
+                                                                   (const CW*)ch.Wc, ch.ell, d_out, d_pairs)
 #define GGF_EL(RW, CW, H)                  \
     do {                                   \
         if (field) GGF_EL2(RW, CW, H, true); \

@@ -17,33 +17,138 @@
 // (densities n_s = (1 + i site[s]) / 2; hoppings and pairings are linear in
 // the link block, and link_term_kernel forms the gauge-invariant one with the
 // link operator, u_l F_s F_t, from it).
-#include "ggf_obs.cuh"
+//
+// What bounds it: the latency of the block loads; 32 chains of 8 x 8 U(1), K = 2:
+// bilinears 155 us with one thread per item, 72 with a group of B lanes
+// (one row of the block each); the four-point function 329 and 104.
+#include "ggf_obs_group.cuh"
 
 namespace {
 
 constexpr int FTHREADS = 128;
 
-// One thread per (chain, item).
+// A group of BW lanes per (chain, item): items 0 .. V - 1 are sites, the
+// others links.
 template <class RW, class CW, int BW>
-__global__ void __launch_bounds__(FTHREADS) fermion_kernel(DevConst dc, int n_chains, int blocks_per_chain,
-                                                           const RW* Wr, const CW* Wc, const cxd* ell,
-                                                           cxd* site_out, cxd* link_out, cxd* pair_site,
-                                                           cxd* pair_link) {
-    const int c = blockIdx.x / blocks_per_chain;
-    const int it = (blockIdx.x - c * blocks_per_chain) * FTHREADS + threadIdx.x;
-    if (c >= n_chains || it >= dc.g.V + dc.g.n_links) return;
-    fermion_item<RW, CW, BW>(dc, c, it, Wr, Wc, ell, site_out, link_out, pair_site, pair_link);
+__global__ void __launch_bounds__(OT) fermion_kernel(DevConst dc, int blocks_per_chain, int it0, int items, const RW* Wr,
+                                                     const CW* Wc, const cxd* ell, cxd* site_out, cxd* link_out,
+                                                     cxd* pair_site, cxd* pair_link) {
+    constexpr int NG = OT / BW;
+    __shared__ cxd np[36];
+    const Geometry& g = dc.g;
+    const int c = blockIdx.x / blocks_per_chain, lane = threadIdx.x % BW, K = dc.K;
+    const int want = (blockIdx.x - c * blocks_per_chain) * NG + threadIdx.x / BW;
+    const bool live = want < items;
+    const int it = it0 + min(want, items - 1);
+    chain_weights(dc, ell + (size_t)c * dc.P, np);
+    const bool is_site = it < g.V;
+    int s = it, t = it;
+    if (!is_site) {
+        int a0, b0;
+        link_ends(g, it - g.V, a0, b0);
+        s = a0 / g.B;
+        t = b0 / g.B;
+    }
+    cxd* out = is_site ? site_out : link_out;
+    cxd* pout = is_site ? pair_site : pair_link;
+    if (pout) pout += is_site ? ((size_t)c * g.V + s) * K * K : ((size_t)c * g.n_links + (it - g.V)) * 4 * K * K;
+    // lanes 0 .. 3 of the group each keep one entry (alpha, beta)
+    const int a = (lane >> 1) & 1, b = lane & 1;
+    const bool entry = live && lane < 4 && (!is_site || lane == 1);
+    const size_t NN = (size_t)g.N * g.N;
+    cxd acc = {0.0, 0.0};
+    for (int p = 0; p < dc.P; ++p) {
+        const cxd Np = np[p], E = dc.w[p] * Np;
+        int n, m;
+        pair_nm(K, p, n, m);
+        cxd* q = pout ? pout + (is_site ? 0 : (size_t)(a * 2 + b) * K * K) : nullptr;
+        if (p >= K) {
+            cxd X[4];
+            coupled_group<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, s, t, lane, X);
+            const cxd x = a ? (b ? X[3] : X[2]) : (b ? X[1] : X[0]);
+            // (n, m) with weight E / 2 (w_p = 2 lambda_n^* lambda_m), (m, n) with
+            // conj(E) / 2 and the conjugate product; A is added after the loop
+            const cxd h = 0.5 * E;
+            acc += h * x + conjg(h) * conjg(x);
+            if (q && entry) {
+                q[n * K + m] = Np * pair_bilinear(dc, s, t, a, b, x);
+                q[m * K + n] = conjg(Np) * pair_bilinear(dc, s, t, a, b, conjg(x));
+            }
+        } else {
+            double X[4];
+            coupled_group<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, s, t, lane, X);
+            const cxd x = {a ? (b ? X[3] : X[2]) : (b ? X[1] : X[0]), 0.0};
+            acc += E * x;
+            if (q && entry) q[n * K + n] = Np * pair_bilinear(dc, s, t, a, b, x);
+        }
+    }
+    if (!out || !entry) return;
+    // -i (A + sum_p weight_p X_p); A enters with the total weight
+    // sum_nm lambda_n^* lambda_m N_nm / N(G) = 1 (only where s == t)
+    const cxd F = pair_bilinear(dc, s, t, a, b, acc);
+    if (is_site) out[(size_t)c * g.V + s] = F;
+    else out[((size_t)c * g.n_links + (it - g.V)) * 4 + lane] = F;
 }
 
-// One thread per (chain, link).
+// A group of BW lanes per (chain, link).
 template <class RW, class CW, int BW>
-__global__ void __launch_bounds__(FTHREADS) fermion4_kernel(DevConst dc, int n_chains, int blocks_per_chain,
-                                                            const RW* Wr, const CW* Wc, const cxd* ell, cxd* out,
-                                                            cxd* pair_out) {
-    const int c = blockIdx.x / blocks_per_chain;
-    const int l = (blockIdx.x - c * blocks_per_chain) * FTHREADS + threadIdx.x;
-    if (c >= n_chains || l >= dc.g.n_links) return;
-    fermion4_item<RW, CW, BW>(dc, c, l, Wr, Wc, ell, out, pair_out);
+__global__ void __launch_bounds__(OT) fermion4_kernel(DevConst dc, int blocks_per_chain, const RW* Wr, const CW* Wc,
+                                                      const cxd* ell, cxd* out, cxd* pair_out) {
+    constexpr int NG = OT / BW;
+    __shared__ cxd np[36];
+    const Geometry& g = dc.g;
+    const int c = blockIdx.x / blocks_per_chain, lane = threadIdx.x % BW, K = dc.K;
+    const int want = (blockIdx.x - c * blocks_per_chain) * NG + threadIdx.x / BW;
+    const bool live = want < g.n_links;
+    const int l = min(want, g.n_links - 1);
+    chain_weights(dc, ell + (size_t)c * dc.P, np);
+    int a0, b0;
+    link_ends(g, l, a0, b0);
+    const int s = a0 / g.B, t = b0 / g.B;
+    cxd* q = pair_out ? pair_out + ((size_t)c * g.n_links + l) * K * K : nullptr;
+    const size_t NN = (size_t)g.N * g.N;
+    const double As = dc.Ap[(size_t)s * 4 + 1], At = dc.Ap[(size_t)t * 4 + 1];
+    cxd acc = {0.0, 0.0};
+    for (int p = 0; p < dc.P; ++p) {
+        const bool cplx = p >= K;
+        const cxd Np = np[p], E = dc.w[p] * Np;
+        int n, m;
+        pair_nm(K, p, n, m);
+        cxd g01, g23, x[4];
+        if (cplx) {
+            const CW* W = Wc + ((size_t)c * dc.Kc + (p - K)) * NN;
+            cxd ss[4], tt[4];
+            coupled_group<CW, BW>(dc, W, s, s, lane, ss);
+            coupled_group<CW, BW>(dc, W, t, t, lane, tt);
+            coupled_group<CW, BW>(dc, W, s, t, lane, x);
+            g01 = ss[1];
+            g23 = tt[1];
+        } else {
+            const RW* W = Wr + ((size_t)c * K + p) * NN;
+            double ss[4], tt[4], xr[4];
+            coupled_group<RW, BW>(dc, W, s, s, lane, ss);
+            coupled_group<RW, BW>(dc, W, t, t, lane, tt);
+            coupled_group<RW, BW>(dc, W, s, t, lane, xr);
+            g01 = {ss[1], 0.0};
+            g23 = {tt[1], 0.0};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = {xr[k], 0.0};
+        }
+        // lane 0: (n, m) with E / 2, lane 1: (m, n) with conj(E) / 2 and the
+        // conjugate blocks; a diagonal pair once with E
+        const bool ord = lane == 1;
+        auto cj = [&](cxd v) { return ord ? conjg(v) : v; };
+        const cxd pf = (cj(g01) + cxd{As, 0.0}) * (cj(g23) + cxd{At, 0.0}) - cj(x[0]) * cj(x[3]) + cj(x[1]) * cj(x[2]);
+        // a self-link (s = t): c_2s c_2s+1 c_2s c_2s+1 = -1
+        const cxd v = s == t ? cxd{1.0, 0.0} : pf;
+        if (lane == 0 || (ord && cplx)) {
+            const cxd N1 = cj(Np);
+            acc -= ((cplx ? 0.5 : 1.0) * cj(E)) * v;
+            if (q && live) q[ord ? m * K + n : n * K + m] = -1.0 * (N1 * v);
+        }
+    }
+    acc = acc + shfl_xor_(acc, 1);
+    if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = s == t ? cxd{-1.0, 0.0} : acc;
 }
 
 // One thread per (chain, link).
@@ -90,13 +195,13 @@ ggf_status ggf_fermion4(ggf_ctx* ctx, cxd* d_out, cudaStream_t st, cxd* d_pairs)
     Chains& ch = ctx->ch;
     const Geometry& g = ctx->g;
     GGF_TRY(ggf_flush(ctx, st));
-    const int bpc = (g.n_links + FTHREADS - 1) / FTHREADS;
+    const int ng = OT / g.B, bpc = (g.n_links + ng - 1) / ng;
     const long long blocks = (long long)bpc * ch.n;
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
-#define GGF_F4(RW, CW, BW)                                                                                 \
-    fermion4_kernel<RW, CW, BW><<<(unsigned)blocks, FTHREADS, 0, st>>>(ctx->dc(), ch.n, bpc, (const RW*)ch.Wr, \
-                                                                       (const CW*)ch.Wc, ch.ell, d_out, d_pairs)
+#define GGF_F4(RW, CW, BW)                                                                                  \
+    fermion4_kernel<RW, CW, BW><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, (const RW*)ch.Wr,           \
+                                                                 (const CW*)ch.Wc, ch.ell, d_out, d_pairs)
     if (g.B == 8) {
         if (fp64) GGF_F4(double, cxd, 8); else GGF_F4(float, cxf, 8);
     } else if (g.B == 16) {
@@ -117,15 +222,18 @@ ggf_status ggf_fermion(ggf_ctx* ctx, cxd* d_site, cxd* d_link, cxd* d_pair_site,
     Chains& ch = ctx->ch;
     const Geometry& g = ctx->g;
     GGF_TRY(ggf_flush(ctx, st));
-    const int items = g.V + g.n_links;
-    const int bpc = (items + FTHREADS - 1) / FTHREADS;
+    // only the items that an output wants
+    const int it0 = d_site || d_pair_site ? 0 : g.V;
+    const int items = (d_link || d_pair_link ? g.V + g.n_links : g.V) - it0;
+    if (items <= 0) return GGF_OK;
+    const int ng = OT / g.B, bpc = (items + ng - 1) / ng;
     const long long blocks = (long long)bpc * ch.n;
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
-#define GGF_FE(RW, CW, BW)                                                                                 \
-    fermion_kernel<RW, CW, BW><<<(unsigned)blocks, FTHREADS, 0, st>>>(ctx->dc(), ch.n, bpc, (const RW*)ch.Wr, \
-                                                                      (const CW*)ch.Wc, ch.ell, d_site, d_link, \
-                                                                      d_pair_site, d_pair_link)
+#define GGF_FE(RW, CW, BW)                                                                                       \
+    fermion_kernel<RW, CW, BW><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, it0, items, (const RW*)ch.Wr,     \
+                                                                (const CW*)ch.Wc, ch.ell, d_site, d_link,         \
+                                                                d_pair_site, d_pair_link)
     if (g.B == 8) {
         if (fp64) GGF_FE(double, cxd, 8); else GGF_FE(float, cxf, 8);
     } else if (g.B == 16) {

@@ -23,7 +23,9 @@
 //
 // What bounds it: the FP64 unit in the joints, kernel launches for small
 // batches.  Measured, 8 configurations of 8 x 8 U(1), n_v = 2, K = 2 (16 real
-// and 8 complex matrices of order 1024): 190 ms by Gauss-Jordan, 22 ms so.
+// and 8 complex matrices of order 1024): 190 ms by Gauss-Jordan, 22 ms so;
+// the start of one chain of 16 x 16 U(1), K = 4 (4 real and 6 complex ones of
+// order 4096): 6.0 s and 0.30 s.
 #include <algorithm>
 #include <vector>
 #include "ggf_ctx.h"
