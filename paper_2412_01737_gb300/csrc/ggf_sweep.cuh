@@ -40,6 +40,16 @@ __device__ __forceinline__ void fmsc(cxd& r, cxd a, cxd b) {
 __device__ __forceinline__ cxd to_c(double v) { return {v, 0.0}; }
 __device__ __forceinline__ cxd to_c(cxd v) { return v; }
 
+// acc + a b and acc - a b as the FP32 chains have always rounded them (the
+// product first); FP64 as fused steps, half the instructions of a unit that
+// issues two FMAs per clock and SM.
+template <class T> __device__ __forceinline__ void acc_add(T& r, T a, T b) { r += a * b; }
+template <> __device__ __forceinline__ void acc_add<double>(double& r, double a, double b) { fmac(r, a, b); }
+template <> __device__ __forceinline__ void acc_add<cxd>(cxd& r, cxd a, cxd b) { fmac(r, a, b); }
+template <class T> __device__ __forceinline__ void acc_sub(T& r, T a, T b) { r -= a * b; }
+template <> __device__ __forceinline__ void acc_sub<double>(double& r, double a, double b) { fmsc(r, a, b); }
+template <> __device__ __forceinline__ void acc_sub<cxd>(cxd& r, cxd a, cxd b) { fmsc(r, a, b); }
+
 // Lane of the largest magnitude among the lanes that take part (ties: the
 // lowest lane), one warp, all lanes call: a redux over the upper words of the
 // FP64 magnitudes, and over the lower words where those tie, instead of five

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256) batch_apply(int N, int fam_pairs, int KRM
 #pragma unroll
                 for (int u = 0; u < RPT; ++u)
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) acc[u][t] += v[u] * x[t];
+                    for (int t = 0; t < 8; ++t) acc_add(acc[u][t], v[u], x[t]);
             }
         }
 #pragma unroll

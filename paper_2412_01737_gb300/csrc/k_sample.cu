@@ -327,7 +327,11 @@ __global__ void __launch_bounds__(128) gather_kernel(Geometry g, int P, int fam_
 // W <- W - U V over the pending panels (rank pend[c] * R), SIMT tiled product
 // (FP64 chains, and FP32 when the tensor-core flush is not used).
 // Grid (tiles_i * tiles_j, family pairs, chains), 256 threads as 16 x 16, each
-// a 4 x 4 block of a 64 x 64 tile of W.
+// four rows by four columns (16 apart, so that neighbouring threads touch
+// neighbouring elements) of a 64 x 64 tile of W.  Bound: the FP64 unit; with the
+// complex product formed before it is added (six instructions instead of four
+// fused ones) a rank-128 flush of 24 complex matrices of order 1024 took 35.3
+// ms, 20.9 fused.
 template <class T, int R>
 __global__ void __launch_bounds__(256) flush_kernel(int N, int fam_pairs, T* W, const typename Sc<T>::R* Pan,
                                                     const int* pend, int kmax, int tiles) {
@@ -366,11 +370,11 @@ __global__ void __launch_bounds__(256) flush_kernel(int N, int fam_pairs, T* W, 
 #pragma unroll
             for (int a = 0; a < 4; ++a) av[a] = As[qq][ty * 4 + a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[qq][tx * 4 + b];
+            for (int b = 0; b < 4; ++b) bv[b] = Bs[qq][tx + 16 * b];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
+                for (int b = 0; b < 4; ++b) acc_add(acc[a][b], av[a], bv[b]);
         }
         __syncthreads();
     }
@@ -380,7 +384,7 @@ __global__ void __launch_bounds__(256) flush_kernel(int N, int fam_pairs, T* W, 
         if (i >= N) continue;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            int j = j0 + tx * 4 + b;
+            int j = j0 + tx + 16 * b;
             if (j < N) Wp[(size_t)i * N + j] -= acc[a][b];
         }
     }

@@ -116,16 +116,6 @@ __device__ __forceinline__ float narrow(double v, float) { return (float)v; }
 __device__ __forceinline__ cxd narrow(cxd v, cxd) { return v; }
 __device__ __forceinline__ cxf narrow(cxd v, cxf) { return {(float)v.x, (float)v.y}; }
 
-// acc + a b and acc - a b as the FP32 chains have always rounded them (the
-// product first); FP64 as fused steps, half the instructions of a unit that
-// issues two FMAs per clock and SM.
-template <class T> __device__ __forceinline__ void acc_add(T& r, T a, T b) { r += a * b; }
-template <> __device__ __forceinline__ void acc_add<double>(double& r, double a, double b) { fmac(r, a, b); }
-template <> __device__ __forceinline__ void acc_add<cxd>(cxd& r, cxd a, cxd b) { fmac(r, a, b); }
-template <class T> __device__ __forceinline__ void acc_sub(T& r, T a, T b) { r -= a * b; }
-template <> __device__ __forceinline__ void acc_sub<double>(double& r, double a, double b) { fmsc(r, a, b); }
-template <> __device__ __forceinline__ void acc_sub<cxd>(cxd& r, cxd a, cxd b) { fmsc(r, a, b); }
-
 // Element (xi, yi) of Delta = O' G O'^T - O G O^T of link l for pair p of its family.
 template <class Z>
 __device__ __forceinline__ Z delta_elem(const DevConst& dc, int p, int l, int xi, int yi, const Proposal& q,
