@@ -2,11 +2,44 @@
 // the one-link-per-launch kernels (k_sample.cu) and the batched link steps
 // on the small matrix W[T, T] (k_batch.cu).
 #pragma once
+#include <algorithm>
 #include "ggf_ctx.h"
 #include "ggf_geom.cuh"
 
 namespace {
 constexpr int NWARP = 8;
+constexpr int MAXP = 36;           // pairs at K = 8
+constexpr int MAXCS = 8;           // portable cluster size
+
+// How a chain's pairs are dealt to the CTAs of its cluster: pairs
+// ord[first[b]] .. ord[first[b + 1] - 1] belong to CTA b, real ones first.
+struct PairBins {
+    unsigned char first[MAXCS + 1], ord[MAXP];
+};
+
+// Bins of about one complex or two real pairs (a complex pair costs four real
+// ones), at most MAXCS, the heaviest dealt first to the lightest bin.  Returns
+// the number of CTAs.
+inline int deal_pairs(int K, int Kc, PairBins& a) {
+    const int P = K + Kc;
+    const int CS = std::max(1, std::min(MAXCS, Kc + (K + 1) / 2));
+    int load[MAXCS] = {0}, bin[MAXP], n = 0;
+    for (int k = 0; k < P; ++k) {
+        const int p = k < Kc ? K + k : k - Kc;       // complex pairs first
+        int b = 0;
+        for (int q = 1; q < CS; ++q)
+            if (load[q] < load[b]) b = q;
+        bin[p] = b;
+        load[b] += p >= K ? 4 : 1;
+    }
+    for (int b = 0; b < CS; ++b) {
+        a.first[b] = (unsigned char)n;
+        for (int p = 0; p < P; ++p)
+            if (bin[p] == b) a.ord[n++] = (unsigned char)p;
+    }
+    a.first[CS] = (unsigned char)n;
+    return CS;
+}
 
 __device__ __forceinline__ double magc(cxd v) { return fabs(v.x) + fabs(v.y); }
 
@@ -36,6 +69,17 @@ __device__ __forceinline__ void fmsc(double& r, double a, double b) { r = fma(-a
 __device__ __forceinline__ void fmsc(cxd& r, cxd a, cxd b) {
     r.x = fma(-a.x, b.x, r.x); r.x = fma(a.y, b.y, r.x);
     r.y = fma(-a.x, b.y, r.y); r.y = fma(-a.y, b.x, r.y);
+}
+// a / d from id ~ 1 / d: the quotient a id, corrected once by its remainder
+__device__ __forceinline__ double quotient(double a, double d, double id) {
+    const double q = a * id;
+    return fma(fma(-q, d, a), id, q);
+}
+__device__ __forceinline__ cxd quotient(cxd a, cxd d, cxd id) {
+    cxd q = a * id, r = a;
+    fmsc(r, q, d);
+    fmac(q, r, id);
+    return q;
 }
 __device__ __forceinline__ cxd to_c(double v) { return {v, 0.0}; }
 __device__ __forceinline__ cxd to_c(cxd v) { return v; }
@@ -152,7 +196,7 @@ __device__ __forceinline__ bool warp_solve(T* A, int r, T* fcol) {
         if (is_zero(d)) return false;
         const T id = recip(d);
         __syncwarp();
-        if (lane > k && lane < w) A[k * w + lane] = A[k * w + lane] * id;
+        if (lane > k && lane < w) A[k * w + lane] = quotient(A[k * w + lane], d, id);
         if (lane < r) fcol[lane] = A[lane * w + k];
         __syncwarp();
         const int cols = w - k - 1;
@@ -229,27 +273,6 @@ __device__ __forceinline__ Proposal draw_proposal(const Geometry& g, const void*
     return q;
 }
 
-// Change of pair p's twisted link block, Delta = O' G O'^T - O G O^T on the
-// r Majoranas of link l (r x r, one warp).
-// cs: cos, sin of q_j theta for the old angle (cs[0 .. 2 n_v)) and the new
-// one (cs[4 ..]), from twist_table.
-__device__ __forceinline__ void pair_delta(const DevConst& dc, int p, int l, const Proposal& q, const double* cs,
-                                           cxd* D) {
-    const int r = dc.g.r, lane = threadIdx.x & 31;
-    for (int e = lane; e < r * r; e += 32) {
-        int xi = e / r, yi = e % r;
-        cxd nv, ov;
-        if (p < dc.K) {
-            nv = {twisted_tab<double>(dc, p, l, xi, yi, q.g_new, cs + 4), 0.0};
-            ov = {twisted_tab<double>(dc, p, l, xi, yi, q.g_old, cs), 0.0};
-        } else {
-            nv = twisted_tab<cxd>(dc, p - dc.K, l, xi, yi, q.g_new, cs + 4);
-            ov = twisted_tab<cxd>(dc, p - dc.K, l, xi, yi, q.g_old, cs);
-        }
-        D[e] = nv - ov;
-    }
-}
-
 // SU(2) proposal (n_v = 2, one doublet per link end), thread-local: with
 // Philox words (u_acc, u_prop, u_z, u_phi) of counter (sweep, l, 0, 0) and
 // key (seed, chain), g -> r g with r = cos d + i sin d (n . sigma),
@@ -280,36 +303,28 @@ GGF_HD double draw_su2(const Geometry& g, const void* links, int c, int l,
     return u53(out[0]);
 }
 
-// Delta of pair p for an SU(2) proposal (rotations Rold, Rnew of the source
-// doublet), r x r, one warp.
-__device__ __forceinline__ void pair_delta_su2(const DevConst& dc, int p, int l, const double* Rold,
-                                               const double* Rnew, cxd* D) {
-    const int r = dc.g.r, lane = threadIdx.x & 31;
-    for (int e = lane; e < r * r; e += 32) {
-        int xi = e / r, yi = e % r;
-        cxd nv, ov;
-        if (p < dc.K) {
-            nv = {twisted_su2<double>(dc, p, l, xi, yi, Rnew), 0.0};
-            ov = {twisted_su2<double>(dc, p, l, xi, yi, Rold), 0.0};
-        } else {
-            nv = twisted_su2<cxd>(dc, p - dc.K, l, xi, yi, Rnew);
-            ov = twisted_su2<cxd>(dc, p - dc.K, l, xi, yi, Rold);
-        }
-        D[e] = nv - ov;
-    }
-}
+template <class T> struct Fp64Of;
+template <> struct Fp64Of<double> { typedef double Z; };
+template <> struct Fp64Of<float> { typedef double Z; };
+template <> struct Fp64Of<cxd> { typedef cxd Z; };
+template <> struct Fp64Of<cxf> { typedef cxd Z; };
 
-// cos, sin of q_j theta for the old and the new angle of a U(1) proposal
-// (threads 0 .. 2 n_v - 1 of the block; cs holds 8 doubles).
-__device__ __forceinline__ void twist_table(const Geometry& g, const Proposal& q, double* cs) {
-    const int t = threadIdx.x;
-    if (g.group == GGF_U1 && t < 2 * g.n_v) {
-        const int j = t % g.n_v, nw = t / g.n_v;
-        double sv, cv;
-        sincos(g.q[j] * (nw ? q.th_new : q.th_old), &sv, &cv);
-        cs[4 * nw + 2 * j] = cv;
-        cs[4 * nw + 2 * j + 1] = sv;
-    }
+template <class T> __device__ __forceinline__ typename Fp64Of<T>::Z wide(T v);
+template <> __device__ __forceinline__ double wide<double>(double v) { return v; }
+template <> __device__ __forceinline__ double wide<float>(float v) { return v; }
+template <> __device__ __forceinline__ cxd wide<cxd>(cxd v) { return v; }
+template <> __device__ __forceinline__ cxd wide<cxf>(cxf v) { return {(double)v.x, (double)v.y}; }
+__device__ __forceinline__ double narrow(double v, double) { return v; }
+__device__ __forceinline__ float narrow(double v, float) { return (float)v; }
+__device__ __forceinline__ cxd narrow(cxd v, cxd) { return v; }
+__device__ __forceinline__ cxf narrow(cxd v, cxf) { return {(float)v.x, (float)v.y}; }
+
+// Element (xi, yi) of Delta = O' G O'^T - O G O^T of link l for pair p of its family.
+template <class Z>
+__device__ __forceinline__ Z delta_elem(const DevConst& dc, int p, int l, int xi, int yi, const Proposal& q,
+                                        const double* tw, bool su2) {
+    if (su2) return twisted_su2<Z>(dc, p, l, xi, yi, tw + 20) - twisted_su2<Z>(dc, p, l, xi, yi, tw + 4);
+    return twisted_tab<Z>(dc, p, l, xi, yi, q.g_new, tw + 4) - twisted_tab<Z>(dc, p, l, xi, yi, q.g_old, tw);
 }
 
 // Pf(M') / Pf(M) = Pf([[Delta, -1], [1, W_SS]]) (r/2 = 2 n_v even: no extra
@@ -365,24 +380,6 @@ GGF_HD cxd pair_norm(const DevConst& dc, const cxd* ell_c, int p, double amax, d
     if (p < dc.K) e.y = 0.0;
     e.x -= amax;
     return iden * cexp_(e);
-}
-
-// Numerator and denominator of N(G')/N(G) = Re sum_p w_p e^{logc_p + ell_p} rho_p
-// / Re sum_p w_p e^{logc_p + ell_p}, scaled by the largest modulus (FP64).
-__device__ __forceinline__ void combine_pairs(const DevConst& dc, const cxd* ell_c, const cxd* rho, double& sn,
-                                              double& so) {
-    double amax = -INFINITY;
-    for (int p = 0; p < dc.P; ++p) amax = fmax(amax, dc.logc[p].x + ell_c[p].x);
-    so = 0.0;
-    sn = 0.0;
-    for (int p = 0; p < dc.P; ++p) {
-        cxd e = dc.logc[p] + ell_c[p];
-        if (p < dc.K) e.y = 0.0;
-        e.x -= amax;
-        cxd tt = dc.w[p] * cexp_(e);
-        so += tt.x;
-        sn += (tt * rho[p]).x;
-    }
 }
 
 // Z = (1 + Delta W_SS)^{-1} Delta (r x r) into Zout, one warp; Aug is r x 2r

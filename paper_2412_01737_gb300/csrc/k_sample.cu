@@ -1,7 +1,7 @@
 // Metropolis sweep kernels of libggf (Sec. 5.1 sampling of p(G) = N(G)/N).
 //
 // Per link step, for every chain in lockstep:
-//  ratio_kernel   one CTA per chain.  Draws the Philox numbers, forms the
+//  ratio_kernel   one cluster per chain.  Draws the Philox numbers, forms the
 //                 change Delta of the twisted link block for every pair
 //                 (n, m), gathers W_SS from the cached inverse W = M^{-1},
 //                 evaluates the Pfaffian ratio
@@ -16,10 +16,13 @@
 //                 (exact for an antisymmetric W) lets the rounding error's
 //                 symmetric part grow geometrically from update to update.
 //  observe_kernel per sweep: plaquette mean, log N(G), acceptance rate.
+#include <cooperative_groups.h>
 #include "ggf_ctx.h"
 #include "ggf_geom.cuh"
 
 #include "ggf_sweep.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -52,155 +55,337 @@ struct SweepArgs {
     const double* forced;
     int forced_k;
     int* dead;
+    PairBins bins;
 };
 
+// 16-byte pieces of a run of reals
+template <int n>
+__device__ __forceinline__ void load_reals(const float* p, float* o) {
+#pragma unroll
+    for (int k = 0; k < n; k += 4) {
+        const float4 v = *(const float4*)(p + k);
+        o[k] = v.x; o[k + 1] = v.y; o[k + 2] = v.z; o[k + 3] = v.w;
+    }
+}
+template <int n>
+__device__ __forceinline__ void load_reals(const double* p, double* o) {
+#pragma unroll
+    for (int k = 0; k < n; k += 2) {
+        const double2 v = *(const double2*)(p + k);
+        o[k] = v.x; o[k + 1] = v.y;
+    }
+}
+template <int n>
+__device__ __forceinline__ void store_reals(float* p, const float* o) {
+#pragma unroll
+    for (int k = 0; k < n; k += 4) *(float4*)(p + k) = make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
+}
+template <int n>
+__device__ __forceinline__ void store_reals(double* p, const double* o) {
+#pragma unroll
+    for (int k = 0; k < n; k += 2) *(double2*)(p + k) = make_double2(o[k], o[k + 1]);
+}
+__device__ __forceinline__ double real_of(double v) { return v; }
+__device__ __forceinline__ float real_of(float v) { return v; }
+template <class Q> __device__ __forceinline__ Q real_of(cx<Q> v) { return v.x; }
+__device__ __forceinline__ double imag_of(double) { return 0.0; }
+__device__ __forceinline__ float imag_of(float) { return 0.f; }
+template <class Q> __device__ __forceinline__ Q imag_of(cx<Q> v) { return v.y; }
+template <class T, class Q> __device__ __forceinline__ T from_parts(Q x, Q y) {
+    if constexpr (Sc<T>::CPLX) return T{x, y};
+    else return x;
+}
+
+// n consecutive rank columns (n a multiple of the 16-byte piece, within one
+// chunk of eight) of one panel row
+template <class T, int n>
+__device__ __forceinline__ void panel_load(const typename Sc<T>::R* p, size_t plane, T* o) {
+    typename Sc<T>::R re[n], im[n];
+    load_reals<n>(p, re);
+    if constexpr (Sc<T>::CPLX) load_reals<n>(p + plane, im);
+#pragma unroll
+    for (int k = 0; k < n; ++k) o[k] = from_parts<T>(re[k], Sc<T>::CPLX ? im[k] : re[k]);
+}
+template <class T, int n>
+__device__ __forceinline__ void panel_store(typename Sc<T>::R* p, size_t plane, const T* o) {
+    typename Sc<T>::R re[n], im[n];
+#pragma unroll
+    for (int k = 0; k < n; ++k) { re[k] = real_of(o[k]); im[k] = imag_of(o[k]); }
+    store_reals<n>(p, re);
+    if constexpr (Sc<T>::CPLX) store_reals<n>(p + plane, im);
+}
+
+// Byte offsets of ratio_kernel's shared arrays.
+struct RatioLayout {
+    size_t rho, term, tw, pair, task, part, stage, total;
+    size_t pair_bytes, task_bytes;
+};
+__host__ __device__ inline RatioLayout ratio_layout(int P, int r, int np, int KRM, size_t cw) {
+    RatioLayout s;
+    size_t o = 0;
+    auto take = [&](size_t& at, size_t bytes) { at = o; o = (o + bytes + 15) & ~(size_t)15; };
+    take(s.rho, (size_t)P * sizeof(cxd));
+    take(s.term, (size_t)P * sizeof(cxd));
+    take(s.tw, 36 * sizeof(double));
+    s.pair_bytes = (size_t)3 * r * r * sizeof(cxd);            // Delta, W_SS, Z
+    take(s.pair, np * s.pair_bytes);
+    s.task_bytes = (size_t)(4 * r * r + r) * sizeof(cxd);      // bordered matrix or [A | B], a column
+    take(s.task, (size_t)(2 * np < NWARP ? 2 * np : NWARP) * s.task_bytes);
+    take(s.part, KRM ? (size_t)(NWARP * 32) * sizeof(cxd) : 0);
+    take(s.stage, KRM ? (size_t)2 * r * (KRM + 1) * cw : 0);    // pending rows of U and V on S
+    s.total = o;
+    return s;
+}
+
+// W_SS of one pair (FP64, shared), less the pending updates where there are
+// any: W_eff[S, S] = W[S, S] - U[S, :] V[:, S].  The pending rows on S are
+// staged once, and the sums of an entry are split over the CTA's threads.
+template <class T, int R>
+__device__ __forceinline__ void load_wss(const Geometry& g, int a0, int b0, const T* W, typename Fp64Of<T>::Z* Ws) {
+    for (int e = threadIdx.x; e < R * R; e += NWARP * 32)
+        Ws[e] = wide(W[(size_t)link_majorana(g, a0, b0, e / R) * g.N + link_majorana(g, a0, b0, e % R)]);
+}
+template <class T, int R>
+__device__ __forceinline__ void subtract_pending(const Geometry& g, int a0, int b0, const typename Sc<T>::R* U, size_t NK,
+                                                 int NP, int kr, void* stage, void* part, typename Fp64Of<T>::Z* Ws) {
+    typedef typename Fp64Of<T>::Z Z;
+    constexpr int PARTS = NWARP * 32 / (R * R);
+    const typename Sc<T>::R* Vt = U + PanelIO<T>::PLANES * NK;
+    const int ld = kr + 1;
+    T* Us = (T*)stage;
+    T* Vs = Us + (size_t)R * ld;
+    for (int e = threadIdx.x; e < R * kr; e += NWARP * 32) {
+        const int x = e / kr, q = e - x * kr;
+        const size_t at = pidx(link_majorana(g, a0, b0, x), q, NP);
+        Us[x * ld + q] = PanelIO<T>::ld(U, NK, at);
+        Vs[x * ld + q] = PanelIO<T>::ld(Vt, NK, at);
+    }
+    __syncthreads();
+    Z* ps = (Z*)part;
+    {
+        const int en = threadIdx.x % (R * R), pt = threadIdx.x / (R * R);
+        const T* u = Us + (en / R) * ld;
+        const T* v = Vs + (en % R) * ld;
+        Z acc = Sc<Z>::zero();
+        for (int q = pt; q < kr; q += PARTS) fmac(acc, wide(u[q]), wide(v[q]));
+        ps[threadIdx.x] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x < R * R) {
+        Z acc = ps[threadIdx.x];
+        for (int k = 1; k < PARTS; ++k) acc += ps[k * R * R + threadIdx.x];
+        Ws[threadIdx.x] -= acc;
+    }
+    __syncthreads();
+}
+
+// Rows Y = W[S, :] and columns C^T = W[:, S]^T of one pair into yb [2][R][N],
+// by `cnt` threads from `first`.
+template <class T, int R>
+__device__ __forceinline__ void gather_rows_cols(int N, int a0, int b0, const T* W, T* yb, int first, int cnt) {
+    constexpr int H = R / 2, E = 16 / sizeof(T);
+    const int pieces = N / E;                       // N is a multiple of 8
+    for (int e = first; e < R * pieces; e += cnt) {
+        const int xi = e / pieces, k = e - xi * pieces;
+        const int gi = xi < H ? a0 + xi : b0 + xi - H;
+        ((float4*)(yb + (size_t)xi * N))[k] = ((const float4*)(W + (size_t)gi * N))[k];
+    }
+    for (int e = first; e < 2 * N; e += cnt) {
+        const int end = e >= N, j = end ? e - N : e;
+        const T* src = W + (size_t)j * N + (end ? b0 : a0);
+#pragma unroll
+        for (int k = 0; k < H; ++k) yb[(size_t)(R + end * H + k) * N + j] = src[k];
+    }
+}
+
+// One proposal of every chain; a cluster per chain, its pairs dealt to the CTAs
+// (deal_pairs).  The Pfaffian ratio and Z of a pair run side by side on two
+// warps, the pair terms on the last one, and in immediate mode the warps in
+// between already copy the rows and columns that an accepted update needs.
+// Bound: the latency of that chain of FP64 steps; one CTA that drew, formed
+// Delta, W_SS, ratio, terms, Z and copies in turn took 134 us for 1024 chains of
+// 8 x 8 Z2 and 185 us for a block-move link of 32 chains of 8 x 8 U(1), K = 2;
+// 78 and 53 us so.
 // SU2: SU(2) links (quaternion proposal and doublet twist); the Z2 and U(1)
 // instantiations (SU2 = false) do not contain that code.
-template <class RW, class CW, bool SU2>
-__global__ void __launch_bounds__(NWARP * 32) ratio_kernel(SweepArgs a) {
-    extern __shared__ cxd sm[];
+template <class RW, class CW, bool SU2, int R>
+__global__ void __launch_bounds__(NWARP * 32, 2) ratio_kernel(SweepArgs a) {
+    extern __shared__ __align__(16) unsigned char smr[];
+    typedef typename Sc<RW>::R QR;
     const Geometry& g = a.dc.g;
-    const int P = a.dc.P, K = a.dc.K, r = g.r, N = g.N;
-    const int c = blockIdx.x;
+    const int P = a.dc.P, K = a.dc.K, Kc = P - K, N = g.N, KRM = a.kmax > 1 ? a.kmax * R : 0;
+    const int CS = cg::this_cluster().num_blocks(), rank = cg::this_cluster().block_rank();
+    const int c = blockIdx.x / CS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    cxd* Delta = sm;                       // [P][r][r]
-    cxd* Wss = Delta + P * r * r;          // [P][r][r]
-    cxd* Bord = Wss + P * r * r;           // [NWARP][2r][2r]
-    cxd* rho = Bord + NWARP * 4 * r * r;   // [P]
-    cxd* fcol = rho + P;                   // [NWARP][r]
+    const int p0 = a.bins.first[rank], np = a.bins.first[rank + 1] - p0;
+    const RatioLayout lay = ratio_layout(P, R, np, KRM, sizeof(CW));
+    cxd* rho = (cxd*)(smr + lay.rho);
+    cxd* term = (cxd*)(smr + lay.term);
+    double* tw = (double*)(smr + lay.tw);
+    auto slot = [&](int s, int k) { return (cxd*)(smr + lay.pair + s * lay.pair_bytes) + k * R * R; };
     __shared__ Proposal s_q;
-    __shared__ double s_cs[8];
-    __shared__ int s_accept;
-    __shared__ double s_su2[36];          // SU2: new quaternion, old and new doublet rotations
+    __shared__ int s_accept, s_okz[MAXP];
 
     const int l = a.link_of_chain ? a.link_of_chain[c] : a.link;
+    const int dead = a.forced ? a.dead[c] : 0;
+    const int kr = KRM ? a.pend[c] * R : 0;
     int a0, b0;
     link_ends(g, l, a0, b0);
-
-    if constexpr (SU2) {
-        if (threadIdx.x == 0) {
-            Proposal q{};
-            q.u_acc = draw_su2(g, a.links, c, l, *a.d_sweep, a.seed, a.width, s_su2, s_su2 + 4, s_su2 + 20,
-                                   a.coff);
-            s_q = q;
-        }
-        __syncthreads();
-    } else {
-        if (threadIdx.x == 0) {
-            Proposal q = draw_proposal(g, a.links, c, l, *a.d_sweep, a.seed, a.width, a.coff);
-            if (a.forced && g.group == GGF_U1) q.th_new = a.forced[(size_t)c * 32 + a.forced_k];   // block move
-            s_q = q;
-        }
-        __syncthreads();
-    }
-    const Proposal q = s_q;
-    if constexpr (!SU2) twist_table(g, q, s_cs);
-    __syncthreads();
-
-    for (int p = warp; p < P; p += NWARP) {
-        cxd* D = Delta + p * r * r;
-        cxd* Ws = Wss + p * r * r;
-        if constexpr (SU2) pair_delta_su2(a.dc, p, l, s_su2 + 4, s_su2 + 20, D);
-        else pair_delta(a.dc, p, l, q, s_cs, D);
-        for (int e = lane; e < r * r; e += 32) {
-            const int gi = link_majorana(g, a0, b0, e / r), gj = link_majorana(g, a0, b0, e % r);
-            cxd wv;
-            if (p < K) wv = loadc((const RW*)a.Wr + (((size_t)c * K + p) * N + gi) * N + gj);
-            else wv = loadc((const CW*)a.Wc + (((size_t)c * (P - K) + (p - K)) * N + gi) * N + gj);
-            if (a.kmax > 1) {
-                // pending updates: W_eff[S, S] = W[S, S] - U[S, :] V[:, S]
-                const int kr = a.pend[c] * r;
-                const int KRM = a.kmax * r, NP = panel_rows(N);
-                const size_t NK = panel_plane(N, KRM);
-                typedef typename Sc<RW>::R R;
-                if (p < K) {
-                    const R* U = (const R*)a.Pr + ((size_t)c * K + p) * 2 * NK;
-                    const R* Vt = U + NK;
-                    for (int qq = 0; qq < kr; ++qq)
-                        wv -= Sc<RW>::to(PanelIO<RW>::ld(U, NK, pidx(gi, qq, NP))) *
-                              Sc<RW>::to(PanelIO<RW>::ld(Vt, NK, pidx(gj, qq, NP)));
-                } else {
-                    const R* U = (const R*)a.Pc + ((size_t)c * (P - K) + (p - K)) * 4 * NK;
-                    const R* Vt = U + 2 * NK;
-                    for (int qq = 0; qq < kr; ++qq)
-                        wv -= Sc<CW>::to(PanelIO<CW>::ld(U, NK, pidx(gi, qq, NP))) *
-                              Sc<CW>::to(PanelIO<CW>::ld(Vt, NK, pidx(gj, qq, NP)));
-                }
-            }
-            Ws[e] = wv;
-        }
-        __syncwarp();
-        cxd pf = bordered_ratio(D, Ws, Bord + warp * 4 * r * r, r);
-        if (lane == 0) rho[p] = pf;
-        __syncwarp();
-    }
-    __syncthreads();
+    auto w_real = [&](int p) { return (const RW*)a.Wr + ((size_t)c * K + p) * N * N; };
+    auto w_cplx = [&](int p) { return (const CW*)a.Wc + ((size_t)c * Kc + (p - K)) * N * N; };
 
     if (threadIdx.x == 0) {
-        double sn, so;
-        combine_pairs(a.dc, a.ell + (size_t)c * P, rho, sn, so);
+        Proposal q{};
+        if constexpr (SU2) {
+            q.u_acc = draw_su2(g, a.links, c, l, *a.d_sweep, a.seed, a.width, tw, tw + 4, tw + 20, a.coff);
+        } else {
+            q = draw_proposal(g, a.links, c, l, *a.d_sweep, a.seed, a.width, a.coff);
+            if (a.forced && g.group == GGF_U1) q.th_new = a.forced[(size_t)c * 32 + a.forced_k];   // block move
+            if (g.group == GGF_U1)
+                for (int t = 0; t < 2 * g.n_v; ++t) {
+                    const int md = t % g.n_v, nw = t / g.n_v;
+                    double sv, cv;
+                    sincos(g.q[md] * (nw ? q.th_new : q.th_old), &sv, &cv);
+                    tw[4 * nw + 2 * md] = cv;
+                    tw[4 * nw + 2 * md + 1] = sv;
+                }
+        }
+        s_q = q;
+    }
+    for (int s = 0; s < np; ++s) {
+        const int p = a.bins.ord[p0 + s];
+        if (p < K) load_wss<RW, R>(g, a0, b0, w_real(p), (double*)slot(s, 1));
+        else load_wss<CW, R>(g, a0, b0, w_cplx(p), slot(s, 1));
+    }
+    __syncthreads();
+    const Proposal q = s_q;
+    const size_t NK = panel_plane(N, KRM ? KRM : R);
+    const int NP = panel_rows(N);
+    for (int s = 0; s < np; ++s) {
+        const int p = a.bins.ord[p0 + s];
+        if (kr > 0) {
+            if (p < K)
+                subtract_pending<RW, R>(g, a0, b0, (const QR*)a.Pr + ((size_t)c * K + p) * 2 * NK, NK, NP, kr,
+                                        smr + lay.stage, smr + lay.part, (double*)slot(s, 1));
+            else
+                subtract_pending<CW, R>(g, a0, b0, (const QR*)a.Pc + ((size_t)c * Kc + (p - K)) * 4 * NK, NK, NP, kr,
+                                        smr + lay.stage, smr + lay.part, slot(s, 1));
+        }
+        for (int e = threadIdx.x; e < R * R; e += NWARP * 32) {
+            if (p < K) ((double*)slot(s, 0))[e] = delta_elem<double>(a.dc, p, l, e / R, e % R, q, tw, SU2);
+            else slot(s, 0)[e] = delta_elem<cxd>(a.dc, p - K, l, e / R, e % R, q, tw, SU2);
+        }
+    }
+    // every CTA of the cluster is running before the first remote write
+    if (CS > 1) cg::this_cluster().sync();
+    else __syncthreads();
+
+    const int spare0 = min(2 * np, NWARP - 1), spare = NWARP - 1 - spare0;
+    if (warp == NWARP - 1) {
+        double amax = -INFINITY;
+        for (int p = lane; p < P; p += 32) amax = fmax(amax, a.dc.logc[p].x + a.ell[(size_t)c * P + p].x);
+        for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        for (int p = lane; p < P; p += 32) {
+            cxd e = a.dc.logc[p] + a.ell[(size_t)c * P + p];
+            if (p < K) e.y = 0.0;
+            e.x -= amax;
+            term[p] = a.dc.w[p] * cexp_(e);
+        }
+    }
+    for (int t = warp; t < 2 * np; t += NWARP) {
+        const int s = t >> 1, p = a.bins.ord[p0 + s];
+        void* scr = smr + lay.task + (size_t)warp * lay.task_bytes;
+        if (t & 1) {
+            const bool ok = p < K ? pair_z((const double*)slot(s, 0), (const double*)slot(s, 1), (double*)scr,
+                                           (double*)scr + 4 * R * R, R, slot(s, 2))
+                                  : pair_z(slot(s, 0), slot(s, 1), (cxd*)scr, (cxd*)scr + 4 * R * R, R, slot(s, 2));
+            if (lane == 0) s_okz[s] = ok;
+        } else {
+            const cxd pf = p < K ? cxd{bordered_ratio((const double*)slot(s, 0), (const double*)slot(s, 1), (double*)scr, R), 0.0}
+                                 : bordered_ratio(slot(s, 0), slot(s, 1), (cxd*)scr, R);
+            if (lane < CS) {
+                cxd* dst = rho + p;
+                if (CS > 1) dst = cg::this_cluster().map_shared_rank(dst, lane);
+                *dst = pf;
+            }
+            __syncwarp();
+        }
+    }
+    auto copy_rows = [&](int first, int cnt) {
+        for (int s = 0; s < np; ++s) {
+            const int p = a.bins.ord[p0 + s];
+            if (p < K) gather_rows_cols<RW, R>(N, a0, b0, w_real(p), (RW*)a.ybuf_r + ((size_t)c * K + p) * 2 * R * N, first, cnt);
+            else gather_rows_cols<CW, R>(N, a0, b0, w_cplx(p), (CW*)a.ybuf_c + ((size_t)c * Kc + (p - K)) * 2 * R * N, first, cnt);
+        }
+    };
+    if (a.kmax <= 1 && spare > 0 && warp >= spare0 && warp < NWARP - 1)
+        copy_rows((warp - spare0) * 32 + lane, spare * 32);
+    if (CS > 1) cg::this_cluster().sync();
+    else __syncthreads();
+
+    if (warp == 0) {
         int acc;
         if (a.forced) {
             // block move: every link of the block is taken tentatively; the move is
             // decided once the whole block's ratio is known
-            bool ok = a.dead[c] == 0;
-            for (int p = 0; p < P; ++p) ok = ok && isfinite(rho[p].x) && isfinite(rho[p].y) && (rho[p].x != 0.0 || rho[p].y != 0.0);
-            if (!ok) a.dead[c] = 1;
-            acc = ok ? 1 : 0;
+            bool ok = dead == 0;
+            for (int p = lane; p < P; p += 32) ok = ok && is_fin(rho[p]) && !is_zero(rho[p]);
+            acc = __all_sync(0xffffffffu, ok) ? 1 : 0;
         } else {
-            acc = (sn > 0.0 && so > 0.0 && q.u_acc < sn / so) ? 1 : 0;
-            atomicAdd(&a.counters[0], 1ULL);
-        }
-        s_accept = acc;
-        a.accept[c] = acc;
-        if (acc) {
-            if (a.kmax > 1) a.pend[c] += 1;
-            if (!a.forced) {
-                atomicAdd(&a.counters[1], 1ULL);
-                a.since_refresh[c] += 1;
-                a.sweep_acc[c] += 1;
+            double so = 0.0, sn = 0.0;
+            for (int p = lane; p < P; p += 32) {
+                so += term[p].x;
+                sn += (term[p] * rho[p]).x;
             }
-            if constexpr (SU2) {
-                double* dst = (double*)a.links + ((size_t)c * g.n_links + l) * 4;
-                for (int k = 0; k < 4; ++k) dst[k] = s_su2[k];
+            for (int o = 16; o > 0; o >>= 1) {
+                so += __shfl_xor_sync(0xffffffffu, so, o);
+                sn += __shfl_xor_sync(0xffffffffu, sn, o);
+            }
+            acc = (sn > 0.0 && so > 0.0 && q.u_acc < sn / so) ? 1 : 0;
+        }
+        if (lane == 0) s_accept = acc;
+        if (rank == 0 && lane == 0) {
+            a.accept[c] = acc;
+            if (a.forced) {
+                if (!acc) a.dead[c] = 1;
             } else {
-                if (g.group == GGF_Z2) ((int8_t*)a.links)[(size_t)c * g.n_links + l] = (int8_t)q.g_new;
-                else ((double*)a.links)[(size_t)c * g.n_links + l] = q.th_new;
+                atomicAdd(&a.counters[0], 1ULL);
+            }
+            if (acc) {
+                if (a.kmax > 1) a.pend[c] += 1;
+                if (!a.forced) {
+                    atomicAdd(&a.counters[1], 1ULL);
+                    a.since_refresh[c] += 1;
+                    a.sweep_acc[c] += 1;
+                }
+                if constexpr (SU2) {
+                    double* dst = (double*)a.links + ((size_t)c * g.n_links + l) * 4;
+                    for (int k = 0; k < 4; ++k) dst[k] = tw[k];
+                } else {
+                    if (g.group == GGF_Z2) ((int8_t*)a.links)[(size_t)c * g.n_links + l] = (int8_t)q.g_new;
+                    else ((double*)a.links)[(size_t)c * g.n_links + l] = q.th_new;
+                }
             }
         }
     }
     __syncthreads();
     if (!s_accept) return;
-
-    for (int p = warp; p < P; p += NWARP) {
-        const bool ok = pair_z(Delta + p * r * r, Wss + p * r * r, Bord + warp * 4 * r * r, fcol + warp * r, r,
-                               a.zbuf + ((size_t)c * P + p) * r * r);
-        if (!ok && a.forced && lane == 0) a.dead[c] = 1;
-        if (lane == 0) ell_add(a.ell[(size_t)c * P + p], rho[p], p < K);
-        __syncwarp();
+    if (rank == 0 && warp == NWARP - 1)
+        for (int p = lane; p < P; p += 32) ell_add(a.ell[(size_t)c * P + p], rho[p], p < K);
+    for (int s = 0; s < np; ++s) {
+        const int p = a.bins.ord[p0 + s];
+        for (int e = threadIdx.x; e < R * R; e += NWARP * 32) a.zbuf[((size_t)c * P + p) * R * R + e] = slot(s, 2)[e];
+        if (!s_okz[s] && a.forced && threadIdx.x == 0) a.dead[c] = 1;
     }
-    // rows Y = W[S, :] and columns C^T = W[:, S]^T for the update kernel,
-    // stored per (chain, pair) as [2][r][N] (delayed mode: gather_kernel)
-    if (a.kmax > 1) return;
-    for (int p = 0; p < P; ++p) {
-        for (int e = threadIdx.x; e < r * N; e += blockDim.x) {
-            int xi = e / N, j = e - xi * N;
-            int gi = xi < g.h2 ? a0 + xi : b0 + xi - g.h2;
-            if (p < K) {
-                const RW* W = (const RW*)a.Wr + ((size_t)c * K + p) * N * N;
-                RW* yb = (RW*)a.ybuf_r + ((size_t)c * K + p) * 2 * r * N;
-                yb[(size_t)xi * N + j] = W[(size_t)gi * N + j];
-                yb[(size_t)(r + xi) * N + j] = W[(size_t)j * N + gi];
-            } else {
-                const CW* W = (const CW*)a.Wc + ((size_t)c * (P - K) + (p - K)) * N * N;
-                CW* yb = (CW*)a.ybuf_c + ((size_t)c * (P - K) + (p - K)) * 2 * r * N;
-                yb[(size_t)xi * N + j] = W[(size_t)gi * N + j];
-                yb[(size_t)(r + xi) * N + j] = W[(size_t)j * N + gi];
-            }
-        }
-    }
+    // (delayed mode: gather_kernel forms the rows and columns)
+    if (a.kmax <= 1 && spare == 0) copy_rows(threadIdx.x, NWARP * 32);
 }
 
+// W <- W - C Z Y of the accepted chains.  Bound: the traffic of W, read and
+// written once; each thread takes 16 bytes of a row and four rows at a time, so
+// that four independent loads are in flight (one element of one row at a time
+// moved 3.9 TB/s: 1024 chains of 8 x 8 Z2 took 530 us per accepted link,
+// 285 us so, 6.9 TB/s).
 template <class T, int R>
 __global__ void __launch_bounds__(256) update_kernel(int N, int P, int fam_pairs, int pair_off, T* W,
                                                      const T* ybuf, const cxd* zbuf, const int* accept, int TI) {
@@ -226,102 +411,135 @@ __global__ void __launch_bounds__(256) update_kernel(int N, int P, int fam_pairs
         Pr[i * R + b] = acc;
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        T yv[R];
+    constexpr int E = 16 / sizeof(T);       // elements per piece; N is a multiple of 8
+    const int pieces = N / E, width = min(pieces, 256), rows = 256 / width;
+    const int t = threadIdx.x % width, r0 = threadIdx.x / width;
+    if (r0 >= rows) return;
+    union Piece { float4 v; T e[E]; };
+    for (int k = t; k < pieces; k += width) {
+        T y[R][E];
 #pragma unroll
-        for (int b = 0; b < R; ++b) yv[b] = Y[(size_t)b * N + j];
-        for (int i = 0; i < ti; ++i) {
-            T acc = Wp[(size_t)(i0 + i) * N + j];
+        for (int b = 0; b < R; ++b) {
+            Piece u;
+            u.v = ((const float4*)(Y + (size_t)b * N))[k];
 #pragma unroll
-            for (int b = 0; b < R; ++b) acc -= Pr[i * R + b] * yv[b];
-            Wp[(size_t)(i0 + i) * N + j] = acc;
+            for (int x = 0; x < E; ++x) y[b][x] = u.e[x];
+        }
+        for (int i = r0; i < ti; i += 4 * rows) {
+            Piece w[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (i + m * rows < ti) w[m].v = ((const float4*)(Wp + (size_t)(i0 + i + m * rows) * N))[k];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int ii = i + m * rows;
+                if (ii >= ti) break;
+#pragma unroll
+                for (int x = 0; x < E; ++x) {
+                    T acc = w[m].e[x];
+#pragma unroll
+                    for (int b = 0; b < R; ++b) acc -= Pr[ii * R + b] * y[b][x];
+                    w[m].e[x] = acc;
+                }
+                ((float4*)(Wp + (size_t)(i0 + ii) * N))[k] = w[m].v;
+            }
         }
     }
 }
 
-// Delayed mode, accepted chains: rows Y = W_eff[S, :] and columns
+// Block moves, accepted chains: rows Y = W_eff[S, :] and columns
 // C = W_eff[:, S] of the effective inverse W_eff = W - U V, then the new
 // panel entries U[:, slot] = C Z and V[slot, :] = Y (stored as V^T rows).
-// Grid (ceil(N / 128), family pairs, chains), 128 threads, one index each.
+// Grid (ceil(N / 128), pairs, chains), 128 threads, one index each: its panel
+// rows are read straight from the chunk-major panels (eight rank columns of
+// neighbouring rows are one run), the rows on S from shared memory.
+// Bound: panel reads from L2 and FP32 arithmetic at high rank; with the panel
+// rows staged element by element, and a launch per family, a block-move link of
+// 32 chains of 8 x 8 U(1), K = 2 took 150 us, 59 so.
 template <class T, int R>
-__global__ void __launch_bounds__(128) gather_kernel(Geometry g, int P, int fam_pairs, int pair_off, int link_all,
-                                                     const int* link_of_chain, const T* W,
-                                                     typename Sc<T>::R* Pan, const cxd* zbuf,
-                                                     const int* accept, const int* pend, int kmax) {
+__device__ __forceinline__ void gather_pair(const Geometry& g, const int* S, const T* Wp, typename Sc<T>::R* U,
+                                            const cxd* Z, int kr, int KRM, unsigned char* smraw) {
     typedef typename Sc<T>::R RR;
-    const int c = blockIdx.z;
-    if (!accept[c]) return;
-    const int p = blockIdx.y, N = g.N;
-    const int slot = pend[c] - 1, kr = slot * R;
-    const int KRM = kmax * R, NP = panel_rows(N);
+    const int N = g.N, NP = panel_rows(N);
     const size_t NK = panel_plane(N, KRM);
-    extern __shared__ unsigned char smraw[];
-    constexpr int QC = 128 / sizeof(T);  // rank chunk staged per step
     T* UtS = (T*)smraw;            // [kr][R]  U[S_a, q]
-    T* VS = UtS + kmax * R * R;    // [kr][R]  V[q, S_a]
-    T* Zs = VS + kmax * R * R;     // [R][R]
-    T* Uc = Zs + R * R;            // [128][QC + 1] panel rows j0.., rank chunk
-    T* Vc = Uc + 128 * (QC + 1);
-    __shared__ int S[R];
-    const int link = link_of_chain ? link_of_chain[c] : link_all;
-    const int s = link >> 1, d = link & 1, x = s % g.L, y = s / g.L;
-    const int t = d == 0 ? y * g.L + (x + 1) % g.L : ((y + 1) % g.L) * g.L + x;
-    const int a0 = s * g.B + (2 * d + 1) * g.h2, b0 = t * g.B + (2 * d) * g.h2;
-    if (threadIdx.x < R) S[threadIdx.x] = threadIdx.x < g.h2 ? a0 + threadIdx.x : b0 + threadIdx.x - g.h2;
-    __syncthreads();
-    const size_t base = ((size_t)c * fam_pairs + p);
-    const T* Wp = W + base * N * N;
-    RR* U = Pan + base * 2 * PanelIO<T>::PLANES * NK;
+    T* VS = UtS + (size_t)KRM * R; // [kr][R]  V[q, S_a]
+    T* Zs = VS + (size_t)KRM * R;  // [R][R]
     RR* Vt = U + PanelIO<T>::PLANES * NK;
-    const cxd* Z = zbuf + ((size_t)c * P + pair_off + p) * R * R;
     for (int e = threadIdx.x; e < kr * R; e += blockDim.x) {
-        int q = e / R, a = e % R;
-        UtS[e] = PanelIO<T>::ld(U, NK, pidx(S[a], q, NP));
-        VS[e] = PanelIO<T>::ld(Vt, NK, pidx(S[a], q, NP));
+        const int a = e / kr, q = e - a * kr;
+        UtS[q * R + a] = PanelIO<T>::ld(U, NK, pidx(S[a], q, NP));
+        VS[q * R + a] = PanelIO<T>::ld(Vt, NK, pidx(S[a], q, NP));
     }
     for (int e = threadIdx.x; e < R * R; e += blockDim.x) Zs[e] = Sc<T>::from(Z[e]);
     __syncthreads();
-    const int j0 = blockIdx.x * blockDim.x;
-    const int j = j0 + threadIdx.x;
-    const bool live = j < N;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= N) return;
     T yv[R], cv[R];
 #pragma unroll
     for (int a = 0; a < R; ++a) {
-        yv[a] = live ? Wp[(size_t)S[a] * N + j] : Sc<T>::zero();
-        cv[a] = live ? Wp[(size_t)j * N + S[a]] : Sc<T>::zero();
+        yv[a] = Wp[(size_t)S[a] * N + j];
+        cv[a] = Wp[(size_t)j * N + S[a]];
     }
-    // panel rows j0 .. j0+127 staged chunk by chunk with coalesced loads
-    for (int q0 = 0; q0 < kr; q0 += QC) {
-        const int qn = min(QC, kr - q0);
-        __syncthreads();
-        for (int e = threadIdx.x; e < 128 * QC; e += blockDim.x) {
-            int row = e / QC, qq = e % QC;
-            bool ok = qq < qn && j0 + row < N;
-            size_t idx = pidx(j0 + row, q0 + qq, NP);
-            Uc[row * (QC + 1) + qq] = ok ? PanelIO<T>::ld(U, NK, idx) : Sc<T>::zero();
-            Vc[row * (QC + 1) + qq] = ok ? PanelIO<T>::ld(Vt, NK, idx) : Sc<T>::zero();
+    // R rank columns per step (kr is a multiple of R, and R of them stay within a
+    // chunk), the next step's loaded before this one's products
+    T un[R], vn[R];
+    if (kr > 0) {
+        panel_load<T, R>(U + pidx(j, 0, NP), NK, un);
+        panel_load<T, R>(Vt + pidx(j, 0, NP), NK, vn);
+    }
+    for (int q0 = 0; q0 < kr; q0 += R) {
+        T uq[R], vq[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) { uq[k] = un[k]; vq[k] = vn[k]; }
+        if (q0 + R < kr) {
+            const size_t at = pidx(j, q0 + R, NP);
+            panel_load<T, R>(U + at, NK, un);
+            panel_load<T, R>(Vt + at, NK, vn);
         }
-        __syncthreads();
-        for (int qq = 0; qq < qn; ++qq) {
-            const T vq = Vc[threadIdx.x * (QC + 1) + qq];
-            const T uq = Uc[threadIdx.x * (QC + 1) + qq];
-            const int q = q0 + qq;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
 #pragma unroll
             for (int a = 0; a < R; ++a) {
-                yv[a] -= UtS[q * R + a] * vq;
-                cv[a] -= uq * VS[q * R + a];
+                acc_sub(yv[a], UtS[(q0 + k) * R + a], vq[k]);
+                acc_sub(cv[a], uq[k], VS[(q0 + k) * R + a]);
             }
         }
     }
-    if (!live) return;
+    T u[R];
 #pragma unroll
     for (int b = 0; b < R; ++b) {
-        T u = Sc<T>::zero();
+        u[b] = Sc<T>::zero();
 #pragma unroll
-        for (int a = 0; a < R; ++a) u += cv[a] * Zs[a * R + b];
-        PanelIO<T>::st(U, NK, pidx(j, kr + b, NP), u);
-        PanelIO<T>::st(Vt, NK, pidx(j, kr + b, NP), yv[b]);
+        for (int a = 0; a < R; ++a) acc_add(u[b], cv[a], Zs[a * R + b]);
     }
+    const size_t at = pidx(j, kr, NP);
+    panel_store<T, R>(U + at, NK, u);
+    panel_store<T, R>(Vt + at, NK, yv);
+}
+
+template <class RW, class CW, int R>
+__global__ void __launch_bounds__(128) gather_kernel(Geometry g, int K, int Kc, int link_all, const int* link_of_chain,
+                                                     const RW* Wr, const CW* Wc, typename Sc<RW>::R* Pr,
+                                                     typename Sc<RW>::R* Pc, const cxd* zbuf, const int* accept,
+                                                     const int* pend, int kmax) {
+    const int c = blockIdx.z;
+    if (!accept[c]) return;
+    const int p = blockIdx.y, N = g.N, P = K + Kc;
+    const int kr = (pend[c] - 1) * R, KRM = kmax * R;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int S[R];
+    int a0, b0;
+    link_ends(g, link_of_chain ? link_of_chain[c] : link_all, a0, b0);
+    if (threadIdx.x < R) S[threadIdx.x] = link_majorana(g, a0, b0, threadIdx.x);
+    __syncthreads();
+    const size_t NK = panel_plane(N, KRM), NN = (size_t)N * N;
+    const cxd* Z = zbuf + ((size_t)c * P + p) * R * R;
+    if (p < K)
+        gather_pair<RW, R>(g, S, Wr + ((size_t)c * K + p) * NN, Pr + ((size_t)c * K + p) * 2 * NK, Z, kr, KRM, smraw);
+    else
+        gather_pair<CW, R>(g, S, Wc + ((size_t)c * Kc + (p - K)) * NN, Pc + ((size_t)c * Kc + (p - K)) * 4 * NK, Z, kr, KRM,
+                           smraw);
 }
 
 // W <- W - U V over the pending panels (rank pend[c] * R), SIMT tiled product
@@ -452,10 +670,6 @@ __global__ void mark_refresh(int n_chains, int R, const int* since, int* list) {
 ggf_status ggf_flush(ggf_ctx* ctx, cudaStream_t st);
 ggf_status ggf_flush_tc(ggf_ctx* ctx, cudaStream_t st, int* launches);
 
-size_t ggf_ratio_smem(int P, int r) {
-    return (size_t)(2 * P * r * r + NWARP * 4 * r * r + P + NWARP * r) * sizeof(cxd);
-}
-
 ggf_status ggf_link_step_ex(ggf_ctx* ctx, int link, cudaStream_t st, const int* link_of_chain, const double* forced,
                             int forced_k, int* dead);
 
@@ -498,42 +712,47 @@ ggf_status ggf_link_step_ex(ggf_ctx* ctx, int link, cudaStream_t st, const int* 
     a.dead = dead;
     a.pend = ch.pend;
     a.kmax = ch.kmax;
-    size_t smem = ggf_ratio_smem(ctx->P, g.r);
+    const int CS = deal_pairs(ctx->K, ctx->Kc, a.bins);
+    size_t smem = 0;
+    for (int b = 0; b < CS; ++b)
+        smem = std::max(smem, ratio_layout(ctx->P, g.r, a.bins.first[b + 1] - a.bins.first[b],
+                                           ch.kmax > 1 ? ch.kmax * g.r : 0, 2 * rsz).total);
     const int ev0 = ctx->prof_mark(st);
     ctx->launches += 2 + (ctx->Kc ? 1 : 0);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ch.n * CS);
+    cfg.blockDim = dim3(NWARP * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CS;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CS > 1 ? 1 : 0;
     if (g.group == GGF_SU2) {
-        if (fp64) ratio_kernel<double, cxd, true><<<ch.n, NWARP * 32, smem, st>>>(a);
-        else ratio_kernel<float, cxf, true><<<ch.n, NWARP * 32, smem, st>>>(a);
+        if (fp64) GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<double, cxd, true, 8>, a));
+        else GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<float, cxf, true, 8>, a));
+    } else if (g.r == 4) {
+        if (fp64) GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<double, cxd, false, 4>, a));
+        else GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<float, cxf, false, 4>, a));
     } else {
-        if (fp64) ratio_kernel<double, cxd, false><<<ch.n, NWARP * 32, smem, st>>>(a);
-        else ratio_kernel<float, cxf, false><<<ch.n, NWARP * 32, smem, st>>>(a);
+        if (fp64) GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<double, cxd, false, 8>, a));
+        else GGF_CK(cudaLaunchKernelEx(&cfg, ratio_kernel<float, cxf, false, 8>, a));
     }
-    GGF_CK(cudaGetLastError());
     const int ev1 = ctx->prof_mark(st);
     ctx->prof_pair(GGF_KT_RATIO, ev0, ev1);
     const int N = g.N;
     if (ch.kmax > 1) {
-        dim3 gg((N + 127) / 128, ctx->K, ch.n), gc2((N + 127) / 128, ctx->Kc, ch.n);
-#define GGF_GATH(T, R_, grid, fam, off, Wp, Pp)                                                               \
-    gather_kernel<T, R_><<<grid, 128, (2 * ch.kmax * R_ * R_ + R_ * R_ + 2 * 128 * (128 / sizeof(T) + 1)) * sizeof(T), st>>>( \
-        g, ctx->P, fam, off, link, link_of_chain, (const T*)(Wp), (typename Sc<T>::R*)(Pp), a.zbuf, ch.accept, \
-        ch.pend, ch.kmax)
+        dim3 gg((N + 127) / 128, ctx->P, ch.n);
+#define GGF_GATH(RW, CW, R_)                                                                                         \
+    gather_kernel<RW, CW, R_><<<gg, 128, (2 * (size_t)ch.kmax * R_ * R_ + R_ * R_) * sizeof(CW), st>>>(                \
+        g, ctx->K, ctx->Kc, link, link_of_chain, (const RW*)ch.Wr, (const CW*)ch.Wc, (typename Sc<RW>::R*)ch.Pr,       \
+        (typename Sc<RW>::R*)ch.Pc, a.zbuf, ch.accept, ch.pend, ch.kmax)
         if (g.r == 4) {
-            if (fp64) {
-                GGF_GATH(double, 4, gg, ctx->K, 0, ch.Wr, ch.Pr);
-                if (ctx->Kc) GGF_GATH(cxd, 4, gc2, ctx->Kc, ctx->K, ch.Wc, ch.Pc);
-            } else {
-                GGF_GATH(float, 4, gg, ctx->K, 0, ch.Wr, ch.Pr);
-                if (ctx->Kc) GGF_GATH(cxf, 4, gc2, ctx->Kc, ctx->K, ch.Wc, ch.Pc);
-            }
+            if (fp64) GGF_GATH(double, cxd, 4); else GGF_GATH(float, cxf, 4);
         } else {
-            if (fp64) {
-                GGF_GATH(double, 8, gg, ctx->K, 0, ch.Wr, ch.Pr);
-                if (ctx->Kc) GGF_GATH(cxd, 8, gc2, ctx->Kc, ctx->K, ch.Wc, ch.Pc);
-            } else {
-                GGF_GATH(float, 8, gg, ctx->K, 0, ch.Wr, ch.Pr);
-                if (ctx->Kc) GGF_GATH(cxf, 8, gc2, ctx->Kc, ctx->K, ch.Wc, ch.Pc);
-            }
+            if (fp64) GGF_GATH(double, cxd, 8); else GGF_GATH(float, cxf, 8);
         }
 #undef GGF_GATH
         GGF_CK(cudaGetLastError());
@@ -542,7 +761,8 @@ ggf_status ggf_link_step_ex(ggf_ctx* ctx, int link, cudaStream_t st, const int* 
         if (++ch.steps_since_flush >= ch.kmax) GGF_TRY(ggf_flush(ctx, st));
         return GGF_OK;
     }
-    const int TI = 8;
+    // rows per CTA: 32 amortise its rank columns where they still fill the chip
+    const int TI = (long long)ch.n * ctx->P * (N / 32) >= 8LL * ctx->n_sms ? 32 : 8;
     dim3 gr((N + TI - 1) / TI, ctx->K, ch.n);
     dim3 gc((N + TI - 1) / TI, ctx->Kc, ch.n);
 #define GGF_UPD(T, R_, grid, fam, off, Wp, Yp)                                                         \
@@ -612,7 +832,6 @@ ggf_status ggf_prepare_sampler(ggf_ctx* ctx) {
     if (ctx->device >= 0 && ctx->device < 64 && done[ctx->device]) return GGF_OK;
     int mx = 0;
     GGF_CK(cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-    if (ggf_ratio_smem(36, 8) > (size_t)mx) return ggf_fail(ctx, GGF_EINVAL, "shared memory too small for K = 8");
     // dynamic cap = opt-in limit minus the kernel's static shared memory
     auto cap = [&](const void* fn) -> ggf_status {
         cudaFuncAttributes fa;
@@ -620,18 +839,16 @@ ggf_status ggf_prepare_sampler(ggf_ctx* ctx) {
         GGF_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, mx - (int)fa.sharedSizeBytes));
         return GGF_OK;
     };
-    GGF_TRY(cap((const void*)ratio_kernel<double, cxd, false>));
-    GGF_TRY(cap((const void*)ratio_kernel<float, cxf, false>));
-    GGF_TRY(cap((const void*)ratio_kernel<double, cxd, true>));
-    GGF_TRY(cap((const void*)ratio_kernel<float, cxf, true>));
-    GGF_TRY(cap((const void*)gather_kernel<double, 4>));
-    GGF_TRY(cap((const void*)gather_kernel<double, 8>));
-    GGF_TRY(cap((const void*)gather_kernel<float, 4>));
-    GGF_TRY(cap((const void*)gather_kernel<float, 8>));
-    GGF_TRY(cap((const void*)gather_kernel<cxd, 4>));
-    GGF_TRY(cap((const void*)gather_kernel<cxd, 8>));
-    GGF_TRY(cap((const void*)gather_kernel<cxf, 4>));
-    GGF_TRY(cap((const void*)gather_kernel<cxf, 8>));
+    GGF_TRY(cap((const void*)ratio_kernel<double, cxd, false, 4>));
+    GGF_TRY(cap((const void*)ratio_kernel<double, cxd, false, 8>));
+    GGF_TRY(cap((const void*)ratio_kernel<float, cxf, false, 4>));
+    GGF_TRY(cap((const void*)ratio_kernel<float, cxf, false, 8>));
+    GGF_TRY(cap((const void*)ratio_kernel<double, cxd, true, 8>));
+    GGF_TRY(cap((const void*)ratio_kernel<float, cxf, true, 8>));
+    GGF_TRY(cap((const void*)gather_kernel<double, cxd, 4>));
+    GGF_TRY(cap((const void*)gather_kernel<double, cxd, 8>));
+    GGF_TRY(cap((const void*)gather_kernel<float, cxf, 4>));
+    GGF_TRY(cap((const void*)gather_kernel<float, cxf, 8>));
     if (ctx->device >= 0 && ctx->device < 64) done[ctx->device] = true;
     return GGF_OK;
 }

@@ -35,8 +35,6 @@ namespace {
 
 constexpr int ST = 256;            // threads per CTA
 constexpr int SWARPS = ST / 32;
-constexpr int MAXP = 36;           // pairs at K = 8
-constexpr int MAXCS = 8;           // portable cluster size
 
 struct StepArgs {
     DevConst dc;
@@ -53,11 +51,11 @@ struct StepArgs {
     int* pend;
     void* Sr;         // small matrices [n][K][2][KRM][KRM]: G0 then X
     void* Sc_;        // [n][Kc][2][KRM][KRM]
-    // pairs ord[first[b]] .. ord[first[b + 1] - 1] belong to CTA b of the
-    // cluster; resident[b]: their matrices live in shared memory; tables[b]: so
+    PairBins bins;
+    // resident[b]: the matrices of CTA b's pairs live in shared memory; tables[b]: so
     // do every link's Delta and the slices of G0 (else Delta link by link, and
     // the slices read in place)
-    unsigned char first[MAXCS + 1], ord[MAXP], resident[MAXCS], tables[MAXCS];
+    unsigned char resident[MAXCS], tables[MAXCS];
 };
 
 // Byte offsets of a CTA's shared arrays (host and device compute the same).
@@ -98,30 +96,6 @@ __host__ __device__ inline StepLayout step_layout(int P, int r, int kb, int KRM,
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
-}
-
-template <class T> struct Fp64Of;
-template <> struct Fp64Of<double> { typedef double Z; };
-template <> struct Fp64Of<float> { typedef double Z; };
-template <> struct Fp64Of<cxd> { typedef cxd Z; };
-template <> struct Fp64Of<cxf> { typedef cxd Z; };
-
-template <class T> __device__ __forceinline__ typename Fp64Of<T>::Z wide(T v);
-template <> __device__ __forceinline__ double wide<double>(double v) { return v; }
-template <> __device__ __forceinline__ double wide<float>(float v) { return v; }
-template <> __device__ __forceinline__ cxd wide<cxd>(cxd v) { return v; }
-template <> __device__ __forceinline__ cxd wide<cxf>(cxf v) { return {(double)v.x, (double)v.y}; }
-__device__ __forceinline__ double narrow(double v, double) { return v; }
-__device__ __forceinline__ float narrow(double v, float) { return (float)v; }
-__device__ __forceinline__ cxd narrow(cxd v, cxd) { return v; }
-__device__ __forceinline__ cxf narrow(cxd v, cxf) { return {(float)v.x, (float)v.y}; }
-
-// Element (xi, yi) of Delta = O' G O'^T - O G O^T of link l for pair p of its family.
-template <class Z>
-__device__ __forceinline__ Z delta_elem(const DevConst& dc, int p, int l, int xi, int yi, const Proposal& q,
-                                        const double* tw, bool su2) {
-    if (su2) return twisted_su2<Z>(dc, p, l, xi, yi, tw + 20) - twisted_su2<Z>(dc, p, l, xi, yi, tw + 4);
-    return twisted_tab<Z>(dc, p, l, xi, yi, q.g_new, tw + 4) - twisted_tab<Z>(dc, p, l, xi, yi, q.g_old, tw);
 }
 
 // One pair's part of link j before the decision: the ratio (task 0) or Z (task 1).
@@ -288,9 +262,9 @@ __global__ void __launch_bounds__(ST, 2) batch_steps(StepArgs a) {
     const int CS = cg::this_cluster().num_blocks(), rank = cg::this_cluster().block_rank();
     const int c = blockIdx.x / CS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int p0 = a.first[rank], np = a.first[rank + 1] - p0;
+    const int p0 = a.bins.first[rank], np = a.bins.first[rank + 1] - p0;
     int nc = 0;
-    for (int s = 0; s < np; ++s) nc += a.ord[p0 + s] >= K;
+    for (int s = 0; s < np; ++s) nc += a.bins.ord[p0 + s] >= K;
     const bool resident = a.resident[rank], tables = a.tables[rank];
     const StepLayout lay = step_layout(P, R, kb, KRM, np, nc, sizeof(RW), sizeof(CW), resident, tables);
     const int kbt = tables ? kb : 1;
@@ -307,8 +281,8 @@ __global__ void __launch_bounds__(ST, 2) batch_steps(StepArgs a) {
 
     // the CTA's real pairs come before its complex ones (nr of them)
     const int nr = np - nc;
-    auto g0_real = [&](int s) { return (RW*)a.Sr + ((size_t)c * K + a.ord[p0 + s]) * 2 * SS; };
-    auto g0_cplx = [&](int s) { return (CW*)a.Sc_ + ((size_t)c * Kc + (a.ord[p0 + s] - K)) * 2 * SS; };
+    auto g0_real = [&](int s) { return (RW*)a.Sr + ((size_t)c * K + a.bins.ord[p0 + s]) * 2 * SS; };
+    auto g0_cplx = [&](int s) { return (CW*)a.Sc_ + ((size_t)c * Kc + (a.bins.ord[p0 + s] - K)) * 2 * SS; };
     auto mat_real = [&](int s) {
         return resident ? (RW*)(sm + lay.mat) + (size_t)s * KRM * ldr : g0_real(s) + SS;
     };
@@ -366,7 +340,7 @@ __global__ void __launch_bounds__(ST, 2) batch_steps(StepArgs a) {
     // Delta of the links j0 .. j0 + kbt - 1
     auto fill_delta = [&](int j0) {
         for (int s = 0; s < np; ++s) {
-            const int p = a.ord[p0 + s];
+            const int p = a.bins.ord[p0 + s];
             for (int e = threadIdx.x; e < kbt * R * R; e += ST) {
                 const int j = j0 + e / (R * R), x = e % (R * R);
                 if (s < nr) del_real(s)[e] = delta_elem<double>(a.dc, p, a.l0 + j, x / R, x % R, props[j], tws + j * 36, SU2);
@@ -409,7 +383,7 @@ __global__ void __launch_bounds__(ST, 2) batch_steps(StepArgs a) {
             }
         }
         for (int t = warp; t < 2 * np; t += SWARPS) {
-            const int s = t >> 1, p = a.ord[p0 + s];
+            const int s = t >> 1, p = a.bins.ord[p0 + s];
             void* scr = sm + lay.task + (size_t)warp * lay.task_bytes;
             if (s < nr) {
                 const double* D = del_real(s) + dj * R * R;
@@ -511,40 +485,24 @@ __global__ void __launch_bounds__(ST, 2) batch_steps(StepArgs a) {
     }
 }
 
-// Pairs to CTAs: bins of about one complex or two real pairs (a complex pair
-// costs four real ones), at most MAXCS, the heaviest dealt first to the
-// lightest bin; in each bin real pairs come first.  Returns the CTAs and the
-// shared memory of the largest.
+// Bins of the pairs (deal_pairs), and for each CTA how much of its data fits in
+// shared memory.  Returns the CTAs and the shared memory of the largest.
 int step_bins(int K, int Kc, int r, int kb, int KRM, size_t rw, size_t cw, size_t smem_max, StepArgs& a, size_t& smem) {
-    const int P = K + Kc;
-    const int CS = std::max(1, std::min(MAXCS, Kc + (K + 1) / 2));
-    int load[MAXCS] = {0}, bin[MAXP];
-    for (int k = 0; k < P; ++k) {
-        const int p = k < Kc ? K + k : k - Kc;       // complex pairs first
-        int b = 0;
-        for (int q = 1; q < CS; ++q)
-            if (load[q] < load[b]) b = q;
-        bin[p] = b;
-        load[b] += p >= K ? 4 : 1;
-    }
-    int n = 0;
+    const int CS = deal_pairs(K, Kc, a.bins);
     smem = 0;
     for (int b = 0; b < CS; ++b) {
-        a.first[b] = (unsigned char)n;
+        const int np = a.bins.first[b + 1] - a.bins.first[b];
         int nc = 0;
-        for (int p = 0; p < P; ++p)
-            if (bin[p] == b) { a.ord[n++] = (unsigned char)p; nc += p >= K; }
-        const int np = n - a.first[b];
+        for (int s = 0; s < np; ++s) nc += a.bins.ord[a.bins.first[b] + s] >= K;
         size_t need = 0;
         for (int level = 0; level < 3; ++level) {
             a.resident[b] = level == 0;
             a.tables[b] = level < 2;
-            need = step_layout(P, r, kb, KRM, np, nc, rw, cw, level == 0, level < 2).total;
+            need = step_layout(K + Kc, r, kb, KRM, np, nc, rw, cw, level == 0, level < 2).total;
             if (need <= smem_max) break;
         }
         smem = std::max(smem, need);
     }
-    a.first[CS] = (unsigned char)n;
     return CS;
 }
 
