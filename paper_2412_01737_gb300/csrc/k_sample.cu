@@ -447,6 +447,38 @@ __global__ void __launch_bounds__(256) update_kernel(int N, int P, int fam_pairs
     }
 }
 
+// Products of the block-move gather.  FP32 complex ones with their roundings
+// written out (which of the two terms of the imaginary part is rounded first
+// shows in the last bit of the panels, and through a block move's low-weight
+// configurations far above it): im = fma(ax, by, ay bx) for MF = false,
+// fma(ay, bx, ax by) for MF = true; re = fma(ax, bx, -(ay by)).
+template <bool MF, class T> __device__ __forceinline__ T gather_mul(T a, T b) {
+    if constexpr (sizeof(T) == sizeof(cxf) && Sc<T>::CPLX) {
+        T r;
+        r.x = __fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y));
+        r.y = MF ? __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)) : __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x));
+        return r;
+    } else {
+        return a * b;
+    }
+}
+template <bool MF, class T> __device__ __forceinline__ void gather_sub(T& r, T a, T b) {
+    if constexpr (sizeof(T) == sizeof(cxf) && Sc<T>::CPLX) {
+        const T t = gather_mul<MF>(a, b);
+        r = {__fsub_rn(r.x, t.x), __fsub_rn(r.y, t.y)};
+    } else {
+        acc_sub(r, a, b);
+    }
+}
+template <bool MF, class T> __device__ __forceinline__ void gather_add(T& r, T a, T b) {
+    if constexpr (sizeof(T) == sizeof(cxf) && Sc<T>::CPLX) {
+        const T t = gather_mul<MF>(a, b);
+        r = {__fadd_rn(r.x, t.x), __fadd_rn(r.y, t.y)};
+    } else {
+        acc_add(r, a, b);
+    }
+}
+
 // Block moves, accepted chains: rows Y = W_eff[S, :] and columns
 // C = W_eff[:, S] of the effective inverse W_eff = W - U V, then the new
 // panel entries U[:, slot] = C Z and V[slot, :] = Y (stored as V^T rows).
@@ -501,8 +533,8 @@ __device__ __forceinline__ void gather_pair(const Geometry& g, const int* S, con
         for (int k = 0; k < R; ++k) {
 #pragma unroll
             for (int a = 0; a < R; ++a) {
-                acc_sub(yv[a], UtS[(q0 + k) * R + a], vq[k]);
-                acc_sub(cv[a], uq[k], VS[(q0 + k) * R + a]);
+                gather_sub<false>(yv[a], UtS[(q0 + k) * R + a], vq[k]);
+                gather_sub<true>(cv[a], uq[k], VS[(q0 + k) * R + a]);
             }
         }
     }
@@ -511,7 +543,7 @@ __device__ __forceinline__ void gather_pair(const Geometry& g, const int* S, con
     for (int b = 0; b < R; ++b) {
         u[b] = Sc<T>::zero();
 #pragma unroll
-        for (int a = 0; a < R; ++a) acc_add(u[b], cv[a], Zs[a * R + b]);
+        for (int a = 0; a < R; ++a) gather_add<true>(u[b], cv[a], Zs[a * R + b]);
     }
     const size_t at = pidx(j, kr, NP);
     panel_store<T, R>(U + at, NK, u);
