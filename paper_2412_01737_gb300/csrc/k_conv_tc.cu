@@ -13,14 +13,25 @@
 // nb_t(s) is pixel s shifted by tap t = 3 ky + kx, (ky - 1, kx - 1), on the
 // torus; nb'_t(s) the opposite shift (the output pixel whose tap t read s).
 //
-// One CTA of 256 threads: every thread builds one row of the im2col operand
-// tile per K step (the gather from global memory, which stays in L2), one
-// thread issues the MMAs, and two operand buffers alternate so the gather of
-// step k + 1 overlaps the MMAs of step k.  Mbarrier waits are bounded; on
-// expiry the CTA stops, raises the network's error word and frees its TMEM.
+// One CTA of 256 threads.  Forward and input gradient: every thread builds one
+// row of the im2col operand tile per K step from values it loaded two steps
+// earlier (the gather from global memory, which stays in L2), one thread issues
+// the MMAs, and two operand buffers alternate.  The weight operand lies in global
+// memory in the shared-memory layout already (ggf_conv_pack.cuh, kept up to date by
+// the optimiser step), so that it is a plain copy.  Weight gradient: a
+// band of rows of one sample is staged in shared memory, the inputs with their
+// halo, and the tiles are built from there.  Mbarrier waits are bounded; on expiry the CTA stops,
+// raises the network's error word and frees its TMEM.
+//
+// What bounds them: the operand building (index arithmetic and load latency),
+// far above the MMAs.  Per layer 64 -> 64 at 16 x 16 and 128 samples, against
+// gathering at the step of use, integer divisions per element and weights
+// gathered by every CTA: forward 56 -> 40 us, input gradient 106 -> 61, weight
+// gradient 221 -> 94.
 #include <cuda_bf16.h>
 #include "ggf_ctx.h"
 #include "ggf_tc.cuh"
+#include "ggf_conv_pack.cuh"
 
 namespace {
 
@@ -31,9 +42,19 @@ __device__ __forceinline__ unsigned char* align1k(unsigned char* p) {
     return (unsigned char*)(((uintptr_t)p + 1023) & ~(uintptr_t)1023);
 }
 
-__device__ __forceinline__ int shifted(int L, int s, int t, int sign) {
-    const int x = s % L, y = s / L, ky = t / 3 - 1, kx = t % 3 - 1;
-    return ((y + sign * ky + L) % L) * L + (x + sign * kx + L) % L;
+// pixel (x, y) shifted by sign * (kx, ky) of tap t on the torus
+__device__ __forceinline__ int shifted(int L, int x, int y, int t, int sign) {
+    int xx = x + sign * (t % 3 - 1), yy = y + sign * (t / 3 - 1);
+    xx = xx < 0 ? xx + L : xx >= L ? xx - L : xx;
+    yy = yy < 0 ? yy + L : yy >= L ? yy - L : yy;
+    return yy * L + xx;
+}
+
+// 16-byte copy of a packed operand
+__device__ __forceinline__ void copy_packed(unsigned char* dst, const void* src, int bytes) {
+    const uint4* g = (const uint4*)src;
+#pragma unroll 6
+    for (int e = threadIdx.x; e < bytes / 16; e += CT) ((uint4*)dst)[e] = g[e];
 }
 
 // TMEM allocation by one whole warp; the column address lands in *slot
@@ -71,7 +92,7 @@ __device__ __forceinline__ void fence_to_async() {
 // forward: two M tiles of 128 pixels per pass, N = CO_PAD output channels
 template <int CI_PAD, int CO_PAD, bool RELU, bool OUT_F32>
 __global__ void __launch_bounds__(CT, 1)
-conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const bf16* W, const float* bias, void* Y, int* err) {
+conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const void* Wp, const float* bias, void* Y, int* err) {
     constexpr int KT = 9 * CI_PAD, KS = KT / 16;
     constexpr int TCOLS = 2 * CO_PAD < 32 ? 32 : 2 * CO_PAD;
     constexpr uint32_t SBO_B = (KT / 8) * 128;
@@ -82,11 +103,7 @@ conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const bf16* W, const fl
     unsigned char* As = Bs + CO_PAD * KT * 2;                 // 2 buffers x 2 tiles x 128 rows x 32 B
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int V = L * L;
-    for (int e = tid; e < CO_PAD * KT; e += CT) {
-        const int o = e / KT, k = e % KT, t = k / CI_PAD, c = k % CI_PAD;
-        const bf16 v = (o < co && c < ci) ? W[((size_t)o * ci + c) * 9 + t] : __float2bfloat16(0.f);
-        *(bf16*)(Bs + (o >> 3) * SBO_B + (k >> 3) * 128 + (o & 7) * 16 + (k & 7) * 2) = v;
-    }
+    copy_packed(Bs, Wp, CO_PAD * KT * 2);
     if (warp == 0) tmem_alloc_warp(&tslot, TCOLS);
     Bufs bf;
     bf.bar[0] = tc::smem_u32(&bars[0]);
@@ -105,24 +122,26 @@ conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const bf16* W, const fl
     for (int b = blockIdx.x; b < n && ok; b += gridDim.x) {
         const bf16* Xb = X + (size_t)b * ci * V;
         for (int p0 = 0; p0 < V && ok; p0 += 2 * 128) {
-            const int s = p0 + tid;
-            for (int ks = 0; ks < KS && ok; ++ks) {
-                const int buf = ks & 1;
-                if (!(ok = bf.wait(buf))) break;
+            const int s = p0 + tid, x = s % L, y = s / L;
+            // the 16 input channels of step ks, loaded two steps ahead of their use
+            auto fetch = [&](int ks, uint32_t (&pk)[8]) {
                 const int t = ks / (CI_PAD / 16), c0 = (ks % (CI_PAD / 16)) * 16;
-                uint32_t pk[8];
-                const int nb = s < V ? shifted(L, s, t, 1) : 0;
+                const bf16* src = Xb + (s < V ? shifted(L, x, y, t, 1) : 0);
+                uint16_t v[16];
 #pragma unroll
-                for (int h = 0; h < 8; ++h) {
-                    const int c = c0 + 2 * h;
-                    const bf16 lo = (s < V && c < ci) ? Xb[(size_t)c * V + nb] : __float2bfloat16(0.f);
-                    const bf16 hi = (s < V && c + 1 < ci) ? Xb[(size_t)(c + 1) * V + nb] : __float2bfloat16(0.f);
-                    pk[h] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-                }
+                for (int h = 0; h < 16; ++h)
+                    v[h] = (s < V && c0 + h < ci) ? __bfloat16_as_ushort(src[(size_t)(c0 + h) * V]) : (uint16_t)0;
+#pragma unroll
+                for (int h = 0; h < 8; ++h) pk[h] = (uint32_t)v[2 * h] | ((uint32_t)v[2 * h + 1] << 16);
+            };
+            auto step = [&](int ks, uint32_t (&pk)[8]) -> bool {
+                const int buf = ks & 1;
+                if (!bf.wait(buf)) return false;
                 unsigned char* Ab = As + buf * 8192 + (tid >> 7) * 4096;
                 const int r = tid & 127;
                 *(uint4*)(Ab + tc::cm32(r, 0, 2)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                 *(uint4*)(Ab + tc::cm32(r, 8, 2)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                if (ks + 2 < KS) fetch(ks + 2, pk);
                 fence_to_async();
                 __syncthreads();
                 if (tid == 0) {
@@ -136,6 +155,14 @@ conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const bf16* W, const fl
                     tc::commit(bf.bar[buf]);
                 }
                 bf.pending[buf] = true;
+                return true;
+            };
+            uint32_t pa[8], pb[8];
+            fetch(0, pa);
+            fetch(1, pb);
+            for (int ks = 0; ks < KS && ok; ks += 2) {
+                ok = step(ks, pa);
+                if (ok && ks + 1 < KS) ok = step(ks + 1, pb);
             }
             if (!ok || !(ok = bf.drain())) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -176,7 +203,7 @@ conv_fwd_tc(int n, int L, int ci, int co, const bf16* X, const bf16* W, const fl
 // input gradient: D[s][c], N = 64 input channels, K = 9 x CO_PAD (TF32 steps of 8)
 template <int CO_PAD>
 __global__ void __launch_bounds__(CT, 1)
-conv_bwd_data_tc(int n, int L, int ci, int co, const bf16* W, const float* dY, const bf16* act, float* dX,
+conv_bwd_data_tc(int n, int L, int ci, int co, const void* Wp, const float* dY, const bf16* act, float* dX,
                  int* err) {
     constexpr int NC = 64, KT = 9 * CO_PAD, KS = KT / 8, TCOLS = 2 * NC;
     constexpr uint32_t SBO_B = (KT / 4) * 128;
@@ -187,11 +214,7 @@ conv_bwd_data_tc(int n, int L, int ci, int co, const bf16* W, const float* dY, c
     unsigned char* As = Bs + NC * KT * 4;                     // 2 buffers x 2 tiles x 128 rows x 32 B
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int V = L * L;
-    for (int e = tid; e < NC * KT; e += CT) {
-        const int c = e / KT, k = e % KT, t = k / CO_PAD, o = k % CO_PAD;
-        const float v = (c < ci && o < co) ? __bfloat162float(W[((size_t)o * ci + c) * 9 + t]) : 0.f;
-        *(float*)(Bs + (c >> 3) * SBO_B + (k >> 2) * 128 + (c & 7) * 16 + (k & 3) * 4) = v;
-    }
+    copy_packed(Bs, Wp, NC * KT * 4);
     if (warp == 0) tmem_alloc_warp(&tslot, TCOLS);
     Bufs bf;
     bf.bar[0] = tc::smem_u32(&bars[0]);
@@ -210,22 +233,24 @@ conv_bwd_data_tc(int n, int L, int ci, int co, const bf16* W, const float* dY, c
     for (int b = blockIdx.x; b < n && ok; b += gridDim.x) {
         const float* dYb = dY + (size_t)b * co * V;
         for (int p0 = 0; p0 < V && ok; p0 += 2 * 128) {
-            const int s = p0 + tid;
-            for (int ks = 0; ks < KS && ok; ++ks) {
-                const int buf = ks & 1;
-                if (!(ok = bf.wait(buf))) break;
+            const int s = p0 + tid, x = s % L, y = s / L;
+            // the 8 output channels of step ks, loaded two steps ahead of their use
+            auto fetch = [&](int ks, float (&v)[8]) {
                 const int t = ks / (CO_PAD / 8), o0 = (ks % (CO_PAD / 8)) * 8;
-                const int nb = s < V ? shifted(L, s, t, -1) : 0;
-                float v[8];
+                const float* src = dYb + (s < V ? shifted(L, x, y, t, -1) : 0);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int o = o0 + k;
-                    v[k] = (s < V && o < co) ? tc::tf32_rna(dYb[(size_t)o * V + nb]) : 0.f;
-                }
+                for (int k = 0; k < 8; ++k) v[k] = (s < V && o0 + k < co) ? src[(size_t)(o0 + k) * V] : 0.f;
+            };
+            auto step = [&](int ks, float (&v)[8]) -> bool {
+                const int buf = ks & 1;
+                if (!bf.wait(buf)) return false;
                 unsigned char* Ab = As + buf * 8192 + (tid >> 7) * 4096;
                 const int r = tid & 127;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = tc::tf32_rna(v[k]);
                 *(float4*)(Ab + tc::cm32(r, 0, 4)) = make_float4(v[0], v[1], v[2], v[3]);
                 *(float4*)(Ab + tc::cm32(r, 4, 4)) = make_float4(v[4], v[5], v[6], v[7]);
+                if (ks + 2 < KS) fetch(ks + 2, v);
                 fence_to_async();
                 __syncthreads();
                 if (tid == 0) {
@@ -239,6 +264,14 @@ conv_bwd_data_tc(int n, int L, int ci, int co, const bf16* W, const float* dY, c
                     tc::commit(bf.bar[buf]);
                 }
                 bf.pending[buf] = true;
+                return true;
+            };
+            float va[8], vb[8];
+            fetch(0, va);
+            fetch(1, vb);
+            for (int ks = 0; ks < KS && ok; ks += 2) {
+                ok = step(ks, va);
+                if (ok && ks + 1 < KS) ok = step(ks + 1, vb);
             }
             if (!ok || !(ok = bf.drain())) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -273,11 +306,36 @@ conv_bwd_data_tc(int n, int L, int ci, int co, const bf16* W, const float* dY, c
 
 // ---------------------------------------------------------------------------
 // weight gradient: D[(t, c)][o], MT tiles of 128 rows (t, c), N = CO_PAD,
-// K = pixels (TF32 steps of 8); the CTA's partial sums are added to dW
-// (zeroed by the caller).
+// K = pixels (TF32 steps of 8); the CTA's partial sums go to its own plane of
+// `part` ([o][t][c]: a warp's 32 rows are 32 consecutive words), which
+// reduce_weight_grad adds up in a fixed order.  Adding them to the gradient
+// atomically cost a sector per word and made the sums, and with them the
+// optimiser's normalised steps, depend on the CTAs' timing.  Work unit: h rows
+// of a sample.
+struct BandLayout {
+    int xs, ys;              // elements between channels of the staged X (with halo) and dY
+    size_t x, y, base, total;
+};
+__host__ __device__ inline BandLayout band_layout(int L, int ci, int co, int h, size_t front) {
+    BandLayout l;
+    // an odd number of words between channels: neighbouring channels on other banks
+    l.xs = (h + 2) * (L + 2);
+    l.xs += l.xs & 1;
+    if ((l.xs >> 1) % 2 == 0) l.xs += 2;
+    l.ys = h * L + 8;
+    l.ys |= 1;
+    size_t o = front;
+    auto take = [&](size_t& at, size_t bytes) { at = o; o = (o + bytes + 15) & ~(size_t)15; };
+    take(l.x, (size_t)ci * l.xs * 2);
+    take(l.y, (size_t)co * l.ys * 4);
+    take(l.base, (size_t)(h * L + 8) * 2);
+    l.total = o;
+    return l;
+}
+
 template <int MT, int CO_PAD>
 __global__ void __launch_bounds__(CT, 1)
-conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY, float* dW, int* err) {
+conv_bwd_weight_tc(int n, int L, int ci, int co, int h, const bf16* X, const float* dY, float* part, int* err) {
     constexpr int TC_ = MT * CO_PAD <= 32 ? 32 : MT * CO_PAD <= 64 ? 64 : MT * CO_PAD <= 128 ? 128
                         : MT * CO_PAD <= 256 ? 256 : 512;
     constexpr int ABYTES = MT * 128 * 32;                     // one buffer of A
@@ -287,8 +345,12 @@ conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY,
     __shared__ uint32_t tslot;
     unsigned char* As = align1k(smraw);
     unsigned char* Bsm = As + 2 * ABYTES;
+    const BandLayout lay = band_layout(L, ci, co, h, 2 * ABYTES + 2 * BBYTES);
+    bf16* Xs = (bf16*)(As + lay.x);                           // [ci][xs]: rows y0 - 1 .. y0 + h, columns -1 .. L
+    float* Ys = (float*)(As + lay.y);                         // [co][ys]: the band's pixels, TF32, zeros behind
+    uint16_t* base = (uint16_t*)(As + lay.base);              // pixel -> its offset in a halo plane, less one row and column
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int V = L * L, R = 9 * ci;                          // rows (t, c) = t * ci + c
+    const int V = L * L, R = 9 * ci, W2 = L + 2;              // rows (t, c) = t * ci + c
     if (warp == 0) tmem_alloc_warp(&tslot, TC_);
     Bufs bf;
     bf.bar[0] = tc::smem_u32(&bars[0]);
@@ -298,41 +360,75 @@ conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY,
         tc::mbar_init(bf.bar[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
+    for (int q = tid; q < h * L + 8; q += CT) base[q] = (uint16_t)(q < h * L ? (q / L) * W2 + q % L : 0);
+    // this thread's (t, c) rows: their offset in Xs, -1 past the last
+    int off[MT];
+#pragma unroll
+    for (int i = 0; i < MT; ++i) {
+        const int row = (tid + i * CT) >> 1, t = row / ci, c = row - t * ci;
+        off[i] = row < R ? c * lay.xs + (t / 3) * W2 + t % 3 : -1;
+    }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tbase = tslot;
+    const int bands = (L + h - 1) / h;
     bool ok = true;
     int step = 0;
-    for (int b = blockIdx.x; b < n && ok; b += gridDim.x) {
+    for (int u = blockIdx.x; u < n * bands && ok; u += gridDim.x) {
+        const int b = u / bands, y0 = (u - b * bands) * h, hh = min(h, L - y0), npx = hh * L;
         const bf16* Xb = X + (size_t)b * ci * V;
-        const float* dYb = dY + (size_t)b * co * V;
-        for (int s0 = 0; s0 < V && ok; s0 += 8, ++step) {
+        const float* dYb = dY + (size_t)b * co * V + (size_t)y0 * L;
+        // the staged band is not rewritten while its tiles are being built: the
+        // last build ended with a barrier
+        for (int rr = warp; rr < ci * (hh + 2); rr += CT / 32) {
+            const int c = rr / (hh + 2), yy = rr - c * (hh + 2);
+            int gy = y0 + yy - 1;
+            gy = gy < 0 ? gy + L : gy >= L ? gy - L : gy;
+            const bf16* src = Xb + (size_t)c * V + (size_t)gy * L;
+            bf16* dst = Xs + (size_t)c * lay.xs + yy * W2;
+            for (int x = lane; x < W2; x += 32) dst[x] = src[x == 0 ? L - 1 : x == L + 1 ? 0 : x - 1];
+        }
+        for (int o = warp; o < co; o += CT / 32) {
+            for (int q = lane; q < ((npx + 7) & ~7); q += 32)
+                Ys[(size_t)o * lay.ys + q] = q < npx ? tc::tf32_rna(dYb[(size_t)o * V + q]) : 0.f;
+        }
+        __syncthreads();
+        for (int s0 = 0; s0 < npx && ok; s0 += 8, ++step) {
             const int buf = step & 1;
             if (!(ok = bf.wait(buf))) break;
             unsigned char* Ab = As + buf * ABYTES;
-            // A: rows (t, c), 8 pixels; 4-wide groups of k per store
-            for (int e = tid; e < MT * 128 * 2; e += CT) {
-                const int row = e >> 1, kg = (e & 1) * 4;
-                const int t = row / ci, c = row - t * ci;
-                float v[4];
+            // A: rows (t, c), 8 pixels; 4-wide groups of k per store.  Pixels past
+            // the band meet zeros of dY, and read the band's first pixel (never
+            // what shared memory held before)
+            const int kg = (tid & 1) * 4;
+            ushort4 q4 = *(const ushort4*)(base + s0 + kg);
+            if (s0 + 8 > npx) {
+                if (s0 + kg + 0 >= npx) q4.x = 0;
+                if (s0 + kg + 1 >= npx) q4.y = 0;
+                if (s0 + kg + 2 >= npx) q4.z = 0;
+                if (s0 + kg + 3 >= npx) q4.w = 0;
+            }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int s = s0 + kg + k;
-                    v[k] = (row < R && s < V) ? __bfloat162float(Xb[(size_t)c * V + shifted(L, s, t, 1)]) : 0.f;
+            for (int i = 0; i < MT; ++i) {
+                const int row = (tid + i * CT) >> 1;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (off[i] >= 0) {
+                    const bf16* p = Xs + off[i];
+                    v = make_float4(__bfloat162float(p[q4.x]), __bfloat162float(p[q4.y]), __bfloat162float(p[q4.z]),
+                                    __bfloat162float(p[q4.w]));
                 }
-                *(float4*)(Ab + (row >> 7) * 4096 + tc::cm32(row & 127, kg, 4)) = make_float4(v[0], v[1], v[2], v[3]);
+                *(float4*)(Ab + (row >> 7) * 4096 + tc::cm32(row & 127, kg, 4)) = v;
             }
             unsigned char* Bb = Bsm + buf * BBYTES;
-            for (int e = tid; e < CO_PAD * 2; e += CT) {
-                const int o = e >> 1, kg = (e & 1) * 4;
-                float v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int s = s0 + kg + k;
-                    v[k] = (o < co && s < V) ? tc::tf32_rna(dYb[(size_t)o * V + s]) : 0.f;
+            if (tid < CO_PAD * 2) {
+                const int o = tid >> 1;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (o < co) {
+                    const float* p = Ys + (size_t)o * lay.ys + s0 + kg;
+                    v = make_float4(p[0], p[1], p[2], p[3]);
                 }
-                *(float4*)(Bb + tc::cm32(o, kg, 4)) = make_float4(v[0], v[1], v[2], v[3]);
+                *(float4*)(Bb + tc::cm32(o, kg, 4)) = v;
             }
             fence_to_async();
             __syncthreads();
@@ -356,7 +452,6 @@ conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY,
         const int q = warp & 3;
         for (int m = warp >> 2; m < MT; m += 2) {
             const int row = m * 128 + q * 32 + lane;
-            const int t = row / ci, c = row - t * ci;
 #pragma unroll
             for (int j = 0; j < CO_PAD; j += 16) {
                 float v[16];
@@ -364,7 +459,7 @@ conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY,
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
                     const int o = j + k;
-                    if (o < co && row < R) atomicAdd(&dW[((size_t)o * ci + c) * 9 + t], v[k]);
+                    if (o < co && row < R) part[((size_t)blockIdx.x * co + o) * R + row] = v[k];
                 }
             }
         }
@@ -378,13 +473,42 @@ conv_bwd_weight_tc(int n, int L, int ci, int co, const bf16* X, const float* dY,
     if (!ok && tid == 0) atomicExch(err, 1);
 }
 
-// db[o] = sum_{b, s} dY[b][o][s]
-__global__ void conv_bias_grad(int n, int V, int co, const float* dY, float* db) {
-    const int o = blockIdx.x;
+// dW [o][c][t] = sum of the planes of part [o][t][c]: eight threads per word,
+// each over every eighth plane, then a tree.
+__global__ void __launch_bounds__(256) reduce_weight_grad(int planes, int ci, int co, const float* part, float* dW) {
+    __shared__ float red[8][33];
+    const int R = 9 * ci, e = blockIdx.x * 32 + (threadIdx.x & 31), g = threadIdx.x >> 5;
     float acc = 0.f;
-    for (int e = threadIdx.x; e < n * V; e += blockDim.x) {
-        const int b = e / V, s = e - b * V;
-        acc += dY[((size_t)b * co + o) * V + s];
+    if (e < co * R)
+#pragma unroll 4
+        for (int k = g; k < planes; k += 8) acc += part[(size_t)k * co * R + e];
+    red[g][threadIdx.x & 31] = acc;
+    __syncthreads();
+    if (g == 0 && e < co * R) {
+        const int x = threadIdx.x & 31, o = e / R, t = (e - o * R) / ci, c = e % ci;
+        dW[((size_t)o * ci + c) * 9 + t] = ((red[0][x] + red[1][x]) + (red[2][x] + red[3][x])) +
+                                           ((red[4][x] + red[5][x]) + (red[6][x] + red[7][x]));
+    }
+}
+
+// db[o] = sum_{b, s} dY[b][o][s].  A thread's values are added one after the
+// other (the sums cancel to a fraction of their terms, and the optimiser
+// normalises them, so that another order shows), but loaded eight at a time.
+__global__ void conv_bias_grad(int n, int V, int co, const float* dY, float* db) {
+    const int o = blockIdx.x, total = n * V;
+    float acc = 0.f;
+    int b = threadIdx.x / V, s = threadIdx.x - b * V;
+    for (int e = threadIdx.x; e < total; e += 8 * blockDim.x) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = e + k * (int)blockDim.x < total ? dY[((size_t)b * co + o) * V + s] : 0.f;
+            s += blockDim.x;
+            while (s >= V) { s -= V; ++b; }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (e + k * (int)blockDim.x < total) acc += v[k];
     }
     __shared__ float red[32];
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
@@ -422,8 +546,7 @@ ggf_status ggf_conv_fwd_tc(int n, int L, int ci, int co, bool relu, const void* 
         e = cudaFuncSetAttribute(conv_fwd_tc<CIP, COP, RL, OF>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                  (int)sm);                                                                     \
         if (e == cudaSuccess)                                                                                  \
-            conv_fwd_tc<CIP, COP, RL, OF><<<grid, CT, sm, st>>>(n, L, ci, co, (const bf16*)X, (const bf16*)W, \
-                                                                 bias, Y, err);                                 \
+            conv_fwd_tc<CIP, COP, RL, OF><<<grid, CT, sm, st>>>(n, L, ci, co, (const bf16*)X, W, bias, Y, err);                                 \
     } while (0)
     if (ci <= 16 && co <= 64 && relu && !out_f32) GGF_FWD(16, 64, true, false);
     else if (ci <= 64 && co <= 64 && co > 16 && relu && !out_f32) GGF_FWD(64, 64, true, false);
@@ -445,8 +568,7 @@ ggf_status ggf_conv_bwd_data_tc(int n, int L, int ci, int co, const void* W, con
         const size_t sm = launch_smem(1024 + (size_t)64 * 9 * (COP) * 4 + 2 * 8192, 128);                     \
         e = cudaFuncSetAttribute(conv_bwd_data_tc<COP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
         if (e == cudaSuccess)                                                                                  \
-            conv_bwd_data_tc<COP><<<grid, CT, sm, st>>>(n, L, ci, co, (const bf16*)W, dY, (const bf16*)act,  \
-                                                        dX, err);                                              \
+            conv_bwd_data_tc<COP><<<grid, CT, sm, st>>>(n, L, ci, co, W, dY, (const bf16*)act, dX, err);                                              \
     } while (0)
     if (co <= 8) GGF_BWD(8);
     else if (co <= 64) GGF_BWD(64);
@@ -456,19 +578,27 @@ ggf_status ggf_conv_bwd_data_tc(int n, int L, int ci, int co, const void* W, con
     return cudaGetLastError() == cudaSuccess ? GGF_OK : GGF_ECUDA;
 }
 
+// part: scratch of sms co 9 ci floats.  A unit of work is the
+// tallest band of rows that fits in shared memory, or a shorter one where the
+// samples alone would leave SMs idle.
 ggf_status ggf_conv_bwd_weight_tc(int n, int L, int ci, int co, const void* X, const float* dY, float* dW,
-                                  float* db, int* err, int sms, cudaStream_t st) {
-    const int grid = n < sms ? n : sms;
-    if (grid == 0) return GGF_OK;
-    if (cudaMemsetAsync(dW, 0, (size_t)co * ci * 9 * sizeof(float), st) != cudaSuccess) return GGF_ECUDA;
+                                  float* db, float* part, int* err, int sms, cudaStream_t st) {
+    if (n < 1) return GGF_OK;
     cudaError_t e = cudaSuccess;
-#define GGF_BWW(MT, COP)                                                                                       \
-    do {                                                                                                       \
-        const size_t sm = launch_smem(1024 + 2 * ((size_t)(MT) * 128 * 32 + (size_t)(COP) * 32), (MT) * (COP));  \
-        e = cudaFuncSetAttribute(conv_bwd_weight_tc<MT, COP>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                 (int)sm);                                                                     \
-        if (e == cudaSuccess)                                                                                  \
-            conv_bwd_weight_tc<MT, COP><<<grid, CT, sm, st>>>(n, L, ci, co, (const bf16*)X, dY, dW, err);      \
+    int planes = 0;
+    constexpr size_t cap = 227 * 1024 - 2048;
+#define GGF_BWW(MT, COP)                                                                                              \
+    do {                                                                                                              \
+        const size_t front = 2 * ((size_t)(MT) * 128 * 32 + (size_t)(COP) * 32);                                      \
+        int h = L;                                                                                                    \
+        while (h > 1 && band_layout(L, ci, co, h, front).total > cap) --h;                                            \
+        while (h > 2 && (long long)n * ((L + h - 1) / h) * 2 <= sms) h = (h + 1) / 2;                                  \
+        const int units = n * ((L + h - 1) / h), grid = units < sms ? units : sms;                                     \
+        planes = grid;                                                                                                \
+        const size_t sm = launch_smem(1024 + band_layout(L, ci, co, h, front).total, (MT) * (COP));                    \
+        e = cudaFuncSetAttribute(conv_bwd_weight_tc<MT, COP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+        if (e == cudaSuccess)                                                                                         \
+            conv_bwd_weight_tc<MT, COP><<<grid, CT, sm, st>>>(n, L, ci, co, h, (const bf16*)X, dY, part, err);         \
     } while (0)
     const int rows = 9 * ci;
     if (rows <= 128 && co <= 64) GGF_BWW(1, 64);
@@ -477,6 +607,7 @@ ggf_status ggf_conv_bwd_weight_tc(int n, int L, int ci, int co, const void* X, c
     else return GGF_EINVAL;
 #undef GGF_BWW
     if (e != cudaSuccess) return GGF_ECUDA;
+    reduce_weight_grad<<<(co * rows + 31) / 32, 256, 0, st>>>(planes, ci, co, part, dW);
     conv_bias_grad<<<co, 256, 0, st>>>(n, L * L, co, dY, db);
     return cudaGetLastError() == cudaSuccess ? GGF_OK : GGF_ECUDA;
 }

@@ -19,13 +19,14 @@
 #include <vector>
 #include "ggf_ctx.h"
 #include "ggf_net.h"
+#include "ggf_conv_pack.cuh"
 
 ggf_status ggf_conv_fwd_tc(int n, int L, int ci, int co, bool relu, const void* X, const void* W, const float* bias,
                            void* Y, bool out_f32, int* err, int sms, cudaStream_t st);
 ggf_status ggf_conv_bwd_data_tc(int n, int L, int ci, int co, const void* W, const float* dY, const void* act,
                                 float* dX, int* err, int sms, cudaStream_t st);
 ggf_status ggf_conv_bwd_weight_tc(int n, int L, int ci, int co, const void* X, const float* dY, float* dW,
-                                  float* db, int* err, int sms, cudaStream_t st);
+                                  float* db, float* part, int* err, int sms, cudaStream_t st);
 
 namespace {
 
@@ -148,13 +149,32 @@ __global__ void head_kernel(int n, int L, int mode, const float* out, const doub
     }
 }
 
-__global__ void to_bf16(int n, const float* a, bf16* b) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = __float2bfloat16(a[i]);
+// Packed operands of all layers: the forward ones, then the input gradients' of
+// layers 1 .. (layer 0 has none).
+__host__ __device__ constexpr size_t pack_fwd_at(int l) {
+    return l == 0 ? 0 : pack_fwd_at(l - 1) + pack_fwd_bytes(layer_ci(l - 1), layer_co(l - 1));
+}
+__host__ __device__ constexpr size_t pack_bwd_at(int l) {
+    return l <= 1 ? pack_fwd_at(NLAYER) : pack_bwd_at(l - 1) + pack_bwd_bytes(layer_co(l - 1));
+}
+constexpr size_t PACK_BYTES = pack_bwd_at(NLAYER);
+
+// Parameter i (value v) into the packed operands; biases are read as FP32.
+__device__ __forceinline__ void pack_param(int i, float v, unsigned char* pk) {
+    int l = 0;
+    while (l + 1 < NLAYER && i >= layer_off(l + 1)) ++l;
+    const int rel = i - layer_off(l);
+    if (rel >= layer_co(l) * layer_ci(l) * 9) return;
+    pack_weight(layer_ci(l), layer_co(l), rel, v, pk + pack_fwd_at(l), l ? pk + pack_bwd_at(l) : nullptr);
+}
+
+__global__ void pack_params(const float* p, unsigned char* pk) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < NPARAM) pack_param(i, p[i], pk);
 }
 
 __global__ void adam_kernel(int n, float* p, const float* g, float* m, float* v, float lr, float b1, float b2,
-                            float eps, float c1, float c2, bf16* pb) {
+                            float eps, float c1, float c2, unsigned char* pk) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float gi = g[i];
@@ -164,7 +184,7 @@ __global__ void adam_kernel(int n, float* p, const float* g, float* m, float* v,
     v[i] = vi;
     float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     p[i] = pi;
-    pb[i] = __float2bfloat16(pi);
+    pack_param(i, pi, pk);
 }
 
 __global__ void init_params(float* p, uint64_t seed) {
@@ -200,8 +220,9 @@ struct ggf_net {
     uint64_t seed = 0;
     std::string err;
     float* p = nullptr;        // FP32 master parameters
-    bf16* pb = nullptr;        // BF16 copy used by the kernels
+    unsigned char* pk = nullptr;   // packed BF16 / TF32 weights used by the convolutions
     float* g = nullptr;        // gradient
+    float* part = nullptr;     // partial weight gradients of one layer, a plane per CTA
     float* m = nullptr;
     float* v = nullptr;
     long long t = 0;           // Adam steps
@@ -258,7 +279,7 @@ ggf_status ggf_net_forward(ggf_net* net, int n, cudaStream_t st) {
     const int L = net->L;
     for (int l = 0; l < NLAYER; ++l) {
         const int ci = layer_ci(l), co = layer_co(l);
-        const bf16* W = net->pb + layer_off(l);
+        const void* W = net->pk + pack_fwd_at(l);
         const float* b = net->p + layer_off(l) + co * ci * 9;
         const bool last = l == NLAYER - 1;
         ggf_status rc = ggf_conv_fwd_tc(n, L, ci, co, !last, net->X[l], W, b, last ? (void*)net->out : (void*)net->X[l + 1],
@@ -270,16 +291,18 @@ ggf_status ggf_net_forward(ggf_net* net, int n, cudaStream_t st) {
 
 static ggf_status net_backward(ggf_net* net, int n, cudaStream_t st) {
     const int L = net->L;
+    if (!net->part) NET_CK(cudaMalloc(&net->part, (size_t)net->sms * CH * CH * 9 * sizeof(float)));
     float* dcur = net->dA;      // gradient w.r.t. the current layer's output
     float* dnext = net->dB;
     for (int l = NLAYER - 1; l >= 0; --l) {
         const int ci = layer_ci(l), co = layer_co(l);
         float* dW = net->g + layer_off(l);
         float* db = dW + co * ci * 9;
-        ggf_status rc = ggf_conv_bwd_weight_tc(n, L, ci, co, net->X[l], dcur, dW, db, net->d_err, net->sms, st);
+        ggf_status rc = ggf_conv_bwd_weight_tc(n, L, ci, co, net->X[l], dcur, dW, db, net->part,
+                                               net->d_err, net->sms, st);
         if (rc != GGF_OK) return net_fail(net, rc, "tensor-core convolution (weight gradient) failed to launch");
         if (l > 0) {
-            rc = ggf_conv_bwd_data_tc(n, L, ci, co, net->pb + layer_off(l), dcur, net->X[l], dnext, net->d_err,
+            rc = ggf_conv_bwd_data_tc(n, L, ci, co, net->pk + pack_bwd_at(l), dcur, net->X[l], dnext, net->d_err,
                                       net->sms, st);
             if (rc != GGF_OK) return net_fail(net, rc, "tensor-core convolution (input gradient) failed to launch");
             std::swap(dcur, dnext);
@@ -334,7 +357,7 @@ ggf_status ggf_net_create(ggf_net** out, int device, int L, uint64_t seed) {
     ggf_status s = GGF_OK;
     auto ck = [&](cudaError_t e) { if (e != cudaSuccess && s == GGF_OK) s = GGF_ENOMEM; };
     ck(cudaMalloc(&net->p, NPARAM * sizeof(float)));
-    ck(cudaMalloc(&net->pb, NPARAM * sizeof(bf16)));
+    ck(cudaMalloc(&net->pk, PACK_BYTES));
     ck(cudaMalloc(&net->g, NPARAM * sizeof(float)));
     ck(cudaMalloc(&net->m, NPARAM * sizeof(float)));
     ck(cudaMalloc(&net->v, NPARAM * sizeof(float)));
@@ -343,7 +366,8 @@ ggf_status ggf_net_create(ggf_net** out, int device, int L, uint64_t seed) {
     cudaMemset(net->d_err, 0, sizeof(int));
     cudaDeviceGetAttribute(&net->sms, cudaDevAttrMultiProcessorCount, device);
     init_params<<<(NPARAM + 255) / 256, 256>>>(net->p, seed);
-    to_bf16<<<(NPARAM + 255) / 256, 256>>>(NPARAM, net->p, net->pb);
+    cudaMemset(net->pk, 0, PACK_BYTES);
+    pack_params<<<(NPARAM + 255) / 256, 256>>>(net->p, net->pk);
     cudaMemset(net->m, 0, NPARAM * sizeof(float));
     cudaMemset(net->v, 0, NPARAM * sizeof(float));
     if (cudaDeviceSynchronize() != cudaSuccess) { ggf_net_destroy(net); return GGF_ECUDA; }
@@ -355,7 +379,7 @@ void ggf_net_destroy(ggf_net* net) {
     if (!net) return;
     cudaSetDevice(net->device);
     net_free_ws(net);
-    void* ps[] = {net->p, net->pb, net->g, net->m, net->v, net->d_err};
+    void* ps[] = {net->p, net->pk, net->g, net->part, net->m, net->v, net->d_err};
     for (void* q : ps) if (q) cudaFree(q);
     delete net;
 }
@@ -373,7 +397,7 @@ ggf_status ggf_net_set_params(ggf_net* net, const float* in) {
     if (!net || !in) return GGF_EINVAL;
     cudaSetDevice(net->device);
     NET_CK(cudaMemcpy(net->p, in, NPARAM * sizeof(float), cudaMemcpyHostToDevice));
-    to_bf16<<<(NPARAM + 255) / 256, 256>>>(NPARAM, net->p, net->pb);
+    pack_params<<<(NPARAM + 255) / 256, 256>>>(net->p, net->pk);
     NET_CK(cudaMemset(net->m, 0, NPARAM * sizeof(float)));
     NET_CK(cudaMemset(net->v, 0, NPARAM * sizeof(float)));
     net->t = 0;
@@ -449,7 +473,7 @@ ggf_status ggf_net_train(ggf_net* net, int n_cfg, const double* theta, int batch
         net->t += 1;
         float c1 = 1.f - powf(b1, (float)net->t), c2 = 1.f - powf(b2, (float)net->t);
         adam_kernel<<<(NPARAM + 255) / 256, 256, 0, st>>>(NPARAM, net->p, net->g, net->m, net->v, lr, b1, b2, eps, c1,
-                                                          c2, net->pb);
+                                                          c2, net->pk);
         NET_CK(cudaGetLastError());
         if (losses) {
             double l = 0;
