@@ -46,15 +46,17 @@ __device__ __forceinline__ double magc(cxd v) { return fabs(v.x) + fabs(v.y); }
 // ---- FP64 scalars of the link steps: double for the diagonal pairs, cxd for
 // the pairs n < m ----
 __device__ __forceinline__ double magc(double v) { return fabs(v); }
-__device__ __forceinline__ bool is_zero(double v) { return v == 0.0; }
-__device__ __forceinline__ bool is_zero(cxd v) { return v.x == 0.0 && v.y == 0.0; }
+// (on the words: an FP64 comparison takes the unit's 64 cycles too)
+__device__ __forceinline__ bool is_zero(double v) { return ((__double2hiint(v) << 1) | __double2loint(v)) == 0; }
+__device__ __forceinline__ bool is_zero(cxd v) { return is_zero(v.x) && is_zero(v.y); }
 __device__ __forceinline__ bool is_fin(double v) { return isfinite(v); }
 __device__ __forceinline__ bool is_fin(cxd v) { return isfinite(v.x) && isfinite(v.y); }
 __device__ __forceinline__ double recip(double v) { return 1.0 / v; }
 // one division where |v|^2 is well inside the range, Smith's method elsewhere
 __device__ __forceinline__ cxd recip(cxd v) {
     const double m = v.x * v.x + v.y * v.y;
-    if (m > 1e-280 && m < 1e280) {
+    const int e = __double2hiint(m) >> 20;          // biased exponent: 2^-930 <= m < 2^930
+    if (e >= 1023 - 930 && e < 1023 + 930) {
         const double t = 1.0 / m;
         return {v.x * t, -v.y * t};
     }
@@ -408,11 +410,10 @@ __device__ __forceinline__ bool pair_z(const T* D, const T* Ws, T* Aug, T* fcol,
 // ell_p += log rho_p: modulus only for diagonal pairs, phase wrapped into
 // (-pi, pi] for pairs n < m.
 __device__ __forceinline__ void ell_add(cxd& el, cxd rho, bool real_pair) {
-    cxd lr = clog_(rho);
     if (real_pair) {
-        el.x += lr.x;
+        el.x += log(fabs(rho.x));        // a real ratio
     } else {
-        el = el + lr;
+        el = el + clog_(rho);
         if (el.y > M_PI) el.y -= 2 * M_PI;
         else if (el.y <= -M_PI) el.y += 2 * M_PI;
     }
