@@ -460,10 +460,11 @@ ggf_status chain_ell(ggf_ctx* ctx, const std::vector<int>& chains, bool init, cu
 }
 
 // Factor the listed chains: log-weights from the site-by-site FP64 Pfaffian
-// (init: set; refresh: drift recorded), inverses in FP64 along the lattice at
-// the start and for FP64 chains (Gauss-Jordan below four rows and where that
-// is not accurate enough), by a Newton step on the tensor cores for FP32
-// chains (the FP64 inverse where the residual is too large for it).
+// (init: set; refresh: drift recorded).  Inverses of FP64 chains in FP64 along
+// the lattice (Gauss-Jordan below four rows and where that is not accurate
+// enough); of FP32 chains by Gauss-Jordan in FP64 at the start and a Newton
+// step on the tensor cores afterwards (Gauss-Jordan again where the residual is
+// too large for it).
 ggf_status factor_chains(ggf_ctx* ctx, const std::vector<int>& chains, bool init, cudaStream_t st) {
     if (chains.empty()) return GGF_OK;
     GGF_TRY(chain_ell(ctx, chains, init, st));
@@ -475,7 +476,9 @@ ggf_status factor_chains(ggf_ctx* ctx, const std::vector<int>& chains, bool init
     } else {
         dense = chains;
     }
-    if (dense.empty() || !ggf_lattice_inverse_use(ctx)) return dense_inverse(ctx, dense, st);
+    // (an FP32 chain starts from the elimination's rounding, see ZOps)
+    const bool fp32 = ctx->ch.opts.precision == GGF_FP32;
+    if (dense.empty() || fp32 || !ggf_lattice_inverse_use(ctx)) return dense_inverse(ctx, dense, st);
     std::vector<int> rest;
     GGF_TRY(lattice_inverse(ctx, dense, rest, st));
     return dense_inverse(ctx, rest, st);

@@ -83,6 +83,30 @@ __device__ __forceinline__ cxd quotient(cxd a, cxd d, cxd id) {
     fmac(q, r, id);
     return q;
 }
+// The arithmetic of Z = (1 + Delta W_SS)^{-1} Delta.  Z of an FP32 chain is
+// rounded to FP32, and one of some ten million elements lies so near the middle
+// of two FP32 numbers that the last FP64 bits decide it; the chain then carries
+// an FP32 rounding more or less.  So these chains keep one way of rounding
+// (APART: the product first, then the sum; the quotient from a division);
+// FP64 chains take fused sums and one reciprocal per row.
+template <bool APART> struct ZOps {
+    template <class T> __device__ static void add(T& r, T a, T b) { fmac(r, a, b); }
+    template <class T> __device__ static void sub(T& r, T a, T b) { fmsc(r, a, b); }
+    template <class T> __device__ static T inv(T d) { return recip(d); }
+    template <class T> __device__ static T div(T a, T d, T id) { return quotient(a, d, id); }
+};
+template <> struct ZOps<true> {
+    __device__ static double mul(double a, double b) { return __dmul_rn(a, b); }
+    __device__ static cxd mul(cxd a, cxd b) {
+        return {__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y))};
+    }
+    __device__ static void add(double& r, double a, double b) { r = __dadd_rn(r, mul(a, b)); }
+    __device__ static void sub(double& r, double a, double b) { r = __dsub_rn(r, mul(a, b)); }
+    __device__ static void add(cxd& r, cxd a, cxd b) { const cxd t = mul(a, b); r = {__dadd_rn(r.x, t.x), __dadd_rn(r.y, t.y)}; }
+    __device__ static void sub(cxd& r, cxd a, cxd b) { const cxd t = mul(a, b); r = {__dsub_rn(r.x, t.x), __dsub_rn(r.y, t.y)}; }
+    template <class T> __device__ static T inv(T d) { return d; }
+    template <class T> __device__ static T div(T a, T d, T) { return a / d; }
+};
 __device__ __forceinline__ cxd to_c(double v) { return {v, 0.0}; }
 __device__ __forceinline__ cxd to_c(cxd v) { return v; }
 
@@ -183,7 +207,7 @@ __device__ __forceinline__ T warp_pfaffian(T* A, int n) {
 // Solve [A | B] (r x 2r, row-major, stride 2r) in place by Gauss-Jordan with
 // partial pivoting; the right half becomes A^{-1} B (columns up to the pivot
 // are not read again and keep their values).  fcol: r scratch.
-template <class T>
+template <bool APART, class T>
 __device__ __forceinline__ bool warp_solve(T* A, int r, T* fcol) {
     const int lane = threadIdx.x & 31;
     const int w = 2 * r;
@@ -196,15 +220,15 @@ __device__ __forceinline__ bool warp_solve(T* A, int r, T* fcol) {
         }
         const T d = A[k * w + k];
         if (is_zero(d)) return false;
-        const T id = recip(d);
+        const T id = ZOps<APART>::inv(d);
         __syncwarp();
-        if (lane > k && lane < w) A[k * w + lane] = quotient(A[k * w + lane], d, id);
+        if (lane > k && lane < w) A[k * w + lane] = ZOps<APART>::div(A[k * w + lane], d, id);
         if (lane < r) fcol[lane] = A[lane * w + k];
         __syncwarp();
         const int cols = w - k - 1;
         for (int e = lane; e < r * cols; e += 32) {
             const int i = e / cols, j = k + 1 + e % cols;
-            if (i != k) fmsc(A[i * w + j], fcol[i], A[k * w + j]);
+            if (i != k) ZOps<APART>::sub(A[i * w + j], fcol[i], A[k * w + j]);
         }
         __syncwarp();
     }
@@ -385,19 +409,19 @@ GGF_HD cxd pair_norm(const DevConst& dc, const cxd* ell_c, int p, double amax, d
 }
 
 // Z = (1 + Delta W_SS)^{-1} Delta (r x r) into Zout, one warp; Aug is r x 2r
-// scratch, fcol r.  Returns false for a singular system.
-template <class T, class Z>
+// scratch, fcol r; APART for FP32 chains (ZOps).  Returns false for a singular system.
+template <bool APART, class T, class Z>
 __device__ __forceinline__ bool pair_z(const T* D, const T* Ws, T* Aug, T* fcol, int r, Z* Zout) {
     const int lane = threadIdx.x & 31, w2 = 2 * r;
     for (int e = lane; e < r * r; e += 32) {
         const int i = e / r, j = e % r;
         T v = i == j ? Sc<T>::one() : Sc<T>::zero();
-        for (int z = 0; z < r; ++z) fmac(v, D[i * r + z], Ws[z * r + j]);
+        for (int z = 0; z < r; ++z) ZOps<APART>::add(v, D[i * r + z], Ws[z * r + j]);
         Aug[i * w2 + j] = v;
         Aug[i * w2 + r + j] = D[e];
     }
     __syncwarp();
-    const bool ok = warp_solve(Aug, r, fcol);
+    const bool ok = warp_solve<APART>(Aug, r, fcol);
     for (int e = lane; e < r * r; e += 32) {
         const T v = Aug[(e / r) * w2 + r + e % r];
         if constexpr (sizeof(Z) == sizeof(T)) Zout[e] = v;

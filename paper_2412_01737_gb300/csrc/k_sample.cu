@@ -296,9 +296,9 @@ __global__ void __launch_bounds__(NWARP * 32, 2) ratio_kernel(SweepArgs a) {
         const int s = t >> 1, p = a.bins.ord[p0 + s];
         void* scr = smr + lay.task + (size_t)warp * lay.task_bytes;
         if (t & 1) {
-            const bool ok = p < K ? pair_z((const double*)slot(s, 0), (const double*)slot(s, 1), (double*)scr,
+            const bool ok = p < K ? pair_z<sizeof(RW) == 4>((const double*)slot(s, 0), (const double*)slot(s, 1), (double*)scr,
                                            (double*)scr + 4 * R * R, R, slot(s, 2))
-                                  : pair_z(slot(s, 0), slot(s, 1), (cxd*)scr, (cxd*)scr + 4 * R * R, R, slot(s, 2));
+                                  : pair_z<sizeof(RW) == 4>(slot(s, 0), slot(s, 1), (cxd*)scr, (cxd*)scr + 4 * R * R, R, slot(s, 2));
             if (lane == 0) s_okz[s] = ok;
         } else {
             const cxd pf = p < K ? cxd{bordered_ratio((const double*)slot(s, 0), (const double*)slot(s, 1), (double*)scr, R), 0.0}

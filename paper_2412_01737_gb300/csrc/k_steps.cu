@@ -27,8 +27,8 @@
 // left factor: 39, 3, 21 - 49).
 // Measured per batch of 16 links, against one CTA per chain that took its
 // pairs in turn with G and X in L2: 16 chains of 16 x 16 U(1), K = 4 (rank
-// 128) 8.70 -> 0.89 ms (two waves: 15 clusters of 8 fit); 96 chains of 5 x 5
-// SU(2), K = 2 (rank 64) 0.92 -> 0.22 ms; 24 FP64 chains of 8 x 8 U(1), K = 2
+// 128) 8.70 -> 0.97 ms (two waves: 15 clusters of 8 fit); 96 chains of 5 x 5
+// SU(2), K = 2 (rank 64) 0.92 -> 0.23 ms; 24 FP64 chains of 8 x 8 U(1), K = 2
 // (rank 128) 9.7 -> 3.6 ms.  Rolled loops and calls in place of expanded code
 // (half the instructions) were 10% slower.
 #include <algorithm>
@@ -153,7 +153,7 @@ __device__ __forceinline__ void z_task(const T* M, int ld, int jr, const typenam
     Z* fcol = Aug + 4 * R * R;
     for (int e = lane; e < R * R; e += 32) Ws[e] = wide(M[(size_t)(jr + e / R) * ld + jr + e % R]);
     __syncwarp();
-    pair_z(D, Ws, Aug, fcol, R, Zw);
+    pair_z<sizeof(typename Sc<T>::R) == 4>(D, Ws, Aug, fcol, R, Zw);
     for (int e = lane; e < R * R; e += 32) Zout[e] = narrow(Zw[e], T{});
 }
 
@@ -166,6 +166,7 @@ template <class T, int R>
 __device__ __forceinline__ void z_task_two(const T* M, int ld, int jr, const typename Fp64Of<T>::Z* D, void* scratch,
                                            T* Zout, int part) {
     typedef typename Fp64Of<T>::Z Z;
+    typedef ZOps<sizeof(typename Sc<T>::R) == 4> Ops;
     constexpr int W2 = 2 * R;
     const int lane = threadIdx.x & 31, l2 = part * 32 + lane;
     Z* Ws = (Z*)scratch;
@@ -178,7 +179,7 @@ __device__ __forceinline__ void z_task_two(const T* M, int ld, int jr, const typ
         const int i = e / R, j = e % R;
         Z v = i == j ? Sc<Z>::one() : Sc<Z>::zero();
 #pragma unroll
-        for (int z = 0; z < R; ++z) fmac(v, D[i * R + z], Ws[z * R + j]);
+        for (int z = 0; z < R; ++z) Ops::add(v, D[i * R + z], Ws[z * R + j]);
         A[i * W2 + j] = v;
         A[i * W2 + R + j] = D[e];
     }
@@ -189,11 +190,11 @@ __device__ __forceinline__ void z_task_two(const T* M, int ld, int jr, const typ
         const Z d = A[p * W2 + k];
         if (is_zero(d)) break;       // alike in both warps; the ratio is 0 then
         if (part == 0) {
-            const Z id = recip(d);
+            const Z id = Ops::inv(d);
             if (lane > k && lane < W2) {
                 const Z t = A[p * W2 + lane], u = A[k * W2 + lane];
                 A[p * W2 + lane] = u;
-                A[k * W2 + lane] = quotient(t, d, id);
+                A[k * W2 + lane] = Ops::div(t, d, id);
             }
         } else if (lane < R) {
             fcol[lane] = A[(lane == p ? k : lane) * W2 + k];
@@ -201,7 +202,7 @@ __device__ __forceinline__ void z_task_two(const T* M, int ld, int jr, const typ
         both();
         const int j = l2 % W2;
         for (int i = l2 / W2; i < R; i += 64 / W2)
-            if (i != k && j > k) fmsc(A[i * W2 + j], fcol[i], A[k * W2 + j]);
+            if (i != k && j > k) Ops::sub(A[i * W2 + j], fcol[i], A[k * W2 + j]);
         both();
     }
     for (int e = l2; e < R * R; e += 64) {
