@@ -579,7 +579,7 @@ def run_ggf(args):
         props = sp1.proposals - sp0.proposals
         roof = {"kernel": "batch_steps (link steps on W[T, T], FP64 ratios)", "bound": "latency",
                 "achieved": props / (kt["ratio"][0] * 1e-3), "peak": None, "unit": "link proposals/s",
-                "peak_source": "latency-bound (one CTA per chain, sequential links); no peak applies"}
+                "peak_source": "latency-bound (one cluster per chain, sequential links); no peak applies"}
     else:
         roof = {"kernel": "ratio_kernel", "bound": "alu", "achieved": None, "peak": None, "unit": None}
     roof["frac"] = (roof["achieved"] / roof["peak"]) if roof.get("achieved") and roof.get("peak") else None
