@@ -1,5 +1,5 @@
-// FP64 inverses W = M_nm(G)^{-1} along the lattice (chain start, and the
-// refresh of FP64 chains).
+// FP64 inverses W = M_nm(G)^{-1} along the lattice (start and refresh of FP64
+// chains).
 //
 // Without its y links, M falls into L blocks of one lattice row each (size
 // b = L B).  Those are inverted densely (b^3 each), and neighbouring groups of
