@@ -11,8 +11,10 @@
 // the block of one eliminated pair (k, p),
 //     Pf(M) = M_kp Pf(C + (v u^T - u v^T) / M_kp),   u = M[k, rest], v = M[p, rest]
 // (Schur complement of a skew matrix), after moving k, p to the front, which
-// multiplies Pf by the sign of that permutation.  Pairs are chosen within the
-// closed set by the largest |entry| (pivoting restricted to the closed set).
+// multiplies Pf by the sign of that permutation.  Pairs are chosen by the
+// largest |entry| within a panel of the closed set, as long as that is no
+// smaller than 1/16 of what the closed set offers; else the panel ends there
+// and the largest entry of the whole remaining closed set comes next (below).
 //
 // The front of a periodic L x L lattice holds two rows of link ends (the
 // +y ends of the last L sites and the -y ends of row 0, which wait for the
@@ -27,11 +29,22 @@
 // sequence (k_1, p_1, k_2, p_2, ...): the sign of the schedule's own sequence
 // (known on the host) times one factor -1 per exchange a pivot choice makes.
 //
-// What bounds it: the FP64 unit (two FMAs per clock and SM).  The closed set is
+// What bounds it: the FP64 unit (two FMAs per clock and SM).  The closed set (at
+// most four links, 32 Majoranas) is
 // eliminated in chunks of at most 16 Majoranas: their rows are copied into a
 // dense panel over the live slots, the pivoted pairs update the panel only,
 // and the rest of the front then takes the chunk's rank-16 update in one
-// pass, 2 x 2 register tiles over a list of the live slots.  Against a rank-2
+// pass, 2 x 2 register tiles over a list of the live slots.
+//
+// A chunk of a larger closed set can be nearly singular by itself although the
+// closed set is not (the complex pairs n < m; a pivot of 1e-8 then costs eight
+// digits).  So a pivot below 1/16 ends such a chunk, its remaining rows go back
+// to the front, and the next chunk starts from the largest entry of all that
+// is left of the closed set, against which its other pivots are measured.
+// Random states of every group have pivots of 0.2 and more there and never
+// take that turn.
+//
+// Against a rank-2
 // update of the whole triangle per pair (33 % of the FP64 slots useful: dead
 // slots, ragged rows, a shared-memory round trip per product pair) 64 real
 // and 96 complex items of 16 x 16, n_v = 2 took 113 ms and take 50,
@@ -49,6 +62,8 @@ namespace {
 
 constexpr int CHUNK = 16;          // closed Majoranas per panel
 constexpr int SMALL_FRONT = 48;    // slots up to which an item takes 64 threads
+constexpr int MAX_CLOSED = 32;     // Majoranas closed by one site (four links)
+constexpr double PIVOT_FLOOR = 1.0 / 256.0;    // smallest |pivot|^2 of a chunk, over the largest there is
 
 __host__ __device__ __forceinline__ int tri_row(int i, int F) { return i * (2 * F - i - 1) / 2 - i - 1; }
 
@@ -80,6 +95,37 @@ __device__ __forceinline__ T sget(const T* S, int F, int a, int b) {
     if (a < b) return S[tri_row(a, F) + b];
     if (a > b) return fneg(S[tri_row(b, F) + a]);
     return Sc<T>::zero();
+}
+
+// Largest |get(x, y)|^2 over x < y < n (n <= 32, one warp): best in every lane,
+// at = 32 x + y.  NaN orders above all others.
+template <class Get>
+__device__ __forceinline__ void warp_best_pair(int n, Get get, double& best, int& at) {
+    best = -1.0;
+    at = 1;
+    for (int p = threadIdx.x & 31; p < n * (n - 1) / 2; p += 32) {
+        int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
+        if (y * (y - 1) / 2 > p) --y;
+        if ((y + 1) * y / 2 <= p) ++y;
+        const int x = p - y * (y - 1) / 2;
+        const double m = fsq(get(x, y));
+        if (m > best || !(m == m)) { best = m; at = x * 32 + y; }
+    }
+    const unsigned key = best >= 0.0 || !(best == best) ? (unsigned)__double2hiint(best) & 0x7fffffffu : 0u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, key);
+    const int src = __ffs(__ballot_sync(0xffffffffu, key == top && !(best < 0.0))) - 1;
+    best = __shfl_sync(0xffffffffu, best, src);
+    at = __shfl_sync(0xffffffffu, at, src);
+}
+
+// The pair (x, y), x < y, of list a to its first two positions; whether that is an odd permutation.
+__device__ __forceinline__ bool pair_to_front(int* a, int x, int y) {
+    const int k = a[x], p = a[y];
+    a[x] = a[0];
+    a[0] = k;
+    a[y] = a[1];
+    a[1] = p;
+    return (x > 0) != (y > 1);
 }
 
 struct FrontArgs {
@@ -144,10 +190,10 @@ __global__ void __launch_bounds__(NT, NT == 64 ? 8 : (sizeof(T) == 8 ? 2 : 1))
 front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains, int npf, int pair_off,
                 const void* links, cxd* ell, int* bad, T* gws, size_t tri_elems, int in_smem) {
     extern __shared__ __align__(16) unsigned char fsm[];
-    __shared__ int s_bad, s_nl;
+    __shared__ int s_bad, s_nl, s_stop;
     __shared__ T s_inv;
     __shared__ T s_scale[CHUNK];
-    __shared__ int ord[CHUNK], es[CHUNK];
+    __shared__ int ord[CHUNK], es[CHUNK], cl[MAX_CLOSED];
     constexpr int NW = NT / 32;
     const int F = fa.F, B = fa.B, V = fa.V;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -184,6 +230,8 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                 }
             }
             for (int k = tid; k < B; k += NT) idx[fa.slot[s * B + k]] = s * B + k;
+            const int first = fa.eoff[s], ne = fa.eoff[s + 1] - first;
+            for (int k = tid; k < ne; k += NT) cl[k] = fa.elim[first + k];
             __syncthreads();
             for (int k = warp; k < B; k += NW) {
                 const int a = fa.slot[s * B + k];
@@ -198,10 +246,23 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
             }
             __syncthreads();
             // ---- eliminate the closed Majoranas, a chunk at a time
-            const int e1 = fa.eoff[s + 1];
-            for (int e0 = fa.eoff[s]; e0 < e1; e0 += CHUNK) {
-                const int c = min(CHUNK, e1 - e0);
-                if (tid < c) { es[tid] = fa.elim[e0 + tid]; ord[tid] = tid; }
+            int e = 0;
+            bool search = false;       // the last chunk ended at a small pivot
+            while (e < ne) {
+                const int c = min(CHUNK, ne - e);
+                double low = PIVOT_FLOOR;      // (warp 0) |pivot|^2 below which this chunk ends
+                if (search) {
+                    if (warp == 0) {
+                        double best;
+                        int bq;
+                        warp_best_pair(ne - e, [&](int x, int y) { return sget(S, F, cl[e + x], cl[e + y]); }, best, bq);
+                        low = PIVOT_FLOOR * best;
+                        if (lane == 0 && pair_to_front(cl + e, bq / 32, bq % 32)) pr = -pr;
+                    }
+                    __syncthreads();
+                }
+                if (tid == 0) s_stop = 0;
+                if (tid < c) { es[tid] = cl[e + tid]; ord[tid] = tid; }
                 __syncthreads();
                 if (tid < c) idx[es[tid]] = -1;
                 __syncthreads();
@@ -221,49 +282,34 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     for (int w = lane; w < W; w += 32)
                         Pn[(size_t)t * F + w] = sget(S, F, es[t], w < c ? es[w] : lv[w - c]);
                 __syncthreads();
-                for (int t = 0; t < c; t += 2) {
+                int te = 0;            // eliminated rows of the chunk
+                for (; te < c; te += 2) {
+                    const int t = te;
                     if (warp == 0) {
                         // pivot: the largest entry among the chunk's remaining pairs
-                        const int ne = c - t;
-                        double best = -1.0;
-                        int bq = 1;
-                        for (int p = lane; p < ne * (ne - 1) / 2; p += 32) {
-                            int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
-                            if (y * (y - 1) / 2 > p) --y;
-                            if ((y + 1) * y / 2 <= p) ++y;
-                            const int x = p - y * (y - 1) / 2;
-                            const double m = fsq(Pn[(size_t)ord[t + x] * F + ord[t + y]]);
-                            if (m > best || !(m == m)) { best = m; bq = x * 32 + y; }
-                        }
-                        const unsigned key = best >= 0.0 || !(best == best) ? (unsigned)__double2hiint(best) & 0x7fffffffu : 0u;
-                        const unsigned top = __reduce_max_sync(0xffffffffu, key);
-                        const int src = __ffs(__ballot_sync(0xffffffffu, key == top && !(best < 0.0))) - 1;
-                        best = __shfl_sync(0xffffffffu, best, src);
-                        bq = __shfl_sync(0xffffffffu, bq, src);
-                        if (lane == 0) {
-                            const int x = bq / 32, y = bq % 32;
+                        double best;
+                        int bq;
+                        warp_best_pair(c - t, [&](int x, int y) { return Pn[(size_t)ord[t + x] * F + ord[t + y]]; }, best, bq);
+                        if (e + c < ne && best < low && !(search && t == 0)) {
+                            if (lane == 0) s_stop = 1;           // better ones may lie outside the chunk
+                        } else if (lane == 0) {
                             if (!(best > 1e-16) || !isfinite(best)) s_bad = 1;   // no usable pivot: refactor densely
-                            // the pair to positions t, t + 1 (x < y: the first exchange leaves t + y alone)
-                            const int k = ord[t + x], p = ord[t + y];
-                            ord[t + x] = ord[t];
-                            ord[t] = k;
-                            ord[t + y] = ord[t + 1];
-                            ord[t + 1] = p;
+                            if (pair_to_front(ord + t, bq / 32, bq % 32)) pr = -pr;
+                            const int k = ord[t], p = ord[t + 1];
                             const T akp = Pn[(size_t)k * F + p];
                             const T inv = finv(akp);
                             s_inv = inv;
                             s_scale[t] = inv;
                             pr = pr * as_c(akp);
-                            if ((x > 0) != (y > 1)) pr = -pr;
                             // keep the product in range by its own power of two
-                            const int e = ((__double2hiint(fmax(fabs(pr.x), fabs(pr.y))) >> 20) & 0x7ff) - 1023;
-                            const double sc = __hiloint2double((1023 - e) << 20, 0);
+                            const int ep = ((__double2hiint(fmax(fabs(pr.x), fabs(pr.y))) >> 20) & 0x7ff) - 1023;
+                            const double sc = __hiloint2double((1023 - ep) << 20, 0);
                             pr = {pr.x * sc, pr.y * sc};
-                            ex += e;
+                            ex += ep;
                         }
                     }
                     __syncthreads();
-                    if (s_bad) break;
+                    if (s_bad || s_stop) break;
                     // the remaining rows of the chunk: R += (v_R / a) k - (k_R / a) v
                     const T* rk = Pn + (size_t)ord[t] * F;
                     const T* rp = Pn + (size_t)ord[t + 1] * F;
@@ -281,8 +327,22 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     __syncthreads();
                 }
                 if (s_bad) break;
+                // the rows that the chunk leaves behind, back to the front
+                for (int i = te + warp; i < c; i += NW) {
+                    const int row = ord[i], a = es[row];
+                    for (int w = i + 1 + lane; w < W; w += 32) {
+                        const int col = w < c ? ord[w] : w, b = w < c ? es[col] : lv[w - c];
+                        const T val = Pn[(size_t)row * F + col];
+                        if (a < b) S[tri_row(a, F) + b] = val;
+                        else S[tri_row(b, F) + a] = fneg(val);
+                    }
+                    if (lane == 0) {
+                        cl[e + i] = a;
+                        idx[a] = 0;        // live again (which Majorana it is matters only to later sites)
+                    }
+                }
                 // u_t = row k_t / a_t over the live columns
-                for (int t = 2 * warp; t < c; t += 2 * NW) {
+                for (int t = 2 * warp; t < te; t += 2 * NW) {
                     T* r = Pn + (size_t)ord[t] * F + c;
                     const T inv = s_scale[t];
                     for (int w = lane; w < nl; w += 32) r[w] = fmul(r[w], inv);
@@ -302,7 +362,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     const bool diag = i == j;
                     T a00 = diag ? Sc<T>::zero() : S0[c0], a01 = S0[c1];
                     T a10 = diag ? Sc<T>::zero() : S1[c0], a11 = diag ? Sc<T>::zero() : S1[c1];
-                    for (int t = 0; t < c; t += 2) {
+                    for (int t = 0; t < te; t += 2) {
                         const T* u = Pn + (size_t)ord[t] * F + c;
                         const T* v = Pn + (size_t)ord[t + 1] * F + c;
                         const T ui0 = u[i], ui1 = u[i + 1], vi0 = v[i], vi1 = v[i + 1];
@@ -316,6 +376,8 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     if (!diag) { S0[c0] = a00; S1[c0] = a10; S1[c1] = a11; }
                 }
                 __syncthreads();
+                search = te < c;
+                e += te;
             }
             if (s_bad) break;
         }
@@ -415,6 +477,8 @@ ggf_status ggf_front_prepare(ggf_ctx* ctx) {
     std::vector<int> slot, eoff, elim;
     build_schedule(g, F, slot, eoff, elim, sign);
     if ((int)elim.size() != g.N) return ggf_fail(ctx, GGF_ESTATE, "front schedule does not close every Majorana");
+    for (int s = 0; s < g.V; ++s)
+        if (eoff[s + 1] - eoff[s] > MAX_CLOSED) return ggf_fail(ctx, GGF_ESTATE, "front schedule closes too many Majoranas");
     std::vector<int> all;
     all.insert(all.end(), slot.begin(), slot.end());
     all.insert(all.end(), eoff.begin(), eoff.end());
