@@ -56,6 +56,7 @@ struct SweepArgs {
     int forced_k;
     int* dead;
     PairBins bins;
+    unsigned char early[MAXCS];     // immediate mode: CTA b copies beside the Pfaffian (copy_early)
 };
 
 // 16-byte pieces of a run of reals
@@ -201,7 +202,8 @@ __device__ __forceinline__ void gather_rows_cols(int N, int a0, int b0, const T*
 // One proposal of every chain; a cluster per chain, its pairs dealt to the CTAs
 // (deal_pairs).  The Pfaffian ratio and Z of a pair run side by side on two
 // warps, the pair terms on the last one, and in immediate mode the warps in
-// between already copy the rows and columns that an accepted update needs.
+// between already copy the rows and columns that an accepted update needs,
+// where that is done before the Pfaffian is (copy_early).
 // Bound: the latency of that chain of FP64 steps; one CTA that drew, formed
 // Delta, W_SS, ratio, terms, Z and copies in turn took 134 us for 1024 chains of
 // 8 x 8 Z2 and 185 us for a block-move link of 32 chains of 8 x 8 U(1), K = 2;
@@ -318,7 +320,7 @@ __global__ void __launch_bounds__(NWARP * 32, 2) ratio_kernel(SweepArgs a) {
             else gather_rows_cols<CW, R>(N, a0, b0, w_cplx(p), (CW*)a.ybuf_c + ((size_t)c * Kc + (p - K)) * 2 * R * N, first, cnt);
         }
     };
-    if (a.kmax <= 1 && spare > 0 && warp >= spare0 && warp < NWARP - 1)
+    if (a.early[rank] && warp >= spare0 && warp < NWARP - 1)
         copy_rows((warp - spare0) * 32 + lane, spare * 32);
     if (CS > 1) cg::this_cluster().sync();
     else __syncthreads();
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(NWARP * 32, 2) ratio_kernel(SweepArgs a) {
         if (!s_okz[s] && a.forced && threadIdx.x == 0) a.dead[c] = 1;
     }
     // (delayed mode: gather_kernel forms the rows and columns)
-    if (a.kmax <= 1 && spare == 0) copy_rows(threadIdx.x, NWARP * 32);
+    if (a.kmax <= 1 && !a.early[rank]) copy_rows(threadIdx.x, NWARP * 32);
 }
 
 // W <- W - C Z Y of the accepted chains.  Bound: the traffic of W, read and
@@ -697,6 +699,25 @@ __global__ void mark_refresh(int n_chains, int R, const int* since, int* list) {
     }
 }
 
+// Whether a CTA copies the rows and columns of its nr real and nc complex pairs
+// before the decision, on `spare` warps beside the Pfaffian: only where the
+// Pfaffian hides it, or a rejected proposal pays for a copy that nobody reads.
+// The line is the loop trips of a spare thread (16-byte pieces of the rows,
+// entries of the columns) against the order R of the blocks, in proportion to
+// which the Pfaffian grows.  Microseconds per link, early and after
+// the decision, accepted / rejected: 10 trips of R = 4 (8 x 8 Z2) 17 / 14 and
+// 19 / 14, 26 of R = 8 (8 x 8 U(1), K = 1, FP32) 34 / 28 and 41 / 27, 32 (4 x 4
+// U(1), K = 2, FP64) 48 / 36 and 52 / 33; but 38 of R = 4 (16 x 16 Z2) 41 / 27 and
+// 37 / 15, 85 of R = 8 (8 x 8 U(1), K = 2, FP32) 83 / 64 and 70 / 40, 288
+// (12 x 12, FP64) 202 / 185 and 118 / 33.  (Where the chains alone fill the chip,
+// 1024 of 8 x 8 Z2, early is better from 75 % accepted on: 73 / 58 and 79 / 43.)
+// rsz: bytes of a real element of W.
+bool copy_early(int N, int R, int nr, int nc, int rsz) {
+    const int spare = NWARP - 1 - std::min(2 * (nr + nc), NWARP - 1);
+    const long long work = (long long)N * ((nr + 2 * nc) * R * rsz / 16 + 2 * (nr + nc));
+    return spare > 0 && work <= 4LL * R * 32 * spare;
+}
+
 }  // namespace
 
 ggf_status ggf_flush(ggf_ctx* ctx, cudaStream_t st);
@@ -746,9 +767,13 @@ ggf_status ggf_link_step_ex(ggf_ctx* ctx, int link, cudaStream_t st, const int* 
     a.kmax = ch.kmax;
     const int CS = deal_pairs(ctx->K, ctx->Kc, a.bins);
     size_t smem = 0;
-    for (int b = 0; b < CS; ++b)
-        smem = std::max(smem, ratio_layout(ctx->P, g.r, a.bins.first[b + 1] - a.bins.first[b],
-                                           ch.kmax > 1 ? ch.kmax * g.r : 0, 2 * rsz).total);
+    for (int b = 0; b < CS; ++b) {
+        const int np = a.bins.first[b + 1] - a.bins.first[b];
+        int nc = 0;
+        for (int s = 0; s < np; ++s) nc += a.bins.ord[a.bins.first[b] + s] >= ctx->K;
+        smem = std::max(smem, ratio_layout(ctx->P, g.r, np, ch.kmax > 1 ? ch.kmax * g.r : 0, 2 * rsz).total);
+        a.early[b] = ch.kmax <= 1 && copy_early(g.N, g.r, np - nc, nc, (int)rsz);
+    }
     const int ev0 = ctx->prof_mark(st);
     ctx->launches += 2 + (ctx->Kc ? 1 : 0);
     cudaLaunchConfig_t cfg{};
