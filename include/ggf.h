@@ -414,6 +414,12 @@ typedef struct {
 
 ggf_status ggf_chains_stats(ggf_ctx* ctx, ggf_chain_stats* out);
 
+/* FP64 chains: inverses since ggf_chains_init (start and refreshes) that the
+ * elimination along the lattice left to FP64 Gauss-Jordan, because an open row
+ * of the lattice was too badly conditioned or the workspace too small
+ * (ggf_chain_stats keeps its layout). */
+ggf_status ggf_chains_dense_inverses(ggf_ctx* ctx, uint64_t* matrices);
+
 /* Per-chain failure report (the aggregate counters above say that something
  * failed, this says which chain): status[n_chains] (int32, host or device per
  * mem) gets GGF_ESINGULAR for a chain whose factorisation met a singular

@@ -344,6 +344,7 @@ ggf_status lattice_inverse(ggf_ctx* ctx, const std::vector<int>& chains, std::ve
         const int cap = ggf_lattice_inverse_plan(ctx, cplx, (int)cfg.size(), std::max(budget_bytes(), ctx->work_bytes), bytes);
         if (cap < 1) {                       // no room for one matrix's workspace
             for (int c : chains) bad[c] = 1;
+            ctx->dense_inverses += cfg.size();
             break;
         }
         GGF_TRY(ggf_workspace(ctx, bytes));
@@ -357,7 +358,10 @@ ggf_status lattice_inverse(ggf_ctx* ctx, const std::vector<int>& chains, std::ve
             GGF_TRY(place_inverses(ctx, cplx, n, d_chain, d_pair, A, st));
             GGF_CK(cudaStreamSynchronize(st));   // the workspace is reused by the next batch
             for (int i = 0; i < n; ++i)
-                if (!ok[i]) bad[cfg[i0 + i]] = 1;
+                if (!ok[i]) {
+                    bad[cfg[i0 + i]] = 1;
+                    ctx->dense_inverses += 1;
+                }
         }
     }
     for (int c : chains)
@@ -702,7 +706,7 @@ ggf_status ggf_chains_init(ggf_ctx* ctx, int n_chains, const void* links, const 
     cudaStream_t st = (cudaStream_t)stream;
     ggf_free_chains(ctx);
     ctx->refine_rmax = 0.0;
-    ctx->dense_refreshes = ctx->dense_pfaffians = ctx->refine_steps = 0;
+    ctx->dense_refreshes = ctx->dense_pfaffians = ctx->refine_steps = ctx->dense_inverses = 0;
     Chains& ch = ctx->ch;
     ch.opts = *opts;
     ch.n = n_chains;
@@ -1431,6 +1435,13 @@ ggf_status ggf_chains_stats(ggf_ctx* ctx, ggf_chain_stats* out) {
     out->dense_pfaffians = ctx->dense_pfaffians;
     out->flush_wave = ctx->ch.ps ? (uint64_t)ctx->ch.ps_wave : 0;
     if (h[3]) return ggf_fail(ctx, GGF_ESINGULAR, "a refresh met a singular M(G)");
+    return GGF_OK;
+}
+
+ggf_status ggf_chains_dense_inverses(ggf_ctx* ctx, uint64_t* matrices) {
+    GGF_TRY(require(ctx, true, true));
+    if (!matrices) return ggf_fail(ctx, GGF_EINVAL, "null count");
+    *matrices = ctx->dense_inverses;
     return GGF_OK;
 }
 

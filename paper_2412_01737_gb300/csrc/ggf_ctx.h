@@ -117,10 +117,10 @@ struct ggf_ctx {
     void* front_ws = nullptr;
     size_t front_ws_bytes = 0;
     // refresh bookkeeping since ggf_chains_init: largest Newton residual
-    // |I - M W| seen, chains refreshed by dense Gauss-Jordan instead, and
-    // Pfaffian items that fell back to the dense elimination
+    // |I - M W| seen, chains refreshed by dense Gauss-Jordan instead, Pfaffian
+    // items that fell back to the dense elimination, and FP64 inverses that did
     double refine_rmax = 0.0;
-    unsigned long long dense_refreshes = 0, dense_pfaffians = 0, refine_steps = 0;
+    unsigned long long dense_refreshes = 0, dense_pfaffians = 0, refine_steps = 0, dense_inverses = 0;
     // event timing (ggf_profile)
     bool prof = false;
     std::vector<cudaEvent_t> ev;            // event pool

@@ -57,7 +57,7 @@ EXPORTS = ["ggf_create", "ggf_destroy", "ggf_last_error", "ggf_init_lattice", "g
            "ggf_chains_fermion4", "ggf_chains_link_score", "ggf_wilson_loop", "ggf_polyakov_loop",
            "ggf_debug_poison_inverse", "ggf_chains_refine", "ggf_debug_scale_inverse", "ggf_chains_status", "ggf_chains_state_size", "ggf_chains_save_state", "ggf_chains_load_state",
            "ggf_chains_electric_field", "ggf_chains_link_terms",
-           "ggf_chains_stats",
+           "ggf_chains_stats", "ggf_chains_dense_inverses",
            "ggf_checkpoint",
            "ggf_resume", "ggf_profile", "ggf_kernel_time", "ggf_sync", "ggf_logweight_noalloc",
            "ggf_selftest_flush", "ggf_selftest_flush_data", "ggf_net_create", "ggf_net_destroy", "ggf_net_last_error", "ggf_net_get_params",
@@ -111,6 +111,7 @@ def load():
         "ggf_chains_save_state": ([P, P, I, P], I),
         "ggf_chains_load_state": ([P, P, I, P], I),
         "ggf_chains_stats": ([P, ctypes.POINTER(ChainStats)], I),
+        "ggf_chains_dense_inverses": ([P, ctypes.POINTER(ctypes.c_uint64)], I),
         "ggf_checkpoint": ([P, ctypes.c_char_p], I),
         "ggf_resume": ([P, ctypes.c_char_p, P], I),
         "ggf_profile": ([P, I], I),
@@ -453,6 +454,12 @@ class GGF:
         s = ChainStats()
         self._ck(self.lib.ggf_chains_stats(self.h, ctypes.byref(s)))
         return s
+
+    def chains_dense_inverses(self):
+        """Inverses of FP64 chains that fell back from the lattice to Gauss-Jordan."""
+        n = ctypes.c_uint64()
+        self._ck(self.lib.ggf_chains_dense_inverses(self.h, ctypes.byref(n)))
+        return n.value
 
     def state_size(self):
         """Bytes of the in-memory chain state (save_state / load_state)."""
