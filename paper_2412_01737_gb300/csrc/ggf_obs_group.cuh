@@ -1,7 +1,9 @@
-// Cooperative bodies of the observable kernels: a group of lanes (one per
-// virtual Majorana of a site: B = 8 n_v) evaluates one (chain, item).  What
-// each item is, and the one-thread form of the same arithmetic, is in
-// ggf_obs.cuh.
+// The observable kernels' bodies (electric, Sec. 5.3; fermionic, Sec. 5.2; scores
+// and per-pair norms): a group of lanes (one per virtual Majorana of a site:
+// B = 8 n_v) evaluates one (chain, item).  Each body is cut into phases, what a
+// lane does between two barriers; the kernels run the phases with a warp's
+// lanes side by side, ggf_obs.cuh one lane after the other on the host, so
+// that CPU tests check the kernels' own arithmetic and indices.
 //
 // One thread per item walked its W block row by row: dependent scattered
 // loads, the pair weights' exponentials formed again by every thread, complex
@@ -10,7 +12,8 @@
 // the weights are formed once per CTA, real pairs stay real, and the two
 // orders of a pair share their products (below).
 #pragma once
-#include "ggf_obs.cuh"
+#include "ggf_ctx.h"
+#include "ggf_sweep.cuh"
 
 namespace {
 
@@ -22,19 +25,19 @@ template <> struct Wide<float> { typedef double Z; };
 template <> struct Wide<cxd> { typedef cxd Z; };
 template <> struct Wide<cxf> { typedef cxd Z; };
 
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) { return (double)v; }
-__device__ __forceinline__ cxd widen(cxd v) { return v; }
-__device__ __forceinline__ cxd widen(cxf v) { return {(double)v.x, (double)v.y}; }
+GGF_HD double widen(double v) { return v; }
+GGF_HD double widen(float v) { return (double)v; }
+GGF_HD cxd widen(cxd v) { return v; }
+GGF_HD cxd widen(cxf v) { return {(double)v.x, (double)v.y}; }
 
-__device__ __forceinline__ void axpy(double& r, double a, double b) { r = fma(a, b, r); }
-__device__ __forceinline__ void axpy(cxd& r, double a, cxd b) { r.x = fma(a, b.x, r.x); r.y = fma(a, b.y, r.y); }
-__device__ __forceinline__ void axpy(cxd& r, cxd a, cxd b) {
+GGF_HD void axpy(double& r, double a, double b) { r = fma(a, b, r); }
+GGF_HD void axpy(cxd& r, double a, cxd b) { r.x = fma(a, b.x, r.x); r.y = fma(a, b.y, r.y); }
+GGF_HD void axpy(cxd& r, cxd a, cxd b) {
     r.x = fma(a.x, b.x, r.x); r.x = fma(-a.y, b.y, r.x);
     r.y = fma(a.x, b.y, r.y); r.y = fma(a.y, b.x, r.y);
 }
-__device__ __forceinline__ cxd as_cx(double v) { return {v, 0.0}; }
-__device__ __forceinline__ cxd as_cx(cxd v) { return v; }
+GGF_HD cxd as_cx(double v) { return {v, 0.0}; }
+GGF_HD cxd as_cx(cxd v) { return v; }
 __device__ __forceinline__ double shfl_xor_(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ cxd shfl_xor_(cxd v, int o) {
     return {__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
@@ -43,7 +46,7 @@ __device__ __forceinline__ cxd shfl_xor_(cxd v, int o) {
 // n consecutive elements of W (n sizeof(T) a multiple of 8; 16-byte pieces
 // where the run allows: every run starts on a multiple of its length)
 template <int n, class T>
-__device__ __forceinline__ void load_run(const T* p, typename Wide<T>::Z* out) {
+GGF_HD void load_run(const T* p, typename Wide<T>::Z* out) {
     constexpr int bytes = n * sizeof(T);
     if constexpr (bytes % 16 == 0) {
         union { float4 v[bytes / 16]; T t[n]; } u;
@@ -82,7 +85,62 @@ __device__ __forceinline__ void chain_weights(const DevConst& dc, const cxd* el,
     __syncthreads();
 }
 
-// ---- electric ------------------------------------------------------------------
+// ---- electric (the derivation is in k_electric.cu) ---------------------------
+
+// Pfaffian of an H x H antisymmetric matrix (H = 2 n_v = 2 or 4), closed form.
+template <int H>
+GGF_HD cxd small_pf(const cxd (&A)[H][H]);
+template <>
+GGF_HD cxd small_pf<2>(const cxd (&A)[2][2]) { return A[0][1]; }
+template <>
+GGF_HD cxd small_pf<4>(const cxd (&A)[4][4]) {
+    return A[0][1] * A[2][3] - A[0][2] * A[1][3] + A[0][3] * A[1][2];
+}
+
+// Normalised expectation of the insertion from G = Gamma_O[S, S]; FIELD: the
+// U(1) twist charge Q_l itself (the electric field) instead of Q_l^2.
+template <int H, bool FIELD = false>
+GGF_HD cxd insertion(const Geometry& g, const cxd (&G)[H][H]) {
+    if constexpr (FIELD) {
+        cxd val = {0.0, 0.0};
+#pragma unroll
+        for (int j = 0; j < H / 2; ++j) {
+            cxd occ = G[2 * j][2 * j + 1];
+            occ.x += 1.0;
+            val += (0.5 * (double)g.q[j]) * occ;       // q_j <n_j>
+        }
+        return val;
+    }
+    if (g.group == GGF_Z2) {
+        const double sg = (H / 2) % 2 ? -1.0 : 1.0;    // (-1)^{n_v}
+        return sg * small_pf<H>(G);
+    }
+    if constexpr (H == 4) {
+        if (g.group == GGF_SU2) {
+            // sum_a (Q^a)^2 on the doublet = (3/4)(n_0 + n_1 - 2 n_0 n_1)
+            cxd o = G[0][1] + G[2][3];
+            o.x += 2.0;                                  // 2 (<n_0> + <n_1>)
+            cxd pr = G[0][1] + G[2][3] + small_pf<H>(G);
+            pr.x += 1.0;                                 // 4 <n_0 n_1>
+            return 0.375 * (o - pr);                     // (3/4)(o / 2 - 2 pr / 4)
+        }
+    }
+    cxd val = {0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j < H / 2; ++j) {
+        const double qj = g.q[j];
+        cxd occ = G[2 * j][2 * j + 1];
+        occ.x += 1.0;
+        val += (0.5 * qj * qj) * occ;
+    }
+    if constexpr (H == 4) {
+        cxd pr = G[0][1] + G[2][3] + small_pf<H>(G);
+        pr.x += 1.0;
+        val += (0.5 * g.q[0] * g.q[1]) * pr;            // 2 q_0 q_1 <n_0 n_1>
+    }
+    return val;
+}
+
 // With A the columns S of the block W[site, link] and G = W[site, link]
 // Gamma_tw[link, S], the two orders of a pair are
 //   X_f = U + i V,  X_r = conj(U - i V),  U = A_S - D_S G,  V = G_S + D_S A
@@ -95,74 +153,208 @@ template <int H> struct ElectricShared {
     double tw[16];
 };
 
-template <class T, int H, bool FIELD>
-__device__ __forceinline__ cxd electric_pair(const DevConst& dc, int pf, int l, const T* W, int lane, double gval,
-                                             ElectricShared<H>& sh) {
+// The link's twist into sh.tw (SU(2): lane 0; U(1): a lane per mode); the value of a Z2 link.
+template <int H>
+GGF_HD double electric_twist(const Geometry& g, const void* links, int c, int l, int lane, ElectricShared<H>& sh) {
+    if (g.group == GGF_SU2) {
+        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), sh.tw);
+    } else if (g.group == GGF_U1) {
+        const double th = ((const double*)links)[(size_t)c * g.n_links + l];
+        if (lane < g.n_v) sincos(g.q[lane] * th, &sh.tw[2 * lane + 1], &sh.tw[2 * lane]);
+    } else {
+        return (double)((const int8_t*)links)[(size_t)c * g.n_links + l];
+    }
+    return 1.0;
+}
+
+// Phase 1: the lane's entries of Gamma_tw and its row of W[site, link] (a0, b0: the link's ends).
+template <class T, int H>
+GGF_HD void electric_load(const DevConst& dc, int pf, int l, int a0, int b0, const T* W, int lane, double gval,
+                          ElectricShared<H>& sh, typename Wide<T>::Z (&w)[2 * H]) {
     typedef typename Wide<T>::Z Z;
     constexpr int R = 2 * H, B = 4 * H;
     const Geometry& g = dc.g;
     Z* gt = (Z*)sh.gt;
-    Z* As = (Z*)sh.A;
-    Z* Gs = (Z*)sh.G;
-    int a0, b0;
-    link_ends(g, l, a0, b0);
-    const int s0 = (l >> 1) * g.B, loc0 = a0 - s0;
     for (int e = lane; e < R * H; e += B)
         gt[e] = g.group == GGF_SU2 ? twisted_su2<Z>(dc, pf, l, e / H, e % H, sh.tw)
                                    : twisted_tab<Z>(dc, pf, l, e / H, e % H, gval, sh.tw);
-    Z w[R];
-    const T* row = W + (size_t)(s0 + lane) * g.N;
+    const T* row = W + (size_t)((l >> 1) * B + lane) * g.N;
     load_run<H>(row + a0, w);
     load_run<H>(row + b0, w + H);
-    __syncwarp();
+}
+
+// Phase 2: the lane's row of A and G.
+template <class T, int H>
+GGF_HD void electric_rows(int lane, const typename Wide<T>::Z (&w)[2 * H], ElectricShared<H>& sh) {
+    typedef typename Wide<T>::Z Z;
+    const Z* gt = (const Z*)sh.gt;
+    Z* As = (Z*)sh.A;
+    Z* Gs = (Z*)sh.G;
 #pragma unroll
     for (int b = 0; b < H; ++b) {
         Z s = Sc<Z>::zero();
 #pragma unroll
-        for (int j = 0; j < R; ++j) axpy(s, w[j], gt[j * H + b]);
+        for (int j = 0; j < 2 * H; ++j) axpy(s, w[j], gt[j * H + b]);
         As[lane * H + b] = w[b];
         Gs[lane * H + b] = s;
     }
-    __syncwarp();
-    if (lane < H * H) {
-        const int a = lane / H, b = lane % H;
-        const double* Dr = dc.D + ((size_t)(l >> 1) * B + loc0 + a) * B;
-        Z u = As[(loc0 + a) * H + b], v = Gs[(loc0 + a) * H + b];
-#pragma unroll 4
-        for (int i = 0; i < B; ++i) {
-            const double d = Dr[i];
-            axpy(u, -d, Gs[i * H + b]);
-            axpy(v, d, As[i * H + b]);
-        }
-        sh.U[lane] = as_cx(u);
-        sh.V[lane] = as_cx(v);
-    }
-    __syncwarp();
-    // lane 0: the (n, m) order, lane 1: (m, n)
-    cxd out = {0.0, 0.0};
-    if (lane < 2) {
-        const double sg = lane ? -1.0 : 1.0;
-        cxd X[H][H];
-#pragma unroll
-        for (int a = 0; a < H; ++a)
-#pragma unroll
-            for (int b = 0; b < H; ++b) {
-                const cxd u = sh.U[a * H + b], v = sh.V[a * H + b];
-                // -(U + i V) or -conj(U - i V), plus i on the diagonal
-                X[a][b] = {-(u.x - sg * v.y), -sg * (u.y + sg * v.x)};
-                if (a == b) X[a][b].y += 1.0;
-            }
-        out = insertion<H, FIELD>(g, X);
-    }
-    __syncwarp();
-    return out;
 }
 
-// ---- fermionic -------------------------------------------------------------------
-// X[alpha][beta] = B_s W[s, t] B_t^T; every lane of the group gets the result.
+// Phase 3: an entry of U and V per lane.
+template <class T, int H>
+GGF_HD void electric_products(const DevConst& dc, int l, int a0, int lane, ElectricShared<H>& sh) {
+    typedef typename Wide<T>::Z Z;
+    constexpr int B = 4 * H;
+    if (lane >= H * H) return;
+    const Z* As = (const Z*)sh.A;
+    const Z* Gs = (const Z*)sh.G;
+    const int a = lane / H, b = lane % H, at = a0 - (l >> 1) * B + a;
+    const double* Dr = dc.D + ((size_t)(l >> 1) * B + at) * B;
+    Z u = As[at * H + b], v = Gs[at * H + b];
+#pragma unroll 4
+    for (int i = 0; i < B; ++i) {
+        const double d = Dr[i];
+        axpy(u, -d, Gs[i * H + b]);
+        axpy(v, d, As[i * H + b]);
+    }
+    sh.U[lane] = as_cx(u);
+    sh.V[lane] = as_cx(v);
+}
+
+// Phase 4: lane 0: the (n, m) order, lane 1: (m, n).
+template <int H, bool FIELD>
+GGF_HD cxd electric_value(const Geometry& g, int lane, const ElectricShared<H>& sh) {
+    if (lane >= 2) return {0.0, 0.0};
+    const double sg = lane ? -1.0 : 1.0;
+    cxd X[H][H];
+#pragma unroll
+    for (int a = 0; a < H; ++a)
+#pragma unroll
+        for (int b = 0; b < H; ++b) {
+            const cxd u = sh.U[a * H + b], v = sh.V[a * H + b];
+            // -(U + i V) or -conj(U - i V), plus i on the diagonal
+            X[a][b] = {-(u.x - sg * v.y), -sg * (u.y + sg * v.x)};
+            if (a == b) X[a][b].y += 1.0;
+        }
+    return insertion<H, FIELD>(g, X);
+}
+
+// The lane's order of pair p (value v, norm Np) into its sum and the per-pair
+// output po [K][K] (or null; not live: nothing is stored).  w_p = 2 lambda_n^* lambda_m: the (n, m) term
+// (lane 0) takes E / 2, the (m, n) term (lane 1) its conjugate; a diagonal pair
+// E once.
+GGF_HD void electric_term(const DevConst& dc, int p, int lane, bool live, cxd Np, cxd v, cxd& num, cxd* po) {
+    const int K = dc.K;
+    const bool cplx = p >= K;
+    const cxd E = dc.w[p] * Np;
+    if (lane == 0) num += (cplx ? 0.5 : 1.0) * (E * v);
+    else if (lane == 1 && cplx) num += 0.5 * (conjg(E) * v);
+    if (po && live) {
+        int n, m;
+        pair_nm(K, p, n, m);
+        if (lane == 0) po[n * K + m] = Np * v;
+        else if (lane == 1 && cplx) po[m * K + n] = conjg(Np) * v;
+    }
+}
+
+template <class T, int H, bool FIELD>
+__device__ __forceinline__ cxd electric_pair(const DevConst& dc, int pf, int l, const T* W, int lane, double gval,
+                                             ElectricShared<H>& sh) {
+    typename Wide<T>::Z w[2 * H];
+    int a0, b0;
+    link_ends(dc.g, l, a0, b0);
+    electric_load<T, H>(dc, pf, l, a0, b0, W, lane, gval, sh, w);
+    __syncwarp();
+    electric_rows<T, H>(lane, w, sh);
+    __syncwarp();
+    electric_products<T, H>(dc, l, a0, lane, sh);
+    __syncwarp();
+    const cxd v = electric_value<H, FIELD>(dc.g, lane, sh);
+    __syncwarp();
+    return v;
+}
+
+// N_nm(G) / N(G) of chain c into out[c][n][m] for every ordered pair.
+__host__ __device__ inline void pair_norm_item(const DevConst& dc, int c, const cxd* ell, cxd* out) {
+    const int K = dc.K;
+    const cxd* el = ell + (size_t)c * dc.P;
+    double amax, iden;
+    pair_scale(dc, el, amax, iden);
+    cxd* o = out + (size_t)c * K * K;
+    for (int p = 0; p < dc.P; ++p) {
+        const cxd Np = pair_norm(dc, el, p, amax, iden);
+        int n, m;
+        pair_nm(K, p, n, m);
+        o[n * K + m] = Np;
+        if (n != m) o[m * K + n] = conjg(Np);
+    }
+}
+
+// ---- fermionic (the derivation is in k_fermion.cu) ---------------------------
+
+GGF_HD cxd times_minus_i(cxd v) { return {v.y, -v.x}; }
+
+// Per-pair expectation -i (A + X)[alpha][beta] of entry (alpha, beta) of item
+// (s, t), with c_a c_a = 1 where both Majoranas coincide (self-links).
+GGF_HD cxd pair_bilinear(const DevConst& dc, int s, int t, int a, int b, cxd x) {
+    if (s == t) {
+        if (a == b) return cxd{1.0, 0.0};
+        x.x += dc.Ap[(size_t)s * 4 + a * 2 + b];
+    }
+    return times_minus_i(x);
+}
+
+// What lane `lane` of item it of chain c keeps: entry (a, b) of the block of
+// sites (s, t), whether it is wanted, and where it goes in the combined and in
+// the per-pair outputs (items 0 .. V - 1 are sites, of which only the entry
+// (0, 1) is kept, then the links).
+struct FermionLane {
+    bool is_site, entry;
+    int s, t, a, b;
+    size_t out, pair;
+};
+GGF_HD FermionLane fermion_lane(const Geometry& g, int K, int c, int it, int lane) {
+    FermionLane f;
+    f.is_site = it < g.V;
+    f.s = f.t = it;
+    if (!f.is_site) {
+        int a0, b0;
+        link_ends(g, it - g.V, a0, b0);
+        f.s = a0 / g.B;
+        f.t = b0 / g.B;
+    }
+    f.a = (lane >> 1) & 1;
+    f.b = lane & 1;
+    f.entry = lane < 4 && (!f.is_site || lane == 1);
+    f.out = f.is_site ? (size_t)c * g.V + f.s : ((size_t)c * g.n_links + (it - g.V)) * 4 + (lane & 3);
+    f.pair = f.is_site ? f.out * K * K : (((size_t)c * g.n_links + (it - g.V)) * 4 + (f.a * 2 + f.b)) * K * K;
+    return f;
+}
+
+// Pair p's block entry x (norm Np) into the lane's sum, and its two orders into
+// the per-pair output q [K][K] (or null).
+GGF_HD void fermion_term(const DevConst& dc, const FermionLane& f, int p, cxd Np, cxd x, cxd& acc, cxd* q) {
+    const cxd E = dc.w[p] * Np;
+    int n, m;
+    pair_nm(dc.K, p, n, m);
+    if (p >= dc.K) {
+        // (n, m) with weight E / 2 (w_p = 2 lambda_n^* lambda_m), (m, n) with
+        // conj(E) / 2 and the conjugate product; A is added after the loop
+        const cxd h = 0.5 * E;
+        acc += h * x + conjg(h) * conjg(x);
+        if (q) {
+            q[n * dc.K + m] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, x);
+            q[m * dc.K + n] = conjg(Np) * pair_bilinear(dc, f.s, f.t, f.a, f.b, conjg(x));
+        }
+    } else {
+        acc += E * x;
+        if (q) q[n * dc.K + n] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, x);
+    }
+}
+
+// X[alpha][beta] = B_s W[s, t] B_t^T: row `lane` of the block's part of the sum.
 template <class T, int BW>
-__device__ __forceinline__ void coupled_group(const DevConst& dc, const T* W, int s, int t, int lane,
-                                              typename Wide<T>::Z (&X)[4]) {
+GGF_HD void coupled_row(const DevConst& dc, const T* W, int s, int t, int lane, typename Wide<T>::Z (&X)[4]) {
     typedef typename Wide<T>::Z Z;
     const double* Bs = dc.Bp + (size_t)s * 2 * BW;
     const double* Bt = dc.Bp + (size_t)t * 2 * BW;
@@ -175,10 +367,180 @@ __device__ __forceinline__ void coupled_group(const DevConst& dc, const T* W, in
     }
     const double b0 = Bs[lane], b1 = Bs[BW + lane];
     X[0] = b0 * u0; X[1] = b0 * u1; X[2] = b1 * u0; X[3] = b1 * u1;
+}
+
+// The whole block product in every lane of the group.
+template <class T, int BW>
+__device__ __forceinline__ void coupled_group(const DevConst& dc, const T* W, int s, int t, int lane,
+                                              typename Wide<T>::Z (&X)[4]) {
+    coupled_row<T, BW>(dc, W, s, t, lane, X);
 #pragma unroll
     for (int o = BW / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k) X[k] = X[k] + shfl_xor_(X[k], o);
+}
+
+// Pair p's part of <c_2s c_2s+1 c_2t c_2t+1> on link (s, t), from the blocks
+// (s, s), (t, t) (entries 0 1) and (s, t): per pair, Wick's theorem gives
+// Pf(-i G4) = -Pf(G4) with G4 the physical covariance A + B W B^T on those four
+// Majoranas ((t, s) = -(s, t)^T), and the pairs combine with lambda_n^* lambda_m
+// N_nm / N(G) as for the bilinears.  Lane 0: (n, m) with E / 2, lane 1: (m, n)
+// with conj(E) / 2 and the conjugate blocks; a diagonal pair once with E.  A
+// self-link (s = t) gives c_2s c_2s+1 c_2s c_2s+1 = -1.
+GGF_HD void four_point_term(const DevConst& dc, int p, int lane, int s, int t, cxd g01, cxd g23, const cxd (&x)[4],
+                            cxd Np, cxd& acc, cxd* q) {
+    const bool cplx = p >= dc.K, ord = lane == 1;
+    const double As = dc.Ap[(size_t)s * 4 + 1], At = dc.Ap[(size_t)t * 4 + 1];
+    const cxd E = dc.w[p] * Np;
+    int n, m;
+    pair_nm(dc.K, p, n, m);
+    auto cj = [&](cxd v) { return ord ? conjg(v) : v; };
+    const cxd pf = (cj(g01) + cxd{As, 0.0}) * (cj(g23) + cxd{At, 0.0}) - cj(x[0]) * cj(x[3]) + cj(x[1]) * cj(x[2]);
+    const cxd v = s == t ? cxd{1.0, 0.0} : pf;
+    if (lane == 0 || (ord && cplx)) {
+        const cxd N1 = cj(Np);
+        acc -= ((cplx ? 0.5 : 1.0) * cj(E)) * v;
+        if (q) q[ord ? m * dc.K + n : n * dc.K + m] = -1.0 * (N1 * v);
+    }
+}
+
+// ---- gauge-invariant link terms ------------------------------------------------
+// A physical bilinear across link l = (s -> t) is gauge invariant together with
+// the link operator u_l (Z2: g_l; U(1): e^{i theta_l}, diagonal in G) when it
+// carries the charge u_l removes: T_l = u_l F_s F_t with F_s = psi_s (q_s > 0)
+// or psi_s^dag (q_s < 0) and F_t = psi_t^dag (q_t > 0) or psi_t (q_t < 0); for
+// staggered charges that is the pair term, and T_l + T_l^dag the link's hopping
+// term.  With psi = (c_0 + i c_1) / 2 and the link block X[alpha][beta] =
+// <c_{2s+alpha} c_{2t+beta}> (entries `stride` apart),
+//   T_l = u_l (1/4) (X00 + i e_t X01 + i e_s X10 - e_s e_t X11),
+// e = +1 for psi, -1 for psi^dag.
+GGF_HD cxd link_term(const cxd* X, size_t stride, int e_s, int e_t, cxd u) {
+    const cxd v = X[0] + cxd{0.0, (double)e_t} * X[stride] + cxd{0.0, (double)e_s} * X[2 * stride] +
+                  (-(double)(e_s * e_t)) * X[3 * stride];
+    return u * (0.25 * v);
+}
+
+// Chain c, link l: T_l from the combined link block blk [n][n_links][2][2]
+// into out[c][l], and from the per-pair blocks pair_blk
+// [n][n_links][2][2][K][K] into pair_out[c][l][n][m] (either pair of pointers
+// may be null); q [V] the sites' physical charges.
+GGF_HD void link_term_item(const DevConst& dc, int c, int l, const void* links, const int* q, const cxd* blk,
+                           const cxd* pair_blk, cxd* out, cxd* pair_out) {
+    const Geometry& g = dc.g;
+    int a0, b0;
+    link_ends(g, l, a0, b0);
+    const int s = a0 / g.B, t = b0 / g.B;
+    const int e_s = q[s] > 0 ? 1 : -1, e_t = q[t] > 0 ? -1 : 1;
+    const size_t cl = (size_t)c * g.n_links + l;
+    cxd u;
+    if (g.group == GGF_Z2) {
+        u = cxd{(double)((const int8_t*)links)[cl], 0.0};
+    } else {
+        const double th = ((const double*)links)[cl];
+        u = cxd{cos(th), sin(th)};
+    }
+    if (blk && out) out[cl] = link_term(blk + cl * 4, 1, e_s, e_t, u);
+    if (pair_blk && pair_out) {
+        const int KK = dc.K * dc.K;
+        for (int nm = 0; nm < KK; ++nm)
+            pair_out[cl * KK + nm] = link_term(pair_blk + cl * 4 * KK + nm, (size_t)KK, e_s, e_t, u);
+    }
+}
+
+// ---- score of the site blocks ------------------------------------------------
+// d log N(G) / d D_s[i][j] of chain c and site s (entries treated as
+// independent).  For pure site states N_nm(G) = const Pf(D + O Gamma_X O^T) and
+// d log Pf(M) = (1/2) tr(M^{-1} dM), so the score is Re sum_p w_p (N_p / N(G))
+// (1/2) W_p[s, s]^T (the (m, n) order of a pair n < m is the conjugate term,
+// hence the real part): entry (i, j) from W_p[s B + j][s B + i].
+template <class RW, class CW, int B>
+GGF_HD double score_entry(const DevConst& dc, int c, int s, int i, int j, const RW* Wr, const CW* Wc, const cxd* np) {
+    const Geometry& g = dc.g;
+    const int K = dc.K;
+    const size_t NN = (size_t)g.N * g.N, off = (size_t)(s * B + j) * g.N + (size_t)s * B + i;
+    double acc = 0.0;
+    for (int p = 0; p < dc.P; ++p) {
+        const cxd E = dc.w[p] * np[p];
+        if (p < K) {
+            acc = fma(0.5 * E.x, widen(Wr[((size_t)c * K + p) * NN + off]), acc);
+        } else {
+            const cxd w = widen(Wc[((size_t)c * dc.Kc + (p - K)) * NN + off]);
+            acc = fma(0.5 * E.x, w.x, acc);
+            acc = fma(-0.5 * E.y, w.y, acc);
+        }
+    }
+    return acc;
+}
+
+// ---- score of the link blocks ------------------------------------------------
+// Pair p, link l of chain c: out[c][p][l] (R x R complex, R = r) =
+// (w_p N_p / N(G)) (1/2) (O_l^T W_p[l, l] O_l)^T with W_p[l, l] the block of the
+// pair's inverse on the link's Majoranas and O_l the link's twist, so that
+// d log N(G) = Re sum_p sum_l tr(U_p[l]^T dGamma_X^p[l]) + the pair constants'
+// terms (none for K = 1, where this is the gradient for the bond blocks).  One
+// warp per (chain, pair, link), in phases.
+
+// Phase 1: the source end's rotation, rows O[x][a] (H x H).
+template <int H>
+GGF_HD void link_score_twist(const DevConst& dc, const void* links, int c, int l, int lane, double* O) {
+    const Geometry& g = dc.g;
+    if (g.group == GGF_SU2) {
+        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), O);
+    } else if (lane < H) {
+        double gval, theta, cs = 1.0, sn = 0.0;
+        link_value<double>(dc, links, c, l, gval, theta);
+        if (g.group == GGF_U1) sincos(g.q[lane >> 1] * theta, &sn, &cs);
+        int i0, i1;
+        double c0, c1;
+        twist_row(g, lane, gval, cs, sn, i0, c0, i1, c1);
+        for (int a = 0; a < H; ++a) O[lane * H + a] = 0.0;
+        O[lane * H + i0] = c0;
+        if (i1 != i0) O[lane * H + i1] = c1;
+    }
+}
+
+// Phase 2: the block of W.
+template <class T, int R>
+GGF_HD void link_score_load(const DevConst& dc, const T* W, int l, int lane, cxd* w) {
+    int a0, b0;
+    link_ends(dc.g, l, a0, b0);
+    for (int e = lane; e < R * R; e += 32)
+        w[e] = as_cx(widen(W[(size_t)link_majorana(dc.g, a0, b0, e / R) * dc.g.N + link_majorana(dc.g, a0, b0, e % R)]));
+}
+
+// Phase 3: W O (the twist mixes the source-end columns only), kept by the lanes.
+template <int R> struct LinkScoreRow { cxd t[(R * (R / 2) + 31) / 32]; };
+template <int R>
+GGF_HD void link_score_mix(const double* O, const cxd* w, int lane, LinkScoreRow<R>& m) {
+    constexpr int H = R / 2;
+    int k = 0;
+    for (int e = lane; e < R * H; e += 32, ++k) {
+        m.t[k] = cxd{0.0, 0.0};
+        for (int b = 0; b < H; ++b) axpy(m.t[k], O[b * H + e % H], w[(e / H) * R + b]);
+    }
+}
+
+// Phase 4: back into the block.
+template <int R>
+GGF_HD void link_score_put(int lane, const LinkScoreRow<R>& m, cxd* w) {
+    constexpr int H = R / 2;
+    int k = 0;
+    for (int e = lane; e < R * H; e += 32, ++k) w[(e / H) * R + e % H] = m.t[k];
+}
+
+// Phase 5: out[x][y] = f (O^T W O)[y][x].
+template <int R>
+GGF_HD void link_score_out(const double* O, const cxd* w, cxd f, int lane, cxd* o) {
+    constexpr int H = R / 2;
+    for (int e = lane; e < R * R; e += 32) {
+        const int x = e / R, y = e % R;
+        cxd v = w[y * R + x];
+        if (y < H) {
+            v = cxd{0.0, 0.0};
+            for (int a = 0; a < H; ++a) axpy(v, O[a * H + y], w[a * R + x]);
+        }
+        o[e] = f * v;
+    }
 }
 
 }  // namespace

@@ -58,15 +58,7 @@ __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_pe
     const int l = min(want, g.n_links - 1);            // idle groups repeat the last link and write nothing
     const bool live = want < g.n_links;
     ElectricShared<H>& sh = shared[grp];
-    double gval = 1.0;
-    if (g.group == GGF_SU2) {
-        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), sh.tw);
-    } else if (g.group == GGF_U1) {
-        const double th = ((const double*)links)[(size_t)c * g.n_links + l];
-        if (lane < g.n_v) sincos(g.q[lane] * th, &sh.tw[2 * lane + 1], &sh.tw[2 * lane]);
-    } else {
-        gval = (double)((const int8_t*)links)[(size_t)c * g.n_links + l];
-    }
+    const double gval = electric_twist<H>(g, links, c, l, lane, sh);
     chain_weights(dc, ell + (size_t)c * dc.P, np);
     const int K = dc.K;
     const size_t NN = (size_t)g.N * g.N;
@@ -76,17 +68,7 @@ __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_pe
         const bool cplx = p >= K;
         const cxd v = cplx ? electric_pair<CW, H, FIELD>(dc, p - K, l, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, lane, gval, sh)
                            : electric_pair<RW, H, FIELD>(dc, p, l, Wr + ((size_t)c * K + p) * NN, lane, gval, sh);
-        // w_p = 2 lambda_n^* lambda_m: the (n, m) term (lane 0) takes E / 2, the
-        // (m, n) term (lane 1) its conjugate; a diagonal pair E once
-        const cxd Np = np[p], E = dc.w[p] * Np;
-        if (lane == 0) num += (cplx ? 0.5 : 1.0) * (E * v);
-        else if (lane == 1 && cplx) num += 0.5 * (conjg(E) * v);
-        if (po && live) {
-            int n, m;
-            pair_nm(K, p, n, m);
-            if (lane == 0) po[n * K + m] = Np * v;
-            else if (lane == 1 && cplx) po[m * K + n] = conjg(Np) * v;
-        }
+        electric_term(dc, p, lane, live, np[p], v, num, po);
     }
     num = num + shfl_xor_(num, 1);
     if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = num;

@@ -41,53 +41,29 @@ __global__ void __launch_bounds__(OT) fermion_kernel(DevConst dc, int blocks_per
     const bool live = want < items;
     const int it = it0 + min(want, items - 1);
     chain_weights(dc, ell + (size_t)c * dc.P, np);
-    const bool is_site = it < g.V;
-    int s = it, t = it;
-    if (!is_site) {
-        int a0, b0;
-        link_ends(g, it - g.V, a0, b0);
-        s = a0 / g.B;
-        t = b0 / g.B;
-    }
-    cxd* out = is_site ? site_out : link_out;
-    cxd* pout = is_site ? pair_site : pair_link;
-    if (pout) pout += is_site ? ((size_t)c * g.V + s) * K * K : ((size_t)c * g.n_links + (it - g.V)) * 4 * K * K;
-    // lanes 0 .. 3 of the group each keep one entry (alpha, beta)
-    const int a = (lane >> 1) & 1, b = lane & 1;
-    const bool entry = live && lane < 4 && (!is_site || lane == 1);
+    // (lanes 0 .. 3 of the group each keep one entry)
+    const FermionLane f = fermion_lane(g, K, c, it, lane);
+    cxd* out = f.is_site ? site_out : link_out;
+    cxd* pout = f.is_site ? pair_site : pair_link;
+    cxd* q = pout && live && f.entry ? pout + f.pair : nullptr;
     const size_t NN = (size_t)g.N * g.N;
     cxd acc = {0.0, 0.0};
     for (int p = 0; p < dc.P; ++p) {
-        const cxd Np = np[p], E = dc.w[p] * Np;
-        int n, m;
-        pair_nm(K, p, n, m);
-        cxd* q = pout ? pout + (is_site ? 0 : (size_t)(a * 2 + b) * K * K) : nullptr;
+        cxd x;
         if (p >= K) {
             cxd X[4];
-            coupled_group<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, s, t, lane, X);
-            const cxd x = a ? (b ? X[3] : X[2]) : (b ? X[1] : X[0]);
-            // (n, m) with weight E / 2 (w_p = 2 lambda_n^* lambda_m), (m, n) with
-            // conj(E) / 2 and the conjugate product; A is added after the loop
-            const cxd h = 0.5 * E;
-            acc += h * x + conjg(h) * conjg(x);
-            if (q && entry) {
-                q[n * K + m] = Np * pair_bilinear(dc, s, t, a, b, x);
-                q[m * K + n] = conjg(Np) * pair_bilinear(dc, s, t, a, b, conjg(x));
-            }
+            coupled_group<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, f.s, f.t, lane, X);
+            x = f.a ? (f.b ? X[3] : X[2]) : (f.b ? X[1] : X[0]);
         } else {
             double X[4];
-            coupled_group<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, s, t, lane, X);
-            const cxd x = {a ? (b ? X[3] : X[2]) : (b ? X[1] : X[0]), 0.0};
-            acc += E * x;
-            if (q && entry) q[n * K + n] = Np * pair_bilinear(dc, s, t, a, b, x);
+            coupled_group<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, f.s, f.t, lane, X);
+            x = {f.a ? (f.b ? X[3] : X[2]) : (f.b ? X[1] : X[0]), 0.0};
         }
+        fermion_term(dc, f, p, np[p], x, acc, q);
     }
-    if (!out || !entry) return;
     // -i (A + sum_p weight_p X_p); A enters with the total weight
     // sum_nm lambda_n^* lambda_m N_nm / N(G) = 1 (only where s == t)
-    const cxd F = pair_bilinear(dc, s, t, a, b, acc);
-    if (is_site) out[(size_t)c * g.V + s] = F;
-    else out[((size_t)c * g.n_links + (it - g.V)) * 4 + lane] = F;
+    if (out && live && f.entry) out[f.out] = pair_bilinear(dc, f.s, f.t, f.a, f.b, acc);
 }
 
 // A group of BW lanes per (chain, link).
@@ -107,13 +83,9 @@ __global__ void __launch_bounds__(OT) fermion4_kernel(DevConst dc, int blocks_pe
     const int s = a0 / g.B, t = b0 / g.B;
     cxd* q = pair_out ? pair_out + ((size_t)c * g.n_links + l) * K * K : nullptr;
     const size_t NN = (size_t)g.N * g.N;
-    const double As = dc.Ap[(size_t)s * 4 + 1], At = dc.Ap[(size_t)t * 4 + 1];
     cxd acc = {0.0, 0.0};
     for (int p = 0; p < dc.P; ++p) {
         const bool cplx = p >= K;
-        const cxd Np = np[p], E = dc.w[p] * Np;
-        int n, m;
-        pair_nm(K, p, n, m);
         cxd g01, g23, x[4];
         if (cplx) {
             const CW* W = Wc + ((size_t)c * dc.Kc + (p - K)) * NN;
@@ -134,18 +106,7 @@ __global__ void __launch_bounds__(OT) fermion4_kernel(DevConst dc, int blocks_pe
 #pragma unroll
             for (int k = 0; k < 4; ++k) x[k] = {xr[k], 0.0};
         }
-        // lane 0: (n, m) with E / 2, lane 1: (m, n) with conj(E) / 2 and the
-        // conjugate blocks; a diagonal pair once with E
-        const bool ord = lane == 1;
-        auto cj = [&](cxd v) { return ord ? conjg(v) : v; };
-        const cxd pf = (cj(g01) + cxd{As, 0.0}) * (cj(g23) + cxd{At, 0.0}) - cj(x[0]) * cj(x[3]) + cj(x[1]) * cj(x[2]);
-        // a self-link (s = t): c_2s c_2s+1 c_2s c_2s+1 = -1
-        const cxd v = s == t ? cxd{1.0, 0.0} : pf;
-        if (lane == 0 || (ord && cplx)) {
-            const cxd N1 = cj(Np);
-            acc -= ((cplx ? 0.5 : 1.0) * cj(E)) * v;
-            if (q && live) q[ord ? m * K + n : n * K + m] = -1.0 * (N1 * v);
-        }
+        four_point_term(dc, p, lane, s, t, g01, g23, x, np[p], acc, live ? q : nullptr);
     }
     acc = acc + shfl_xor_(acc, 1);
     if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = s == t ? cxd{-1.0, 0.0} : acc;

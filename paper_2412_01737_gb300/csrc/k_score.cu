@@ -1,5 +1,5 @@
 // Score of the site blocks: d log N(G) / d D_s for every chain and site, from
-// the chains' inverses (the per-thread item is score_item in ggf_obs.cuh).
+// the chains' inverses (score_entry in ggf_obs_group.cuh).
 // With it the gradient of a Wilson-loop energy with respect to the site
 // parameters is the covariance E_p[(W(G) - E) sum_s tr(S_s^T dD_s)].
 //
@@ -19,21 +19,9 @@ __global__ void __launch_bounds__(B * B) score_kernel(DevConst dc, const RW* Wr,
                                                       double* out) {
     __shared__ double tr[B][B + 1];
     __shared__ cxd np[36];
-    const Geometry& g = dc.g;
-    const int c = blockIdx.x / g.V, s = blockIdx.x % g.V, j = threadIdx.x / B, i = threadIdx.x % B, K = dc.K;
+    const int c = blockIdx.x / dc.g.V, s = blockIdx.x % dc.g.V, j = threadIdx.x / B, i = threadIdx.x % B;
     chain_weights(dc, ell + (size_t)c * dc.P, np);
-    const size_t NN = (size_t)g.N * g.N, off = (size_t)(s * B + j) * g.N + (size_t)s * B + i;
-    double acc = 0.0;
-    for (int p = 0; p < dc.P; ++p) {
-        const cxd E = dc.w[p] * np[p];
-        if (p < K) {
-            acc = fma(0.5 * E.x, widen(Wr[((size_t)c * K + p) * NN + off]), acc);
-        } else {
-            const cxd w = widen(Wc[((size_t)c * dc.Kc + (p - K)) * NN + off]);
-            acc = fma(0.5 * E.x, w.x, acc);
-            acc = fma(-0.5 * E.y, w.y, acc);
-        }
-    }
+    const double acc = score_entry<RW, CW, B>(dc, c, s, i, j, Wr, Wc, np);
     tr[i][j] = acc;
     __syncthreads();
     out[(size_t)blockIdx.x * B * B + threadIdx.x] = tr[threadIdx.x / B][threadIdx.x % B];
@@ -43,35 +31,15 @@ __global__ void __launch_bounds__(B * B) score_kernel(DevConst dc, const RW* Wr,
 template <class T, int R>
 __device__ __forceinline__ void link_score_warp(const DevConst& dc, const T* W, int l, cxd f, const double* O, cxd* w,
                                                 cxd* o) {
-    constexpr int H = R / 2;
-    const Geometry& g = dc.g;
     const int lane = threadIdx.x & 31;
-    int a0, b0;
-    link_ends(g, l, a0, b0);
-    for (int e = lane; e < R * R; e += 32)
-        w[e] = as_cx(widen(W[(size_t)link_majorana(g, a0, b0, e / R) * g.N + link_majorana(g, a0, b0, e % R)]));
+    LinkScoreRow<R> m;
+    link_score_load<T, R>(dc, W, l, lane, w);
     __syncwarp();
-    // W O: the twist mixes the source-end columns only
-    cxd t[(R * H + 31) / 32];
-    int k = 0;
-    for (int e = lane; e < R * H; e += 32, ++k) {
-        t[k] = cxd{0.0, 0.0};
-        for (int b = 0; b < H; ++b) axpy(t[k], O[b * H + e % H], w[(e / H) * R + b]);
-    }
+    link_score_mix<R>(O, w, lane, m);
     __syncwarp();
-    k = 0;
-    for (int e = lane; e < R * H; e += 32, ++k) w[(e / H) * R + e % H] = t[k];
+    link_score_put<R>(lane, m, w);
     __syncwarp();
-    // out[x][y] = f (O^T W O)[y][x]
-    for (int e = lane; e < R * R; e += 32) {
-        const int x = e / R, y = e % R;
-        cxd v = w[y * R + x];
-        if (y < H) {
-            v = cxd{0.0, 0.0};
-            for (int a = 0; a < H; ++a) axpy(v, O[a * H + y], w[a * R + x]);
-        }
-        o[e] = f * v;
-    }
+    link_score_out<R>(O, w, f, lane, o);
 }
 
 template <class RW, class CW, int R>
@@ -86,20 +54,7 @@ __global__ void __launch_bounds__(OT) link_score_kernel(DevConst dc, int blocks_
     chain_weights(dc, ell + (size_t)c * dc.P, np);
     if (item >= dc.P * g.n_links) return;
     const int p = item / g.n_links, l = item % g.n_links;
-    // the source end's rotation, rows O[x][a]
-    if (g.group == GGF_SU2) {
-        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), Os[warp]);
-    } else if (lane < H) {
-        double gval, theta, cs = 1.0, sn = 0.0;
-        link_value<double>(dc, links, c, l, gval, theta);
-        if (g.group == GGF_U1) sincos(g.q[lane >> 1] * theta, &sn, &cs);
-        int i0, i1;
-        double c0, c1;
-        twist_row(g, lane, gval, cs, sn, i0, c0, i1, c1);
-        for (int a = 0; a < H; ++a) Os[warp][lane * H + a] = 0.0;
-        Os[warp][lane * H + i0] = c0;
-        if (i1 != i0) Os[warp][lane * H + i1] = c1;
-    }
+    link_score_twist<H>(dc, links, c, l, lane, Os[warp]);
     __syncwarp();
     const size_t NN = (size_t)g.N * g.N;
     const cxd f = 0.5 * (dc.w[p] * np[p]);
