@@ -1,6 +1,6 @@
 // Warp-level helpers and per-link pieces of a Metropolis link step, shared by
 // the one-link-per-launch kernels (k_sample.cu) and the batched link steps
-// on the small matrix W[T, T] (k_batch.cu).
+// on the small matrix W[T, T] (k_steps.cu).
 #pragma once
 #include <algorithm>
 #include "ggf_ctx.h"
@@ -234,9 +234,6 @@ __device__ __forceinline__ bool warp_solve(T* A, int r, T* fcol) {
     }
     return true;
 }
-
-template <class T>
-__device__ __forceinline__ cxd loadc(const T* p) { return Sc<T>::to(*p); }
 
 // Pending-update panels of one (chain, pair): U (N x KRM) followed by V^T
 // (N x KRM), K-major (row index first, rank index contiguous); complex

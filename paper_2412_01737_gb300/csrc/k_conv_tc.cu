@@ -8,8 +8,8 @@
 //                D[s][c] (K = taps x output channels), TF32 operands
 //                (kind::tf32: dY is FP32, rounded to TF32 once);
 //   weight grad  dW[o][c][t] = sum_{b, s} X[b][c][nb_t(s)] dY[b][o][s]
-//                D[(t, c)][o] (K = pixels of the CTA's samples), TF32,
-//                partial sums of the CTAs added atomically.
+//                D[(t, c)][o] (K = pixels of the CTA's bands), TF32, a plane
+//                of partial sums per CTA, added up in a fixed order.
 // nb_t(s) is pixel s shifted by tap t = 3 ky + kx, (ky - 1, kx - 1), on the
 // torus; nb'_t(s) the opposite shift (the output pixel whose tap t read s).
 //
@@ -27,7 +27,7 @@
 // far above the MMAs.  Per layer 64 -> 64 at 16 x 16 and 128 samples, against
 // gathering at the step of use, integer divisions per element and weights
 // gathered by every CTA: forward 56 -> 40 us, input gradient 106 -> 61, weight
-// gradient 221 -> 94.
+// gradient 221 -> 96 with the sum of its planes.
 #include <cuda_bf16.h>
 #include "ggf_ctx.h"
 #include "ggf_tc.cuh"

@@ -200,7 +200,8 @@ size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 // Plans a batch of at most `items` matrices: their number (at least one), the
 // workspace they need, and whether their pre-split operands go into the
 // chains' flush scratch (idle outside a sweep) or into the workspace.  A batch
-// stays within 1 GiB and a quarter of the free memory.
+// makes the workspace no larger than 1 GiB and a quarter of the free memory
+// (one matrix is always taken); a workspace that is larger already is used whole.
 void ggf_refine_plan(ggf_ctx* ctx, bool cplx, int items, RefineBatch& b) {
     const int N = ctx->g.N;
     const Chains& ch = ctx->ch;

@@ -16,15 +16,15 @@
 // of its use.
 //
 // What bounds it: the chain of dependent FP64 steps of a proposal (a Pfaffian
-// of order 2 r, a solve of order r, the combination).  An FP64 instruction
-// holds one of the SM's four sub-units for 64 cycles, so the tasks of a
+// of order 2 r, a solve of order r, the combination).  The FP64 unit takes two
+// lanes per clock and SM, so a warp's instruction holds one of the four
+// sub-units for 64 cycles, and the tasks of a
 // proposal run on different ones: the Pfaffian on a warp, the solve on two
 // whether or not the proposal will be accepted, the log-weights one link later
 // on another.  What does not depend on the decision runs beside them: P and Q,
 // the next link's Delta, the next slices of G0.  Thousand cycles per link of a
-// complex pair of rank 128 in FP32: Pfaffian 31 - 39, barrier and decision 3,
-// update 14 - 17 (with P and Q after the decision and one row per read of the
-// left factor: 39, 3, 21 - 49).
+// complex pair of rank 128 in FP32: Pfaffian 32 - 39, solve 34 - 48, barrier and
+// decision 4, update 14 - 18 (29 on the first link).
 // Measured per batch of 16 links, against one CTA per chain that took its
 // pairs in turn with G and X in L2: 16 chains of 16 x 16 U(1), K = 4 (rank
 // 128) 8.70 -> 0.97 ms (two waves: 15 clusters of 8 fit); 96 chains of 5 x 5
@@ -267,8 +267,8 @@ template <int N, class T> __device__ __forceinline__ void load_row(T (&v)[N], co
 // this is thread t.  A thread keeps the r sums of RB rows (columns): each value
 // of X is read once per product, and the reads, which wait in the same queue
 // as the FP64 instructions of the Pfaffian beside them, are few per product
-// (one row per thread and half of the sums each took 75 instead of 37 thousand
-// cycles at rank 120).  P's rows fill whole warps before Q's columns begin.
+// (one row per thread and half of the sums each took twice as long at rank
+// 120).  P's rows fill whole warps before Q's columns begin.
 // SLICED: the slices of G0 from g0_fetch, else G0 itself.
 template <class T, int R, bool SLICED>
 __device__ __forceinline__ void pair_pq(const T* M, int ld, int jr, int KRM, const T* Gc, const T* Gr, T* Pm, T* Qm,
