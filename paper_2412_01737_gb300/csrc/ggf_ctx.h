@@ -112,6 +112,7 @@ struct ggf_ctx {
     // fronts too large for shared memory
     int* d_front = nullptr;
     int front_F = 0, front_L = -1, front_B = -1, front_sign = 1;
+    bool front_wide = false;                // a site closes more Majoranas than one panel takes
     cudaStream_t front_st = nullptr;        // the real family's items run beside the complex ones
     cudaEvent_t front_fork = nullptr, front_join = nullptr;
     void* front_ws = nullptr;

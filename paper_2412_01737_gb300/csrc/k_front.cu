@@ -63,6 +63,7 @@ namespace {
 constexpr int CHUNK = 16;          // closed Majoranas per panel
 constexpr int SMALL_FRONT = 48;    // slots up to which an item takes 64 threads
 constexpr int MAX_CLOSED = 32;     // Majoranas closed by one site (four links)
+enum { SMALL_PIVOT = 1, NO_PIVOT = 2 };
 constexpr double PIVOT_FLOOR = 1.0 / 256.0;    // smallest |pivot|^2 of a chunk, over the largest there is
 
 __host__ __device__ __forceinline__ int tri_row(int i, int F) { return i * (2 * F - i - 1) / 2 - i - 1; }
@@ -185,12 +186,14 @@ __host__ __device__ inline FrontLayout front_layout(int F, size_t elem, bool tri
 // One CTA per item (grid-stride); item = q npf + pair of configuration
 // chains[q] (or q).  Its log-weight goes to ell[q][pair_off + pair]; items
 // without a usable pivot are appended to bad[1 ..], counted in bad[0].
-template <class T, int NT>
+// WIDE: some site closes more than CHUNK Majoranas (n_v = 2); without it every
+// chunk is a whole closed set.
+template <class T, int NT, bool WIDE>
 __global__ void __launch_bounds__(NT, NT == 64 ? 8 : (sizeof(T) == 8 ? 2 : 1))
 front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains, int npf, int pair_off,
                 const void* links, cxd* ell, int* bad, T* gws, size_t tri_elems, int in_smem) {
     extern __shared__ __align__(16) unsigned char fsm[];
-    __shared__ int s_bad, s_nl, s_stop;
+    __shared__ int s_end, s_nl;        // s_end: how the chunk ended
     __shared__ T s_inv;
     __shared__ T s_scale[CHUNK];
     __shared__ int ord[CHUNK], es[CHUNK], cl[MAX_CLOSED];
@@ -208,7 +211,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
         const int q = (int)(item / npf), pair = (int)(item - (long long)q * npf);
         const int cfg = chains ? chains[q] : q;
         for (int a = tid; a < F; a += NT) idx[a] = -1;
-        if (tid == 0) s_bad = 0;
+        if (tid == 0) s_end = 0;
         __syncthreads();
         // lane 0 of warp 0: prod of the pivots as pr 2^ex
         cxd pr = {(double)fa.sign, 0.0};
@@ -231,7 +234,8 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
             }
             for (int k = tid; k < B; k += NT) idx[fa.slot[s * B + k]] = s * B + k;
             const int first = fa.eoff[s], ne = fa.eoff[s + 1] - first;
-            for (int k = tid; k < ne; k += NT) cl[k] = fa.elim[first + k];
+            if constexpr (WIDE)
+                for (int k = tid; k < ne; k += NT) cl[k] = fa.elim[first + k];
             __syncthreads();
             for (int k = warp; k < B; k += NW) {
                 const int a = fa.slot[s * B + k];
@@ -251,7 +255,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
             while (e < ne) {
                 const int c = min(CHUNK, ne - e);
                 double low = PIVOT_FLOOR;      // (warp 0) |pivot|^2 below which this chunk ends
-                if (search) {
+                if (WIDE && search) {
                     if (warp == 0) {
                         double best;
                         int bq;
@@ -261,8 +265,8 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     }
                     __syncthreads();
                 }
-                if (tid == 0) s_stop = 0;
-                if (tid < c) { es[tid] = cl[e + tid]; ord[tid] = tid; }
+                if (WIDE && tid == 0) s_end = 0;
+                if (tid < c) { es[tid] = WIDE ? cl[e + tid] : fa.elim[first + e + tid]; ord[tid] = tid; }
                 __syncthreads();
                 if (tid < c) idx[es[tid]] = -1;
                 __syncthreads();
@@ -290,10 +294,10 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                         double best;
                         int bq;
                         warp_best_pair(c - t, [&](int x, int y) { return Pn[(size_t)ord[t + x] * F + ord[t + y]]; }, best, bq);
-                        if (e + c < ne && best < low && !(search && t == 0)) {
-                            if (lane == 0) s_stop = 1;           // better ones may lie outside the chunk
+                        if (WIDE && e + c < ne && best < low && !(search && t == 0)) {
+                            if (lane == 0) s_end = SMALL_PIVOT;  // better ones may lie outside the chunk
                         } else if (lane == 0) {
-                            if (!(best > 1e-16) || !isfinite(best)) s_bad = 1;   // no usable pivot: refactor densely
+                            if (!(best > 1e-16) || !isfinite(best)) s_end = NO_PIVOT;   // no usable pivot: refactor densely
                             if (pair_to_front(ord + t, bq / 32, bq % 32)) pr = -pr;
                             const int k = ord[t], p = ord[t + 1];
                             const T akp = Pn[(size_t)k * F + p];
@@ -309,7 +313,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                         }
                     }
                     __syncthreads();
-                    if (s_bad || s_stop) break;
+                    if (s_end) break;
                     // the remaining rows of the chunk: R += (v_R / a) k - (k_R / a) v
                     const T* rk = Pn + (size_t)ord[t] * F;
                     const T* rp = Pn + (size_t)ord[t + 1] * F;
@@ -326,23 +330,25 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     }
                     __syncthreads();
                 }
-                if (s_bad) break;
-                // the rows that the chunk leaves behind, back to the front
-                for (int i = te + warp; i < c; i += NW) {
-                    const int row = ord[i], a = es[row];
-                    for (int w = i + 1 + lane; w < W; w += 32) {
-                        const int col = w < c ? ord[w] : w, b = w < c ? es[col] : lv[w - c];
-                        const T val = Pn[(size_t)row * F + col];
-                        if (a < b) S[tri_row(a, F) + b] = val;
-                        else S[tri_row(b, F) + a] = fneg(val);
-                    }
-                    if (lane == 0) {
-                        cl[e + i] = a;
-                        idx[a] = 0;        // live again (which Majorana it is matters only to later sites)
+                if (s_end == NO_PIVOT) break;
+                if constexpr (WIDE) {
+                    // the rows that the chunk leaves behind, back to the front
+                    for (int i = te + warp; i < c; i += NW) {
+                        const int row = ord[i], a = es[row];
+                        for (int w = i + 1 + lane; w < W; w += 32) {
+                            const int col = w < c ? ord[w] : w, b = w < c ? es[col] : lv[w - c];
+                            const T val = Pn[(size_t)row * F + col];
+                            if (a < b) S[tri_row(a, F) + b] = val;
+                            else S[tri_row(b, F) + a] = fneg(val);
+                        }
+                        if (lane == 0) {
+                            cl[e + i] = a;
+                            idx[a] = 0;        // live again (which Majorana it is matters only to later sites)
+                        }
                     }
                 }
                 // u_t = row k_t / a_t over the live columns
-                for (int t = 2 * warp; t < te; t += 2 * NW) {
+                for (int t = 2 * warp; t < (WIDE ? te : c); t += 2 * NW) {
                     T* r = Pn + (size_t)ord[t] * F + c;
                     const T inv = s_scale[t];
                     for (int w = lane; w < nl; w += 32) r[w] = fmul(r[w], inv);
@@ -362,7 +368,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     const bool diag = i == j;
                     T a00 = diag ? Sc<T>::zero() : S0[c0], a01 = S0[c1];
                     T a10 = diag ? Sc<T>::zero() : S1[c0], a11 = diag ? Sc<T>::zero() : S1[c1];
-                    for (int t = 0; t < te; t += 2) {
+                    for (int t = 0; t < (WIDE ? te : c); t += 2) {
                         const T* u = Pn + (size_t)ord[t] * F + c;
                         const T* v = Pn + (size_t)ord[t + 1] * F + c;
                         const T ui0 = u[i], ui1 = u[i + 1], vi0 = v[i], vi1 = v[i + 1];
@@ -377,13 +383,13 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                 }
                 __syncthreads();
                 search = te < c;
-                e += te;
+                e += WIDE ? te : c;
             }
-            if (s_bad) break;
+            if (s_end == NO_PIVOT) break;
         }
         if (tid == 0) {
             cxd* dst = ell + (size_t)q * dc.P + pair_off + pair;
-            if (s_bad) {
+            if (s_end == NO_PIVOT) {
                 *dst = {NAN, 0.0};
                 bad[1 + atomicAdd(bad, 1)] = (int)((long long)q * dc.P + pair_off + pair);
             } else {
@@ -462,7 +468,8 @@ const size_t kSmemMax = 227 * 1024 - 1024;
 
 template <class T, int NT>
 ggf_status raise_cap(ggf_ctx* ctx) {
-    GGF_CK(cudaFuncSetAttribute(front_pf_kernel<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    GGF_CK(cudaFuncSetAttribute(front_pf_kernel<T, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    GGF_CK(cudaFuncSetAttribute(front_pf_kernel<T, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     return GGF_OK;
 }
 
@@ -477,8 +484,9 @@ ggf_status ggf_front_prepare(ggf_ctx* ctx) {
     std::vector<int> slot, eoff, elim;
     build_schedule(g, F, slot, eoff, elim, sign);
     if ((int)elim.size() != g.N) return ggf_fail(ctx, GGF_ESTATE, "front schedule does not close every Majorana");
-    for (int s = 0; s < g.V; ++s)
-        if (eoff[s + 1] - eoff[s] > MAX_CLOSED) return ggf_fail(ctx, GGF_ESTATE, "front schedule closes too many Majoranas");
+    int closed = 0;
+    for (int s = 0; s < g.V; ++s) closed = std::max(closed, eoff[s + 1] - eoff[s]);
+    if (closed > MAX_CLOSED) return ggf_fail(ctx, GGF_ESTATE, "front schedule closes too many Majoranas");
     std::vector<int> all;
     all.insert(all.end(), slot.begin(), slot.end());
     all.insert(all.end(), eoff.begin(), eoff.end());
@@ -491,6 +499,7 @@ ggf_status ggf_front_prepare(ggf_ctx* ctx) {
         GGF_CK(cudaEventCreateWithFlags(&ctx->front_join, cudaEventDisableTiming));
     }
     ctx->front_F = F;
+    ctx->front_wide = closed > CHUNK;
     ctx->front_sign = sign;
     ctx->front_L = g.L;
     ctx->front_B = g.B;
@@ -564,19 +573,28 @@ ggf_status ggf_front_pfaffian(ggf_ctx* ctx, int n, const int* d_chains, const vo
         GGF_CK(cudaStreamWaitEvent(ctx->front_st, ctx->front_fork, 0));
     }
     const bool small = F <= SMALL_FRONT;
-#define GGF_FRONT(T, NT, f, npf, off_p, stream)                                                                  \
-    front_pf_kernel<T, NT><<<grid[f], NT, front_layout(F, sizeof(T), in_smem[f]).total, stream>>>(                \
+#define GGF_FRONT(T, NT, W, f, npf, off_p, stream)                                                               \
+    front_pf_kernel<T, NT, W><<<grid[f], NT, front_layout(F, sizeof(T), in_smem[f]).total, stream>>>(                \
         ctx->dc(), fa, (long long)n * (npf), d_chains, npf, off_p, d_links, d_ell, d_bad,                         \
         (T*)((unsigned char*)ctx->front_ws + off[f]), tri, in_smem[f] ? 1 : 0)
+#define GGF_FRONTS(T, f, npf, off_p, stream)                                                                      \
+    do {                                                                                                          \
+        if (ctx->front_wide) {                                                                                    \
+            if (small) GGF_FRONT(T, 64, true, f, npf, off_p, stream);                                             \
+            else GGF_FRONT(T, 256, true, f, npf, off_p, stream);                                                  \
+        } else {                                                                                                  \
+            if (small) GGF_FRONT(T, 64, false, f, npf, off_p, stream);                                            \
+            else GGF_FRONT(T, 256, false, f, npf, off_p, stream);                                                 \
+        }                                                                                                         \
+    } while (0)
     if (both) {      // the complex items, four times as long, are placed first
-        if (small) GGF_FRONT(cxd, 64, 1, ctx->Kc, ctx->K, st);
-        else GGF_FRONT(cxd, 256, 1, ctx->Kc, ctx->K, st);
+        GGF_FRONTS(cxd, 1, ctx->Kc, ctx->K, st);
         GGF_CK(cudaGetLastError());
     }
     cudaStream_t rs = both ? ctx->front_st : st;
-    if (small) GGF_FRONT(double, 64, 0, ctx->K, 0, rs);
-    else GGF_FRONT(double, 256, 0, ctx->K, 0, rs);
+    GGF_FRONTS(double, 0, ctx->K, 0, rs);
     GGF_CK(cudaGetLastError());
+#undef GGF_FRONTS
 #undef GGF_FRONT
     ctx->launches += both ? 2 : 1;
     if (both) {
