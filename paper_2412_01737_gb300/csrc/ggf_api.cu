@@ -720,7 +720,8 @@ ggf_status ggf_chains_init(ggf_ctx* ctx, int n_chains, const void* links, const 
     GGF_CK(cudaMalloc(&ch.links, lb));
     GGF_CK(cudaMalloc(&ch.Wr, std::max<size_t>(16, (size_t)n_chains * ctx->K * NN * rsz)));
     GGF_CK(cudaMalloc(&ch.Wc, std::max<size_t>(16, (size_t)n_chains * ctx->Kc * NN * 2 * rsz)));
-    GGF_CK(cudaMalloc(&ch.ell, (size_t)n_chains * ctx->P * sizeof(cxd)));
+    GGF_CK(cudaMalloc(&ch.ell, (size_t)n_chains * 3 * ctx->P * sizeof(cxd)));
+    ch.obs_w = ch.ell + (size_t)n_chains * ctx->P;
     GGF_CK(cudaMalloc(&ch.zbuf, (size_t)n_chains * ctx->P * g.r * g.r * sizeof(cxd)));
     ch.kmax = opts->delay > 1 ? opts->delay : 1;
     if (ch.kmax > 64) return ggf_fail(ctx, GGF_EINVAL, "delay must be <= 64");

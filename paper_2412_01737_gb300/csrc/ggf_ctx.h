@@ -38,6 +38,7 @@ struct Chains {
     void* Wr = nullptr;           // [n][K][N][N]   double or float
     void* Wc = nullptr;           // [n][Kc][N][N]  cxd or cxf
     cxd* ell = nullptr;           // [n][P]
+    cxd* obs_w = nullptr;         // [n][2][P] pair weights of one observable call (behind ell)
     void* zbuf = nullptr;         // [n][P][r][r]  W-precision scalars (complex slot size)
     void* ybuf = nullptr;         // [n][P][r][N]
     int* accept = nullptr;        // [n]
@@ -223,6 +224,9 @@ ggf_status ggf_invert_batched(ggf_ctx* ctx, bool cplx, int n, int batch, void* A
 ggf_status ggf_front_pfaffian(ggf_ctx* ctx, int n, const int* d_chains, const void* d_links, cxd* d_ell, int* d_bad,
                               cudaStream_t st);
 void ggf_front_free(ggf_ctx* ctx);
+// Pair weights of the chains, formed ahead of an observable kernel of `blocks`
+// CTAs, or null where its CTAs form them (k_electric.cu).
+const cxd* ggf_obs_weights(ggf_ctx* ctx, long long blocks, cudaStream_t st);
 // Combine per-config pair log-Pfaffians into log N (device, n_cfg items).
 ggf_status ggf_combine(ggf_ctx* ctx, int n_cfg, const cxd* d_ell, double* d_logN, cudaStream_t st);
 ggf_status ggf_plaquette(ggf_ctx* ctx, int n_cfg, const void* d_links, double* d_out, cudaStream_t st);

@@ -9,8 +9,10 @@
 // loads, the pair weights' exponentials formed again by every thread, complex
 // arithmetic for the real pairs and both orders of a complex pair from
 // scratch.  Here a lane owns a row of the block (whole 16-byte pieces of it),
-// the weights are formed once per CTA, real pairs stay real, and the two
-// orders of a pair share their products (below).
+// the weights are formed once per CTA or, for many CTAs, once per chain, real
+// pairs stay real, and the two orders of a pair share their products (below).
+// With many chains the FP64 unit is what is left, and it takes a warp's
+// instruction at the same price whatever the number of its lanes.
 #pragma once
 #include "ggf_ctx.h"
 #include "ggf_sweep.cuh"
@@ -63,24 +65,53 @@ GGF_HD void load_run(const T* p, typename Wide<T>::Z* out) {
     }
 }
 
-// N_nm(G) / N(G) of every pair of one chain into np (shared), by warp 0.
-__device__ __forceinline__ void chain_weights(const DevConst& dc, const cxd* el, cxd* np) {
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        double amax = -INFINITY, den = 0.0;
-        for (int p = lane; p < dc.P; p += 32) amax = fmax(amax, dc.logc[p].x + el[p].x);
-        for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        for (int p = lane; p < dc.P; p += 32) {
-            cxd e = dc.logc[p] + el[p];
-            if (p < dc.K) e.y = 0.0;
-            e.x -= amax;
-            const cxd t = cexp_(e);
-            np[p] = t;
-            den += (dc.w[p] * t).x;
+// The weights of one chain's pairs: N_nm(G) / N(G), and w_p N_nm(G) / N(G).
+struct PairWeights {
+    cxd np[36], E[36];
+};
+
+// By G lanes (a power of two, P <= G or G = 32) of a warp whose lanes all call;
+// np, E: [P], in any memory; nothing is stored where live is false.
+__device__ __forceinline__ void warp_weights(const DevConst& dc, const cxd* el, int G, bool live, cxd* np, cxd* E) {
+    const int lane = (threadIdx.x & 31) & (G - 1);
+    double amax = -INFINITY, den = 0.0;
+    for (int p = lane; p < dc.P; p += G) amax = fmax(amax, dc.logc[p].x + el[p].x);
+    for (int o = G / 2; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    // (P <= 36: a lane has two pairs at most, the second one seldom)
+    auto term = [&](int p) {
+        cxd e = dc.logc[p] + el[p];
+        if (p < dc.K) e.y = 0.0;
+        e.x -= amax;
+        const cxd t = cexp_(e);
+        den += (dc.w[p] * t).x;
+        return t;
+    };
+    cxd t0 = {0.0, 0.0}, t1 = {0.0, 0.0};
+    if (lane < dc.P) t0 = term(lane);
+    if (lane + G < dc.P) t1 = term(lane + G);
+    for (int o = G / 2; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    const double iden = 1.0 / den;
+    auto put = [&](int p, cxd t) {
+        const cxd v = iden * t;
+        np[p] = v;
+        E[p] = dc.w[p] * v;
+    };
+    if (live && lane < dc.P) put(lane, t0);
+    if (live && lane + G < dc.P) put(lane + G, t1);
+}
+
+// The weights of chain c into shared memory: from `ready` [n][2][P]
+// (ggf_obs_weights), or formed by the CTA's first warp.
+__device__ __forceinline__ void chain_weights(const DevConst& dc, int c, const cxd* ell, const cxd* ready,
+                                              PairWeights& pw) {
+    if (ready) {
+        const cxd* r = ready + (size_t)c * 2 * dc.P;
+        for (int p = threadIdx.x; p < dc.P; p += blockDim.x) {
+            pw.np[p] = r[p];
+            pw.E[p] = r[dc.P + p];
         }
-        for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
-        const double iden = 1.0 / den;
-        for (int p = lane; p < dc.P; p += 32) np[p] = iden * np[p];
+    } else if (threadIdx.x < 32) {
+        warp_weights(dc, ell + (size_t)c * dc.P, 32, true, pw.np, pw.E);
     }
     __syncthreads();
 }
@@ -112,8 +143,7 @@ GGF_HD cxd insertion(const Geometry& g, const cxd (&G)[H][H]) {
         return val;
     }
     if (g.group == GGF_Z2) {
-        const double sg = (H / 2) % 2 ? -1.0 : 1.0;    // (-1)^{n_v}
-        return sg * small_pf<H>(G);
+        return (H / 2) % 2 ? -small_pf<H>(G) : small_pf<H>(G);    // (-1)^{n_v}
     }
     if constexpr (H == 4) {
         if (g.group == GGF_SU2) {
@@ -175,9 +205,12 @@ GGF_HD void electric_load(const DevConst& dc, int pf, int l, int a0, int b0, con
     constexpr int R = 2 * H, B = 4 * H;
     const Geometry& g = dc.g;
     Z* gt = (Z*)sh.gt;
-    for (int e = lane; e < R * H; e += B)
-        gt[e] = g.group == GGF_SU2 ? twisted_su2<Z>(dc, pf, l, e / H, e % H, sh.tw)
-                                   : twisted_tab<Z>(dc, pf, l, e / H, e % H, gval, sh.tw);
+    for (int e = lane; e < R * H; e += B) {
+        const int j = e / H, b = e % H;
+        if (g.group == GGF_Z2) gt[e] = mulc((j < H ? gval : 1.0) * gval, bond_elem<Z>(dc, pf, l, j, b));
+        else if (g.group == GGF_SU2) gt[e] = twisted_su2<Z>(dc, pf, l, j, b, sh.tw);
+        else gt[e] = twisted_tab<Z>(dc, pf, l, j, b, gval, sh.tw);
+    }
     const T* row = W + (size_t)((l >> 1) * B + lane) * g.N;
     load_run<H>(row + a0, w);
     load_run<H>(row + b0, w + H);
@@ -200,55 +233,75 @@ GGF_HD void electric_rows(int lane, const typename Wide<T>::Z (&w)[2 * H], Elect
     }
 }
 
-// Phase 3: an entry of U and V per lane.
+// Phase 3: an entry of U and of V per lane, or of one of them where the group
+// has lanes for both (an FP64 instruction costs a warp the same whatever the
+// number of its lanes).
 template <class T, int H>
 GGF_HD void electric_products(const DevConst& dc, int l, int a0, int lane, ElectricShared<H>& sh) {
     typedef typename Wide<T>::Z Z;
-    constexpr int B = 4 * H;
-    if (lane >= H * H) return;
+    constexpr int B = 4 * H, E = H * H;
     const Z* As = (const Z*)sh.A;
     const Z* Gs = (const Z*)sh.G;
-    const int a = lane / H, b = lane % H, at = a0 - (l >> 1) * B + a;
+    const int e = lane % E, a = e / H, b = e % H, at = a0 - (l >> 1) * B + a;
     const double* Dr = dc.D + ((size_t)(l >> 1) * B + at) * B;
-    Z u = As[at * H + b], v = Gs[at * H + b];
+    if constexpr (2 * E <= B) {
+        const bool second = lane >= E;
+        const Z* other = second ? As : Gs;
+        Z s = second ? Gs[at * H + b] : As[at * H + b];
 #pragma unroll 4
-    for (int i = 0; i < B; ++i) {
-        const double d = Dr[i];
-        axpy(u, -d, Gs[i * H + b]);
-        axpy(v, d, As[i * H + b]);
+        for (int i = 0; i < B; ++i) axpy(s, second ? Dr[i] : -Dr[i], other[i * H + b]);
+        (second ? (Z*)sh.V : (Z*)sh.U)[e] = s;
+    } else {
+        Z u = As[at * H + b], v = Gs[at * H + b];
+#pragma unroll 4
+        for (int i = 0; i < B; ++i) {
+            const double d = Dr[i];
+            axpy(u, -d, Gs[i * H + b]);
+            axpy(v, d, As[i * H + b]);
+        }
+        ((Z*)sh.U)[e] = u;
+        ((Z*)sh.V)[e] = v;
     }
-    sh.U[lane] = as_cx(u);
-    sh.V[lane] = as_cx(v);
 }
 
-// Phase 4: lane 0: the (n, m) order, lane 1: (m, n).
-template <int H, bool FIELD>
+// Phase 4: lane 0: the (n, m) order, lane 1: (m, n); a diagonal pair's orders are one.
+template <class T, int H, bool FIELD>
 GGF_HD cxd electric_value(const Geometry& g, int lane, const ElectricShared<H>& sh) {
-    if (lane >= 2) return {0.0, 0.0};
-    const double sg = lane ? -1.0 : 1.0;
+    typedef typename Wide<T>::Z Z;
+    if (lane >= (Sc<Z>::CPLX ? 2 : 1)) return {0.0, 0.0};
+    const Z* U = (const Z*)sh.U;
+    const Z* V = (const Z*)sh.V;
     cxd X[H][H];
 #pragma unroll
     for (int a = 0; a < H; ++a)
 #pragma unroll
         for (int b = 0; b < H; ++b) {
-            const cxd u = sh.U[a * H + b], v = sh.V[a * H + b];
             // -(U + i V) or -conj(U - i V), plus i on the diagonal
-            X[a][b] = {-(u.x - sg * v.y), -sg * (u.y + sg * v.x)};
+            if constexpr (Sc<Z>::CPLX) {
+                const double sg = lane ? -1.0 : 1.0;
+                const cxd u = U[a * H + b], v = V[a * H + b];
+                X[a][b] = {-(u.x - sg * v.y), -sg * (u.y + sg * v.x)};
+            } else {
+                X[a][b] = {-U[a * H + b], -V[a * H + b]};
+            }
             if (a == b) X[a][b].y += 1.0;
         }
     return insertion<H, FIELD>(g, X);
 }
 
-// The lane's order of pair p (value v, norm Np) into its sum and the per-pair
+// The lane's order of pair p (value v, norm Np, weight E) into its sum and the per-pair
 // output po [K][K] (or null; not live: nothing is stored).  w_p = 2 lambda_n^* lambda_m: the (n, m) term
 // (lane 0) takes E / 2, the (m, n) term (lane 1) its conjugate; a diagonal pair
 // E once.
-GGF_HD void electric_term(const DevConst& dc, int p, int lane, bool live, cxd Np, cxd v, cxd& num, cxd* po) {
+GGF_HD void electric_term(const DevConst& dc, int p, int lane, bool live, cxd Np, cxd E, cxd v, cxd& num,
+                         cxd* po) {
     const int K = dc.K;
     const bool cplx = p >= K;
-    const cxd E = dc.w[p] * Np;
-    if (lane == 0) num += (cplx ? 0.5 : 1.0) * (E * v);
-    else if (lane == 1 && cplx) num += 0.5 * (conjg(E) * v);
+    if (!cplx) {
+        if (lane == 0) num += E * v;
+    } else if (lane < 2) {
+        num += 0.5 * ((lane ? conjg(E) : E) * v);
+    }
     if (po && live) {
         int n, m;
         pair_nm(K, p, n, m);
@@ -269,7 +322,7 @@ __device__ __forceinline__ cxd electric_pair(const DevConst& dc, int pf, int l, 
     __syncwarp();
     electric_products<T, H>(dc, l, a0, lane, sh);
     __syncwarp();
-    const cxd v = electric_value<H, FIELD>(dc.g, lane, sh);
+    const cxd v = electric_value<T, H, FIELD>(dc.g, lane, sh);
     __syncwarp();
     return v;
 }
@@ -304,8 +357,8 @@ GGF_HD cxd pair_bilinear(const DevConst& dc, int s, int t, int a, int b, cxd x) 
     return times_minus_i(x);
 }
 
-// What lane `lane` of item it of chain c keeps: entry (a, b) of the block of
-// sites (s, t), whether it is wanted, and where it goes in the combined and in
+// What lane `lane` of the BW of item it of chain c keeps: entry (a, b) of the
+// block of sites (s, t), each held by BW / 4 lanes of which the first writes, and where it goes in the combined and in
 // the per-pair outputs (items 0 .. V - 1 are sites, of which only the entry
 // (0, 1) is kept, then the links).
 struct FermionLane {
@@ -313,8 +366,10 @@ struct FermionLane {
     int s, t, a, b;
     size_t out, pair;
 };
+template <int BW>
 GGF_HD FermionLane fermion_lane(const Geometry& g, int K, int c, int it, int lane) {
     FermionLane f;
+    const int e = lane / (BW / 4);
     f.is_site = it < g.V;
     f.s = f.t = it;
     if (!f.is_site) {
@@ -323,33 +378,31 @@ GGF_HD FermionLane fermion_lane(const Geometry& g, int K, int c, int it, int lan
         f.s = a0 / g.B;
         f.t = b0 / g.B;
     }
-    f.a = (lane >> 1) & 1;
-    f.b = lane & 1;
-    f.entry = lane < 4 && (!f.is_site || lane == 1);
-    f.out = f.is_site ? (size_t)c * g.V + f.s : ((size_t)c * g.n_links + (it - g.V)) * 4 + (lane & 3);
+    f.a = e >> 1;
+    f.b = e & 1;
+    f.entry = lane % (BW / 4) == 0 && (!f.is_site || e == 1);
+    f.out = f.is_site ? (size_t)c * g.V + f.s : ((size_t)c * g.n_links + (it - g.V)) * 4 + e;
     f.pair = f.is_site ? f.out * K * K : (((size_t)c * g.n_links + (it - g.V)) * 4 + (f.a * 2 + f.b)) * K * K;
     return f;
 }
 
-// Pair p's block entry x (norm Np) into the lane's sum, and its two orders into
-// the per-pair output q [K][K] (or null).
-GGF_HD void fermion_term(const DevConst& dc, const FermionLane& f, int p, cxd Np, cxd x, cxd& acc, cxd* q) {
-    const cxd E = dc.w[p] * Np;
-    int n, m;
-    pair_nm(dc.K, p, n, m);
-    if (p >= dc.K) {
-        // (n, m) with weight E / 2 (w_p = 2 lambda_n^* lambda_m), (m, n) with
-        // conj(E) / 2 and the conjugate product; A is added after the loop
-        const cxd h = 0.5 * E;
-        acc += h * x + conjg(h) * conjg(x);
-        if (q) {
-            q[n * dc.K + m] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, x);
-            q[m * dc.K + n] = conjg(Np) * pair_bilinear(dc, f.s, f.t, f.a, f.b, conjg(x));
-        }
-    } else {
-        acc += E * x;
-        if (q) q[n * dc.K + n] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, x);
+// Pair p's block entry x (norm Np, weight E) into the lane's sum, and its two
+// orders into the per-pair output q [K][K] (or null): of a complex pair
+// (n, m) with weight E / 2 (w_p = 2 lambda_n^* lambda_m), (m, n) with conj(E) / 2
+// and the conjugate product; A is added after the loop.
+GGF_HD void fermion_term(const DevConst& dc, const FermionLane& f, int p, cxd Np, cxd E, cxd x, cxd& acc, cxd* q) {
+    const cxd h = 0.5 * E;
+    acc += h * x + conjg(h) * conjg(x);
+    if (q) {
+        int n, m;
+        pair_nm(dc.K, p, n, m);
+        q[n * dc.K + m] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, x);
+        q[m * dc.K + n] = conjg(Np) * pair_bilinear(dc, f.s, f.t, f.a, f.b, conjg(x));
     }
+}
+GGF_HD void fermion_term(const DevConst& dc, const FermionLane& f, int p, cxd Np, cxd E, double x, cxd& acc, cxd* q) {
+    axpy(acc, x, E);
+    if (q) q[p * dc.K + p] = Np * pair_bilinear(dc, f.s, f.t, f.a, f.b, cxd{x, 0.0});
 }
 
 // X[alpha][beta] = B_s W[s, t] B_t^T: row `lane` of the block's part of the sum.
@@ -369,15 +422,59 @@ GGF_HD void coupled_row(const DevConst& dc, const T* W, int s, int t, int lane, 
     X[0] = b0 * u0; X[1] = b0 * u1; X[2] = b1 * u0; X[3] = b1 * u1;
 }
 
-// The whole block product in every lane of the group.
+// Entry (0, 1) of X on a site's own block: row `lane`'s part of the sum.
 template <class T, int BW>
-__device__ __forceinline__ void coupled_group(const DevConst& dc, const T* W, int s, int t, int lane,
-                                              typename Wide<T>::Z (&X)[4]) {
+GGF_HD typename Wide<T>::Z coupled_row01(const DevConst& dc, const T* W, int s, int lane) {
+    typedef typename Wide<T>::Z Z;
+    const double* Bs = dc.Bp + (size_t)s * 2 * BW;
+    Z w[BW], u1 = Sc<Z>::zero();
+    load_run<BW>(W + (size_t)(s * BW + lane) * dc.g.N + (size_t)s * BW, w);
+#pragma unroll
+    for (int j = 0; j < BW; ++j) axpy(u1, Bs[BW + j], w[j]);
+    return Bs[lane] * u1;
+}
+
+// Sums over the group's lanes: every round halves the values a lane carries as
+// long as it has several, so that four values take 4 or 5 additions instead of
+// 12 or 16 (the additions are those of a butterfly over all lanes).
+template <class Z>
+__device__ __forceinline__ Z fold_(Z low, Z high, int lane, int o) {
+    const bool up = lane & o;
+    return (up ? high : low) + shfl_xor_(up ? low : high, o);
+}
+__device__ __forceinline__ double from_lane_(double v, int src, int width) { return __shfl_sync(0xffffffffu, v, src, width); }
+__device__ __forceinline__ cxd from_lane_(cxd v, int src, int width) {
+    return {__shfl_sync(0xffffffffu, v.x, src, width), __shfl_sync(0xffffffffu, v.y, src, width)};
+}
+
+// The block product's entry lane / (BW / 4).
+template <class T, int BW>
+__device__ __forceinline__ typename Wide<T>::Z coupled_entry(const DevConst& dc, const T* W, int s, int t, int lane) {
+    typedef typename Wide<T>::Z Z;
+    Z X[4];
     coupled_row<T, BW>(dc, W, s, t, lane, X);
+    const Z y0 = fold_(X[0], X[2], lane, BW / 2), y1 = fold_(X[1], X[3], lane, BW / 2);
+    Z x = fold_(y0, y1, lane, BW / 4);
 #pragma unroll
-    for (int o = BW / 2; o > 0; o >>= 1)
+    for (int o = BW / 8; o > 0; o >>= 1) x = x + shfl_xor_(x, o);
+    return x;
+}
+
+// What the four-point function of link (s, t) needs of a pair's inverse, in
+// every lane of the group: X of (s, t), and its entries (0, 1) of (s, s) and (t, t).
+template <class T, int BW>
+__device__ __forceinline__ void four_point_blocks(const DevConst& dc, const T* W, int s, int t, int lane,
+                                                  typename Wide<T>::Z& g01, typename Wide<T>::Z& g23,
+                                                  typename Wide<T>::Z (&x)[4]) {
+    typedef typename Wide<T>::Z Z;
+    Z own = fold_(coupled_row01<T, BW>(dc, W, s, lane), coupled_row01<T, BW>(dc, W, t, lane), lane, BW / 2);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) X[k] = X[k] + shfl_xor_(X[k], o);
+    for (int o = BW / 4; o > 0; o >>= 1) own = own + shfl_xor_(own, o);
+    const Z e = coupled_entry<T, BW>(dc, W, s, t, lane);
+    g01 = from_lane_(own, 0, BW);
+    g23 = from_lane_(own, BW / 2, BW);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = from_lane_(e, k * (BW / 4), BW);
 }
 
 // Pair p's part of <c_2s c_2s+1 c_2t c_2t+1> on link (s, t), from the blocks
@@ -388,20 +485,28 @@ __device__ __forceinline__ void coupled_group(const DevConst& dc, const T* W, in
 // with conj(E) / 2 and the conjugate blocks; a diagonal pair once with E.  A
 // self-link (s = t) gives c_2s c_2s+1 c_2s c_2s+1 = -1.
 GGF_HD void four_point_term(const DevConst& dc, int p, int lane, int s, int t, cxd g01, cxd g23, const cxd (&x)[4],
-                            cxd Np, cxd& acc, cxd* q) {
-    const bool cplx = p >= dc.K, ord = lane == 1;
+                            cxd Np, cxd E, cxd& acc, cxd* q) {
+    if (lane > 1) return;
+    const bool ord = lane == 1;
     const double As = dc.Ap[(size_t)s * 4 + 1], At = dc.Ap[(size_t)t * 4 + 1];
-    const cxd E = dc.w[p] * Np;
-    int n, m;
-    pair_nm(dc.K, p, n, m);
     auto cj = [&](cxd v) { return ord ? conjg(v) : v; };
     const cxd pf = (cj(g01) + cxd{As, 0.0}) * (cj(g23) + cxd{At, 0.0}) - cj(x[0]) * cj(x[3]) + cj(x[1]) * cj(x[2]);
     const cxd v = s == t ? cxd{1.0, 0.0} : pf;
-    if (lane == 0 || (ord && cplx)) {
-        const cxd N1 = cj(Np);
-        acc -= ((cplx ? 0.5 : 1.0) * cj(E)) * v;
-        if (q) q[ord ? m * dc.K + n : n * dc.K + m] = -1.0 * (N1 * v);
+    acc -= (0.5 * cj(E)) * v;
+    if (q) {
+        int n, m;
+        pair_nm(dc.K, p, n, m);
+        q[ord ? m * dc.K + n : n * dc.K + m] = -1.0 * (cj(Np) * v);
     }
+}
+GGF_HD void four_point_term(const DevConst& dc, int p, int lane, int s, int t, double g01, double g23,
+                            const double (&x)[4], cxd Np, cxd E, cxd& acc, cxd* q) {
+    if (lane > 0) return;
+    const double As = dc.Ap[(size_t)s * 4 + 1], At = dc.Ap[(size_t)t * 4 + 1];
+    const double pf = (g01 + As) * (g23 + At) - x[0] * x[3] + x[1] * x[2];
+    const double v = s == t ? 1.0 : pf;
+    axpy(acc, -v, E);
+    if (q) q[p * dc.K + p] = -1.0 * (v * Np);
 }
 
 // ---- gauge-invariant link terms ------------------------------------------------
@@ -454,13 +559,14 @@ GGF_HD void link_term_item(const DevConst& dc, int c, int l, const void* links, 
 // (1/2) W_p[s, s]^T (the (m, n) order of a pair n < m is the conjugate term,
 // hence the real part): entry (i, j) from W_p[s B + j][s B + i].
 template <class RW, class CW, int B>
-GGF_HD double score_entry(const DevConst& dc, int c, int s, int i, int j, const RW* Wr, const CW* Wc, const cxd* np) {
+GGF_HD double score_entry(const DevConst& dc, int c, int s, int i, int j, const RW* Wr, const CW* Wc,
+                          const cxd* Es) {
     const Geometry& g = dc.g;
     const int K = dc.K;
     const size_t NN = (size_t)g.N * g.N, off = (size_t)(s * B + j) * g.N + (size_t)s * B + i;
     double acc = 0.0;
     for (int p = 0; p < dc.P; ++p) {
-        const cxd E = dc.w[p] * np[p];
+        const cxd E = Es[p];
         if (p < K) {
             acc = fma(0.5 * E.x, widen(Wr[((size_t)c * K + p) * NN + off]), acc);
         } else {

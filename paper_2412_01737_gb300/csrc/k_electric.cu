@@ -38,20 +38,33 @@
 //
 // What bounds it: latency of short dependent phases (load a block, two small
 // products, the insertion) over many independent items; 32 chains of 8 x 8
-// U(1), K = 2 took 508 us with one thread per (chain, link) and take 93
-// with a group of B lanes (ggf_obs_group.cuh).
+// U(1), K = 2 took 508 us with one thread per (chain, link) and take 88
+// with a group of B lanes (ggf_obs_group.cuh).  Where the chains fill the chip,
+// the FP64 unit, 83 % busy: 1024 chains of 8 x 8 Z2 take 98 us (95 with one
+// thread per item, 148 with the weights formed in every CTA and complex
+// products for the real pairs).
 #include "ggf_obs_group.cuh"
 
 namespace {
+
+// CTAs of an observable kernel above which the pair weights are formed once per
+// chain ahead of it: a launch of about 2 us against some hundred FP64
+// instructions per CTA.  Microseconds, in the CTAs and ahead of them: 1024 CTAs
+// 21 and 23 (128 chains of 8 x 8 Z2, electric), 19 and 19 (16 of 8 x 8 U(1),
+// K = 2, site scores); 2048 CTAs 38 and 34 (256 of 8 x 8 Z2, electric), 32 and 27
+// (32 of 8 x 8 U(1), K = 2, site scores); 65536 CTAs 305 and 46 (1024 of 8 x 8 Z2,
+// site scores).
+constexpr long long OBS_WEIGHTS_ABOVE = 1024;
 
 // A group of B = 4 H lanes per (chain, link); FIELD: the U(1) electric field
 // instead of J^2.
 template <class RW, class CW, int H, bool FIELD>
 __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_per_chain, const void* links, const RW* Wr,
-                                                      const CW* Wc, const cxd* ell, cxd* out, cxd* pair_out) {
+                                                      const CW* Wc, const cxd* ell, const cxd* ready, cxd* out,
+                                                      cxd* pair_out) {
     constexpr int B = 4 * H, NG = OT / B;
     __shared__ ElectricShared<H> shared[NG];
-    __shared__ cxd np[36];
+    __shared__ PairWeights pw;
     const Geometry& g = dc.g;
     const int c = blockIdx.x / blocks_per_chain, grp = threadIdx.x / B, lane = threadIdx.x % B;
     const int want = (blockIdx.x - c * blocks_per_chain) * NG + grp;
@@ -59,7 +72,7 @@ __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_pe
     const bool live = want < g.n_links;
     ElectricShared<H>& sh = shared[grp];
     const double gval = electric_twist<H>(g, links, c, l, lane, sh);
-    chain_weights(dc, ell + (size_t)c * dc.P, np);
+    chain_weights(dc, c, ell, ready, pw);
     const int K = dc.K;
     const size_t NN = (size_t)g.N * g.N;
     cxd num = {0.0, 0.0};
@@ -68,10 +81,19 @@ __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_pe
         const bool cplx = p >= K;
         const cxd v = cplx ? electric_pair<CW, H, FIELD>(dc, p - K, l, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, lane, gval, sh)
                            : electric_pair<RW, H, FIELD>(dc, p, l, Wr + ((size_t)c * K + p) * NN, lane, gval, sh);
-        electric_term(dc, p, lane, live, np[p], v, num, po);
+        electric_term(dc, p, lane, live, pw.np[p], pw.E[p], v, num, po);
     }
-    num = num + shfl_xor_(num, 1);
+    if (dc.Kc > 0) num = num + shfl_xor_(num, 1);
     if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = num;
+}
+
+// A group of G lanes per chain, the smallest power of two that holds the pairs
+// (an FP64 instruction costs a warp the same whatever the number of its lanes):
+// out [n][2][P].
+__global__ void __launch_bounds__(OT) obs_weights_kernel(DevConst dc, int n_chains, int G, const cxd* ell, cxd* out) {
+    const int want = (blockIdx.x * OT + threadIdx.x) / G, c = min(want, n_chains - 1);
+    cxd* o = out + (size_t)c * 2 * dc.P;
+    warp_weights(dc, ell + (size_t)c * dc.P, G, want < n_chains, o, o + dc.P);
 }
 
 // One thread per chain.
@@ -84,6 +106,19 @@ __global__ void pair_norm_kernel(DevConst dc, int n_chains, const cxd* ell, cxd*
 }  // namespace
 
 ggf_status ggf_flush(ggf_ctx* ctx, cudaStream_t st);
+
+// The chains' pair weights for an observable kernel of `blocks` CTAs, formed
+// once per chain ahead of it, or null where its CTAs form their chain's
+// themselves (OBS_WEIGHTS_ABOVE).
+const cxd* ggf_obs_weights(ggf_ctx* ctx, long long blocks, cudaStream_t st) {
+    const Chains& ch = ctx->ch;
+    if (blocks <= OBS_WEIGHTS_ABOVE) return nullptr;
+    int G = 1;
+    while (G < 32 && G < ctx->P) G *= 2;
+    obs_weights_kernel<<<(unsigned)(((long long)ch.n * G + OT - 1) / OT), OT, 0, st>>>(ctx->dc(), ch.n, G, ch.ell,
+                                                                                        ch.obs_w);
+    return ch.obs_w;
+}
 
 // N_nm(G) / N(G) of every chain into d_out [n_chains][K][K] (device).
 ggf_status ggf_pair_norm(ggf_ctx* ctx, cxd* d_out, cudaStream_t st) {
@@ -106,9 +141,10 @@ ggf_status ggf_electric(ggf_ctx* ctx, cxd* d_out, cxd* d_pairs, cudaStream_t st,
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
     const void* lk = ch.links;
+    const cxd* ready = ggf_obs_weights(ctx, blocks, st);
 #define GGF_EL2(RW, CW, H, F)                                                                                       \
     electric_kernel<RW, CW, H, F><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, lk, (const RW*)ch.Wr,             \
-                                                                   (const CW*)ch.Wc, ch.ell, d_out, d_pairs)
+                                                                   (const CW*)ch.Wc, ch.ell, ready, d_out, d_pairs)
 #define GGF_EL(RW, CW, H)                  \
     do {                                   \
         if (field) GGF_EL2(RW, CW, H, true); \

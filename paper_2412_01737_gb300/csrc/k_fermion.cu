@@ -19,8 +19,10 @@
 // link operator, u_l F_s F_t, from it).
 //
 // What bounds it: the latency of the block loads; 32 chains of 8 x 8 U(1), K = 2:
-// bilinears 155 us with one thread per item, 72 with a group of B lanes
-// (one row of the block each); the four-point function 329 and 104.
+// bilinears 155 us with one thread per item, 60 with a group of B lanes
+// (one row of the block each); the four-point function 329 and 89.  Where the
+// chains fill the chip, the FP64 unit: 1024 chains of 8 x 8 Z2 178 -> 114 and
+// 188 -> 165 us.
 #include "ggf_obs_group.cuh"
 
 namespace {
@@ -31,35 +33,30 @@ constexpr int FTHREADS = 128;
 // others links.
 template <class RW, class CW, int BW>
 __global__ void __launch_bounds__(OT) fermion_kernel(DevConst dc, int blocks_per_chain, int it0, int items, const RW* Wr,
-                                                     const CW* Wc, const cxd* ell, cxd* site_out, cxd* link_out,
+                                                     const CW* Wc, const cxd* ell, const cxd* ready, cxd* site_out, cxd* link_out,
                                                      cxd* pair_site, cxd* pair_link) {
     constexpr int NG = OT / BW;
-    __shared__ cxd np[36];
+    __shared__ PairWeights pw;
     const Geometry& g = dc.g;
     const int c = blockIdx.x / blocks_per_chain, lane = threadIdx.x % BW, K = dc.K;
     const int want = (blockIdx.x - c * blocks_per_chain) * NG + threadIdx.x / BW;
     const bool live = want < items;
     const int it = it0 + min(want, items - 1);
-    chain_weights(dc, ell + (size_t)c * dc.P, np);
-    // (lanes 0 .. 3 of the group each keep one entry)
-    const FermionLane f = fermion_lane(g, K, c, it, lane);
+    chain_weights(dc, c, ell, ready, pw);
+    const FermionLane f = fermion_lane<BW>(g, K, c, it, lane);
     cxd* out = f.is_site ? site_out : link_out;
     cxd* pout = f.is_site ? pair_site : pair_link;
     cxd* q = pout && live && f.entry ? pout + f.pair : nullptr;
     const size_t NN = (size_t)g.N * g.N;
     cxd acc = {0.0, 0.0};
     for (int p = 0; p < dc.P; ++p) {
-        cxd x;
         if (p >= K) {
-            cxd X[4];
-            coupled_group<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, f.s, f.t, lane, X);
-            x = f.a ? (f.b ? X[3] : X[2]) : (f.b ? X[1] : X[0]);
+            const cxd x = coupled_entry<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, f.s, f.t, lane);
+            fermion_term(dc, f, p, pw.np[p], pw.E[p], x, acc, q);
         } else {
-            double X[4];
-            coupled_group<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, f.s, f.t, lane, X);
-            x = {f.a ? (f.b ? X[3] : X[2]) : (f.b ? X[1] : X[0]), 0.0};
+            const double x = coupled_entry<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, f.s, f.t, lane);
+            fermion_term(dc, f, p, pw.np[p], pw.E[p], x, acc, q);
         }
-        fermion_term(dc, f, p, np[p], x, acc, q);
     }
     // -i (A + sum_p weight_p X_p); A enters with the total weight
     // sum_nm lambda_n^* lambda_m N_nm / N(G) = 1 (only where s == t)
@@ -69,15 +66,15 @@ __global__ void __launch_bounds__(OT) fermion_kernel(DevConst dc, int blocks_per
 // A group of BW lanes per (chain, link).
 template <class RW, class CW, int BW>
 __global__ void __launch_bounds__(OT) fermion4_kernel(DevConst dc, int blocks_per_chain, const RW* Wr, const CW* Wc,
-                                                      const cxd* ell, cxd* out, cxd* pair_out) {
+                                                      const cxd* ell, const cxd* ready, cxd* out, cxd* pair_out) {
     constexpr int NG = OT / BW;
-    __shared__ cxd np[36];
+    __shared__ PairWeights pw;
     const Geometry& g = dc.g;
     const int c = blockIdx.x / blocks_per_chain, lane = threadIdx.x % BW, K = dc.K;
     const int want = (blockIdx.x - c * blocks_per_chain) * NG + threadIdx.x / BW;
     const bool live = want < g.n_links;
     const int l = min(want, g.n_links - 1);
-    chain_weights(dc, ell + (size_t)c * dc.P, np);
+    chain_weights(dc, c, ell, ready, pw);
     int a0, b0;
     link_ends(g, l, a0, b0);
     const int s = a0 / g.B, t = b0 / g.B;
@@ -85,28 +82,16 @@ __global__ void __launch_bounds__(OT) fermion4_kernel(DevConst dc, int blocks_pe
     const size_t NN = (size_t)g.N * g.N;
     cxd acc = {0.0, 0.0};
     for (int p = 0; p < dc.P; ++p) {
-        const bool cplx = p >= K;
-        cxd g01, g23, x[4];
-        if (cplx) {
-            const CW* W = Wc + ((size_t)c * dc.Kc + (p - K)) * NN;
-            cxd ss[4], tt[4];
-            coupled_group<CW, BW>(dc, W, s, s, lane, ss);
-            coupled_group<CW, BW>(dc, W, t, t, lane, tt);
-            coupled_group<CW, BW>(dc, W, s, t, lane, x);
-            g01 = ss[1];
-            g23 = tt[1];
+        cxd* po = live ? q : nullptr;
+        if (p >= K) {
+            cxd g01, g23, x[4];
+            four_point_blocks<CW, BW>(dc, Wc + ((size_t)c * dc.Kc + (p - K)) * NN, s, t, lane, g01, g23, x);
+            four_point_term(dc, p, lane, s, t, g01, g23, x, pw.np[p], pw.E[p], acc, po);
         } else {
-            const RW* W = Wr + ((size_t)c * K + p) * NN;
-            double ss[4], tt[4], xr[4];
-            coupled_group<RW, BW>(dc, W, s, s, lane, ss);
-            coupled_group<RW, BW>(dc, W, t, t, lane, tt);
-            coupled_group<RW, BW>(dc, W, s, t, lane, xr);
-            g01 = {ss[1], 0.0};
-            g23 = {tt[1], 0.0};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) x[k] = {xr[k], 0.0};
+            double g01, g23, x[4];
+            four_point_blocks<RW, BW>(dc, Wr + ((size_t)c * K + p) * NN, s, t, lane, g01, g23, x);
+            four_point_term(dc, p, lane, s, t, g01, g23, x, pw.np[p], pw.E[p], acc, po);
         }
-        four_point_term(dc, p, lane, s, t, g01, g23, x, np[p], acc, live ? q : nullptr);
     }
     acc = acc + shfl_xor_(acc, 1);
     if (out && live && lane == 0) out[(size_t)c * g.n_links + l] = s == t ? cxd{-1.0, 0.0} : acc;
@@ -160,9 +145,10 @@ ggf_status ggf_fermion4(ggf_ctx* ctx, cxd* d_out, cudaStream_t st, cxd* d_pairs)
     const long long blocks = (long long)bpc * ch.n;
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
+    const cxd* ready = ggf_obs_weights(ctx, blocks, st);
 #define GGF_F4(RW, CW, BW)                                                                                  \
     fermion4_kernel<RW, CW, BW><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, (const RW*)ch.Wr,           \
-                                                                 (const CW*)ch.Wc, ch.ell, d_out, d_pairs)
+                                                                 (const CW*)ch.Wc, ch.ell, ready, d_out, d_pairs)
     if (g.B == 8) {
         if (fp64) GGF_F4(double, cxd, 8); else GGF_F4(float, cxf, 8);
     } else if (g.B == 16) {
@@ -191,9 +177,10 @@ ggf_status ggf_fermion(ggf_ctx* ctx, cxd* d_site, cxd* d_link, cxd* d_pair_site,
     const long long blocks = (long long)bpc * ch.n;
     if (blocks > 0x7fffffffLL) return ggf_fail(ctx, GGF_EINVAL, "too many chains for one launch");
     const bool fp64 = ch.opts.precision == GGF_FP64;
+    const cxd* ready = ggf_obs_weights(ctx, blocks, st);
 #define GGF_FE(RW, CW, BW)                                                                                       \
     fermion_kernel<RW, CW, BW><<<(unsigned)blocks, OT, 0, st>>>(ctx->dc(), bpc, it0, items, (const RW*)ch.Wr,     \
-                                                                (const CW*)ch.Wc, ch.ell, d_site, d_link,         \
+                                                                (const CW*)ch.Wc, ch.ell, ready, d_site, d_link,         \
                                                                 d_pair_site, d_pair_link)
     if (g.B == 8) {
         if (fp64) GGF_FE(double, cxd, 8); else GGF_FE(float, cxf, 8);
