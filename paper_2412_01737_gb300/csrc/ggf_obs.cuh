@@ -40,8 +40,8 @@ void electric_item(const DevConst& dc, int c, int l, const void* links, const RW
     const int K = dc.K;
     const size_t NN = (size_t)g.N * g.N;
     ElectricShared<H> sh;
-    double gval = 1.0;
-    for (int lane = 0; lane < 4 * H; ++lane) gval = electric_twist<H>(g, links, c, l, lane, sh);
+    const double gval = electric_link(g, links, c, l);
+    for (int mode = 0; mode < electric_modes(g); ++mode) electric_twist<H>(g, links, c, l, mode, sh);
     PairWeights pw;
     cxd num[2] = {{0.0, 0.0}, {0.0, 0.0}};
     item_weights(dc, ell + (size_t)c * dc.P, pw);

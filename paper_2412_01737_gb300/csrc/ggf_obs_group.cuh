@@ -183,18 +183,20 @@ template <int H> struct ElectricShared {
     double tw[16];
 };
 
-// The link's twist into sh.tw (SU(2): lane 0; U(1): a lane per mode); the value of a Z2 link.
+// The twists of a link's modes (U(1): one per virtual mode, SU(2): the doublet's)
+// into sh.tw, mode by mode, and the value of a Z2 link.
+GGF_HD int electric_modes(const Geometry& g) { return g.group == GGF_SU2 ? 1 : g.group == GGF_U1 ? g.n_v : 0; }
 template <int H>
-GGF_HD double electric_twist(const Geometry& g, const void* links, int c, int l, int lane, ElectricShared<H>& sh) {
+GGF_HD void electric_twist(const Geometry& g, const void* links, int c, int l, int mode, ElectricShared<H>& sh) {
     if (g.group == GGF_SU2) {
-        if (lane == 0) doublet_rotation(link_quat(g, links, c, l), sh.tw);
-    } else if (g.group == GGF_U1) {
-        const double th = ((const double*)links)[(size_t)c * g.n_links + l];
-        if (lane < g.n_v) sincos(g.q[lane] * th, &sh.tw[2 * lane + 1], &sh.tw[2 * lane]);
+        doublet_rotation(link_quat(g, links, c, l), sh.tw);
     } else {
-        return (double)((const int8_t*)links)[(size_t)c * g.n_links + l];
+        const double th = ((const double*)links)[(size_t)c * g.n_links + l];
+        sincos(g.q[mode] * th, &sh.tw[2 * mode + 1], &sh.tw[2 * mode]);
     }
-    return 1.0;
+}
+GGF_HD double electric_link(const Geometry& g, const void* links, int c, int l) {
+    return g.group == GGF_Z2 ? (double)((const int8_t*)links)[(size_t)c * g.n_links + l] : 1.0;
 }
 
 // Phase 1: the lane's entries of Gamma_tw and its row of W[site, link] (a0, b0: the link's ends).

@@ -38,11 +38,11 @@
 //
 // What bounds it: latency of short dependent phases (load a block, two small
 // products, the insertion) over many independent items; 32 chains of 8 x 8
-// U(1), K = 2 took 508 us with one thread per (chain, link) and take 88
+// U(1), K = 2 took 508 us with one thread per (chain, link) and take 85
 // with a group of B lanes (ggf_obs_group.cuh).  Where the chains fill the chip,
-// the FP64 unit, 83 % busy: 1024 chains of 8 x 8 Z2 take 98 us (95 with one
-// thread per item, 148 with the weights formed in every CTA and complex
-// products for the real pairs).
+// the FP64 unit, 83 % busy: 1024 chains of 8 x 8 Z2 take 99 us, of U(1) 129 (95
+// and 122 with one thread per item; 148 for Z2 with the weights formed in every
+// CTA and complex products for the real pairs).
 #include "ggf_obs_group.cuh"
 
 namespace {
@@ -71,7 +71,13 @@ __global__ void __launch_bounds__(OT) electric_kernel(DevConst dc, int blocks_pe
     const int l = min(want, g.n_links - 1);            // idle groups repeat the last link and write nothing
     const bool live = want < g.n_links;
     ElectricShared<H>& sh = shared[grp];
-    const double gval = electric_twist<H>(g, links, c, l, lane, sh);
+    const double gval = electric_link(g, links, c, l);
+    // the twists of all the CTA's links by the second warp, beside the weights
+    const int modes = electric_modes(g);
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + NG * modes) {
+        const int i = threadIdx.x - 32, of = i / modes;
+        electric_twist<H>(g, links, c, min(want - grp + of, g.n_links - 1), i - of * modes, shared[of]);
+    }
     chain_weights(dc, c, ell, ready, pw);
     const int K = dc.K;
     const size_t NN = (size_t)g.N * g.N;
