@@ -119,9 +119,11 @@ __device__ __forceinline__ void warp_best_pair(int n, Get get, double& best, int
     at = __shfl_sync(0xffffffffu, at, src);
 }
 
-// The pair (x, y), x < y, of list a to its first two positions; whether that is an odd permutation.
-__device__ __forceinline__ bool pair_to_front(int* a, int x, int y) {
-    const int k = a[x], p = a[y];
+// The pair (x, y), x < y, of list a, values (k, p), to its first two positions;
+// whether that is an odd permutation.
+__device__ __forceinline__ bool pair_to_front(int* a, int x, int y, int& k, int& p) {
+    k = a[x];
+    p = a[y];
     a[x] = a[0];
     a[0] = k;
     a[y] = a[1];
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(NT, NT == 64 ? 8 : (sizeof(T) == 8 ? 2 : 1))
 front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains, int npf, int pair_off,
                 const void* links, cxd* ell, int* bad, T* gws, size_t tri_elems, int in_smem) {
     extern __shared__ __align__(16) unsigned char fsm[];
-    __shared__ int s_end, s_nl;        // s_end: how the chunk ended
+    __shared__ int s_end, s_done, s_nl;        // s_end: how the chunk ended, s_done: after how many rows
     __shared__ T s_inv;
     __shared__ T s_scale[CHUNK];
     __shared__ int ord[CHUNK], es[CHUNK], cl[MAX_CLOSED];
@@ -234,7 +236,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
             }
             for (int k = tid; k < B; k += NT) idx[fa.slot[s * B + k]] = s * B + k;
             const int first = fa.eoff[s], ne = fa.eoff[s + 1] - first;
-            if constexpr (WIDE)
+            if (WIDE && ne > CHUNK)
                 for (int k = tid; k < ne; k += NT) cl[k] = fa.elim[first + k];
             __syncthreads();
             for (int k = warp; k < B; k += NW) {
@@ -254,19 +256,22 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
             bool search = false;       // the last chunk ended at a small pivot
             while (e < ne) {
                 const int c = min(CHUNK, ne - e);
-                double low = PIVOT_FLOOR;      // (warp 0) |pivot|^2 below which this chunk ends
+                // (warp 0) |pivot|^2 below which this chunk ends: its upper word, which
+                // orders as an integer and leaves the FP64 unit alone
+                int low = __double2hiint(PIVOT_FLOOR);
                 if (WIDE && search) {
                     if (warp == 0) {
                         double best;
                         int bq;
                         warp_best_pair(ne - e, [&](int x, int y) { return sget(S, F, cl[e + x], cl[e + y]); }, best, bq);
-                        low = PIVOT_FLOOR * best;
-                        if (lane == 0 && pair_to_front(cl + e, bq / 32, bq % 32)) pr = -pr;
+                        low = __double2hiint(PIVOT_FLOOR * best);
+                        int k, p;
+                        if (lane == 0 && pair_to_front(cl + e, bq / 32, bq % 32, k, p)) pr = -pr;
                     }
                     __syncthreads();
                 }
                 if (WIDE && tid == 0) s_end = 0;
-                if (tid < c) { es[tid] = WIDE ? cl[e + tid] : fa.elim[first + e + tid]; ord[tid] = tid; }
+                if (tid < c) { es[tid] = WIDE && ne > CHUNK ? cl[e + tid] : fa.elim[first + e + tid]; ord[tid] = tid; }
                 __syncthreads();
                 if (tid < c) idx[es[tid]] = -1;
                 __syncthreads();
@@ -286,25 +291,24 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     for (int w = lane; w < W; w += 32)
                         Pn[(size_t)t * F + w] = sget(S, F, es[t], w < c ? es[w] : lv[w - c]);
                 __syncthreads();
-                int te = 0;            // eliminated rows of the chunk
-                for (; te < c; te += 2) {
-                    const int t = te;
+                for (int t = 0; t < c; t += 2) {
                     if (warp == 0) {
                         // pivot: the largest entry among the chunk's remaining pairs
                         double best;
                         int bq;
                         warp_best_pair(c - t, [&](int x, int y) { return Pn[(size_t)ord[t + x] * F + ord[t + y]]; }, best, bq);
-                        if (WIDE && e + c < ne && best < low && !(search && t == 0)) {
-                            if (lane == 0) s_end = SMALL_PIVOT;  // better ones may lie outside the chunk
+                        if (WIDE && e + c < ne && __double2hiint(best) < low && !(search && t == 0)) {
+                            if (lane == 0) { s_end = SMALL_PIVOT; s_done = t; }     // better ones may lie outside the chunk
                         } else if (lane == 0) {
                             if (!(best > 1e-16) || !isfinite(best)) s_end = NO_PIVOT;   // no usable pivot: refactor densely
-                            if (pair_to_front(ord + t, bq / 32, bq % 32)) pr = -pr;
-                            const int k = ord[t], p = ord[t + 1];
+                            int k, p;
+                            const bool odd = pair_to_front(ord + t, bq / 32, bq % 32, k, p);
                             const T akp = Pn[(size_t)k * F + p];
                             const T inv = finv(akp);
                             s_inv = inv;
                             s_scale[t] = inv;
                             pr = pr * as_c(akp);
+                            if (odd) pr = -pr;
                             // keep the product in range by its own power of two
                             const int ep = ((__double2hiint(fmax(fabs(pr.x), fabs(pr.y))) >> 20) & 0x7ff) - 1023;
                             const double sc = __hiloint2double((1023 - ep) << 20, 0);
@@ -331,24 +335,30 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     __syncthreads();
                 }
                 if (s_end == NO_PIVOT) break;
-                if constexpr (WIDE) {
-                    // the rows that the chunk leaves behind, back to the front
-                    for (int i = te + warp; i < c; i += NW) {
+                int done = c;
+                if (WIDE && s_end == SMALL_PIVOT) {
+                    // the rows that the chunk leaves behind: back to the front, and zero in
+                    // the panel, so that the update below takes nothing from them
+                    done = s_done;
+                    for (int i = done + warp; i < c; i += NW) {
                         const int row = ord[i], a = es[row];
                         for (int w = i + 1 + lane; w < W; w += 32) {
                             const int col = w < c ? ord[w] : w, b = w < c ? es[col] : lv[w - c];
                             const T val = Pn[(size_t)row * F + col];
                             if (a < b) S[tri_row(a, F) + b] = val;
                             else S[tri_row(b, F) + a] = fneg(val);
+                            if (w >= c) Pn[(size_t)row * F + col] = Sc<T>::zero();
                         }
                         if (lane == 0) {
+                            s_scale[i] = Sc<T>::zero();
                             cl[e + i] = a;
                             idx[a] = 0;        // live again (which Majorana it is matters only to later sites)
                         }
                     }
+                    __syncthreads();
                 }
                 // u_t = row k_t / a_t over the live columns
-                for (int t = 2 * warp; t < (WIDE ? te : c); t += 2 * NW) {
+                for (int t = 2 * warp; t < c; t += 2 * NW) {
                     T* r = Pn + (size_t)ord[t] * F + c;
                     const T inv = s_scale[t];
                     for (int w = lane; w < nl; w += 32) r[w] = fmul(r[w], inv);
@@ -368,7 +378,7 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     const bool diag = i == j;
                     T a00 = diag ? Sc<T>::zero() : S0[c0], a01 = S0[c1];
                     T a10 = diag ? Sc<T>::zero() : S1[c0], a11 = diag ? Sc<T>::zero() : S1[c1];
-                    for (int t = 0; t < (WIDE ? te : c); t += 2) {
+                    for (int t = 0; t < c; t += 2) {
                         const T* u = Pn + (size_t)ord[t] * F + c;
                         const T* v = Pn + (size_t)ord[t + 1] * F + c;
                         const T ui0 = u[i], ui1 = u[i + 1], vi0 = v[i], vi1 = v[i + 1];
@@ -382,8 +392,8 @@ front_pf_kernel(DevConst dc, FrontArgs fa, long long n_items, const int* chains,
                     if (!diag) { S0[c0] = a00; S1[c0] = a10; S1[c1] = a11; }
                 }
                 __syncthreads();
-                search = te < c;
-                e += WIDE ? te : c;
+                search = done < c;
+                e += done;
             }
             if (s_end == NO_PIVOT) break;
         }
